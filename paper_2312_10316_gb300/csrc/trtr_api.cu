@@ -16,7 +16,7 @@ namespace trtr {
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out) {
     out[0] = out[1] = out[2] = 0ull;
     cudaError_t (*units[])(cudaStream_t, unsigned long long*) = {bounds_take_step, bounds_take_aux, bounds_take_batch,
-                                                                  bounds_take_adjoint, bounds_take_step2};
+                                                                  bounds_take_adjoint, bounds_take_step2, bounds_take_sweep};
     for (auto take : units) {
         unsigned long long u[3];
         const cudaError_t e = take(s, u);
@@ -27,6 +27,53 @@ cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out) {
         }
         out[0] += u[0];
     }
+    return cudaSuccess;
+}
+
+// Four steps a launch (trtr_sweep.cu) where the call takes enough of them: the launch that brings the
+// ghost columns up to date costs what two sweeps of a small grid save over two-step launches (200^2
+// FP32, 8 steps: 22 us either way), on a large one it is lost in the first.
+constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 1L << 18;
+
+cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
+    const bool two = most >= 2 && two_step_applies(ctx);
+    const long nodes = (long)ctx->p.nx * ctx->p.ny;
+    const bool four = two && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
+                      sweep_applies(ctx);
+    cudaError_t e = cudaSuccess;
+    if (two && !ctx->fld2_ready) {
+        *what = "field packing launch";
+        e = launch_pack_fields2(ctx);
+        if (e != cudaSuccess) return e;
+        ctx->fld2_ready = true;
+    }
+    *what = "pulse tables launch";
+    *taken = four ? 4 : (two ? 2 : 1);
+    e = ensure_pulse_levels(ctx, ctx->step, *taken);
+    if (e != cudaSuccess) return e;
+    if (four) {
+        *what = "four-step launch";
+        if (!ctx->ghost4_ready) e = launch_ghost_columns(ctx);
+        if (e == cudaSuccess) e = launch_sweep(ctx);
+    } else if (two) {
+        *what = "two-step launch";
+        if (!ctx->ghost2_ready) e = launch_refresh_ghosts2(ctx);  // after one-step launches: complete the two-wide frame
+        if (e == cudaSuccess) e = launch_step2(ctx);
+    } else {
+        *what = "step launch";
+        e = launch_step(ctx);
+    }
+    if (e != cudaSuccess) return e;
+    ctx->launches += 1;
+    if (ctx->p.bc_mode == TRTR_BC_DIRICHLET_NEE) {
+        *what = "boundary launch";
+        e = launch_dirichlet(ctx, ctx->pop[ctx->cur ^ 1]);
+        if (e != cudaSuccess) return e;
+    }
+    ctx->ghost4_ready = four;
+    ctx->ghost2_ready = two;  // the one-step kernel writes the one-wide frame
+    ctx->cur ^= 1;
+    ctx->step += *taken;
     return cudaSuccess;
 }
 }  // namespace trtr
@@ -242,7 +289,7 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         ((p->precision == TRTR_F16_OFS || p->precision == TRTR_BF16_OFS) && p->nx % 2 == 0);
     const bool two_step = two_step_storage && p->bc_mode == TRTR_BC_PERIODIC && p->src_mode != TRTR_SRC_FIELD &&
                           p->nx >= 2 && p->ny >= 2;
-    ctx->lt = trtr::make_layout(p->nx, p->ny, 4, trtr::kGhostP);
+    ctx->lt = trtr::make_layout(p->nx, p->ny, 4, trtr::kGhostT);
 
     cudaError_t e = cudaGetDevice(&ctx->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
@@ -267,6 +314,11 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         {&ctx->S, p->src_mode == TRTR_SRC_FIELD ? 2 * fld_bytes : 0, true},
         {&ctx->tab_x, 2 * (size_t)p->nx * ctx->csize, true},
         {&ctx->tab_y, 2 * (size_t)p->ny * ctx->csize, true},
+        {&ctx->ptab,
+         p->src_mode == TRTR_SRC_PULSE
+             ? trtr::PulseTab::make(p->nx, p->ny).values(trtr::kPulseLevels) * ctx->csize
+             : 0,
+         true},
         {(void**)&ctx->scratch, 2 * (size_t)ctx->red_blocks * sizeof(double), false},
         {(void**)&ctx->dres, 4 * sizeof(double), false},
         {(void**)&ctx->dflag, 4 * sizeof(int), true},  // the timeout flag, then the tile counters
@@ -297,7 +349,7 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         trtr_destroy(ctx);
         return TRTR_ENOMEM;
     }
-    if (trtr::encode_maps(ctx) != cudaSuccess || trtr::encode_maps2(ctx) != cudaSuccess) {
+    if (trtr::encode_maps(ctx) != cudaSuccess || trtr::encode_maps2(ctx) != cudaSuccess || trtr::encode_maps4(ctx) != cudaSuccess) {
         cudaGetLastError();
         trtr_destroy(ctx);
         return TRTR_ECUDA;
@@ -312,7 +364,7 @@ trtr_status trtr_destroy(trtr_ctx* ctx) {
     cudaGetLastError();
     trtr::free_adjoint(ctx);
     void* ptrs[] = {ctx->pop[0], ctx->pop[1],  ctx->uv,   ctx->Dh,    ctx->S,    ctx->tab_x,
-                    ctx->tab_y,  ctx->scratch, ctx->dres, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2};
+                    ctx->tab_y,  ctx->scratch, ctx->dres, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (ctx->hres) cudaFreeHost(ctx->hres);
@@ -433,6 +485,7 @@ trtr_status trtr_set_pulse(trtr_ctx* ctx, double omega, double xc, double yc, do
     trtr_status s = check_launch(ctx, trtr::launch_pulse_fields(ctx), "pulse fields");
     if (s != TRTR_OK) return s;
     ctx->pulse_set = true;
+    ctx->ptab_ready = false;
     ctx->fields_set = true;
     ctx->fld2_ready = false;
     return TRTR_OK;
@@ -453,6 +506,7 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
     trtr_status s = check_launch(ctx, trtr::launch_init_equilibrium(ctx, dev), "init");
     if (s != TRTR_OK) return s;
     ctx->ghost2_ready = true;  // written with the whole ghost frame
+    ctx->ghost4_ready = false;
     ctx->step = 0;
     ctx->initialized = true;
     ctx->S_prev = -1;
@@ -472,41 +526,15 @@ trtr_status trtr_step(trtr_ctx* ctx, long n) {
     const bool nee = ctx->p.bc_mode == TRTR_BC_DIRICHLET_NEE;
     if (nee && !ctx->dirichlet_set)
         return fail(ctx, TRTR_ESTATE, "bc_mode DIRICHLET_NEE needs boundary values (trtr_set_dirichlet)");
-    const bool two = trtr::two_step_applies(ctx);
     const long every = ctx->p.check_every;
     for (long k = 0; k < n;) {
-        // two steps per launch where the kernel applies, unless the step between them is one
-        // that the stability check looks at
-        if (two && n - k >= 2 && !(every > 0 && (ctx->step + 1) % every == 0)) {
-            if (!ctx->fld2_ready) {
-                cudaError_t e = trtr::launch_pack_fields2(ctx);
-                if (e != cudaSuccess) return cuda_fail(ctx, e, "field packing launch");
-                ctx->fld2_ready = true;
-            }
-            if (!ctx->ghost2_ready) {  // after one-step launches: complete the two-wide frame
-                cudaError_t e = trtr::launch_refresh_ghosts2(ctx);
-                if (e != cudaSuccess) return cuda_fail(ctx, e, "ghost refresh launch");
-            }
-            cudaError_t e = trtr::launch_step2(ctx);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "two-step launch");
-            ctx->launches += 1;
-            ctx->ghost2_ready = true;
-            ctx->cur ^= 1;
-            ctx->step += 2;
-            k += 2;
-        } else {
-            cudaError_t e = trtr::launch_step(ctx);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
-            ctx->launches += 1;
-            ctx->ghost2_ready = false;  // the one-step kernel writes the one-wide frame
-            if (nee) {
-                e = trtr::launch_dirichlet(ctx, ctx->pop[ctx->cur ^ 1]);
-                if (e != cudaSuccess) return cuda_fail(ctx, e, "boundary launch");
-            }
-            ctx->cur ^= 1;
-            ctx->step += 1;
-            k += 1;
-        }
+        // no launch passes over a step that the stability check looks at
+        const long most = every > 0 ? (every - ctx->step % every < n - k ? every - ctx->step % every : n - k) : n - k;
+        const char* what = "";
+        int taken = 0;
+        cudaError_t e = trtr::launch_steps(ctx, most, n, &taken, &what);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, what);
+        k += taken;
         if (ctx->p.src_mode == TRTR_SRC_FIELD) ctx->S_prev = ctx->S_cur;
         if (ctx->p.check_every > 0 && (ctx->step % ctx->p.check_every) == 0) {
             double r[2];
@@ -612,6 +640,7 @@ trtr_status trtr_set_populations(trtr_ctx* ctx, const double* g, int on_device, 
     if (s != TRTR_OK) return s;
     s = check_launch(ctx, trtr::launch_set_populations(ctx, dev), "set populations");
     if (s == TRTR_OK) ctx->ghost2_ready = true;
+    ctx->ghost4_ready = false;
     if (s != TRTR_OK) return s;
     ctx->step = step;
     ctx->initialized = true;
@@ -712,6 +741,7 @@ trtr_status trtr_load(trtr_ctx* ctx, const void* host_buf, size_t bytes) {
     }
     TRTR_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "load");
     ctx->step = h.step;
+    ctx->ghost4_ready = false;
     ctx->ghost2_ready = false;  // the saved frame may be the one-step kernels' one-wide one
     ctx->initialized = true;
     return TRTR_OK;

@@ -10,17 +10,6 @@
 
 namespace trtr {
 
-PulseTime pulse_at(const Pulse& p, double t) {
-    PulseTime r;
-    const double c = cos(p.omega * t), s = sin(p.omega * t);
-    r.cx = p.xc * c - p.yc * s;
-    r.cy = p.xc * s + p.yc * c;
-    const double s2 = p.sigma0 * p.sigma0 + 2.0 * p.D0 * t;
-    r.inv_s2 = 1.0 / s2;
-    r.amp = p.sigma0 * p.sigma0 / s2;
-    return r;
-}
-
 PlaneLayout make_layout(int nx, int ny, int elem_bytes, int ghost) {
     PlaneLayout L;
     L.nx = nx;

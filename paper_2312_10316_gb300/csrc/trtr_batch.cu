@@ -9,10 +9,10 @@
 // so the consumers read the arguments after their acquire-wait.  The arithmetic per node is
 // the single-grid step's (Eq. (14)); only the work distribution differs.
 //
-// Time-dependent uniforms (the pulse source at t_n and t_{n-1}, and for two-step launches at
-// t_{n+1}) live in device tables that the last CTA to finish a launch advances, together
-// with a device step clock, so two-launch CUDA graphs can be replayed with no host
-// involvement.
+// The step clock lives in device memory and is advanced by the last CTA to finish a launch; the
+// pulse tables of the next kPulseLevels time levels are filled by one launch for every instance
+// where a step needs a level outside them.  A launch finds its levels from the clock, so
+// two-launch CUDA graphs can be replayed with no host involvement.
 //
 // The autotuner (trtr_batch_tune) times every tile shape x schedule and keeps the fastest.
 #include <math.h>
@@ -36,6 +36,7 @@ struct BatchClock {
     long long n;        // step of the instances
     unsigned int done;  // CTAs of the running launch that have finished
     unsigned int next;  // next work-list entry of a dynamically scheduled launch
+    long long first;    // time level of the pulse tables' first entry
 };
 
 template <typename C>
@@ -43,23 +44,21 @@ struct alignas(64) InstanceDesc {
     CUtensorMap mp[2];    // populations, source buffer 0 / 1
     CUtensorMap mu;       // uhat_x, uhat_y
     CUtensorMap md;       // Dh
-    StepArgs<C> base[2];  // step arguments by source-buffer parity (dst differs); time part unused
-    Pulse pulse;
-    double dt;
+    StepArgs<C> base[2];  // step arguments by source-buffer parity (dst differs); pulse: the tables' first level
 };
 // Two-step launches (FP32 or 2-byte instances): the two-step kernel's maps and arguments per instance.
 struct alignas(64) InstanceDesc2 {
     CUtensorMap mp[2];        // populations, source buffer 0 / 1, the two-step tile's box
     CUtensorMap mf;           // packed fields
-    StepArgs<float> base[2];  // by source-buffer parity; time part unused
+    StepArgs<float> base[2];  // by source-buffer parity; pulse: the tables' first level
+};
+// The table fill of one instance.
+struct InstanceFill {
+    PulseFill fill;
     Pulse pulse;
     double dt;
 };
-// Pulse uniforms of a two-step launch from step n: steps n and n + 1.
-struct alignas(16) TimeFields2 {
-    TimeFields<float> t1, t2;
-};
-static_assert(sizeof(StepArgs<float>) % 16 == 0 && sizeof(TimeFields<float>) % 16 == 0, "16-byte chunks");
+static_assert(sizeof(StepArgs<float>) % 16 == 0, "16-byte chunks");
 static_assert(offsetof(InstanceDesc2, base) % 16 == 0, "16-byte aligned arguments");
 static_assert(offsetof(InstanceDesc<float>, base) % 16 == 0, "16-byte aligned arguments");
 
@@ -82,9 +81,21 @@ constexpr int kBatch2Run = TRTR_BATCH2_RUN;  // work-list entries per take of th
 // kernel mode of a schedule: 0 chunked, 1 interleaved, 2 dynamic
 constexpr int schedule_mode(int schedule) { return schedule == 0 ? 1 : (schedule == 3 ? 2 : 0); }
 
-// Pulse source uniforms of step n (t_n = n dt and t_{n-1}), in double, stored as float.
-__host__ __device__ inline TimeFields<float> time_fields(const Pulse& p, double dt, long long n) {
-    return pulse_time_fields<float>(p, dt, n);
+// Pulse tables of every instance (blockIdx.y) from time level `first` on.
+__global__ void __launch_bounds__(256) batch_pulse_tables_kernel(const InstanceFill* fills, BatchClock* clk, long long first) {
+    __shared__ PulseTime levels[kPulseLevels];
+    const InstanceFill& f = fills[blockIdx.y];
+    if (threadIdx.x < kPulseLevels) levels[threadIdx.x] = pulse_at(f.pulse, (double)(first + threadIdx.x) * f.dt);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) clk->first = first;
+    __syncthreads();
+    fill_pulse_tables<float>(f.fill, levels, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+// Level n - 1 of the pulse tables within them (the clock is advanced only after every CTA of the
+// launch has finished its tiles).
+__device__ __forceinline__ int pulse_level_at(const BatchClock* clk) {
+    const volatile BatchClock* c = clk;
+    return (int)(c->n - 1 - c->first);
 }
 
 // Asynchronous copy of `bytes` (a multiple of 16) from global to shared memory.
@@ -97,6 +108,19 @@ __device__ __forceinline__ void cp_async_16(void* sdst, const void* gsrc, int by
             : "memory");
 }
 
+// A CTA's end of a launch of `steps` steps (one thread): the last CTA to finish advances the step
+// clock and sets the work-list counter back.
+__device__ __forceinline__ void advance_clock(BatchClock* clk, int steps) {
+    __threadfence();
+    if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        clk->n += steps;
+        clk->next = 0;
+        clk->done = 0;
+        __threadfence();
+    }
+}
+
 template <int BY>
 constexpr int min_blocks() {
     return BY >= 16 ? 1 : (BY == 8 ? 2 : 4);  // keeps the register budget at 128 per thread
@@ -105,14 +129,13 @@ constexpr int min_blocks() {
 template <typename S, int SRC, int BX, int BY, int STAGES>
 __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
     batch_kernel(const InstanceDesc<typename Store<S>::C>* __restrict__ desc, const int4* __restrict__ tiles,
-                 int ntiles, TimeFields<float>* tu, TimeFields2* tu2, BatchClock* clk, int count, int parity,
-                 int mode, int sr) {
+                 int ntiles, BatchClock* clk, int parity, int mode, int sr) {
     using C = typename Store<S>::C;
     using T = Tile<S, SRC, BX, BY>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(16) StepArgs<C> sargs[STAGES];
     __shared__ int4 s_t[STAGES];  // the work-list entry loaded into each stage (x = -1: none)
-    __shared__ int s_abort, s_last, s_more;
+    __shared__ int s_abort, s_more;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                            ~static_cast<uintptr_t>(127));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * T::STAGE);
@@ -164,9 +187,7 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
             tma_load_3d(stage + T::POP, &d->mu, bar, t.y + gxf - T::AC, t.z + kGhostF - 1, 0);
         if (tma_ok(stage + T::POP + T::U, t.y + gxf, t.z + kGhostF, kFe))
             tma_load_2d(stage + T::POP + T::U, &d->md, bar, t.y + gxf, t.z + kGhostF);
-        constexpr int kStatic = (int)(sizeof(StepArgs<C>) - sizeof(TimeFields<C>));
-        cp_async_16(&sargs[s], &d->base[parity], kStatic);
-        if (SRC == TRTR_SRC_PULSE) cp_async_16(&sargs[s].tf, &tu[t.x], (int)sizeof(TimeFields<C>));
+        cp_async_16(&sargs[s], &d->base[parity], (int)sizeof(StepArgs<C>));
         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
     };
 
@@ -182,6 +203,7 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
     // stochastic rounding of the 2-byte storages: the key of this step (the clock is advanced
     // only after every CTA of the launch has finished its tiles)
     const uint32_t rkey = sr ? sr_step_key((long)*reinterpret_cast<volatile long long*>(&clk->n)) : 0u;
+    const int level = SRC == TRTR_SRC_PULSE ? pulse_level_at(clk) : 0;
     __syncthreads();  // s_t of the first stages
 
     for (int k = 0;; ++k) {
@@ -190,24 +212,13 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
         if (t.x < 0) break;
         const int i0 = t.y, j0 = t.z, j = j0 + r;
 
-        F2 sx[BX / 64 > 0 ? BX / 64 : 1], cx[BX / 64 > 0 ? BX / 64 : 1];
-        float sy = 0.f, cy = 0.f;
-        if (SRC == TRTR_SRC_PULSE) {  // per-column tables, fetched before the wait
+        F2 psrc[BX / 64 > 0 ? BX / 64 : 1];
+        if (SRC == TRTR_SRC_PULSE) {  // the pulse source of the lane's pairs, before the wait
             const StepArgs<C>& g = desc[t.x].base[0];
-            const int nx = g.lp.nx, ny = g.lp.ny;
-            const float* tx = reinterpret_cast<const float*>(g.tab_x);
+            if (j < g.lp.ny) {
 #pragma unroll
-            for (int m = 0; m < BX / 64; ++m) {
-                const int i = i0 + 64 * m + 2 * lane;
-                const float s0 = i < nx ? __ldg(tx + i) : 0.f, s1 = i + 1 < nx ? __ldg(tx + i + 1) : 0.f;
-                const float c0 = i < nx ? __ldg(tx + nx + i) : 0.f, c1 = i + 1 < nx ? __ldg(tx + nx + i + 1) : 0.f;
-                sx[m] = F2(s0, s1);
-                cx[m] = F2(c0, c1);
-            }
-            if (j < ny) {
-                const float* ty = reinterpret_cast<const float*>(g.tab_y);
-                sy = __ldg(ty + j);
-                cy = __ldg(ty + ny + j);
+                for (int m = 0; m < BX / 64; ++m)
+                    psrc[m] = pulse_source_dt(g.pulse + (size_t)level * g.pt.level, g.pt, i0 + 64 * m + 2 * lane, j);
             }
         }
 
@@ -220,12 +231,12 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
                 if (sr) {
                     args.rkey = rkey;
                     tile_row_pairs<S, SRC, BX, BY, BX / 64, false, 1, true>(smem + s * T::STAGE, r, lane, i0, j, args,
-                                                                          sx, cx, sy, cy);
+                                                                          psrc);
                 } else {
-                    tile_row_pairs<S, SRC, BX, BY>(smem + s * T::STAGE, r, lane, i0, j, args, sx, cx, sy, cy);
+                    tile_row_pairs<S, SRC, BX, BY>(smem + s * T::STAGE, r, lane, i0, j, args, psrc);
                 }
             } else {
-                tile_row_pairs<S, SRC, BX, BY>(smem + s * T::STAGE, r, lane, i0, j, args, sx, cx, sy, cy);
+                tile_row_pairs<S, SRC, BX, BY>(smem + s * T::STAGE, r, lane, i0, j, args, psrc);
             }
         }
         __syncthreads();
@@ -247,48 +258,27 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
         if constexpr (STAGES == 1) __syncthreads();  // s_t[0] is read again at once
     }
 
-    // The last CTA to finish advances the step clock and every instance's time uniforms.
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(&clk->done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        const long long n1 = clk->n + 1;
-        if (SRC == TRTR_SRC_PULSE)
-            for (int k = tid; k < count; k += blockDim.x) {
-                tu[k] = time_fields(desc[k].pulse, desc[k].dt, n1);
-                if (tu2) tu2[k] = TimeFields2{tu[k], time_fields(desc[k].pulse, desc[k].dt, n1 + 1)};
-            }
-        __syncthreads();
-        if (tid == 0) {
-            clk->n = n1;
-            clk->next = 0;
-            clk->done = 0;
-            __threadfence();
-        }
-    }
+    if (tid == 0) advance_clock(clk, 1);
 }
 
 // Two time steps per launch over the work-list of two-step tiles (FP32 or 2-byte instances):
-// per tile the producer issues the instance's two TMA boxes and copies its arguments and the
-// time uniforms of both steps into the stage's slot (the barrier's second arrival), then the
+// per tile the producer issues the instance's two TMA boxes and copies its arguments
+// into the stage's slot (the barrier's second arrival), then the
 // block runs the two-step kernel's two steps on the staged tile (SR: the 2-byte values rounded
 // stochastically with both steps' keys, from the clock).  The last CTA advances the clock by two
-// steps and both time tables.
+// steps.
 template <typename S, int SRC, class G, bool SR>
 __global__ void __launch_bounds__(G::kThreads, G::kCtas)
     batch2_kernel(const InstanceDesc2* __restrict__ desc, const int4* __restrict__ tiles, int ntiles,
-                  TimeFields<float>* tu, TimeFields2* tu2, BatchClock* clk, int count, int parity) {
+                  BatchClock* clk, int parity) {
     constexpr int STAGES = G::kStages, NT = G::kThreads;
     using T = typename G::T;
     const long long n0 = *reinterpret_cast<volatile long long*>(&clk->n);
     const uint32_t rkey1 = SR ? sr_step_key((long)n0) : 0u, rkey2 = SR ? sr_step_key((long)n0 + 1) : 0u;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(16) StepArgs<float> sargs[STAGES];
-    __shared__ __align__(16) TimeFields<float> stf2[STAGES];
-    __shared__ int s_abort, s_last;
+    __shared__ int s_abort;
+    const int level = SRC == TRTR_SRC_PULSE ? pulse_level_at(clk) : 0;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                            ~static_cast<uintptr_t>(127));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * T::Stage);
@@ -325,12 +315,7 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         uint64_t* bar = &full[s];
         mbar_expect_tx(bar, T::TX);
         step2_issue<T>(smem + s * T::Stage, bar, &d->mp[parity], &d->mf, t.y, t.z, t.w & 0xffff, t.w >> 16);
-        constexpr int kStatic = (int)(sizeof(StepArgs<float>) - sizeof(TimeFields<float>));
-        cp_async_16(&sargs[s], &d->base[parity], kStatic);
-        if (SRC == TRTR_SRC_PULSE) {
-            cp_async_16(&sargs[s].tf, &tu2[t.x].t1, (int)sizeof(TimeFields<float>));
-            cp_async_16(&stf2[s], &tu2[t.x].t2, (int)sizeof(TimeFields<float>));
-        }
+        cp_async_16(&sargs[s], &d->base[parity], (int)sizeof(StepArgs<float>));
         asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
     };
 
@@ -352,10 +337,11 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         if (!ok) s_abort = 1;
         S* sp = reinterpret_cast<S*>(smem + s * T::Stage);
         const float* sf = reinterpret_cast<const float*>(smem + s * T::Stage + T::FldOff);
-        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, t.y, t.z, sargs[s], sargs[s].tf, tid, rkey1);
+        auto tables = [&](int l) { return SRC == TRTR_SRC_PULSE ? sargs[s].pulse + (size_t)(level + l) * sargs[s].pt.level : nullptr; };
+        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, t.y, t.z, sargs[s], tables(0), tid, rkey1);
         __syncthreads();  // step 1 complete (and s_abort visible)
         if (ok && !s_abort)
-            step2_second<S, SRC, T, NT, false, SR>(sp, sf, t.y, t.z, sargs[s], stf2[s], tid, nullptr, rkey2);
+            step2_second<S, SRC, T, NT, false, SR>(sp, sf, t.y, t.z, sargs[s], tables(1), tid, nullptr, rkey2);
         __syncthreads();  // stage s and its argument slot fully read
         if (s_abort) {
             if (tid == 0) {
@@ -374,35 +360,13 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         if constexpr (STAGES == 1) __syncthreads();  // s_t[0] is read again at once
     }
 
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(&clk->done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        const long long n2 = clk->n + 2;
-        if (SRC == TRTR_SRC_PULSE)
-            for (int k = tid; k < count; k += blockDim.x) {
-                tu[k] = time_fields(desc[k].pulse, desc[k].dt, n2);
-                tu2[k] = TimeFields2{tu[k], time_fields(desc[k].pulse, desc[k].dt, n2 + 1)};
-            }
-        __syncthreads();
-        if (tid == 0) {
-            clk->n = n2;
-            clk->next = 0;
-            clk->done = 0;
-            __threadfence();
-        }
-    }
+    if (tid == 0) advance_clock(clk, 2);
 }
 
 }  // namespace
 }  // namespace trtr
 
 using trtr::BatchClock;
-using trtr::TimeFields2;
-using TimeUniforms = trtr::TimeFields<float>;
 
 struct trtr_batch {
     int count;
@@ -414,13 +378,14 @@ struct trtr_batch {
     void* d_desc;
     int4* d_tiles;
     int ntiles;
-    TimeUniforms* d_tu;  // per-instance pulse uniforms of the current step
-    // two steps per launch (FP32 instances): descriptors, work-list and time table of the
-    // two-step kernel, its graph, and whether pairs of steps use it
+    void* d_fill;     // InstanceFill of every instance (src PULSE)
+    long ptab_first;  // time level of the pulse tables' first entry
+    bool ptab_ready;
+    // two steps per launch (FP32 instances): descriptors and work-list of the two-step kernel,
+    // its graph, and whether pairs of steps use it
     void* d_desc2;
     int4* d_tiles2;
     int ntiles2;
-    TimeFields2* d_tu2;
     int grid2;
     bool two_step;
     int steps_per_launch;
@@ -437,7 +402,6 @@ struct trtr_batch {
     int parity;
     long long nodes;
     bool sr;  // 2-byte instances rounded stochastically (TRTR_ROUND_STOCHASTIC)
-    std::vector<trtr::Pulse> pulses;
 };
 
 namespace trtr {
@@ -471,8 +435,7 @@ struct BatchLaunch {
     static cudaError_t launch(trtr_batch* b, int parity, int mode) {
         auto kernel = batch_kernel<S, SRC, BX, BY, kStages>;
         kernel<<<b->grid, 32 * BY, smem(), b->stream>>>(static_cast<const InstanceDesc<C>*>(b->d_desc), b->d_tiles,
-                                                         b->ntiles, b->d_tu, b->d_tu2, b->d_clk, b->count, parity,
-                                                         mode, b->sr ? 1 : 0);
+                                                         b->ntiles, b->d_clk, parity, mode, b->sr ? 1 : 0);
         return cudaGetLastError();
     }
     static bool encode_desc(trtr_batch* b, InstanceDesc<C>* h) {
@@ -487,8 +450,8 @@ struct BatchLaunch {
             if (!ok) return false;
             StepArgs<C>& a = d.base[0];
             memset(static_cast<void*>(&a), 0, sizeof(a));
-            a.tab_x = static_cast<const C*>(c->tab_x);
-            a.tab_y = static_cast<const C*>(c->tab_y);
+            a.pt = PulseTab::make(c->p.nx, c->p.ny);
+            a.pulse = c->ptab ? static_cast<const C*>(c->ptab) + kTabGhost : nullptr;
             a.flag = b->d_flag;
             a.lp = c->lp;
             a.lf = c->lf;
@@ -496,16 +459,9 @@ struct BatchLaunch {
             a.magic = C(c->p.magic);
             a.omega2_fixed = C(c->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / c->p.tau2 : 0.0);
             a.phi_ref = C(c->p.phi_ref);
-            a.x0 = C(c->p.x0);
-            a.y0 = C(c->p.y0);
-            a.dx = C(c->p.dx);
-            a.dt = C(c->p.dt);
-            a.dD_amp = C(c->pulse.D0 * c->pulse.D_amp);
             d.base[1] = a;
             d.base[0].dst = c->pop[1];  // source buffer 0 -> write buffer 1
             d.base[1].dst = c->pop[0];
-            d.pulse = c->pulse;
-            d.dt = c->p.dt;
         }
         return true;
     }
@@ -599,8 +555,7 @@ struct Batch2Launch {
     }
     static cudaError_t launch(trtr_batch* b, int parity) {
         batch2_kernel<S, SRC, G, SR><<<b->grid2, G::kThreads, smem(), b->stream>>>(
-            static_cast<const InstanceDesc2*>(b->d_desc2), b->d_tiles2, b->ntiles2, b->d_tu, b->d_tu2, b->d_clk,
-            b->count, parity);
+            static_cast<const InstanceDesc2*>(b->d_desc2), b->d_tiles2, b->ntiles2, b->d_clk, parity);
         return cudaGetLastError();
     }
     static bool encode_desc(trtr_batch* b, InstanceDesc2* h) {
@@ -614,8 +569,8 @@ struct Batch2Launch {
             if (!ok) return false;
             StepArgs<float>& a = d.base[0];
             memset(static_cast<void*>(&a), 0, sizeof(a));
-            a.tab_x = static_cast<const float*>(c->tab_x);
-            a.tab_y = static_cast<const float*>(c->tab_y);
+            a.pt = PulseTab::make(c->p.nx, c->p.ny);
+            a.pulse = c->ptab ? static_cast<const float*>(c->ptab) + kTabGhost : nullptr;
             a.flag = b->d_flag;
             a.lp = c->lp;
             a.lf = c->lt;
@@ -623,16 +578,9 @@ struct Batch2Launch {
             a.magic = (float)c->p.magic;
             a.omega2_fixed = (float)(c->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / c->p.tau2 : 0.0);
             a.phi_ref = (float)c->p.phi_ref;
-            a.x0 = (float)c->p.x0;
-            a.y0 = (float)c->p.y0;
-            a.dx = (float)c->p.dx;
-            a.dt = (float)c->p.dt;
-            a.dD_amp = (float)(c->pulse.D0 * c->pulse.D_amp);
             d.base[1] = a;
             d.base[0].dst = c->pop[1];
             d.base[1].dst = c->pop[0];
-            d.pulse = c->pulse;
-            d.dt = c->p.dt;
         }
         return true;
     }
@@ -756,22 +704,12 @@ trtr_status build_graph(trtr_batch* b) {
 }
 
 trtr_status reset_clock(trtr_batch* b) {
-    std::vector<TimeUniforms> u(b->count);
-    std::vector<TimeFields2> u2(b->count);
-    for (int k = 0; k < b->count; ++k) {
-        u[k] = time_fields(b->pulses[k], b->ctx[k]->p.dt, b->step);
-        u2[k] = TimeFields2{u[k], time_fields(b->pulses[k], b->ctx[k]->p.dt, b->step + 1)};
-    }
-    if (b->d_tu2 && cudaMemcpyAsync(b->d_tu2, u2.data(), u2.size() * sizeof(TimeFields2), cudaMemcpyHostToDevice,
-                                    b->stream) != cudaSuccess)
-        return TRTR_ECUDA;
-    BatchClock c;
+    BatchClock c = {};
+    b->ptab_ready = false;
     c.n = b->step;
     c.done = 0;
     c.next = 0;
-    if (cudaMemcpyAsync(b->d_tu, u.data(), u.size() * sizeof(TimeUniforms), cudaMemcpyHostToDevice, b->stream) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(b->d_clk, &c, sizeof(c), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
+    if (cudaMemcpyAsync(b->d_clk, &c, sizeof(c), cudaMemcpyHostToDevice, b->stream) != cudaSuccess ||
         cudaStreamSynchronize(b->stream) != cudaSuccess)
         return TRTR_ECUDA;
     return TRTR_OK;
@@ -796,15 +734,56 @@ trtr_status build_graph2(trtr_batch* b) {
     return TRTR_OK;
 }
 
+// The pulse tables of the levels step - 1 .. step + steps - 1 in every instance.
+cudaError_t ensure_levels(trtr_batch* b, long step, int steps) {
+    if (b->src != TRTR_SRC_PULSE) return cudaSuccess;
+    if (b->ptab_ready && step - 1 >= b->ptab_first && step + steps <= b->ptab_first + kPulseLevels) return cudaSuccess;
+    for (int k = 0; k < b->count; k += 65535) {
+        const int n = b->count - k < 65535 ? b->count - k : 65535;
+        batch_pulse_tables_kernel<<<dim3(32, n), 256, 0, b->stream>>>(static_cast<const InstanceFill*>(b->d_fill) + k,
+                                                                      b->d_clk, step - 1);
+    }
+    b->ptab_first = step - 1;
+    b->ptab_ready = cudaPeekAtLastError() == cudaSuccess;
+    return cudaGetLastError();
+}
+
+// Instances without tables of their own (src NONE beside PULSE instances) get them; the fills go to
+// the device.
+trtr_status setup_fills(trtr_batch* b) {
+    std::vector<InstanceFill> h(b->count);
+    for (int k = 0; k < b->count; ++k) {
+        trtr_ctx* c = b->ctx[k];
+        if (!c->ptab) {
+            const size_t bytes = PulseTab::make(c->p.nx, c->p.ny).values(kPulseLevels) * sizeof(float);
+            if (cudaMalloc(&c->ptab, bytes) != cudaSuccess || cudaMemsetAsync(c->ptab, 0, bytes, b->stream) != cudaSuccess) {
+                cudaGetLastError();
+                return TRTR_ENOMEM;
+            }
+        }
+        h[k] = InstanceFill{pulse_fill_of(c), c->pulse, c->p.dt};
+    }
+    if (cudaMalloc(&b->d_fill, sizeof(InstanceFill) * b->count) != cudaSuccess) {
+        cudaGetLastError();
+        return TRTR_ENOMEM;
+    }
+    if (cudaMemcpyAsync(b->d_fill, h.data(), sizeof(InstanceFill) * b->count, cudaMemcpyHostToDevice, b->stream) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(b->stream) != cudaSuccess)
+        return TRTR_ECUDA;
+    return TRTR_OK;
+}
+
 // n steps: pairs through the two-step kernel where it applies (steps_per_launch 2), the rest
 // (an odd step, or all with steps_per_launch 1) through the one-step kernel of the configured
-// geometry.  Both kernels advance the device clock and both time tables, so they interleave.
+// geometry.  Both kernels advance the device clock, so they interleave.
 trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
     for (int k = 0; k < b->count; ++k)
         if (b->ctx[k]->step != b->step || b->ctx[k]->cur != b->parity) return TRTR_ESTATE;
     long left = n;
     int par = b->parity;
     bool last_two = false;
+    auto levels = [&](int steps) { return ensure_levels(b, b->step + (n - left), steps) == cudaSuccess; };
     if (b->two_step && steps_per_launch == 2 && left >= 2) {
         for (int k = 0; k < b->count; ++k) {
             trtr_ctx* c = b->ctx[k];  // instances share the batch's stream
@@ -814,28 +793,27 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
             }
             if (!c->ghost2_ready && launch_refresh_ghosts2(c) != cudaSuccess) return TRTR_ECUDA;
         }
-        long pairs = left / 2;
-        left -= 2 * pairs;
         if (par == 1) {
-            if (launch_two(b, 1) != cudaSuccess) return TRTR_ECUDA;
+            if (!levels(2) || launch_two(b, 1) != cudaSuccess) return TRTR_ECUDA;
             par = 0;
-            --pairs;
+            left -= 2;
         }
-        if (pairs >= 2) {
+        if (left >= 4) {
             trtr_status s = build_graph2(b);
             if (s != TRTR_OK) return s;
-            for (; pairs >= 2; pairs -= 2)
-                if (cudaGraphLaunch(b->graph2, b->stream) != cudaSuccess) return TRTR_ECUDA;
+            for (; left >= 4; left -= 4)
+                if (!levels(4) || cudaGraphLaunch(b->graph2, b->stream) != cudaSuccess) return TRTR_ECUDA;
         }
-        if (pairs == 1) {
-            if (launch_two(b, 0) != cudaSuccess) return TRTR_ECUDA;
+        if (left >= 2) {
+            if (!levels(2) || launch_two(b, 0) != cudaSuccess) return TRTR_ECUDA;
             par = 1;
+            left -= 2;
         }
         last_two = true;
     }
     if (left > 0) last_two = false;  // one-step launches follow: the one-wide ghost frame
     if (left > 0 && par == 1) {  // bring the ping-pong to parity 0 for the graph
-        if (launch_one(b, 1) != cudaSuccess) return TRTR_ECUDA;
+        if (!levels(1) || launch_one(b, 1) != cudaSuccess) return TRTR_ECUDA;
         par = 0;
         --left;
     }
@@ -843,10 +821,10 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
         trtr_status s = build_graph(b);
         if (s != TRTR_OK) return s;
         for (; left >= 2; left -= 2)
-            if (cudaGraphLaunch(b->graph, b->stream) != cudaSuccess) return TRTR_ECUDA;
+            if (!levels(2) || cudaGraphLaunch(b->graph, b->stream) != cudaSuccess) return TRTR_ECUDA;
     }
     if (left == 1) {
-        if (launch_one(b, 0) != cudaSuccess) return TRTR_ECUDA;
+        if (!levels(1) || launch_one(b, 0) != cudaSuccess) return TRTR_ECUDA;
         par = 1;
     }
     b->step += n;
@@ -855,6 +833,7 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
         b->ctx[k]->step = b->step;
         b->ctx[k]->cur = b->parity;
         if (n > 0) b->ctx[k]->ghost2_ready = last_two;
+        if (n > 0) b->ctx[k]->ghost4_ready = false;
         b->ctx[k]->launches += n;
     }
     return TRTR_OK;
@@ -912,26 +891,24 @@ trtr_status trtr_batch_create(const trtr_instance* inst, int count, void* cuda_s
         if (s == TRTR_OK) s = trtr_init_equilibrium(b->ctx[k], nullptr, 0);
         if (s == TRTR_OK) {
             b->nodes += (long long)in.p.nx * in.p.ny;
-            b->pulses.push_back(b->ctx[k]->pulse);
         }
     }
     if (s == TRTR_OK &&
         (cudaMalloc(&b->d_desc, trtr::desc_size(prec) * count) != cudaSuccess ||
-         cudaMalloc(&b->d_tu, sizeof(TimeUniforms) * count) != cudaSuccess ||
          cudaMalloc(&b->d_clk, sizeof(BatchClock)) != cudaSuccess || cudaMalloc(&b->d_flag, sizeof(int)) != cudaSuccess ||
          cudaMallocHost(&b->h_flag, sizeof(int)) != cudaSuccess ||
          cudaMemsetAsync(b->d_flag, 0, sizeof(int), b->stream) != cudaSuccess)) {
         cudaGetLastError();
         s = TRTR_ENOMEM;
     }
+    if (s == TRTR_OK && src == TRTR_SRC_PULSE) s = trtr::setup_fills(b);  // before the descriptors (table pointers)
     if (s == TRTR_OK) s = trtr::apply_config(b, b->config);
     // two steps per launch where every instance has the two-step kernel's packed fields
     b->steps_per_launch = 2;
     b->two_step = s == TRTR_OK;  // where every instance has the two-step fields (FP32, or 2-byte with even nx)
     for (int k = 0; k < count && b->two_step; ++k) b->two_step = b->ctx[k]->fld2 != nullptr;
     if (s == TRTR_OK && b->two_step &&
-        (cudaMalloc(&b->d_desc2, sizeof(trtr::InstanceDesc2) * count) != cudaSuccess ||
-         cudaMalloc(&b->d_tu2, sizeof(TimeFields2) * count) != cudaSuccess)) {
+        cudaMalloc(&b->d_desc2, sizeof(trtr::InstanceDesc2) * count) != cudaSuccess) {
         cudaGetLastError();
         s = TRTR_ENOMEM;
     }
@@ -952,7 +929,7 @@ trtr_status trtr_batch_destroy(trtr_batch* b) {
     if (b->graph2_valid) cudaGraphExecDestroy(b->graph2);
     for (int k = 0; k < b->count; ++k)
         if (b->ctx && b->ctx[k]) trtr_destroy(b->ctx[k]);
-    void* ptrs[] = {b->d_desc, b->d_tiles, b->d_tu, b->d_clk, b->d_flag, b->d_desc2, b->d_tiles2, b->d_tu2};
+    void* ptrs[] = {b->d_desc, b->d_tiles, b->d_fill, b->d_clk, b->d_flag, b->d_desc2, b->d_tiles2};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (b->h_flag) cudaFreeHost(b->h_flag);
@@ -1098,6 +1075,7 @@ trtr_status trtr_batch_tune(trtr_batch* b, int trial_steps, int* config_out, flo
             }
             c->cur = cur0[k];
             c->ghost2_ready = ghost0[k] != 0;
+            c->ghost4_ready = false;
             c->step = 0;
         }
         if (s == TRTR_OK && cudaStreamSynchronize(b->stream) != cudaSuccess) {

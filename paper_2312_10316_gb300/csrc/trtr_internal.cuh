@@ -108,6 +108,7 @@ cudaError_t bounds_take_aux(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_batch(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_adjoint(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_step2(cudaStream_t s, unsigned long long* out);
+cudaError_t bounds_take_sweep(cudaStream_t s, unsigned long long* out);
 // All units: the summed count, and the kind and place of the first unit's first access.
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out);
 
@@ -115,6 +116,7 @@ cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out);
 // two-step kernel pulls twice across an edge); the field planes of the one-step kernel one.
 constexpr int kGhostP = 2;
 constexpr int kGhostF = 1;
+constexpr int kGhostT = 4;  // the packed fields of the two- and four-step kernels
 
 struct PlaneLayout {
     int nx, ny;
@@ -177,40 +179,32 @@ struct Store<__nv_bfloat16> {
     static __device__ __forceinline__ __nv_bfloat16 encode(float v, float off) { return __float2bfloat16_rn(v - off); }
 };
 
-// Time-dependent uniforms of the pulse source (centre, 1/s^2, amplitude term at t_n and
-// t_{n-1}); pulse_time_fields fills them.
-template <typename C>
-struct alignas(16) TimeFields {
-    C cx_n, cy_n, inv_s2_n, a_n;     // at t_n
-    C cx_p, cy_p, inv_s2_p, a_p;     // at t_{n-1} (t = -dt at the first step: the closed form)
-};
-
-// The uniforms of step n (t_n = n dt, t_{n-1} = t_n - dt), computed in double.  The amplitude
-// term: FP64 kernels a = s0^2 / s^2; FP32-computing kernels a_n = log2(1.5 dt s0^2 / s_n^4) and
-// a_p = log2(0.5 dt s0^2 / s_p^4), the step's weights of S^n and S^{n-1} in
-// dt S^n + dt/2 (S^n - S^{n-1}) and the 1/s^2 of S folded into the exponent (pulse_source_dt).
-template <typename C>
-__host__ __device__ inline TimeFields<C> pulse_time_fields(const Pulse& p, double dt, long long n) {
-    TimeFields<C> u;
-    const double tn = (double)n * dt, tp = (double)(n - 1) * dt;
-    const double cn = cos(p.omega * tn), sn = sin(p.omega * tn);
-    const double cp = cos(p.omega * tp), sp = sin(p.omega * tp);
-    const double s2n = p.sigma0 * p.sigma0 + 2.0 * p.D0 * tn, s2p = p.sigma0 * p.sigma0 + 2.0 * p.D0 * tp;
-    u.cx_n = (C)(p.xc * cn - p.yc * sn);
-    u.cy_n = (C)(p.xc * sn + p.yc * cn);
-    u.inv_s2_n = (C)(1.0 / s2n);
-    u.cx_p = (C)(p.xc * cp - p.yc * sp);
-    u.cy_p = (C)(p.xc * sp + p.yc * cp);
-    u.inv_s2_p = (C)(1.0 / s2p);
-    if (sizeof(C) == 8) {
-        u.a_n = (C)(p.sigma0 * p.sigma0 / s2n);
-        u.a_p = (C)(p.sigma0 * p.sigma0 / s2p);
-    } else {
-        u.a_n = (C)log2(1.5 * dt * p.sigma0 * p.sigma0 / (s2n * s2n));
-        u.a_p = (C)log2(0.5 * dt * p.sigma0 * p.sigma0 / (s2p * s2p));
+// Tables of the pulse source (TRTR_SRC_PULSE).  With r = x - c(t) the manufactured source is a sum
+// of two products of a function of x and a function of y,
+//   dt S(x, y, t) = P1(x) Q1(y) + P2(x) Q2(y),
+//   P2 = E(r_x) sin(pi x),  P1 = E(r_x) [pi cos(pi x) r_x + sin(pi x) (1 - r_x^2 / s^2)],
+//   Q1 = A E(r_y) sin(pi y),  Q2 = A E(r_y) [pi cos(pi y) r_y + sin(pi y) (1 - r_y^2 / s^2)],
+//   E(r) = exp(-r^2 / (2 s^2)),  A = dt D0 D_amp s0^2 / s^4,
+// so a node's source costs four loads and two multiply-adds a time level instead of an exponential
+// and a dozen operations; the tables of kPulseLevels time levels are filled by one small launch
+// (nx + ny entries a level) when trtr_step leaves the levels they hold.  One level is
+// [P1 over x][P2 over x][(Q1, Q2) over y], each with kTabGhost periodic images before and after
+// the interior (halo nodes read their image's value without wrapping an index) and kTabPad unused
+// entries behind them (ragged tiles).
+constexpr int kPulseLevels = 64;
+constexpr int kTabGhost = 8, kTabPad = 144;
+struct PulseTab {
+    int p2, y, level;  // offsets: P2 from P1, the y part from P1 (both at coordinate 0); stride of a level
+    __host__ __device__ static PulseTab make(int nx, int ny) {
+        const int wx = (kTabGhost + nx + kTabPad + 3) / 4 * 4, wy = (kTabGhost + ny + kTabPad + 3) / 4 * 4;
+        PulseTab t;
+        t.p2 = wx;
+        t.y = 2 * wx + kTabGhost;  // kTabGhost values to P1's coordinate 0, 2 kTabGhost to (Q1, Q2)'s
+        t.level = 2 * wx + 2 * wy;
+        return t;
     }
-    return u;
-}
+    size_t values(int levels) const { return (size_t)level * levels; }
+};
 
 // Tile schedule bits of a step launch.  kSchedDynamic: the CTAs take their tiles from tile_ctr
 // (long launches; kDynMinTilesPerCta).  kSchedReverse: the launch walks the tile order from the
@@ -218,14 +212,13 @@ __host__ __device__ inline TimeFields<C> pulse_time_fields(const Pulse& p, doubl
 // starts on the tiles that the launch before it wrote last, whose lines are still in L2.
 constexpr int kSchedDynamic = 1, kSchedReverse = 2;
 
-// Uniform arguments of the fused step kernel (one launch per time step).  The static part
-// precedes tf and is a whole number of 16-byte chunks, so the batched kernel can copy the
-// two parts into shared memory with asynchronous 16-byte copies.
+// Uniform arguments of the fused step kernel (one launch per time step), a whole number of
+// 16-byte chunks, so the batched kernel can copy them into shared memory with asynchronous
+// 16-byte copies.
 template <typename C>
 struct alignas(16) StepArgs {
     void* dst;              // P written by this step (plain stores, with ghosts)
-    const C* tab_x;         // [2][nx]: sin(pi x_i), cos(pi x_i)
-    const C* tab_y;         // [2][ny]: sin(pi y_j), cos(pi y_j)
+    const C* pulse;         // pulse tables (TRTR_SRC_PULSE): coordinate 0 of level n - 1 (level n follows)
     int* flag;              // set when a bounded wait gives up
     unsigned* tile_ctr;     // [next tile, CTAs done] of kernels that hand out tiles dynamically (zero between launches)
     PlaneLayout lp;         // populations
@@ -235,12 +228,9 @@ struct alignas(16) StepArgs {
     C magic;                // Lambda
     C omega2_fixed;         // 1 / tau2 (TRTR_TAU2_FIXED)
     C phi_ref;
-    // pulse source (TRTR_SRC_PULSE), physical units
-    C x0, y0, dx, dt;
-    C dD_amp;               // D0 * D_amp
+    PulseTab pt;            // layout of the pulse tables
     uint32_t rkey;          // stochastic rounding of the 2-byte storages: the step's key (sr_step_key)
     int sched;              // kSchedDynamic | kSchedReverse (below)
-    TimeFields<C> tf;       // pulse source uniforms of this step (a separate 16-byte block)
 };
 
 // Random bits of the stochastic rounding (TRTR_ROUND_STOCHASTIC): Wellons' "lowbias32"
@@ -273,6 +263,14 @@ constexpr long kDynMinTilesPerCta = 8;
 
 enum MapId { kMapPop0 = 0, kMapPop1 = 1, kMapU = 2, kMapD = 3, kMapS = 4, kNumMaps = 5 };
 
+// What the table fill needs of a context or of a batch's instance.
+struct PulseFill {
+    void* tab;                       // [kPulseLevels][level]
+    const void *tab_x, *tab_y;       // sin and cos of pi x, pi y in the compute type
+    double x0, y0, dx, amp;          // amp: dt D0 D_amp
+    int nx, ny;
+};
+
 }  // namespace trtr
 
 struct trtr_adjoint_state;  // checkpoints and adjoint buffers (trtr_adjoint.cu)
@@ -296,6 +294,9 @@ struct trtr_ctx {
     int S_prev;       // buffer holding S^{n-1} (-1: use S^n)
     void* tab_x;
     void* tab_y;
+    void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
+    long ptab_first;  // time level of its first entry
+    bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
     double* dres;     // device result of the reductions (4 doubles)
@@ -308,9 +309,11 @@ struct trtr_ctx {
     bool small_tiles;  // step kernel geometry for small grids (chosen by encode_maps)
     // two-step kernel (FP32 storage, periodic boundaries, no source or the pulse source)
     CUtensorMap maps2[3];   // populations (buffers 0, 1) and packed fields, its tile boxes
+    CUtensorMap maps4[5];   // four-step kernel: population rows (buffers 0, 1), interior stores (0, 1), field rows
     void* fld2;             // [5][rows][pitch] float: uhat_x, uhat_y, a_x, a_y, Dh, two-wide periodic ghosts
     trtr::PlaneLayout lt;   // layout of fld2
     bool fld2_ready;        // fld2 holds the current fields
+    bool ghost4_ready;      // its four-wide ghost columns are up to date (interior rows)
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
     int steps_per_launch;   // 2: trtr_step uses the two-step kernel where it applies; 1: never
     trtr::Pulse pulse;
@@ -334,7 +337,7 @@ cudaError_t encode_pop_map(trtr_ctx* ctx, void* buffer, CUtensorMap* out);
 // fields (after each change of u or D), and one launch advancing the state by two steps.
 bool two_step_applies(const trtr_ctx* ctx);
 cudaError_t encode_maps2(trtr_ctx* ctx);
-cudaError_t launch_pack_fields2(trtr_ctx* ctx);
+cudaError_t launch_pack_fields2(trtr_ctx* ctx);  // (and the pulse tables from the current step on)
 cudaError_t launch_step2(trtr_ctx* ctx);
 // the distance-2 ghost cells of the current population buffer (or of buffer P) from its
 // interior (periodic)
@@ -344,6 +347,16 @@ cudaError_t launch_refresh_ghosts2_buffer(trtr_ctx* ctx, void* P);
 // dst, as steps `step` and `step + 1`; dst1 (or null) receives the intermediate state
 cudaError_t encode_pop_map2(trtr_ctx* ctx, void* buffer, CUtensorMap* out);
 cudaError_t launch_step2_from(trtr_ctx* ctx, const CUtensorMap* src_map, void* dst, void* dst1, long step);
+// The four-step kernel (trtr_sweep.cu): whether it applies to the context, its maps (at creation),
+// one launch advancing the state by four steps, and the ghost columns that it reads.
+bool sweep_applies(const trtr_ctx* ctx);
+cudaError_t encode_maps4(trtr_ctx* ctx);
+cudaError_t launch_sweep(trtr_ctx* ctx);
+cudaError_t launch_ghost_columns(trtr_ctx* ctx);
+// The next launch of a run that may advance `most` (>= 1) steps, of a call that takes `call` in all:
+// four, two or one steps, with what the launch needs; advances the context's state.  *taken: the
+// steps; *what: names the failing launch on an error.
+cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what);
 // one block whose bounded wait on a barrier that nothing completes gives up after `cycles`
 cudaError_t launch_wait_timeout(trtr_ctx* ctx, long long cycles);
 // one thread that gives the bounds checks four bad arguments and accesses nothing with them
@@ -351,6 +364,9 @@ cudaError_t launch_bounds_probe(trtr_ctx* ctx);
 void free_adjoint(trtr_ctx* ctx);
 cudaError_t launch_convert_fields(trtr_ctx* ctx, const double* ux, const double* uy, const double* D);
 cudaError_t launch_pulse_fields(trtr_ctx* ctx);
+// Pulse tables: makes sure that they hold the time levels step - 1 .. step + steps - 1 (a launch
+// where they do not), and the pointer that a launch from step `step` reads.
+cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps);
 cudaError_t launch_convert_source(trtr_ctx* ctx, const double* S, int buffer);
 cudaError_t launch_init_equilibrium(trtr_ctx* ctx, const double* phi0 /* device or NULL = pulse */);
 cudaError_t launch_moments(trtr_ctx* ctx, double* phi_out_dev);
@@ -367,7 +383,16 @@ cudaError_t launch_dirichlet(trtr_ctx* ctx, void* P);
 // finite and positive (the check of a device-resident D).
 enum ReduceKind { kReduceMass = 0, kReducePulse = 1, kReduceField = 2, kReduceNonFinite = 3, kReduceBadField = 4 };
 
-PulseTime pulse_at(const Pulse& p, double t);
+__host__ __device__ inline PulseTime pulse_at(const Pulse& p, double t) {
+    PulseTime r;
+    const double c = cos(p.omega * t), s = sin(p.omega * t);
+    r.cx = p.xc * c - p.yc * s;
+    r.cy = p.xc * s + p.yc * c;
+    const double s2 = p.sigma0 * p.sigma0 + 2.0 * p.D0 * t;
+    r.inv_s2 = 1.0 / s2;
+    r.amp = p.sigma0 * p.sigma0 / s2;
+    return r;
+}
 
 // Edge nodes of an nx x ny grid (nx, ny >= 3), k in [0, 2 nx + 2 (ny - 2)): the bottom row,
 // the top row, then the left and right columns without their corners.

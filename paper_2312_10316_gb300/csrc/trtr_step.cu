@@ -247,24 +247,12 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
         const int i0 = tile_x0(t), j0 = tile_y0(t);
         const int j = j0 + r;
 
-        // per-column / per-row pulse tables, loaded before the wait so their latency hides
-        F2 sx[kPairsPerLane], cx[kPairsPerLane];
-        float sy = 0.f, cy = 0.f;
-        if (kPairs && SRC == TRTR_SRC_PULSE) {
+        // the pulse source of this lane's pairs, from its tables before the wait (hides their latency)
+        F2 psrc[kPairsPerLane];
+        if (kPairs && SRC == TRTR_SRC_PULSE && j < ny) {
 #pragma unroll
-            for (int m = 0; m < kPairsPerLane; ++m) {
-                const int i = i0 + c0 + 64 * m + 2 * lane;
-                const float* tx = reinterpret_cast<const float*>(a.tab_x);
-                const float s0 = i < nx ? __ldg(tx + i) : 0.f, s1 = i + 1 < nx ? __ldg(tx + i + 1) : 0.f;
-                const float c0 = i < nx ? __ldg(tx + nx + i) : 0.f, c1 = i + 1 < nx ? __ldg(tx + nx + i + 1) : 0.f;
-                sx[m] = F2(s0, s1);
-                cx[m] = F2(c0, c1);
-            }
-            if (j < ny) {
-                const float* ty = reinterpret_cast<const float*>(a.tab_y);
-                sy = __ldg(ty + j);
-                cy = __ldg(ty + ny + j);
-            }
+            for (int m = 0; m < kPairsPerLane; ++m)
+                psrc[m] = pulse_source_dt(reinterpret_cast<const float*>(a.pulse), a.pt, i0 + c0 + 64 * m + 2 * lane, j);
         }
 
         const bool ok = mbar_wait_bounded(&full[s], (k / STAGES) & 1);
@@ -272,8 +260,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
         if (ok && j < ny) {
             const unsigned char* st = smem + s * T::STAGE;
             if constexpr (kPairs)
-                tile_row_pairs<S, SRC, kBX, kBY, kPairsPerLane, kTST, G::UNR, SR>(st, r, lane, i0, j, a, sx, cx, sy,
-                                                                                  cy, c0);
+                tile_row_pairs<S, SRC, kBX, kBY, kPairsPerLane, kTST, G::UNR, SR>(st, r, lane, i0, j, a, psrc, c0);
             else
                 tile_row_f64<SRC, kBX, kBY, 2 * kPairsPerLane, kTST>(st, r, lane, i0, j, a, c0);
         }
@@ -379,8 +366,8 @@ cudaError_t launch_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, l
     }
     StepArgs<C> a;
     a.dst = dst;
-    a.tab_x = static_cast<const C*>(ctx->tab_x);
-    a.tab_y = static_cast<const C*>(ctx->tab_y);
+    a.pt = PulseTab::make(ctx->p.nx, ctx->p.ny);
+    a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<C>(ctx, a.pt, step) : nullptr;
     a.flag = ctx->dflag;
     a.tile_ctr = reinterpret_cast<unsigned*>(ctx->dflag + 2);
     a.lp = ctx->lp;
@@ -391,19 +378,7 @@ cudaError_t launch_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, l
     a.magic = C(ctx->p.magic);
     a.omega2_fixed = C(ctx->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / ctx->p.tau2 : 0.0);
     a.phi_ref = C(ctx->p.phi_ref);
-    a.x0 = C(ctx->p.x0);
-    a.y0 = C(ctx->p.y0);
-    a.dx = C(ctx->p.dx);
-    a.dt = C(ctx->p.dt);
     a.rkey = sr_step_key(step);
-    if (SRC == TRTR_SRC_PULSE) {
-        a.dD_amp = C(ctx->pulse.D0 * ctx->pulse.D_amp);
-        a.tf = pulse_time_fields<C>(ctx->pulse, ctx->p.dt, step);
-    } else {
-        a.dD_amp = C(0);
-        a.tf.cx_n = a.tf.cy_n = a.tf.inv_s2_n = a.tf.a_n = C(0);
-        a.tf.cx_p = a.tf.cy_p = a.tf.inv_s2_p = a.tf.a_p = C(0);
-    }
     const long ntiles = (long)((ctx->lp.nx + kBX - 1) / kBX) * ((ctx->lp.ny + kBY - 1) / kBY);
     const long cap = (long)ctx->num_sms * ctas_per_sm;
     const int grid = (int)(ntiles < cap ? ntiles : cap);
@@ -491,6 +466,29 @@ cudaError_t encode_maps(trtr_ctx* ctx) {
         case TRTR_BF16_OFS: return encode_src<__nv_bfloat16>(ctx);
         default: return cudaErrorInvalidValue;
     }
+}
+
+template <typename C>
+__global__ void pulse_tables_kernel(const PulseFill fill, const __grid_constant__ PulseLevels levels) {
+    fill_pulse_tables<C>(fill, levels.t, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
+    if (ctx->p.src_mode != TRTR_SRC_PULSE) return cudaSuccess;
+    if (ctx->ptab_ready && step - 1 >= ctx->ptab_first && step + steps <= ctx->ptab_first + kPulseLevels) return cudaSuccess;
+    const long entries = (long)kPulseLevels * (ctx->p.nx + ctx->p.ny + 4 * kTabGhost);
+    const long want = (entries + 255) / 256, cap = (long)ctx->num_sms * 8;
+    const unsigned grid = (unsigned)(want < cap ? want : cap);
+    ctx->ptab_ready = false;
+    ctx->launches += 1;
+    if (ctx->csize == 8)
+        pulse_tables_kernel<double><<<grid, 256, 0, ctx->stream>>>(pulse_fill_of(ctx), pulse_levels_of(ctx, step - 1));
+    else
+        pulse_tables_kernel<float><<<grid, 256, 0, ctx->stream>>>(pulse_fill_of(ctx), pulse_levels_of(ctx, step - 1));
+    const cudaError_t e = cudaGetLastError();
+    ctx->ptab_first = step - 1;
+    ctx->ptab_ready = e == cudaSuccess;
+    return e;
 }
 
 cudaError_t launch_wait_timeout(trtr_ctx* ctx, long long cycles) {

@@ -142,10 +142,11 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         if (!ok) s_abort = 1;
         S* sp = reinterpret_cast<S*>(smem + s * T::Stage);
         const float* sf = reinterpret_cast<const float*>(smem + s * T::Stage + T::FldOff);
-        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, i0, j0, a, a.tf, tid, a.rkey);
+        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, i0, j0, a, a.pulse, tid, a.rkey);
         __syncthreads();  // P1 complete (and s_abort visible)
         if (ok && !s_abort)
-            step2_second<S, SRC, T, NT, P1, SR>(sp, sf, i0, j0, a, args.tf2, tid, static_cast<S*>(args.dst1), args.rkey2);
+            step2_second<S, SRC, T, NT, P1, SR>(sp, sf, i0, j0, a, a.pulse + a.pt.level, tid,
+                                                 static_cast<S*>(args.dst1), args.rkey2);
         __syncthreads();  // stage s fully read
         if (s_abort) {
             if (tid == 0) {
@@ -162,16 +163,19 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
     finish();
 }
 
-// Packed fields of the two-step kernel at every node of the two-wide ghost frame, from the
+// Packed fields of the two-step kernel at every node of the four-wide ghost frame, from the
 // one-step kernel's field planes (one-wide ghosts by gradient mode) at the wrapped node, with
 // the one-step kernel's roundings: a_a = uhat_x d_x uhat_a + uhat_y d_y uhat_a, central
 // differences 0.5 (u(+1) - u(-1)).
-__global__ void pack_fields2_kernel(float* f2, const float* uv, const float* Dh, PlaneLayout lt, PlaneLayout lf) {
-    const int gw = lt.nx + 2 * kGhostP, gh = lt.ny + 2 * kGhostP;
+// Fills the pulse tables too (fill.tab not null).
+__global__ void pack_fields2_kernel(float* f2, const float* uv, const float* Dh, PlaneLayout lt, PlaneLayout lf,
+                                    const PulseFill fill, const __grid_constant__ PulseLevels levels) {
+    if (fill.tab) fill_pulse_tables<float>(fill, levels.t, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    const int gw = lt.nx + 2 * kGhostT, gh = lt.ny + 2 * kGhostT;
     const size_t n = (size_t)gw * gh;
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / gw) - kGhostP, i = (int)(k % gw) - kGhostP;
-        const int wi = wrap_clamp(i, lt.nx), wj = wrap_clamp(j, lt.ny);
+        const int j = (int)(k / gw) - kGhostT, i = (int)(k % gw) - kGhostT;
+        const int wi = (i % lt.nx + lt.nx) % lt.nx, wj = (j % lt.ny + lt.ny) % lt.ny;
         const size_t o = lf.at(wi, wj);
         const float* u = uv;
         const float* v = uv + lf.plane;
@@ -237,8 +241,8 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
     memset(static_cast<void*>(&args), 0, sizeof(args));
     a.dst = dst;
     args.dst1 = dst1;
-    a.tab_x = static_cast<const float*>(ctx->tab_x);
-    a.tab_y = static_cast<const float*>(ctx->tab_y);
+    a.pt = PulseTab::make(ctx->p.nx, ctx->p.ny);
+    a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<float>(ctx, a.pt, step) : nullptr;
     a.flag = ctx->dflag;
     a.tile_ctr = reinterpret_cast<unsigned*>(ctx->dflag + 2);
     a.lp = ctx->lp;
@@ -247,17 +251,8 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
     a.magic = (float)ctx->p.magic;
     a.omega2_fixed = (float)(ctx->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / ctx->p.tau2 : 0.0);
     a.phi_ref = (float)ctx->p.phi_ref;
-    a.x0 = (float)ctx->p.x0;
-    a.y0 = (float)ctx->p.y0;
-    a.dx = (float)ctx->p.dx;
-    a.dt = (float)ctx->p.dt;
     a.rkey = sr_step_key(step);
     args.rkey2 = sr_step_key(step + 1);
-    if (SRC == TRTR_SRC_PULSE) {
-        a.dD_amp = (float)(ctx->pulse.D0 * ctx->pulse.D_amp);
-        a.tf = pulse_time_fields<float>(ctx->pulse, ctx->p.dt, step);
-        args.tf2 = pulse_time_fields<float>(ctx->pulse, ctx->p.dt, step + 1);
-    }
     const long ntiles = (long)((ctx->lp.nx + G::T::X - 1) / G::T::X) * ((ctx->lp.ny + G::T::Y - 1) / G::T::Y);
     const long cap = (long)ctx->num_sms * ctas_per_sm;
     const long grid = ntiles < cap ? ntiles : cap;
@@ -327,13 +322,18 @@ cudaError_t encode_maps2(trtr_ctx* ctx) {
 }
 
 cudaError_t launch_pack_fields2(trtr_ctx* ctx) {
-    const size_t n = (size_t)(ctx->p.nx + 2 * kGhostP) * (ctx->p.ny + 2 * kGhostP);
+    const size_t n = (size_t)(ctx->p.nx + 2 * kGhostT) * (ctx->p.ny + 2 * kGhostT);
     const size_t want = (n + 255) / 256, cap = (size_t)ctx->num_sms * 8;
     ctx->launches += 1;
+    PulseLevels levels = {};
+    if (ctx->ptab) levels = pulse_levels_of(ctx, ctx->step - 1);
     pack_fields2_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, ctx->stream>>>(
         static_cast<float*>(ctx->fld2), static_cast<const float*>(ctx->uv), static_cast<const float*>(ctx->Dh),
-        ctx->lt, ctx->lf);
-    return cudaGetLastError();
+        ctx->lt, ctx->lf, pulse_fill_of(ctx), levels);
+    const cudaError_t e = cudaGetLastError();
+    ctx->ptab_first = ctx->step - 1;
+    ctx->ptab_ready = ctx->ptab != nullptr && e == cudaSuccess;
+    return e;
 }
 
 cudaError_t launch_refresh_ghosts2_buffer(trtr_ctx* ctx, void* P) {

@@ -94,8 +94,7 @@ using Geom2Of = typename Geom2For<SRC, ES>::type;
 #endif
 
 struct alignas(16) Step2Args {
-    StepArgs<float> a;  // tf, rkey: the pulse uniforms and rounding key of the first step
-    TimeFields<float> tf2;  // of the second step
+    StepArgs<float> a;  // pulse, rkey: the pulse tables and rounding key of the first step
     void* dst1;             // if not null: also store the first step's state here (one-wide ghosts)
     uint32_t rkey2;         // the second step's rounding key (stochastic rounding of 2-byte storages)
 };
@@ -105,26 +104,6 @@ struct alignas(16) Step2Args {
 __device__ __forceinline__ int wrap_clamp(int v, int n) {
     v = v < 0 ? v + n : (v >= n ? v - n : v);
     return v < 0 ? 0 : (v >= n ? n - 1 : v);
-}
-
-// Source term s = dt S^n + dt/2 (S^n - S^{n-1}) of the pair (xi0, xi1) in row yj: the one-step
-// kernel's expressions, node coordinates from the wrapped indices.
-template <int SRC>
-__device__ __forceinline__ F2 pair_source(const StepArgs<float>& a, const TimeFields<float>& tf, int xi0, int xi1,
-                                          int yj) {
-    if (SRC != TRTR_SRC_PULSE) return F2(0.f);
-    const int nx = a.lp.nx, ny = a.lp.ny;
-    const float* tx = reinterpret_cast<const float*>(a.tab_x);
-    const float* ty = reinterpret_cast<const float*>(a.tab_y);
-    const F2 sxm(__ldg(tx + xi0), __ldg(tx + xi1));
-    const F2 cxm(__ldg(tx + nx + xi0), __ldg(tx + nx + xi1));
-    const float sy = __ldg(ty + yj), cy = __ldg(ty + ny + yj);
-    const F2 x = vfma(F2((float)xi0, (float)xi1), F2(a.dx), F2(a.x0));
-    const F2 y(a.y0 + (float)yj * a.dx);
-    const F2 dD = F2(a.dD_amp * sy) * sxm;
-    const F2 dDx = F2(a.dD_amp * 3.14159265358979323846f * sy) * cxm;
-    const F2 dDy = F2(a.dD_amp * 3.14159265358979323846f * cy) * sxm;
-    return pulse_source_dt(x, y, tf, dD, dDx, dDy);
 }
 
 // The TMA loads of one tile into `stage` (its barrier armed by the caller): the population box of
@@ -145,12 +124,12 @@ __device__ __forceinline__ void step2_issue(unsigned char* stage, uint64_t* bar,
 #if TRTR_STEP2_L2HINT
     const uint64_t keep = l2_evict_last();
     if (tma_ok(stage, xp, j0 + kGhostP - 2, kES)) tma_load_3d_hint(stage, mp, bar, xp, j0 + kGhostP - 2, 0, keep);
-    if (tma_ok(stage + T::FldOff, xf, j0 + kGhostP - 1, 4))
-        tma_load_3d_hint(stage + T::FldOff, mf, bar, xf, j0 + kGhostP - 1, 0, keep);
+    if (tma_ok(stage + T::FldOff, xf, j0 + kGhostT - 1, 4))
+        tma_load_3d_hint(stage + T::FldOff, mf, bar, xf, j0 + kGhostT - 1, 0, keep);
 #else
     if (tma_ok(stage, xp, j0 + kGhostP - 2, kES)) tma_load_3d(stage, mp, bar, xp, j0 + kGhostP - 2, 0);
-    if (tma_ok(stage + T::FldOff, xf, j0 + kGhostP - 1, 4))
-        tma_load_3d(stage + T::FldOff, mf, bar, xf, j0 + kGhostP - 1, 0);
+    if (tma_ok(stage + T::FldOff, xf, j0 + kGhostT - 1, 4))
+        tma_load_3d(stage + T::FldOff, mf, bar, xf, j0 + kGhostT - 1, 0);
 #endif
 }
 
@@ -188,7 +167,7 @@ __device__ __forceinline__ typename Pair<S>::type encode2(F2 v, uint32_t rk, int
 // the wrapped pairs are the one-step kernel's pairs).
 template <typename S, int SRC, class T, int NT, bool SR = false>
 __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int j0, const StepArgs<float>& a,
-                                            const TimeFields<float>& tf, int tid, uint32_t rkey1 = 0u) {
+                                            const float* pulse, int tid, uint32_t rkey1 = 0u) {
     constexpr int kT2W = T::W, kT2WF = T::WF, kT2PopPlane = T::PopPlane, kT2FldPlane = T::FldPlane;
     constexpr bool kOfs = sizeof(S) == 2;  // offsets folded into the moments, as in the one-step kernel
     constexpr int kC = T::HX - 2;          // stage column of R1 column 0
@@ -199,7 +178,7 @@ __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int 
 #define TRTR_STEP2_R1SHIFT 0
 #endif
     constexpr int kShift = TRTR_STEP2_R1SHIFT;
-    static_assert(!kOfs || kShift == 0, "2-byte storages round the one-step kernel's pairs");
+    static_assert((!kOfs && SRC != TRTR_SRC_PULSE) || kShift == 0, "the one-step kernel's pairs, on even columns");
     constexpr int kRowPairs = (T::X + 4 - 2 * kShift) / 2;
     constexpr int kPairs = (T::Y + 2) * kRowPairs;
     const int nx = a.lp.nx, ny = a.lp.ny;
@@ -223,11 +202,11 @@ __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int 
         const F2 ay = ld2(f + 3 * kT2FldPlane, fa);
         const F2 Dh = ld2(f + 4 * kT2FldPlane, fa);
         const int x = i0 - 2 + c, y = j0 - 1 + r;
-        const int wx = wrap_clamp(x, nx), wy = wrap_clamp(y, ny);
-        const F2 src = pair_source<SRC>(a, tf, wx, wrap_clamp(x + 1, nx), wy);
+        F2 src(0.f);  // halo nodes: the tables' periodic images
+        if (SRC == TRTR_SRC_PULSE) src = pulse_source_dt(pulse, a.pt, x, y);
         F2 out[kQ];
         collide_node<F2, kOfs>(g, ux, uy, ax, ay, Dh, src, magic, w2f, a.tau2_fixed, out, F2(a.phi_ref));
-        const uint32_t rk = SR ? sr_pair_key(wx, wy, nx, rkey1) : 0u;
+        const uint32_t rk = SR ? sr_pair_key(wrap_clamp(x, nx), wrap_clamp(y, ny), nx, rkey1) : 0u;
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
             S* d = sp + q * kT2PopPlane + (r + 1 - lattice_ey(q)) * kT2W + c + kC - lattice_ex(q);
@@ -241,7 +220,7 @@ __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int 
 // stored to dst1 too, with the one-wide ghost frame that one-step kernels read.
 template <typename S, int SRC, class T, int NT, bool P1 = false, bool SR = false>
 __device__ __forceinline__ void step2_second(const S* sp, const float* sf, int i0, int j0,
-                                             const StepArgs<float>& a, const TimeFields<float>& tf2, int tid,
+                                             const StepArgs<float>& a, const float* pulse, int tid,
                                              S* dst1 = nullptr, uint32_t rkey2 = 0u) {
     constexpr int kT2X = T::X, kT2W = T::W, kT2WF = T::WF, kT2R2 = T::R2, kT2PopPlane = T::PopPlane,
                   kT2FldPlane = T::FldPlane;
@@ -274,7 +253,8 @@ __device__ __forceinline__ void step2_second(const S* sp, const float* sf, int i
         const F2 ax(*reinterpret_cast<const float2*>(f + 2 * kT2FldPlane));
         const F2 ay(*reinterpret_cast<const float2*>(f + 3 * kT2FldPlane));
         const F2 Dh(*reinterpret_cast<const float2*>(f + 4 * kT2FldPlane));
-        const F2 src = pair_source<SRC>(a, tf2, i, i + 1 < nx ? i + 1 : nx - 1, j);
+        F2 src(0.f);
+        if (SRC == TRTR_SRC_PULSE) src = pulse_source_dt(pulse, a.pt, i, j);
         F2 out[kQ];
         collide_node<F2, kOfs>(g, ux, uy, ax, ay, Dh, src, magic, w2f, a.tau2_fixed, out, F2(a.phi_ref));
         const uint32_t rk = SR ? sr_pair_key(i, j, nx, rkey2) : 0u;

@@ -210,8 +210,6 @@ __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ F2 vdiv(F2 a, F2 b) { return F2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)); }
 __device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
-__device__ __forceinline__ F2 vexp(F2 a) { return F2(__expf(a.v.x), __expf(a.v.y)); }
-__device__ __forceinline__ double vexp(double a) { return exp(a); }
 
 template <class V>
 struct ScalarOf;
@@ -224,42 +222,96 @@ struct ScalarOf<double> {
     using type = double;
 };
 
-// Manufactured pulse source at (x, y) for the time level (cx, cy, inv_s2, amp):
-//   S = phi_a / s^2 [grad D . r - (D - D0)(|r|^2 / s^2 - 2)],  r = x - c(t).
-template <class V>
-__device__ __forceinline__ V pulse_source(V x, V y, V cx, V cy, V inv_s2, V amp, V dD, V dDx, V dDy) {
-    using T = typename ScalarOf<V>::type;
-    const V rx = x - cx, ry = y - cy;
-    const V r2 = vfma(rx, rx, ry * ry);
-    const V e = amp * vexp(r2 * (V(T(-0.5)) * inv_s2));
-    const V br = vfma(dD, vfma(r2, V(T(0)) - inv_s2, V(T(2))), vfma(dDx, rx, dDy * ry));
-    return (e * inv_s2) * br;
+// s = dt S^n + dt/2 (S^n - S^{n-1}) = 1.5 dt S^n - 0.5 dt S^{n-1} (a7, Eqs. (3) and (14)) of the
+// manufactured source at the node pair (i, i + 1) (i even, images included) or the node i of row
+// j, from the tables of the levels n - 1 and n (`lev`: level n - 1).
+__device__ __forceinline__ F2 pulse_source_dt(const float* lev, const PulseTab& t, int i, int j) {
+    auto level = [&](const float* p) {
+        const float2 q = __ldg(reinterpret_cast<const float2*>(p + t.y + 2 * j));
+        const F2 p1(__ldg(reinterpret_cast<const float2*>(p + i))), p2(__ldg(reinterpret_cast<const float2*>(p + t.p2 + i)));
+        return vfma(p1, F2(q.x), p2 * F2(q.y));
+    };
+    return vfma(F2(1.5f), level(lev + t.level), F2(-0.5f) * level(lev));
+}
+__device__ __forceinline__ double pulse_source_dt(const double* lev, const PulseTab& t, int i, int j) {
+    auto level = [&](const double* p) {
+        const double2 q = __ldg(reinterpret_cast<const double2*>(p + t.y + 2 * j));
+        return fma(__ldg(p + i), q.x, __ldg(p + t.p2 + i) * q.y);
+    };
+    return fma(1.5, level(lev + t.level), -0.5 * level(lev));
 }
 
-// 2^a (the hardware's base-2 exponential; results below the normal range flush to zero).
-__device__ __forceinline__ float ex2(float a) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-    return r;
+// The E(r) factor of the pulse tables from its exponent -r^2 / (2 s^2): FP64 as it is; FP32 with the
+// exponent split into an integer and a fraction in FP64, so that a large exponent costs no digits.
+__device__ __forceinline__ double pulse_exp(double z, double) { return exp(z); }
+__device__ __forceinline__ float pulse_exp(double z, float) {
+    const double a = z * 1.4426950408889634074;  // log2(e)
+    const double n = rint(a);
+    return n < -160.0 ? 0.f : scalbnf(exp2f((float)(a - n)), (int)n);
 }
 
-// One time level of the source term, w S(x, t) with the level's weight w folded into lg (see
-// pulse_time_fields): by exp(z) = 2^(z log2 e),
-//   w S = 2^(lg - |r|^2 log2(e) / (2 s^2)) [grad D . r + (D - D0)(2 - |r|^2 / s^2)].
-__device__ __forceinline__ F2 pulse_level(F2 x, F2 y, float cx, float cy, float inv_s2, float lg, F2 dD, F2 dDx,
-                                          F2 dDy) {
-    const F2 rx = x - F2(cx), ry = y - F2(cy);
-    const F2 r2 = vfma(rx, rx, ry * ry);
-    const F2 z = vfma(r2, F2(-0.72134752044448170368f * inv_s2), F2(lg));  // -log2(e) / 2 = -0.7213...
-    const F2 br = vfma(dD, vfma(r2, F2(-inv_s2), F2(2.f)), vfma(dDx, rx, dDy * ry));
-    return F2(ex2(z.v.x), ex2(z.v.y)) * br;
+// Entries k, k + stride, ... of the tables: one coordinate of one level each (levels[l]: the pulse
+// at level l of the table), coordinates outside the grid as their periodic images.
+template <typename C>
+__device__ __forceinline__ void fill_pulse_tables(const PulseFill& f, const PulseTime* levels, unsigned k,
+                                                  unsigned stride) {
+    const PulseTab t = PulseTab::make(f.nx, f.ny);
+    const unsigned gx = f.nx + 2 * kTabGhost, per = gx + f.ny + 2 * kTabGhost;
+    const C pi = C(3.14159265358979323846);
+    for (const unsigned total = per * kPulseLevels; k < total; k += stride) {
+        const unsigned lev = k / per, e = k - lev * per;
+        const bool along_x = e < gx;
+        const int n = along_x ? f.nx : f.ny, at = (int)(along_x ? e : e - gx) - kTabGhost;
+        int w = at % n;
+        w = w < 0 ? w + n : w;
+        const PulseTime pt = levels[lev];
+        const C* tab = static_cast<const C*>(along_x ? f.tab_x : f.tab_y);
+        const C sn = tab[w], cs = tab[n + w];
+        const double r = along_x ? f.x0 + w * f.dx - pt.cx : f.y0 + w * f.dx - pt.cy;
+        const double z = r * r * pt.inv_s2;
+        const C E = pulse_exp(-0.5 * z, C(0));
+        const C slope = E * (pi * cs * C(r) + sn * C(1.0 - z)), value = E * sn;
+        C* out = static_cast<C*>(f.tab) + kTabGhost + (size_t)lev * t.level;
+        if (along_x) {
+            out[at] = slope;
+            out[t.p2 + at] = value;
+        } else {
+            const C A = C(f.amp * pt.amp * pt.inv_s2);
+            out[t.y + 2 * at] = A * value;
+            out[t.y + 2 * at + 1] = A * slope;
+        }
+    }
 }
 
-// s = dt S^n + dt/2 (S^n - S^{n-1}) = 1.5 dt S^n - 0.5 dt S^{n-1} of the manufactured source
-// (a7, Eqs. (3) and (14)) for the FP32-computing kernels.
-__device__ __forceinline__ F2 pulse_source_dt(F2 x, F2 y, const TimeFields<float>& tf, F2 dD, F2 dDx, F2 dDy) {
-    return pulse_level(x, y, tf.cx_n, tf.cy_n, tf.inv_s2_n, tf.a_n, dD, dDx, dDy) -
-           pulse_level(x, y, tf.cx_p, tf.cy_p, tf.inv_s2_p, tf.a_p, dD, dDx, dDy);
+// The pulse at the time levels of one fill of the tables, computed on the host.
+struct PulseLevels {
+    PulseTime t[kPulseLevels];
+};
+inline PulseLevels pulse_levels_of(const trtr_ctx* ctx, long first) {
+    PulseLevels l;
+    for (int k = 0; k < kPulseLevels; ++k) l.t[k] = pulse_at(ctx->pulse, (double)(first + k) * ctx->p.dt);
+    return l;
+}
+
+inline PulseFill pulse_fill_of(const trtr_ctx* ctx) {
+    PulseFill f;
+    memset(static_cast<void*>(&f), 0, sizeof(f));
+    f.tab = ctx->ptab;
+    f.tab_x = ctx->tab_x;
+    f.tab_y = ctx->tab_y;
+    f.x0 = ctx->p.x0;
+    f.y0 = ctx->p.y0;
+    f.dx = ctx->p.dx;
+    f.amp = ctx->p.dt * ctx->pulse.D0 * ctx->pulse.D_amp;
+    f.nx = ctx->p.nx;
+    f.ny = ctx->p.ny;
+    return f;
+}
+
+// The tables of a launch from step `step`: coordinate 0 of level step - 1.
+template <typename C>
+inline const C* pulse_level(const trtr_ctx* ctx, const PulseTab& t, long step) {
+    return static_cast<const C*>(ctx->ptab) + kTabGhost + (size_t)(step - 1 - ctx->ptab_first) * t.level;
 }
 
 // The node update of Eq. (14) in moment space; g: pre-collision populations, out: P_i(x).
@@ -477,13 +529,13 @@ __device__ __forceinline__ void issue_tile(unsigned char* stage, uint64_t* bar, 
 // copy of the row's first `bulk_cols(nx - i0)` columns (16-byte multiples: the row starts are
 // 16-byte aligned in both memories).  The lanes store the few columns past those, and the ghost
 // copies of edge nodes, directly.
+// psrc: the source terms of the lane's pairs (TRTR_SRC_PULSE).
 // UNR: the unroll factor of the pair loop (1: one pair at a time; NM: all pairs interleaved).
 // SR: the 2-byte storages round stochastically (TRTR_ROUND_STOCHASTIC), with the random bits of
 // sr_hash keyed by the node pair and a.rkey.
 template <typename S, int SRC, int BX, int BY, int NM = BX / 64, bool TST = false, int UNR = 1, bool SR = false>
 __device__ __forceinline__ void tile_row_pairs(const unsigned char* st, int r, int lane, int i0, int j,
-                                               const StepArgs<float>& a, const F2* sx, const F2* cx, float sy,
-                                               float cy, int c0 = 0) {
+                                               const StepArgs<float>& a, const F2* psrc, int c0 = 0) {
     static_assert(!TST || NM == BX / 64, "bulk row stores need one warp per tile row");
     using T = Tile<S, SRC, BX, BY>;
     using P = Pair<S>;
@@ -535,19 +587,10 @@ __device__ __forceinline__ void tile_row_pairs(const unsigned char* st, int r, i
             const F2 sp_(*reinterpret_cast<const float2*>(ss + T::S_TILE / sizeof(float) + c));
             src = vfma(F2(1.5f), sn, F2(-0.5f) * sp_);
         } else if (SRC == TRTR_SRC_PULSE) {
-            const F2 x = vfma(F2((float)i, (float)(i + 1)), F2(a.dx), F2(a.x0));
-            const F2 y(a.y0 + (float)j * a.dx);
-            F2 sxm = sx[0], cxm = cx[0];  // compile-time indices only (no local-memory arrays)
+            src = psrc[0];  // compile-time indices only (no local-memory array)
 #pragma unroll
             for (int mm = 1; mm < NM; ++mm)
-                if (m == mm) {
-                    sxm = sx[mm];
-                    cxm = cx[mm];
-                }
-            const F2 dD = F2(a.dD_amp * sy) * sxm;
-            const F2 dDx = F2(a.dD_amp * 3.14159265358979323846f * sy) * cxm;
-            const F2 dDy = F2(a.dD_amp * 3.14159265358979323846f * cy) * sxm;
-            src = pulse_source_dt(x, y, a.tf, dD, dDx, dDy);
+                if (m == mm) src = psrc[mm];
         }
 
         F2 out[kQ];
@@ -624,7 +667,7 @@ __device__ __forceinline__ void tile_row_f64(const unsigned char* st, int r, int
                                              const StepArgs<double>& a, int c0 = 0) {
     static_assert(!TST || NMF == BX / 32, "bulk row stores need one warp per tile row");
     using T = Tile<double, SRC, BX, BY>;
-    const int nx = a.lp.nx, ny = a.lp.ny;
+    const int nx = a.lp.nx;
     const double* sp = reinterpret_cast<const double*>(st) + r * T::PW;
     const double* su = reinterpret_cast<const double*>(st + T::POP) + (r + 1) * T::UW + T::AC;
     const double* sv = su + T::UH * T::UW;
@@ -632,11 +675,6 @@ __device__ __forceinline__ void tile_row_f64(const unsigned char* st, int r, int
     const double* ss = reinterpret_cast<const double*>(st + T::POP + T::U + T::D) + r * BX;
     double* dst = static_cast<double*>(a.dst);
     const size_t pl = a.lp.plane;
-    double sy = 0.0, cy = 0.0;
-    if (SRC == TRTR_SRC_PULSE) {
-        sy = __ldg(a.tab_y + j);
-        cy = __ldg(a.tab_y + ny + j);
-    }
 #pragma unroll 1
     for (int m = 0; m < NMF; ++m) {
         const int c = c0 + 32 * m + lane;
@@ -656,14 +694,7 @@ __device__ __forceinline__ void tile_row_f64(const unsigned char* st, int r, int
         if (SRC == TRTR_SRC_FIELD) {
             src = fma(1.5, ss[c], -0.5 * ss[T::S_TILE / sizeof(double) + c]);
         } else if (SRC == TRTR_SRC_PULSE) {
-            const double x = a.x0 + (double)i * a.dx, y = a.y0 + (double)j * a.dx;
-            const double sx = __ldg(a.tab_x + i), cx = __ldg(a.tab_x + nx + i);
-            const double dD = a.dD_amp * sx * sy;
-            const double dDx = a.dD_amp * 3.14159265358979323846 * cx * sy;
-            const double dDy = a.dD_amp * 3.14159265358979323846 * sx * cy;
-            const double Sn = pulse_source(x, y, a.tf.cx_n, a.tf.cy_n, a.tf.inv_s2_n, a.tf.a_n, dD, dDx, dDy);
-            const double Sp = pulse_source(x, y, a.tf.cx_p, a.tf.cy_p, a.tf.inv_s2_p, a.tf.a_p, dD, dDx, dDy);
-            src = a.dt * fma(1.5, Sn, -0.5 * Sp);
+            src = pulse_source_dt(a.pulse, a.pt, i, j);
         }
         double out[kQ];
         collide_node<double>(g, ux, uy, ax, ay, sd[c], src, a.magic, a.omega2_fixed, a.tau2_fixed, out);
@@ -752,6 +783,20 @@ inline bool encode(CUtensorMap* m, CUtensorMapDataType t, int elem, void* base, 
               kPromotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same with bounds at the interior (coordinate 0 is node 0): loads outside it read zero, stores
+// write nothing there.
+inline bool encode_interior(CUtensorMap* m, CUtensorMapDataType t, int elem, void* base, const PlaneLayout& L, int depth,
+                            int bw, int bh, int bd) {
+    auto fn = get_encoder();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {(cuuint64_t)L.nx, (cuuint64_t)L.ny, (cuuint64_t)depth};
+    const cuuint64_t strides[2] = {(cuuint64_t)L.pitch * elem, (cuuint64_t)L.plane * elem};
+    const cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, (cuuint32_t)bd};
+    const cuuint32_t es[3] = {1, 1, 1};
+    return fn(m, t, 3, static_cast<char*>(base) + ((size_t)L.gy * L.pitch + L.gx) * elem, dims, strides, box, es,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, kPromotion,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 }  // namespace core
 }  // namespace trtr

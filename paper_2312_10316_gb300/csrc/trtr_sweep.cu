@@ -1,0 +1,546 @@
+// trtr_sweep.cu -- four time steps of the evolution equation (14) per launch: each CTA sweeps a
+// strip of columns from bottom to top and carries four time levels behind one another through
+// shared memory (wavefront temporal blocking), for FP32 storage or FP16 / BF16 offset storage
+// (FP32 arithmetic), periodic boundaries and no source or the manufactured pulse source.  The
+// node update is the one-step kernel's, roundings included, so the results have the same bits.
+//
+// Strip: X = 120 output columns from i0; every level computes the 128 columns [i0 - 4, i0 + 124)
+// (two warps a row, a node pair a lane), of which level s is valid on all but s - 1 at each side.
+// Rows arrive through TMA, one box of the nine populations (136 columns from i0 - 8) and one of
+// the five packed fields (128 columns from i0 - 4) a row, into a ring of kRing rows; y wraps by the
+// row index, x through a four-wide ghost frame of columns.  Populations live in place: node x at
+// level s reads and writes the slots x - s e_q of the ring, which no other node touches at that
+// level, so one ring serves every level (level s = 1 .. 4 of row j uses the slot rows j - s, j,
+// j + s).  In iteration k level s works on R rows, kLag rows behind level s - 1, which has then
+// finished the row above them; one CTA barrier an iteration orders everything.  The last level
+// writes its rows to a shared-memory buffer that one TMA store an iteration moves out, clipped to
+// the grid; nodes near an edge also store their ghost copies.
+//
+// Work units are (strip, segment of rows); a segment costs C rows of ramp (its first output row
+// needs C / R iterations), so the host picks the number of segments that ends soonest.
+#include "trtr_step_core.cuh"
+
+namespace trtr {
+namespace {
+
+using namespace core;
+
+constexpr int kT = 4;                 // time levels of a launch
+constexpr int kX = 120, kWC = 128;    // output and computed columns of a strip
+constexpr int kW = kWC + 2 * kT;      // staged population columns
+constexpr int kNF = 5;                // packed fields
+constexpr int kGhostX = 4;            // ghost columns that the strips read
+
+#ifndef TRTR_SWEEP_R
+#define TRTR_SWEEP_R 3
+#endif
+#ifndef TRTR_SWEEP_AHEAD
+#define TRTR_SWEEP_AHEAD 1
+#endif
+#ifndef TRTR_SWEEP_OUTS
+#define TRTR_SWEEP_OUTS 3
+#endif
+#ifndef TRTR_SWEEP_AHEADH
+#define TRTR_SWEEP_AHEADH 3
+#endif
+#ifndef TRTR_SWEEP_RH
+#define TRTR_SWEEP_RH 4
+#endif
+
+template <typename S, int R_>
+struct Sweep {
+    static constexpr int R = R_, ES = (int)sizeof(S);
+    static constexpr int Lag = R + 1;
+    static constexpr int C = ((kT - 1) * (Lag + 1) + R - 1) / R * R;  // ramp rows of a segment
+    static constexpr int Ahead = ES == 2 ? TRTR_SWEEP_AHEADH : TRTR_SWEEP_AHEAD;  // blocks loaded ahead
+    static constexpr int Ring = ((kT - 1) * Lag + kT + 1 + (Ahead + 1) * R + R - 1) / R * R;
+    static constexpr int Blocks = Ring / R;
+    static constexpr int PopRow = kQ * kW * ES, FldRow = kNF * kWC * 4;
+    static constexpr int OutBytes = (kQ * R * kX * ES + 127) / 128 * 128;
+    static constexpr int FldOff = Ring * ((PopRow + 127) / 128 * 128);
+    static constexpr int PopPitch = (PopRow + 127) / 128 * 128;       // TMA destinations on 128 bytes
+    static constexpr int OutOff = FldOff + Ring * FldRow;
+    static constexpr int Outs = ES == 2 ? 3 : TRTR_SWEEP_OUTS;                                    // output buffers
+    static constexpr int BarOff = OutOff + Outs * OutBytes;
+    static constexpr int Depth = 8;                                   // barriers of a level (iterations in flight)
+    static constexpr int Smem = BarOff + (Blocks + kT * Depth + Outs) * 8 + 128;
+    static constexpr int Warps = kT * R;                              // a warp per level and row
+    static constexpr int Threads = (Warps + 1) * 32;                  // and one warp that moves the data
+    static_assert(FldRow % 128 == 0, "TMA destinations on 128 bytes");
+    // level 4 may finish iteration k when level 2 has finished k - 2, and level 1 may then be in k + 1 + Ahead
+    static_assert(Ahead + 2 <= Depth, "a level stays within Depth iterations of the next");
+    static_assert(Smem <= 227 * 1024, "the rings must fit in shared memory");
+};
+
+struct SweepArgs {
+    const float* pulse;  // tables of level n - 1
+    PulseTab pt;
+    void* dst;
+    int* flag;
+    PlaneLayout lp;
+    int gxf, gyf;        // interior origin of the packed fields
+    int strips, seg_rows, units;
+    int tau2_fixed;
+    float magic, omega2_fixed, phi_ref;
+    uint32_t rkey[kT];
+};
+
+// Columns of an nx-wide row in whole 16-byte chunks.
+template <typename T>
+__host__ __device__ __forceinline__ int bulk_cols_of(int nx) {
+    constexpr int kChunk = 16 / (int)sizeof(T);
+    return nx / kChunk * kChunk;
+}
+
+// The ghost copies of one value of interior node (i, j): kGhostX columns, kGhostP rows.
+template <typename T>
+__device__ __forceinline__ void store_sweep_ghosts(T* plane, const PlaneLayout& L, int i, int j, T v) {
+    T* row = plane + (size_t)(j + kGhostP) * L.pitch + L.gx;
+    const int xs = i < kGhostX ? L.nx : (i >= L.nx - kGhostX ? -L.nx : 0);
+    const int ys = j < kGhostP ? L.ny : (j >= L.ny - kGhostP ? -L.ny : 0);
+    if (xs) row[i + xs] = v;
+    if (ys) {
+        row += (ptrdiff_t)ys * L.pitch;
+        row[i] = v;
+        if (xs) row[i + xs] = v;
+    }
+}
+
+// Level LV of row j for one lane: its node pairs at the columns c = 2 lane and c + 64 (h = 0, 1),
+// computed side by side so that each hides the other's latency.  pm / p0 / pp: the ring rows of the
+// slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
+// the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
+// rows within kGhostP of an edge).
+template <typename S, int LV, bool SR, class G>
+__device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[2], const SweepArgs& a,
+                                          const uint32_t rk[2], S* out_row, int lane, int i, int j) {
+    constexpr bool kOfs = sizeof(S) == 2;
+    using S2 = typename Pair<S>::type;
+    F2 out[2][kQ];
+    auto slot = [&](int q, int h) -> S* {
+        S* row = lattice_ey(q) == 1 ? pm : (lattice_ey(q) == -1 ? pp : p0);
+        return row + q * kW - LV * lattice_ex(q) + 64 * h;
+    };
+    auto even = [](int q) { return LV % 2 == 0 || lattice_ex(q) == 0; };
+    F2 g[2][kQ], fld[2][kNF];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+            const S* s = slot(q, h);
+            g[h][q] = even(q) ? Pair<S>::raw(*reinterpret_cast<const S2*>(s)) : Pair<S>::raw(s[0], s[1]);
+        }
+#pragma unroll
+        for (int m = 0; m < kNF; ++m) fld[h][m] = F2(*reinterpret_cast<const float2*>(f + m * kWC + 64 * h));
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        collide_node<F2, kOfs>(g[h], fld[h][0], fld[h][1], fld[h][2], fld[h][3], fld[h][4], src[h], F2(a.magic),
+                               F2(a.omega2_fixed), a.tau2_fixed, out[h], F2(a.phi_ref));
+    auto enc = [&](int q, int h) -> S2 {
+        if constexpr (SR)
+            return Pair<S>::encode_sr(out[h][q], sr_bits(rk[h], q));
+        else
+            return Pair<S>::encode_raw(out[h][q]);
+    };
+    if constexpr (LV < kT) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+                const S2 v = enc(q, h);
+                S* s = slot(q, h);
+                if (even(q)) {
+                    *reinterpret_cast<S2*>(s) = v;
+                } else {
+                    s[0] = reinterpret_cast<const S*>(&v)[0];
+                    s[1] = reinterpret_cast<const S*>(&v)[1];
+                }
+            }
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) *reinterpret_cast<S2*>(out_row + q * (G::R * kX) + 64 * h) = enc(q, h);
+            if (j < kGhostP || j >= a.lp.ny - kGhostP) {
+#pragma unroll 1
+                for (int q = 0; q < kQ; ++q) {
+                    const S* v = out_row + q * (G::R * kX) + 64 * h;
+                    S* plane = static_cast<S*>(a.dst) + q * a.lp.plane;
+                    if (i + 64 * h < a.lp.nx) store_sweep_ghosts(plane, a.lp, i + 64 * h, j, v[0]);
+                    if (i + 64 * h + 1 < a.lp.nx) store_sweep_ghosts(plane, a.lp, i + 64 * h + 1, j, v[1]);
+                }
+            }
+        }
+    }
+}
+
+// The edge columns of the rows y .. y + R - 1 (below j1) of a strip from the output buffer, by one
+// warp: the ghost copies, and the last columns where a row is no whole number of 16-byte chunks (the
+// TMA store's map ends with the last whole one).
+template <typename S, class G>
+__device__ __forceinline__ void copy_edge_columns(const S* buf, const SweepArgs& a, int i0, int y, int j1, int lane) {
+    const int nx = a.lp.nx, nc = bulk_cols_of<S>(nx);
+    const int right = max(i0, min(nc, nx - kGhostX)), left = i0 == 0 ? kGhostX : 0;
+    const int n = left + max(0, min(i0 + kX, nx) - right), t = lane & 15;
+    const int i = t < left ? t : right + t - left;
+    if (t >= n) return;
+    for (int qr = lane >> 4; qr < kQ * G::R; qr += 2) {
+        const int q = qr / G::R, j = y + qr - q * G::R;
+        if (j >= j1) continue;
+        S* row = static_cast<S*>(a.dst) + q * a.lp.plane + (size_t)(j + kGhostP) * a.lp.pitch + a.lp.gx;
+        const S v = buf[qr * kX + i - i0];
+        if (i < kGhostX) row[i + nx] = v;
+        if (i >= nx - kGhostX) row[i - nx] = v;
+        if (i >= nc) row[i] = v;
+    }
+}
+
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(map),
+                 "r"(smem_addr(src)), "r"(x), "r"(y), "r"(z)
+                 : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+template <typename S, int SRC, bool SR, class G>
+__global__ void __launch_bounds__(G::Threads, 1)
+    sweep_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mf,
+                 const __grid_constant__ CUtensorMap mo, const __grid_constant__ SweepArgs a) {
+    constexpr int R = G::R;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ int s_abort;
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
+                                                           ~static_cast<uintptr_t>(127));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + G::BarOff);  // [Blocks]: a block of rows has arrived
+    uint64_t* done = full + G::Blocks;                               // [kT][Depth]: a level has finished an iteration
+    uint64_t* freed = done + kT * G::Depth;                          // [Outs]: an output buffer has been stored
+    const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int nx = a.lp.nx, ny = a.lp.ny;
+    if (tid == 0) {
+        s_abort = 0;
+        for (int b = 0; b < G::Blocks; ++b) mbar_init(&full[b], 1);
+        for (int b = 0; b < kT * G::Depth; ++b) mbar_init(&done[b], R);
+        for (int b = 0; b < G::Outs; ++b) mbar_init(&freed[b], 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // A wait that gives up sets s_abort; every warp then leaves at its next wait.
+    volatile int* abort_flag = &s_abort;
+    auto wait = [&](uint64_t* bar, unsigned parity) -> bool {
+        if (mbar_try_wait(bar, parity)) return true;
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar, parity)) {
+            if (*abort_flag) return false;
+            if (clock64() - t0 > kWaitCycles) {
+                *abort_flag = 1;
+                return false;
+            }
+        }
+        return true;
+    };
+    // Iterations are numbered through all units of the CTA (`it0` before this one): iteration it of a
+    // level completes phase it / Depth of done[level][it % Depth].
+    struct Unit {
+        int i0, j0, j1, iters, a0;
+    };
+    auto unit = [&](int u) {
+        Unit t;
+        const int strip = u % a.strips, seg = u / a.strips;
+        t.i0 = strip * kX;
+        t.j0 = seg * a.seg_rows;
+        t.j1 = min(t.j0 + a.seg_rows, ny);
+        t.iters = (t.j1 - t.j0 + G::C + R - 1) / R;
+        t.a0 = t.j0 + (kT - 1) * G::Lag - G::C;  // level 1's first row
+        return t;
+    };
+
+    if (w == G::Warps) {
+        // The mover: lane 0 loads the blocks (block m of a unit: the rows a0 + 1 - R + m R ..; iteration
+        // k needs the blocks up to k + 1) and stores the rows the last level has finished.
+        unsigned phase = 0, it0 = 0, pending = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+            const Unit t = unit(u);
+            const int blocks = t.iters + 1;
+            auto load = [&](int m) {
+                const unsigned b = (phase + m) % G::Blocks;
+                mbar_expect_tx(&full[b], R * (G::PopRow + G::FldRow));
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    int y = t.a0 + 1 - R + m * R + r;
+                    y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+                    unsigned char* pd = smem + (b * R + r) * G::PopPitch;
+                    unsigned char* fd = smem + G::FldOff + (b * R + r) * G::FldRow;
+                    const int xp = t.i0 - 2 * kT + a.lp.gx, xf = t.i0 - kT + a.gxf;
+                    if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, &mp, &full[b], xp, y + kGhostP, 0);
+                    if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, &mf, &full[b], xf, y + a.gyf, 0);
+                }
+            };
+            const bool edges = t.i0 == 0 || t.i0 + kX > min(nx - kGhostX, bulk_cols_of<S>(nx));
+            int loaded = min(blocks, 2 + G::Ahead);
+            if (lane == 0)
+                for (int m = 0; m < loaded; ++m) load(m);
+            for (int k = 0; k < t.iters; ++k) {
+                const unsigned it = it0 + k, o = it % G::Outs;
+                if (!(ok = wait(&done[(kT - 1) * G::Depth + it % G::Depth], (it / G::Depth) & 1))) break;
+                const int y = t.a0 + k * R - (kT - 1) * G::Lag;  // the last level's rows
+                unsigned char* buf = smem + G::OutOff + o * G::OutBytes;
+                if (lane == 0) {
+                    if (k + 2 + G::Ahead < blocks) {
+                        fence_proxy_async_smem();
+                        load(k + 2 + G::Ahead);
+                    }
+                    if (y >= t.j0) tma_store_3d(&mo, buf, t.i0, y, 0);
+                    bulk_commit();
+                }
+                if (edges && y >= t.j0) copy_edge_columns<S, G>(reinterpret_cast<const S*>(buf), a, t.i0, y, t.j1, lane);
+                __syncwarp();
+                if (lane == 0) {  // the store before this one has left its buffer
+                    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    if (it > 0) mbar_arrive(&freed[(it - 1) % G::Outs]);
+                }
+                loaded = min(blocks, k + 3 + G::Ahead);
+            }
+            pending = phase + loaded;
+            phase += blocks;
+            it0 += t.iters;
+        }
+        if (lane == 0) {
+            if (!ok) {  // let the loads issued into this CTA's shared memory land (bounded)
+                atomicExch(a.flag, 1);
+                const unsigned n = pending < (unsigned)G::Blocks ? pending : (unsigned)G::Blocks;
+                for (unsigned m = pending - n; m < pending; ++m)
+                    mbar_wait_bounded(&full[m % G::Blocks], (m / G::Blocks) & 1);
+            }
+            bulk_wait_all();
+        }
+        return;
+    }
+
+    // Level `level`, row r0 of every iteration.
+    const int level = w / R + 1, r0 = w % R;
+    const uint32_t rkey = a.rkey[level - 1];
+    unsigned phase = 0, it = 0;
+    for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+        const Unit t = unit(u);
+        // per strip: the pairs' columns, their images for the rounding keys, their pulse factors
+        const int i = t.i0 - kT + 2 * lane;
+        F2 p1p[2], p2p[2], p1n[2], p2n[2];
+        int wx[2];
+        const float* lev = a.pulse + (level - 1) * a.pt.level;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (SRC == TRTR_SRC_PULSE) {
+                p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + i + 64 * h)));
+                p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.p2 + i + 64 * h)));
+                p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + i + 64 * h)));
+                p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + a.pt.p2 + i + 64 * h)));
+            }
+            wx[h] = i + 64 * h < 0 ? i + 64 * h + nx : i + 64 * h;
+            wx[h] = wx[h] >= nx ? wx[h] - nx : wx[h];
+        }
+        const float* ty = lev + a.pt.y;
+
+        // the warp's row of the iteration and its ring row (block m = 0 starts at row a0 + 1 - R)
+        int j = t.a0 - (level - 1) * G::Lag + r0;
+        int ring = (int)(phase % G::Blocks) * R + j - (t.a0 + 1 - R);
+        ring = ring < 0 ? ring + G::Ring : (ring >= G::Ring ? ring - G::Ring : ring);
+        unsigned block = phase % G::Blocks, parity = (phase / G::Blocks) & 1;
+        if (level == 1 && !wait(&full[block], parity)) return;
+        for (int k = 0; k < t.iters; ++k, j += R, ++it) {
+            F2 src[2] = {F2(0.f), F2(0.f)};
+            int yw = 0;
+            if (SRC == TRTR_SRC_PULSE || SR) yw = j < 0 ? j + ny : (j >= ny ? j - ny : j);
+            if (SRC == TRTR_SRC_PULSE) {  // as pulse_source_dt
+                const float2 qp = __ldg(reinterpret_cast<const float2*>(ty + 2 * yw));
+                const float2 qn = __ldg(reinterpret_cast<const float2*>(ty + a.pt.level + 2 * yw));
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    src[h] = vfma(F2(1.5f), vfma(p1n[h], F2(qn.x), p2n[h] * F2(qn.y)),
+                                  F2(-0.5f) * vfma(p1p[h], F2(qp.x), p2p[h] * F2(qp.y)));
+            }
+            // level 1 waits for its rows, the others for the level before to have finished the iteration
+            // before this one; the last level also for its output buffer
+            bool ok;
+            if (level == 1) {
+                if (++block == G::Blocks) {
+                    block = 0;
+                    parity ^= 1;
+                }
+                ok = wait(&full[block], parity);
+            } else {
+                ok = it == 0 || wait(&done[(level - 2) * G::Depth + (it - 1) % G::Depth], ((it - 1) / G::Depth) & 1);
+            }
+            const unsigned o = it % G::Outs;
+            if (level == kT && it >= (unsigned)G::Outs) ok = ok && wait(&freed[o], (it / G::Outs - 1) & 1);
+            if (!ok) return;
+            if (j >= t.j0 - (kT - level) && j < t.j1 + (kT - level)) {
+                const int below = ring >= level ? ring - level : ring - level + G::Ring;
+                const int above = ring + level < G::Ring ? ring + level : ring + level - G::Ring;
+                constexpr int kPitch = G::PopPitch / G::ES;
+                S* base = reinterpret_cast<S*>(smem) + 2 * lane + kT;
+                S* pm = base + below * kPitch;
+                S* p0 = base + ring * kPitch;
+                S* pp = base + above * kPitch;
+                const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (kNF * kWC) + 2 * lane;
+                uint32_t rk[2] = {0u, 0u};
+                if (SR) {
+                    rk[0] = sr_pair_key(wx[0], yw, nx, rkey);
+                    rk[1] = sr_pair_key(wx[1], yw, nx, rkey);
+                }
+                S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane - kT;
+                switch (level) {
+                    case 1: sweep_row<S, 1, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 2: sweep_row<S, 2, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 3: sweep_row<S, 3, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    default: sweep_row<S, 4, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                }
+            }
+            if (level == kT) fence_proxy_async_smem();  // the rows, for the TMA store
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&done[(level - 1) * G::Depth + it % G::Depth]);
+            ring += R;
+            if (ring >= G::Ring) ring -= G::Ring;
+        }
+        phase += t.iters + 1;
+    }
+}
+
+// The kGhostX ghost columns of every interior row and plane from the interior (periodic).
+template <typename E>
+__global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
+    const int n = kQ * L.ny * 2 * kGhostX;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int g = k % (2 * kGhostX), row = k / (2 * kGhostX), q = row / L.ny, j = row - q * L.ny;
+        E* p = P + (size_t)q * L.plane + (size_t)(j + kGhostP) * L.pitch + L.gx;
+        const int to = g < kGhostX ? g - kGhostX : L.nx + g - kGhostX;
+        p[to] = p[g < kGhostX ? L.nx + to : to - L.nx];
+    }
+}
+
+template <typename S, int SRC, bool SR>
+cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
+    using G = Sweep<S, sizeof(S) == 2 ? TRTR_SWEEP_RH : TRTR_SWEEP_R>;
+    auto kernel = sweep_kernel<S, SRC, SR, G>;
+    static int configured_device = -1;
+    if (configured_device != ctx->device) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
+        if (e != cudaSuccess) return e;
+        configured_device = ctx->device;
+    }
+    const int nx = ctx->p.nx, ny = ctx->p.ny;
+    SweepArgs a;
+    memset(static_cast<void*>(&a), 0, sizeof(a));
+    a.pt = PulseTab::make(nx, ny);
+    a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<float>(ctx, a.pt, ctx->step) : nullptr;
+    a.dst = ctx->pop[ctx->cur ^ 1];
+    a.flag = ctx->dflag;
+    a.lp = ctx->lp;
+    a.gxf = ctx->lt.gx;
+    a.gyf = ctx->lt.gy;
+    a.strips = (nx + kX - 1) / kX;
+    // the number of segments a strip that ends soonest: rounds of the SMs times a unit's rows
+    long best = 0;
+    int segs = 1;
+    for (int s = 1; s <= (ny + G::R - 1) / G::R && s <= 4 * ctx->num_sms; ++s) {
+        const int rows = ((ny + s - 1) / s + G::R - 1) / G::R * G::R;
+        const long units = (long)a.strips * ((ny + rows - 1) / rows);
+        const long cost = ((units + ctx->num_sms - 1) / ctx->num_sms) * (rows + G::C + 4);
+        if (s == 1 || cost < best) {
+            best = cost;
+            segs = s;
+        }
+    }
+    a.seg_rows = ((ny + segs - 1) / segs + G::R - 1) / G::R * G::R;
+    a.units = a.strips * ((ny + a.seg_rows - 1) / a.seg_rows);
+    a.tau2_fixed = ctx->p.tau2_mode == TRTR_TAU2_FIXED;
+    a.magic = (float)ctx->p.magic;
+    a.omega2_fixed = (float)(ctx->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / ctx->p.tau2 : 0.0);
+    a.phi_ref = (float)ctx->p.phi_ref;
+    for (int s = 0; s < kT; ++s) a.rkey[s] = sr_step_key(ctx->step + s);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.units < ctx->num_sms ? a.units : ctx->num_sms));
+    cfg.blockDim = dim3(G::Threads);
+    cfg.dynamicSmemBytes = G::Smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, ctx->maps4[ctx->cur], ctx->maps4[4], ctx->maps4[2 + (ctx->cur ^ 1)], a);
+}
+
+template <typename S>
+cudaError_t encode4_typed(trtr_ctx* ctx) {
+    using G = Sweep<S, sizeof(S) == 2 ? TRTR_SWEEP_RH : TRTR_SWEEP_R>;
+    bool ok = true;
+    PlaneLayout in = ctx->lp;  // the interior alone, so that stores are clipped to it
+    in.nx = bulk_cols_of<S>(in.nx);
+    for (int b = 0; b < 2; ++b) {
+        ok = ok && encode(&ctx->maps4[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], ctx->lp, kQ, kW, 1, kQ);
+        ok = ok && encode_interior(&ctx->maps4[2 + b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], in, kQ, kX, G::R, kQ);
+    }
+    ok = ok && encode(&ctx->maps4[4], tma_type<float>(), 4, ctx->fld2, ctx->lt, kNF, kWC, 1, kNF);
+    return ok ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+// Rows wrap once around the grid, and a row holds at least one whole 16-byte chunk.
+static bool sweep_size(const trtr_ctx* ctx) { return ctx->p.nx >= 16 && ctx->p.ny >= 32; }
+
+cudaError_t encode_maps4(trtr_ctx* ctx) {
+    if (!ctx->fld2 || !sweep_size(ctx)) return cudaSuccess;
+    switch (ctx->p.precision) {
+        case TRTR_F32: return encode4_typed<float>(ctx);
+        case TRTR_F16_OFS: return encode4_typed<__half>(ctx);
+        case TRTR_BF16_OFS: return encode4_typed<__nv_bfloat16>(ctx);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+bool sweep_applies(const trtr_ctx* ctx) {
+    return two_step_applies(ctx) && sweep_size(ctx);
+}
+
+cudaError_t launch_ghost_columns(trtr_ctx* ctx) {
+    const int n = kQ * ctx->p.ny * 2 * kGhostX, want = (n + 255) / 256, cap = ctx->num_sms * 4;
+    ctx->launches += 1;
+    if (ctx->esize == 4)
+        refresh_ghost_columns_kernel<<<want < cap ? want : cap, 256, 0, ctx->stream>>>(
+            static_cast<float*>(ctx->pop[ctx->cur]), ctx->lp);
+    else
+        refresh_ghost_columns_kernel<<<want < cap ? want : cap, 256, 0, ctx->stream>>>(
+            static_cast<unsigned short*>(ctx->pop[ctx->cur]), ctx->lp);
+    return cudaGetLastError();
+}
+
+template <typename S, bool SR>
+static cudaError_t launch_sweep_src(trtr_ctx* ctx) {
+    return ctx->p.src_mode == TRTR_SRC_PULSE ? launch_sweep_typed<S, TRTR_SRC_PULSE, SR>(ctx)
+                                             : launch_sweep_typed<S, TRTR_SRC_NONE, SR>(ctx);
+}
+
+cudaError_t launch_sweep(trtr_ctx* ctx) {
+    const bool sr = ctx->p.rounding == TRTR_ROUND_STOCHASTIC;
+    switch (ctx->p.precision) {
+        case TRTR_F32: return launch_sweep_src<float, false>(ctx);
+        case TRTR_F16_OFS: return sr ? launch_sweep_src<__half, true>(ctx) : launch_sweep_src<__half, false>(ctx);
+        case TRTR_BF16_OFS:
+            return sr ? launch_sweep_src<__nv_bfloat16, true>(ctx) : launch_sweep_src<__nv_bfloat16, false>(ctx);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+TRTR_BOUNDS_TAKE(sweep)
+
+}  // namespace trtr

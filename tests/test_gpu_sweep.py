@@ -1,0 +1,53 @@
+"""Four steps per launch (strips swept by four time levels behind one another): the bits of one
+launch per step, at the edges of strips (120 columns), of row blocks and of the ghost frames."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2312_10316_gb300 import trtr as T  # noqa: E402
+
+from .test_gpu_step2 import _pulse_solver, _random_solver  # noqa: E402
+
+PREC = {"f32": T.TRTR_F32, "f16": T.TRTR_F16_OFS, "bf16": T.TRTR_BF16_OFS}
+GRIDS = [(16, 32), (38, 40), (120, 64), (122, 35), (124, 33), (240, 34), (250, 300), (37, 50), (1101, 133)]
+
+
+@pytest.mark.parametrize("nx,ny", GRIDS)
+@pytest.mark.parametrize("prec", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("kind", ["none", "pulse"])
+@pytest.mark.parametrize("rounding", [T.TRTR_ROUND_STOCHASTIC, T.TRTR_ROUND_NEAREST])
+def test_sweeps_equal_one_step_launches_bitwise(nx, ny, prec, kind, rounding):
+    if prec == "f32" and rounding == T.TRTR_ROUND_NEAREST:
+        pytest.skip("FP32 storage is not rounded")
+    make = _random_solver if kind == "none" else _pulse_solver
+    kw = dict(precision=PREC[prec], rounding=rounding)
+    if kind == "none" and prec != "f32":
+        kw["phi_ref"] = 0.75
+    out = {}
+    for k in (1, 2):
+        with make(nx, ny, T.TRTR_GRAD_ONESIDED_EDGE, k, **kw) as s:
+            l0 = s.launches
+            s.step(16)  # sweeps only
+            l1 = s.launches
+            s.step(13)  # sweeps and a single step
+            s.step(15)  # sweeps from the one-wide frame that it left, a pair and a single step
+            s.step(66)  # past the levels of the pulse tables' first fill
+            out[k] = (s.get_populations(), s.moments())
+        if k == 2 and (prec == "f32" or nx % 2 == 0):
+            assert l1 - l0 == 2 + 4  # field packing, ghost columns, four sweeps
+    assert np.array_equal(out[1][0], out[2][0], equal_nan=True)
+    assert np.array_equal(out[1][1], out[2][1], equal_nan=True)
+
+
+def test_sweeps_stop_at_the_stability_checks():
+    res = {}
+    for k in (1, 2):
+        with _random_solver(130, 64, T.TRTR_GRAD_PERIODIC, k, check_every=7) as s:
+            s.step(30)
+            res[k] = s.get_populations()
+    assert np.array_equal(res[1], res[2])
