@@ -34,6 +34,13 @@ __constant__ double c_w[kQ] = {4.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0, 1.
 
 constexpr int kThreads = 256;
 
+// The kernels of a time loop are launched with programmatic dependent launch: set up while the kernel
+// before them still runs, they wait here for its completion before they touch memory.
+__device__ __forceinline__ void overlap_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ int wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
 // Value of a field at ghosted position (i, j), i in [-1, nx], j in [-1, ny], from its interior
@@ -97,6 +104,7 @@ __global__ void pulse_fields_kernel(C* uv, C* Dh, C* tab_x, C* tab_y, PlaneLayou
 
 template <typename C>
 __global__ void convert_source_kernel(C* dst, const double* S, PlaneLayout L, double dt) {
+    overlap_launch();
     const size_t n = (size_t)L.nx * L.ny;
     for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
         const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
@@ -146,34 +154,37 @@ __global__ void init_eq_kernel(S* P, const C* uv, const double* phi0, PlaneLayou
 // stored where b pulls it, P_i(b - e_i) (a ghost cell when b - e_i is outside the grid).  A
 // slot P_i(y) is pulled by the node y + e_i alone, so the slots written here (pulled by edge
 // nodes) and the slots read (pulled by interior nodes f) are disjoint: no thread ordering.
+// One thread per edge node and population (threads of a warp share the population), in blocks of one
+// warp: a node's 18 equilibria are 250 FP64 instructions, which on the two SMs of two 256-thread blocks
+// took 20.7 us for the 400 edge nodes of a 101^2 grid, and one population's are 35.
 template <typename S, typename C>
 __global__ void dirichlet_nee_kernel(S* P, const C* uv, const double* phib, PlaneLayout lp, PlaneLayout lf,
                                      C phi_ref) {
+    overlap_launch();
     const int nx = lp.nx, ny = lp.ny, nb = edge_count(nx, ny);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += gridDim.x * blockDim.x) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kQ * nb; e += gridDim.x * blockDim.x) {
+        const int q = e / nb, k = e - q * nb;
         int i, j;
         edge_node(k, nx, ny, &i, &j);
         const int fi = i == 0 ? 1 : (i == nx - 1 ? nx - 2 : i);
         const int fj = j == 0 ? 1 : (j == ny - 1 ? ny - 2 : j);
-        double gf[kQ], phif = 0.0;
+        double gq = 0.0, phif = 0.0;
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            gf[q] = (double)Store<S>::decode(P[q * lp.plane + lp.at(fi - c_ex[q], fj - c_ey[q])],
-                                             (C)(c_w[q]) * phi_ref);
-            phif += gf[q];
+        for (int p = 0; p < kQ; ++p) {
+            const double gf = (double)Store<S>::decode(P[p * lp.plane + lp.at(fi - c_ex[p], fj - c_ey[p])],
+                                                       (C)(c_w[p]) * phi_ref);
+            phif += gf;
+            if (p == q) gq = gf;
         }
         const double ub = (double)uv[lf.at(i, j)], vb = (double)uv[lf.plane + lf.at(i, j)];
         const double uf = (double)uv[lf.at(fi, fj)], vf = (double)uv[lf.plane + lf.at(fi, fj)];
-        const double phi_b = phib[k];
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const double g = equilibrium(q, phi_b, ub, vb) + gf[q] - equilibrium(q, phif, uf, vf);
-            P[q * lp.plane + lp.at(i - c_ex[q], j - c_ey[q])] = Store<S>::encode((C)g, (C)(c_w[q]) * phi_ref);
-        }
+        const double g = equilibrium(q, phib[k], ub, vb) + gq - equilibrium(q, phif, uf, vf);
+        P[q * lp.plane + lp.at(i - c_ex[q], j - c_ey[q])] = Store<S>::encode((C)g, (C)(c_w[q]) * phi_ref);
     }
 }
 
 __global__ void gather_edges_kernel(double* phib, const double* phi, int nx, int ny) {
+    overlap_launch();
     const int nb = edge_count(nx, ny);
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nb; k += gridDim.x * blockDim.x) {
         int i, j;
@@ -321,6 +332,21 @@ int grid_for(const trtr_ctx* ctx, size_t n) {
     return (int)(want < 1 ? 1 : (want > cap ? cap : want));
 }
 
+// A launch that overlaps the tail of the kernel before it (overlap_launch).
+template <typename... P, typename... A>
+void launch_overlapped(trtr_ctx* ctx, void (*kernel)(P...), int grid, int threads, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <typename F>
 cudaError_t dispatch(trtr_ctx* ctx, F&& f) {
     switch (ctx->p.precision) {
@@ -369,8 +395,8 @@ cudaError_t launch_convert_source(trtr_ctx* ctx, const double* S, int buffer) {
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using C = std::remove_pointer_t<decltype(cp)>;
         (void)sp;
-        convert_source_kernel<C><<<grid_for(ctx, n), kThreads, 0, ctx->stream>>>(
-            (C*)ctx->S + (size_t)buffer * ctx->lf.plane, S, ctx->lf, ctx->p.dt);
+        launch_overlapped(ctx, convert_source_kernel<C>, grid_for(ctx, n), kThreads,
+                          (C*)ctx->S + (size_t)buffer * ctx->lf.plane, S, ctx->lf, ctx->p.dt);
     });
 }
 
@@ -447,8 +473,7 @@ cudaError_t launch_sample(trtr_ctx* ctx, const long* nodes, int count, double* o
 cudaError_t launch_gather_edges(trtr_ctx* ctx, const double* phi_b) {
     const int nb = edge_count(ctx->p.nx, ctx->p.ny);
     ctx->launches += 1;
-    gather_edges_kernel<<<(nb + kThreads - 1) / kThreads, kThreads, 0, ctx->stream>>>(ctx->phib, phi_b, ctx->p.nx,
-                                                                                      ctx->p.ny);
+    launch_overlapped(ctx, gather_edges_kernel, (nb + 31) / 32, 32, ctx->phib, phi_b, ctx->p.nx, ctx->p.ny);
     return cudaGetLastError();
 }
 
@@ -458,8 +483,8 @@ cudaError_t launch_dirichlet(trtr_ctx* ctx, void* P) {
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        dirichlet_nee_kernel<S, C><<<(nb + kThreads - 1) / kThreads, kThreads, 0, ctx->stream>>>(
-            (S*)P, (const C*)ctx->uv, ctx->phib, ctx->lp, ctx->lf, (C)ctx->p.phi_ref);
+        launch_overlapped(ctx, dirichlet_nee_kernel<S, C>, (kQ * nb + 31) / 32, 32, (S*)P, (const C*)ctx->uv, ctx->phib,
+                          ctx->lp, ctx->lf, (C)ctx->p.phi_ref);
     });
 }
 
