@@ -317,7 +317,7 @@ trtr_status trtr_adjoint(trtr_ctx* ctx, const double* dJ_dphi, int on_device, do
                 e = trtr::launch_step2_from(ctx, &a->pool_maps2[k], a->pool[k + 2], a->pool[k + 1], a->n0 + s0 + k);
                 k += 2;
             } else {
-                e = trtr::launch_step_from(ctx, &a->pool_maps[k], a->pool[k + 1], a->n0 + s0 + k);
+                e = trtr::launch_step_from(ctx, a->pool[k], &a->pool_maps[k], a->pool[k + 1], a->n0 + s0 + k);
                 k += 1;
             }
         }

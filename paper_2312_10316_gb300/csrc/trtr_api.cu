@@ -16,7 +16,7 @@ namespace trtr {
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out) {
     out[0] = out[1] = out[2] = 0ull;
     cudaError_t (*units[])(cudaStream_t, unsigned long long*) = {bounds_take_step, bounds_take_aux, bounds_take_batch,
-                                                                  bounds_take_adjoint, bounds_take_step2, bounds_take_sweep};
+                                                                  bounds_take_adjoint, bounds_take_step2, bounds_take_sweep, bounds_take_f64};
     for (auto take : units) {
         unsigned long long u[3];
         const cudaError_t e = take(s, u);
@@ -324,6 +324,7 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         {(void**)&ctx->dflag, 4 * sizeof(int), true},  // the timeout flag, then the tile counters
         {(void**)&ctx->phib,
          p->bc_mode == TRTR_BC_DIRICHLET_NEE ? (size_t)trtr::edge_count(p->nx, p->ny) * sizeof(double) : 0, true},
+        {&ctx->pack64, p->precision == TRTR_F64 ? 4 * fld_bytes : 0, true},
         {&ctx->fld2, two_step ? 5 * ctx->lt.plane * sizeof(float) : 0, true},
     };
     // fault injection for tests: TRTR_FAULT_ALLOC=k makes the k-th device allocation here fail
@@ -364,7 +365,7 @@ trtr_status trtr_destroy(trtr_ctx* ctx) {
     cudaGetLastError();
     trtr::free_adjoint(ctx);
     void* ptrs[] = {ctx->pop[0], ctx->pop[1],  ctx->uv,   ctx->Dh,    ctx->S,    ctx->tab_x,
-                    ctx->tab_y,  ctx->scratch, ctx->dres, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab};
+                    ctx->tab_y,  ctx->scratch, ctx->dres, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab, ctx->pack64};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (ctx->hres) cudaFreeHost(ctx->hres);
@@ -456,7 +457,7 @@ trtr_status trtr_set_fields(trtr_ctx* ctx, const double* ux, const double* uy, c
     s = check_launch(ctx, trtr::launch_convert_fields(ctx, dux, duy, dD), "field conversion");
     if (s != TRTR_OK) return s;
     ctx->fields_set = true;
-    ctx->fld2_ready = false;
+    ctx->fld2_ready = ctx->pack64_ready = false;
     if (S) {
         ctx->S_cur = ctx->S_prev = -1;
         // staging slot 0 is reused; the copy into it is ordered after the conversion above
@@ -487,7 +488,7 @@ trtr_status trtr_set_pulse(trtr_ctx* ctx, double omega, double xc, double yc, do
     ctx->pulse_set = true;
     ctx->ptab_ready = false;
     ctx->fields_set = true;
-    ctx->fld2_ready = false;
+    ctx->fld2_ready = ctx->pack64_ready = false;
     return TRTR_OK;
 }
 

@@ -109,6 +109,7 @@ cudaError_t bounds_take_batch(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_adjoint(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_step2(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_sweep(cudaStream_t s, unsigned long long* out);
+cudaError_t bounds_take_f64(cudaStream_t s, unsigned long long* out);
 // All units: the summed count, and the kind and place of the first unit's first access.
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out);
 
@@ -296,6 +297,7 @@ struct trtr_ctx {
     void* tab_y;
     void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
     long ptab_first;  // time level of its first entry
+    bool tables_new;  // filled since the last FP64 step launch
     bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
@@ -315,6 +317,8 @@ struct trtr_ctx {
     bool fld2_ready;        // fld2 holds the current fields
     bool ghost4_ready;      // its four-wide ghost columns are up to date (interior rows)
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
+    void* pack64;           // FP64: [4][rows][pitch] a_x, a_y, k1, k2 (the layout of uv)
+    bool pack64_ready;      // it holds the current fields
     int steps_per_launch;   // 2: trtr_step uses the two-step kernel where it applies; 1: never
     trtr::Pulse pulse;
     long step;
@@ -330,8 +334,9 @@ namespace trtr {
 // return the cudaGetLastError() of the launch.
 cudaError_t encode_maps(trtr_ctx* ctx);
 cudaError_t launch_step(trtr_ctx* ctx);
-// one step from an arbitrary population buffer (its map from encode_pop_map) into dst, as step `step`
-cudaError_t launch_step_from(trtr_ctx* ctx, const CUtensorMap* src_map, void* dst, long step);
+// one step from an arbitrary population buffer src (its map from encode_pop_map) into dst, as step `step`
+cudaError_t launch_step_from(trtr_ctx* ctx, const void* src, const CUtensorMap* src_map, void* dst, long step);
+cudaError_t launch_step_f64(trtr_ctx* ctx, const void* src, void* dst, long step);  // FP64 (trtr_f64.cu)
 cudaError_t encode_pop_map(trtr_ctx* ctx, void* buffer, CUtensorMap* out);
 // The two-step kernel: whether it applies to the context, its maps (at creation), the packed
 // fields (after each change of u or D), and one launch advancing the state by two steps.

@@ -1,4 +1,4 @@
-// trtr_step.cu -- the fused TRT-R time step: one kernel per step does pull-streaming,
+// trtr_step.cu -- the fused TRT-R time step (FP32 and 2-byte storage): one kernel per step does pull-streaming,
 // the phi moment, the TRT-R regularised relaxation, the auxiliary term G and the source
 // term F of the evolution equation (14) of Sec. 2.2, and stores the post-collision values.
 //
@@ -54,14 +54,11 @@ constexpr int kBX = 128;  // nodes per tile along x
 // SMALL_BELOW: grids with fewer than this many of these tiles per SM take the small-grid
 // geometry (SmallPipe below) instead; measured per storage and source mode.
 template <typename S, int SRC>
-struct Geom {  // FP64
-    static constexpr int BY = 8, WPR = 1, CTAS = 2, STAGES = 2, ORDER = 2, TST = 0, SMALL_BELOW = 2;
-    static constexpr bool UNROLL = false;  // UNROLL: the pair loop of the row interleaves both pairs
-};
+struct Geom;
 template <int SRC>
 struct Geom<float, SRC> {  // pulse source
     static constexpr int BY = 16, WPR = 1, CTAS = 1, STAGES = 2, ORDER = 0, TST = 1, SMALL_BELOW = 2;
-    static constexpr bool UNROLL = false;
+    static constexpr bool UNROLL = false;  // UNROLL: the pair loop of the row interleaves both pairs
 };
 template <>
 struct Geom<float, TRTR_SRC_NONE> {  // the small tiles win up to 4096^2 here (not at 8192^2)
@@ -125,7 +122,7 @@ struct Pipe {
                          STAGES = Sweep<S, SRC>::STAGES, ORDER = Sweep<S, SRC>::ORDER;
     static constexpr bool TST = Sweep<S, SRC>::TST != 0 && WPR == 1;
     static constexpr int THREADS = 32 * BY * WPR;
-    static constexpr int PAIRS = BX / 64 / WPR;  // node pairs per lane (FP64: 2 PAIRS nodes)
+    static constexpr int PAIRS = BX / 64 / WPR;  // node pairs per lane
     static constexpr int UNR = Sweep<S, SRC>::UNROLL ? PAIRS : 1;
     static_assert(BY >= 1 && CTAS >= 1 && STAGES >= 1 && THREADS <= 1024, "pipeline geometry");
     static_assert((WPR == 1 || WPR == 2) && PAIRS >= 1, "warps per row");
@@ -158,7 +155,6 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
     constexpr int kBX = G::BX, kBY = G::BY, kWPR = G::WPR, kPairsPerLane = G::PAIRS;
     constexpr bool kTST = G::TST;
     using T = Tile<S, SRC, kBX, kBY>;
-    constexpr bool kPairs = !std::is_same<S, double>::value;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_abort;
     // stages on a 128-byte boundary (TMA destination alignment), barriers after them
@@ -249,7 +245,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
 
         // the pulse source of this lane's pairs, from its tables before the wait (hides their latency)
         F2 psrc[kPairsPerLane];
-        if (kPairs && SRC == TRTR_SRC_PULSE && j < ny) {
+        if (SRC == TRTR_SRC_PULSE && j < ny) {
 #pragma unroll
             for (int m = 0; m < kPairsPerLane; ++m)
                 psrc[m] = pulse_source_dt(reinterpret_cast<const float*>(a.pulse), a.pt, i0 + c0 + 64 * m + 2 * lane, j);
@@ -259,10 +255,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
         if (!ok) s_abort = 1;
         if (ok && j < ny) {
             const unsigned char* st = smem + s * T::STAGE;
-            if constexpr (kPairs)
-                tile_row_pairs<S, SRC, kBX, kBY, kPairsPerLane, kTST, G::UNR, SR>(st, r, lane, i0, j, a, psrc, c0);
-            else
-                tile_row_f64<SRC, kBX, kBY, 2 * kPairsPerLane, kTST>(st, r, lane, i0, j, a, c0);
+            tile_row_pairs<S, SRC, kBX, kBY, kPairsPerLane, kTST, G::UNR, SR>(st, r, lane, i0, j, a, psrc, c0);
         }
         __syncthreads();  // stage s fully read (and s_abort visible)
         if (s_abort) {
@@ -460,7 +453,7 @@ cudaError_t encode_src(trtr_ctx* ctx) {
 // Encodes the context's TMA descriptors and picks its tile geometry (ctx->small_tiles).
 cudaError_t encode_maps(trtr_ctx* ctx) {
     switch (ctx->p.precision) {
-        case TRTR_F64: return encode_src<double>(ctx);
+        case TRTR_F64: return cudaSuccess;  // no TMA (trtr_f64.cu)
         case TRTR_F32: return encode_src<float>(ctx);
         case TRTR_F16_OFS: return encode_src<__half>(ctx);
         case TRTR_BF16_OFS: return encode_src<__nv_bfloat16>(ctx);
@@ -488,6 +481,7 @@ cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
     const cudaError_t e = cudaGetLastError();
     ctx->ptab_first = step - 1;
     ctx->ptab_ready = e == cudaSuccess;
+    ctx->tables_new = true;
     return e;
 }
 
@@ -503,9 +497,9 @@ cudaError_t launch_bounds_probe(trtr_ctx* ctx) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_from(trtr_ctx* ctx, const CUtensorMap* src_map, void* dst, long step) {
+cudaError_t launch_step_from(trtr_ctx* ctx, const void* src, const CUtensorMap* src_map, void* dst, long step) {
     switch (ctx->p.precision) {
-        case TRTR_F64: return launch_src<double>(ctx, *src_map, dst, step);
+        case TRTR_F64: return launch_step_f64(ctx, src, dst, step);
         case TRTR_F32: return launch_src<float>(ctx, *src_map, dst, step);
         case TRTR_F16_OFS: return launch_src<__half>(ctx, *src_map, dst, step);
         case TRTR_BF16_OFS: return launch_src<__nv_bfloat16>(ctx, *src_map, dst, step);
@@ -514,12 +508,12 @@ cudaError_t launch_step_from(trtr_ctx* ctx, const CUtensorMap* src_map, void* ds
 }
 
 cudaError_t launch_step(trtr_ctx* ctx) {
-    return launch_step_from(ctx, &ctx->maps[kMapPop0 + ctx->cur], ctx->pop[ctx->cur ^ 1], ctx->step);
+    return launch_step_from(ctx, ctx->pop[ctx->cur], &ctx->maps[kMapPop0 + ctx->cur], ctx->pop[ctx->cur ^ 1], ctx->step);
 }
 
 cudaError_t encode_pop_map(trtr_ctx* ctx, void* buffer, CUtensorMap* out) {
     switch (ctx->p.precision) {
-        case TRTR_F64: return encode_pop_typed<double>(ctx, buffer, out);
+        case TRTR_F64: return cudaSuccess;
         case TRTR_F32: return encode_pop_typed<float>(ctx, buffer, out);
         case TRTR_F16_OFS: return encode_pop_typed<__half>(ctx, buffer, out);
         case TRTR_BF16_OFS: return encode_pop_typed<__nv_bfloat16>(ctx, buffer, out);

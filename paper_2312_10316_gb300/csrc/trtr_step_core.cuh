@@ -195,7 +195,7 @@ struct TileCursor {
 
 // ---- arithmetic types --------------------------------------------------------------------
 // FP32-computing storages work on pairs of adjacent nodes with the packed FP32 instructions
-// of sm_100-family SMs (two lanes of FP32 per FADD2 / FMUL2 / FFMA2); FP64 works per node.
+// of sm_100-family SMs (two lanes of FP32 per FADD2 / FMUL2 / FFMA2).
 struct F2 {
     float2 v;
     __device__ __forceinline__ F2() {}
@@ -207,20 +207,7 @@ __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(__fadd2_rn(a.v, 
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return F2(__ffma2_rn(b.v, make_float2(-1.f, -1.f), a.v)); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
-__device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ F2 vdiv(F2 a, F2 b) { return F2(__fdividef(a.v.x, b.v.x), __fdividef(a.v.y, b.v.y)); }
-__device__ __forceinline__ double vdiv(double a, double b) { return a / b; }
-
-template <class V>
-struct ScalarOf;
-template <>
-struct ScalarOf<F2> {
-    using type = float;
-};
-template <>
-struct ScalarOf<double> {
-    using type = double;
-};
 
 // s = dt S^n + dt/2 (S^n - S^{n-1}) = 1.5 dt S^n - 0.5 dt S^{n-1} (a7, Eqs. (3) and (14)) of the
 // manufactured source at the node pair (i, i + 1) (i even, images included) or the node i of row
@@ -324,7 +311,7 @@ inline const C* pulse_level(const trtr_ctx* ctx, const PulseTab& t, long step) {
 template <typename V, bool OFS = false>
 __device__ __forceinline__ void collide_node(const V g[kQ], V ux, V uy, V ax, V ay, V Dh, V s, V magic, V w2_fixed,
                                              bool tau2_fixed, V out[kQ], V phi_ref = V(0.f)) {
-    using T = typename ScalarOf<V>::type;
+    using T = float;
     // relaxation rates: tau1 - 1/2 = 3 Dh (Sec. 2.4); tau2 from Lambda (Eq. (28)) or fixed
     const V t1m = V(T(3)) * Dh;
     const V w1 = vdiv(V(T(1)), V(T(0.5)) + t1m);
@@ -660,79 +647,6 @@ __device__ __forceinline__ void tile_row_pairs(const unsigned char* st, int r, i
     }
 }
 
-// One tile row of the FP64 path, or NMF * 32 columns of it from column c0: lane handles nodes
-// i0 + c0 + 32 m + lane, m = 0 .. NMF - 1.  TST: bulk row stores as in tile_row_pairs.
-template <int SRC, int BX, int BY, int NMF = BX / 32, bool TST = false>
-__device__ __forceinline__ void tile_row_f64(const unsigned char* st, int r, int lane, int i0, int j,
-                                             const StepArgs<double>& a, int c0 = 0) {
-    static_assert(!TST || NMF == BX / 32, "bulk row stores need one warp per tile row");
-    using T = Tile<double, SRC, BX, BY>;
-    const int nx = a.lp.nx;
-    const double* sp = reinterpret_cast<const double*>(st) + r * T::PW;
-    const double* su = reinterpret_cast<const double*>(st + T::POP) + (r + 1) * T::UW + T::AC;
-    const double* sv = su + T::UH * T::UW;
-    const double* sd = reinterpret_cast<const double*>(st + T::POP + T::U) + r * BX;
-    const double* ss = reinterpret_cast<const double*>(st + T::POP + T::U + T::D) + r * BX;
-    double* dst = static_cast<double*>(a.dst);
-    const size_t pl = a.lp.plane;
-#pragma unroll 1
-    for (int m = 0; m < NMF; ++m) {
-        const int c = c0 + 32 * m + lane;
-        const int i = i0 + c;
-        if (!TST && i >= nx) break;
-        double g[kQ];
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) g[q] = sp[q * T::PLANE_ELEMS + c + plane_offset<T::A>(q)];
-        const double ux = su[c], uy = sv[c];
-        const double dxux = 0.5 * (su[c + 1] - su[c - 1]);
-        const double dxuy = 0.5 * (sv[c + 1] - sv[c - 1]);
-        const double dyux = 0.5 * (su[c + T::UW] - su[c - T::UW]);
-        const double dyuy = 0.5 * (sv[c + T::UW] - sv[c - T::UW]);
-        const double ax = fma(ux, dxux, uy * dyux);
-        const double ay = fma(ux, dxuy, uy * dyuy);
-        double src = 0.0;
-        if (SRC == TRTR_SRC_FIELD) {
-            src = fma(1.5, ss[c], -0.5 * ss[T::S_TILE / sizeof(double) + c]);
-        } else if (SRC == TRTR_SRC_PULSE) {
-            src = pulse_source_dt(a.pulse, a.pt, i, j);
-        }
-        double out[kQ];
-        collide_node<double>(g, ux, uy, ax, ay, sd[c], src, a.magic, a.omega2_fixed, a.tau2_fixed, out);
-        if constexpr (TST) {
-            __syncwarp();  // every lane has read its inputs of node m
-            double* srow = const_cast<double*>(sp);
-#pragma unroll
-            for (int q = 0; q < kQ; ++q) srow[q * T::PLANE_ELEMS + c] = out[q];
-            if (i < nx) {
-                const bool tail = c >= bulk_cols<double>(nx - i0);
-#pragma unroll
-                for (int q = 0; q < kQ; ++q) {
-                    if (tail) dst[q * pl + a.lp.at_g<kGhostP>(i, j)] = out[q];
-                    store_ghosts<1, kGhostP>(dst + q * pl, a.lp, i, j, out[q]);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < kQ; ++q) store_with_ghosts<1, kGhostP>(dst + q * pl, a.lp, i, j, out[q]);
-        }
-    }
-    if constexpr (TST) {
-        fence_proxy_async_smem();
-        __syncwarp();
-        const int nb = bulk_cols<double>(nx - i0);
-        if (lane == 0 && nb > 0) {
-#pragma unroll
-            for (int q = 0; q < kQ; ++q)
-                if (bulk_ok(dst + q * pl + a.lp.at_g<kGhostP>(i0, j), sp + q * T::PLANE_ELEMS, i0, j, nb, a.lp))
-                    bulk_store(dst + q * pl + a.lp.at_g<kGhostP>(i0, j), sp + q * T::PLANE_ELEMS,
-                               (uint32_t)(nb * sizeof(double)));
-            bulk_commit();
-            bulk_wait_read();
-        }
-    }
-}
-
-
 // ---- host side: TMA descriptors --------------------------------------------------------
 
 // L2 fill granularity of the TMA loads: 0 none, 1 64 B, 2 128 B, 3 256 B.
@@ -742,8 +656,6 @@ __device__ __forceinline__ void tile_row_f64(const unsigned char* st, int r, int
 
 template <typename S>
 CUtensorMapDataType tma_type();
-template <>
-inline CUtensorMapDataType tma_type<double>() { return CU_TENSOR_MAP_DATA_TYPE_FLOAT64; }
 template <>
 inline CUtensorMapDataType tma_type<float>() { return CU_TENSOR_MAP_DATA_TYPE_FLOAT32; }
 template <>
