@@ -164,13 +164,12 @@ trtr_status check_launch(trtr_ctx* ctx, cudaError_t e, const char* what) {
     return TRTR_OK;
 }
 
-// Synchronises the context's stream and reports a step kernel whose bounded wait gave up.  The
-// flag is cleared once reported, so the context stays usable.
-trtr_status sync_and_check(trtr_ctx* ctx, const char* where) {
-    int* hflag = reinterpret_cast<int*>(ctx->hres + 3);
-    TRTR_CUDA(ctx, cudaMemcpyAsync(hflag, ctx->dflag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), where);
+// Synchronises the context's stream and reports a step kernel whose bounded wait gave up, from the
+// pinned copy of the flag that the last kernel wrote.  The flag is cleared once reported, so the
+// context stays usable.
+trtr_status wait_and_check(trtr_ctx* ctx, const char* where) {
     TRTR_CUDA(ctx, cudaStreamSynchronize(ctx->stream), where);
-    if (*hflag != 0) {
+    if (*reinterpret_cast<int*>(ctx->hres + 3) != 0) {
         TRTR_CUDA(ctx, cudaMemsetAsync(ctx->dflag, 0, sizeof(int), ctx->stream), where);
         return fail(ctx, TRTR_ETIMEOUT, "%s: a kernel timed out waiting for its loads", where);
     }
@@ -183,14 +182,17 @@ trtr_status sync_and_check(trtr_ctx* ctx, const char* where) {
 #endif
     return TRTR_OK;
 }
+// The same after work that does not write the copy.
+trtr_status sync_and_check(trtr_ctx* ctx, const char* where) {
+    TRTR_CUDA(ctx, cudaMemcpyAsync(ctx->hres + 3, ctx->dflag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), where);
+    return wait_and_check(ctx, where);
+}
 
 trtr_status reduce(trtr_ctx* ctx, int kind, const double* ref_dev, double out[2]) {
     trtr::TraceRange trace("trtr reduce");
     trtr_status s = check_launch(ctx, trtr::launch_reduce(ctx, kind, ref_dev), "reduction launch");
     if (s != TRTR_OK) return s;
-    TRTR_CUDA(ctx, cudaMemcpyAsync(ctx->hres, ctx->dres, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
-              "reduction result copy");
-    s = sync_and_check(ctx, "reduction");
+    s = wait_and_check(ctx, "reduction");
     if (s != TRTR_OK) return s;
     out[0] = ctx->hres[0];
     out[1] = ctx->hres[1];
@@ -320,7 +322,7 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
              : 0,
          true},
         {(void**)&ctx->scratch, 2 * (size_t)ctx->red_blocks * sizeof(double), false},
-        {(void**)&ctx->dres, 4 * sizeof(double), false},
+        {(void**)&ctx->red_done, sizeof(unsigned), true},
         {(void**)&ctx->dflag, 4 * sizeof(int), true},  // the timeout flag, then the tile counters
         {(void**)&ctx->phib,
          p->bc_mode == TRTR_BC_DIRICHLET_NEE ? (size_t)trtr::edge_count(p->nx, p->ny) * sizeof(double) : 0, true},
@@ -365,7 +367,7 @@ trtr_status trtr_destroy(trtr_ctx* ctx) {
     cudaGetLastError();
     trtr::free_adjoint(ctx);
     void* ptrs[] = {ctx->pop[0], ctx->pop[1],  ctx->uv,   ctx->Dh,    ctx->S,    ctx->tab_x,
-                    ctx->tab_y,  ctx->scratch, ctx->dres, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab, ctx->pack64};
+                    ctx->tab_y,  ctx->scratch, ctx->red_done, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab, ctx->pack64};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (ctx->hres) cudaFreeHost(ctx->hres);
@@ -566,7 +568,7 @@ trtr_status trtr_moments(trtr_ctx* ctx, double* phi_out, int on_device) {
     if (!on_device)
         TRTR_CUDA(ctx, cudaMemcpyAsync(phi_out, dev, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
                   "device-to-host copy");
-    return sync_and_check(ctx, "moments");
+    return wait_and_check(ctx, "moments");
 }
 
 trtr_status trtr_mass(trtr_ctx* ctx, double* sum_phi) {
@@ -628,7 +630,7 @@ trtr_status trtr_get_populations(trtr_ctx* ctx, double* g_out, int on_device) {
     if (!on_device)
         TRTR_CUDA(ctx, cudaMemcpyAsync(g_out, dev, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream),
                   "device-to-host copy");
-    return sync_and_check(ctx, "get populations");
+    return wait_and_check(ctx, "get populations");
 }
 
 trtr_status trtr_set_populations(trtr_ctx* ctx, const double* g, int on_device, long step) {

@@ -6,7 +6,7 @@
 
 #include <type_traits>
 
-#include "trtr_internal.cuh"
+#include "trtr_step_core.cuh"
 
 namespace trtr {
 
@@ -105,9 +105,9 @@ __global__ void pulse_fields_kernel(C* uv, C* Dh, C* tab_x, C* tab_y, PlaneLayou
 template <typename C>
 __global__ void convert_source_kernel(C* dst, const double* S, PlaneLayout L, double dt) {
     overlap_launch();
-    const size_t n = (size_t)L.nx * L.ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
+    const unsigned n = (unsigned)L.nx * L.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
         dst[L.at(i, j)] = C(dt * S[k]);
     }
 }
@@ -127,24 +127,51 @@ __device__ __forceinline__ T equilibrium(int q, T phi, T u, T v) {
            (T(1) + T(3) * eu + T(4.5) * (eu * eu - uu / T(3)) + T(4.5) * (eu * eu * eu - eu * uu));
 }
 
+// Stores value v of population q that node (i, j) pulls, P_q(x - e_q), periodic images included.
+template <typename S>
+__device__ __forceinline__ void store_pulled(S* P, const PlaneLayout& L, int q, int i, int j, bool inner, S v) {
+    S* plane = P + q * L.plane;
+    if (inner)  // the slot and its neighbours are away from the ghost frame
+        plane[L.at(i - c_ex[q], j - c_ey[q])] = v;
+    else
+        store_with_ghosts(plane, L, wrap(i - c_ex[q], L.nx), wrap(j - c_ey[q], L.ny), v);
+}
+__device__ __forceinline__ bool inner_node(const PlaneLayout& L, int i, int j) {
+    return i > L.gy && i < L.nx - 1 - L.gy && j > L.gy && j < L.ny - 1 - L.gy;
+}
+
 // Initial condition g_i(x) = g_i^eq(phi0(x), u(x)) in the pull layout: node x evaluates phi0
 // once (FP64) and its nine equilibria in the compute type, and stores g_i(x) where x pulls it,
-// P_i(x - e_i), periodic images included (each slot has exactly one writer).
+// P_i(x - e_i), periodic images included (each slot has exactly one writer).  A thread takes `rows`
+// rows of one column; the pulse's phi0 is the product of a factor of x, taken once a thread, and one
+// of y, taken once a block and row: an FP64 exponential a node is 45 FP64 instructions and made this
+// kernel 0.9 ms at 4096^2.
+constexpr int kInitRows = 32;
 template <typename S, typename C>
-__global__ void init_eq_kernel(S* P, const C* uv, const double* phi0, PlaneLayout lp, PlaneLayout lf, double x0,
-                               double y0, double dx, PulseTime pt, C phi_ref) {
-    const int nx = lp.nx, ny = lp.ny;
-    const size_t n = (size_t)nx * ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / nx), i = (int)(k - (size_t)j * nx);
-        const C phi = (C)(phi0 ? phi0[k] : pulse_phi(pt, x0 + i * dx, y0 + j * dx));
-        const C u = uv[lf.at(i, j)], v = uv[lf.plane + lf.at(i, j)];
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const int ti = wrap(i - c_ex[q], nx), tj = wrap(j - c_ey[q], ny);
-            store_with_ghosts(P + q * lp.plane, lp, ti, tj,
-                              Store<S>::encode(equilibrium<C>(q, phi, u, v), (C)(c_w[q]) * phi_ref));
+__global__ void __launch_bounds__(128)
+    init_eq_kernel(S* P, const C* uv, const double* phi0, PlaneLayout lp, PlaneLayout lf, double x0, double y0, double dx,
+                   PulseTime pt, C phi_ref, int rows) {
+    __shared__ double fy[kInitRows];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j0 = blockIdx.y * rows;
+    double fx = 0.0;
+    if (!phi0) {
+        const double rx = x0 + i * dx - pt.cx;
+        fx = pt.amp * exp(-0.5 * rx * rx * pt.inv_s2);
+        if (threadIdx.x < (unsigned)rows) {
+            const double ry = y0 + (j0 + (int)threadIdx.x) * dx - pt.cy;
+            fy[threadIdx.x] = exp(-0.5 * ry * ry * pt.inv_s2);
         }
+        __syncthreads();
+    }
+    if (i >= lp.nx) return;
+    for (int r = 0; r < rows && j0 + r < lp.ny; ++r) {
+        const int j = j0 + r;
+        const C phi = (C)(phi0 ? phi0[(size_t)j * lp.nx + i] : fx * fy[r]);
+        const C u = uv[lf.at(i, j)], v = uv[lf.plane + lf.at(i, j)];
+        const bool inner = inner_node(lp, i, j);
+#pragma unroll
+        for (int q = 0; q < kQ; ++q)
+            store_pulled(P, lp, q, i, j, inner, Store<S>::encode(equilibrium<C>(q, phi, u, v), (C)(c_w[q]) * phi_ref));
     }
 }
 
@@ -208,12 +235,92 @@ __device__ __forceinline__ double node_phi(const S* P, int i, int j, const Plane
     return phi;
 }
 
+// The FP32-computing storages: phi of the node pair (i, i + 1) as an unevaluated sum s + c + t of floats,
+// exact to beyond FP64 (two levels of Knuth's error-free two-sum).  Converting the nine floats to
+// FP64 and adding them there takes 17 instructions of the FP64 pipe (16 cycles each), which held
+// these kernels at 36 G nodes/s; s + c + t leaves 5 of them.
+using core::F2;
+struct PhiPair {
+    F2 s, c, t;
+};
+__device__ __forceinline__ F2 two_sum(F2 a, F2 b, F2& e) {
+    const F2 s = a + b, bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+    return s;
+}
+template <typename S>
+__device__ __forceinline__ void pulled_pair(const S* P, int i, int j, const PlaneLayout& L, float phi_ref, F2 g[kQ]) {
+    using S2 = typename core::Pair<S>::type;
+    const S* at = P + L.at(i, j);
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+        const S* p = at + q * L.plane - (ptrdiff_t)lattice_ey(q) * L.pitch - lattice_ex(q);
+        const float off = core::weight<float>(q) * phi_ref;
+        g[q] = lattice_ex(q) == 0 ? core::Pair<S>::decode(*reinterpret_cast<const S2*>(p), off)
+                                  : core::Pair<S>::decode(p[0], p[1], off);
+    }
+}
+template <typename S>
+__device__ __forceinline__ PhiPair pair_phi(const S* P, int i, int j, const PlaneLayout& L, float phi_ref) {
+    F2 g[kQ];
+    pulled_pair(P, i, j, L, phi_ref, g);
+    PhiPair r;
+    r.s = two_sum(g[0], g[1], r.c);
+    r.t = F2(0.f);
+#pragma unroll
+    for (int q = 2; q < kQ; ++q) {
+        F2 e, ee;
+        r.s = two_sum(r.s, g[q], e);
+        r.c = two_sum(r.c, e, ee);
+        r.t = r.t + ee;
+    }
+    return r;
+}
+// The value in FP64; sums near the end of the float range (and beyond it, infinities and NaN) are
+// taken in FP64 from the populations.
+__device__ __forceinline__ bool float_sum_ok(float s) { return fabsf(s) < 1e36f; }
+template <typename S>
+__device__ __forceinline__ double phi_value(float s, float c, float t, const S* P, int i, int j, const PlaneLayout& L,
+                                            float phi_ref) {
+    return float_sum_ok(s) ? (double)s + ((double)c + (double)t) : node_phi<S, float>(P, i, j, L, phi_ref);
+}
+
+// The kernels that a host call waits for put the step kernels' timeout flag into its pinned copy.
+__device__ __forceinline__ void report_flag(const int* flag, int* host_flag) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *host_flag = *flag;
+}
+
 template <typename S, typename C>
-__global__ void moments_kernel(double* out, const S* P, PlaneLayout L, C phi_ref) {
-    const size_t n = (size_t)L.nx * L.ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
-        out[k] = node_phi<S, C>(P, i, j, L, phi_ref);
+__global__ void __launch_bounds__(kThreads)
+    moments_kernel(double* out, const S* P, PlaneLayout L, C phi_ref, const int* flag, int* host_flag) {
+    overlap_launch();
+    report_flag(flag, host_flag);
+    if constexpr (sizeof(S) == 8) {
+        const unsigned n = (unsigned)L.nx * L.ny;
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
+            out[k] = node_phi<S, C>(P, i, j, L, phi_ref);
+        }
+    } else {
+        const unsigned np = (L.nx + 1) / 2, n = np * L.ny;
+        const bool wide = L.nx % 2 == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0u;
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+            const int j = (int)(k / np), i = 2 * (int)(k - (unsigned)j * np);
+            const PhiPair p = pair_phi(P, i, j, L, phi_ref);
+            double* o = out + (size_t)j * L.nx + i;
+            const double a = phi_value(p.s.v.x, p.c.v.x, p.t.v.x, P, i, j, L, phi_ref);
+            if (i + 1 < L.nx) {
+                const double b = phi_value(p.s.v.y, p.c.v.y, p.t.v.y, P, i + 1, j, L, phi_ref);
+                if (wide) {
+                    *reinterpret_cast<double2*>(o) = make_double2(a, b);
+                } else {
+                    o[0] = a;
+                    o[1] = b;
+                }
+            } else {
+                o[0] = a;
+            }
+        }
     }
 }
 
@@ -242,77 +349,146 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
     }
 }
 
-// Per-block FP64 partial sums into scratch[2 * block + {0, 1}]:
-//  kind 0: sum phi;  1: sum (phi - phi_a)^2, sum phi_a^2;  2: same against phi_ref field;
-//  3: number of non-finite populations;  4: number of values of ref that are not finite and > 0.
-template <typename S, typename C>
-__global__ void reduce_kernel(double* partial, const S* P, PlaneLayout L, C phi_ref, int kind, PulseTime pt,
-                              double x0, double y0, double dx, const double* ref) {
-    const size_t n = (size_t)L.nx * L.ny;
-    double a = 0.0, b = 0.0;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
-        if (kind == kReduceBadField) {
+// A thread's part of a reduction of kind KIND:
+//  kReduceMass: sum phi;  kReducePulse: sum (phi - phi_a)^2, sum phi_a^2;  kReduceField: same against
+//  the field ref;  kReduceNonFinite: number of non-finite populations;  kReduceBadField: number of
+//  values of ref that are not finite and > 0.
+template <typename S, typename C, int KIND>
+__device__ __forceinline__ void reduce_nodes(const S* P, const PlaneLayout& L, C phi_ref, const PulseTime& pt, double x0,
+                                             double y0, double dx, const double* ref, double& a, double& b) {
+    const unsigned stride = gridDim.x * blockDim.x, first = blockIdx.x * blockDim.x + threadIdx.x;
+    auto against = [&](double phi, int i, int j) {
+        const double r = KIND == kReducePulse ? pulse_phi(pt, x0 + i * dx, y0 + j * dx) : ref[(size_t)j * L.nx + i];
+        const double d = phi - r;
+        a += d * d;
+        b += r * r;
+    };
+    if constexpr (KIND == kReduceBadField) {
+        const unsigned n = (unsigned)L.nx * L.ny;
+        unsigned bad = 0;
+        for (unsigned k = first; k < n; k += stride) {
             const double v = ref[k];
-            a += (v > 0.0 && isfinite(v)) ? 0.0 : 1.0;
-            continue;
+            bad += (v > 0.0 && isfinite(v)) ? 0u : 1u;
         }
-        if (kind == kReduceNonFinite) {
-            for (int q = 0; q < kQ; ++q) {
-                const double v = (double)pulled<S, C>(P, q, i, j, L, phi_ref);
-                a += isfinite(v) ? 0.0 : 1.0;
+        a = (double)bad;
+    } else if constexpr (sizeof(S) == 8) {
+        const unsigned n = (unsigned)L.nx * L.ny;
+        unsigned bad = 0;
+        for (unsigned k = first; k < n; k += stride) {
+            const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
+            if constexpr (KIND == kReduceNonFinite) {
+#pragma unroll
+                for (int q = 0; q < kQ; ++q) bad += isfinite(pulled<S, C>(P, q, i, j, L, phi_ref)) ? 0u : 1u;
+            } else {
+                const double phi = node_phi<S, C>(P, i, j, L, phi_ref);
+                if constexpr (KIND == kReduceMass)
+                    a += phi;
+                else
+                    against(phi, i, j);
             }
-            continue;
         }
-        const double phi = node_phi<S, C>(P, i, j, L, phi_ref);
-        if (kind == kReduceMass) {
-            a += phi;
-        } else {
-            const double r = kind == kReducePulse ? pulse_phi(pt, x0 + i * dx, y0 + j * dx) : ref[k];
-            const double d = phi - r;
-            a += d * d;
-            b += r * r;
+        if constexpr (KIND == kReduceNonFinite) a = (double)bad;
+    } else {
+        const unsigned np = (L.nx + 1) / 2, n = np * L.ny;
+        unsigned bad = 0;
+        F2 s(0.f), c(0.f), t(0.f);  // mass: the thread's sum as s + c + t too
+        for (unsigned k = first; k < n; k += stride) {
+            const int j = (int)(k / np), i = 2 * (int)(k - (unsigned)j * np);
+            const bool two = i + 1 < L.nx;
+            if constexpr (KIND == kReduceNonFinite) {
+                F2 g[kQ];
+                pulled_pair(P, i, j, L, phi_ref, g);
+#pragma unroll
+                for (int q = 0; q < kQ; ++q) bad += (isfinite(g[q].v.x) ? 0u : 1u) + (two && !isfinite(g[q].v.y) ? 1u : 0u);
+            } else {
+                PhiPair p = pair_phi(P, i, j, L, phi_ref);
+                if constexpr (KIND == kReduceMass) {
+                    if (!float_sum_ok(p.s.v.x)) {
+                        a += node_phi<S, C>(P, i, j, L, phi_ref);
+                        p.s.v.x = p.c.v.x = p.t.v.x = 0.f;
+                    }
+                    if (!two || !float_sum_ok(p.s.v.y)) {
+                        if (two) a += node_phi<S, C>(P, i + 1, j, L, phi_ref);
+                        p.s.v.y = p.c.v.y = p.t.v.y = 0.f;
+                    }
+                    F2 e, f, g;
+                    s = two_sum(s, p.s, e);
+                    c = two_sum(c, p.c, f);
+                    c = two_sum(c, e, g);
+                    t = t + ((p.t + f) + g);
+                    if (!(fabsf(s.v.x) < 1e36f && fabsf(s.v.y) < 1e36f)) {  // long before the float range ends
+                        a += ((double)s.v.x + (double)s.v.y) + ((double)c.v.x + (double)c.v.y);
+                        s = c = F2(0.f);
+                    }
+                } else {
+                    against(phi_value(p.s.v.x, p.c.v.x, p.t.v.x, P, i, j, L, phi_ref), i, j);
+                    if (two) against(phi_value(p.s.v.y, p.c.v.y, p.t.v.y, P, i + 1, j, L, phi_ref), i + 1, j);
+                }
+            }
         }
+        if constexpr (KIND == kReduceNonFinite) a = (double)bad;
+        if constexpr (KIND == kReduceMass)
+            a += (((double)s.v.x + (double)s.v.y) + ((double)c.v.x + (double)c.v.y)) + ((double)t.v.x + (double)t.v.y);
     }
+}
+
+// Per-block FP64 partial sums into partial[2 * block + {0, 1}]; the last block to finish sums them in a
+// fixed order into the pinned host result, beside the timeout flag.
+template <typename S, typename C, int KIND>
+__global__ void __launch_bounds__(kThreads)
+    reduce_kernel(double* partial, unsigned* done, const S* P, PlaneLayout L, C phi_ref, PulseTime pt, double x0, double y0,
+                  double dx, const double* ref, double* result, const int* flag, int* host_flag) {
+    overlap_launch();
+    __shared__ bool last;
+    double a = 0.0, b = 0.0;
+    reduce_nodes<S, C, KIND>(P, L, phi_ref, pt, x0, y0, dx, ref, a, b);
     block_sum2(a, b);
     if (threadIdx.x == 0) {
         partial[2 * blockIdx.x] = a;
         partial[2 * blockIdx.x + 1] = b;
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
     }
-}
-
-__global__ void finish_kernel(double* out, const double* partial, int nblocks) {
-    double a = 0.0, b = 0.0;
-    for (int k = threadIdx.x; k < nblocks; k += blockDim.x) {
-        a += partial[2 * k];
-        b += partial[2 * k + 1];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    a = b = 0.0;
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
+        a += __ldcg(&partial[2 * k]);
+        b += __ldcg(&partial[2 * k + 1]);
     }
+    __syncthreads();  // block_sum2's shared arrays are used again
     block_sum2(a, b);
     if (threadIdx.x == 0) {
-        out[0] = a;
-        out[1] = b;
+        result[0] = a;
+        result[1] = b;
+        *host_flag = *flag;
+        *done = 0u;
     }
 }
 
 template <typename S, typename C>
-__global__ void get_pop_kernel(double* g, const S* P, PlaneLayout L, C phi_ref) {
-    const size_t n = (size_t)L.nx * L.ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
-        for (int q = 0; q < kQ; ++q) g[q * n + k] = (double)pulled<S, C>(P, q, i, j, L, phi_ref);
+__global__ void get_pop_kernel(double* g, const S* P, PlaneLayout L, C phi_ref, const int* flag, int* host_flag) {
+    overlap_launch();
+    report_flag(flag, host_flag);
+    const unsigned n = (unsigned)L.nx * L.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) g[(size_t)q * n + k] = (double)pulled<S, C>(P, q, i, j, L, phi_ref);
     }
 }
 
 template <typename S, typename C>
 __global__ void set_pop_kernel(S* P, const double* g, PlaneLayout L, C phi_ref) {
-    const size_t n = (size_t)L.nx * L.ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
-        const int j = (int)(k / L.nx), i = (int)(k - (size_t)j * L.nx);
-        for (int q = 0; q < kQ; ++q) {
-            const int si = wrap(i + c_ex[q], L.nx), sj = wrap(j + c_ey[q], L.ny);
-            store_with_ghosts(P + q * L.plane, L, i, j,
-                              Store<S>::encode((C)g[q * n + (size_t)sj * L.nx + si], (C)(c_w[q]) * phi_ref));
-        }
+    overlap_launch();
+    const unsigned n = (unsigned)L.nx * L.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
+        const bool inner = inner_node(L, i, j);
+#pragma unroll
+        for (int q = 0; q < kQ; ++q)
+            store_pulled(P, L, q, i, j, inner, Store<S>::encode((C)g[(size_t)q * n + k], (C)(c_w[q]) * phi_ref));
     }
 }
 
@@ -346,6 +522,9 @@ void launch_overlapped(trtr_ctx* ctx, void (*kernel)(P...), int grid, int thread
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+
+// The pinned copy of the timeout flag.
+int* host_flag(trtr_ctx* ctx) { return reinterpret_cast<int*>(ctx->hres + 3); }
 
 template <typename F>
 cudaError_t dispatch(trtr_ctx* ctx, F&& f) {
@@ -401,15 +580,18 @@ cudaError_t launch_convert_source(trtr_ctx* ctx, const double* S, int buffer) {
 }
 
 cudaError_t launch_init_equilibrium(trtr_ctx* ctx, const double* phi0) {
-    const size_t n = (size_t)ctx->p.nx * ctx->p.ny;
+    // rows a thread: as many as leave eight blocks an SM
+    const int columns = (ctx->p.nx + 127) / 128;
+    const long share = (long)ctx->p.ny * columns / (8L * ctx->num_sms);
+    const int rows = share < 1 ? 1 : (share > kInitRows ? kInitRows : (int)share);
     const PulseTime pt = pulse_at(ctx->pulse, 0.0);
     ctx->launches += 1;
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        init_eq_kernel<S, C><<<grid_for(ctx, n), kThreads, 0, ctx->stream>>>(
+        init_eq_kernel<S, C><<<dim3(columns, (ctx->p.ny + rows - 1) / rows), 128, 0, ctx->stream>>>(
             (S*)ctx->pop[ctx->cur], (const C*)ctx->uv, phi0, ctx->lp, ctx->lf, ctx->p.x0, ctx->p.y0, ctx->p.dx, pt,
-            (C)ctx->p.phi_ref);
+            (C)ctx->p.phi_ref, rows);
     });
 }
 
@@ -419,22 +601,33 @@ cudaError_t launch_moments(trtr_ctx* ctx, double* phi_out) {
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        moments_kernel<S, C><<<grid_for(ctx, n), kThreads, 0, ctx->stream>>>(phi_out, (const S*)ctx->pop[ctx->cur],
-                                                                             ctx->lp, (C)ctx->p.phi_ref);
+        launch_overlapped(ctx, moments_kernel<S, C>, grid_for(ctx, sizeof(S) == 8 ? n : (n + 1) / 2), kThreads, phi_out,
+                          (const S*)ctx->pop[ctx->cur], ctx->lp, (C)ctx->p.phi_ref, ctx->dflag, host_flag(ctx));
+    });
+}
+
+template <int KIND>
+cudaError_t launch_reduce_kind(trtr_ctx* ctx, const double* ref) {
+    const PulseTime pt = pulse_at(ctx->pulse, (double)ctx->step * ctx->p.dt);
+    ctx->launches += 1;
+    return dispatch(ctx, [&](auto* sp, auto* cp) {
+        using S = std::remove_pointer_t<decltype(sp)>;
+        using C = std::remove_pointer_t<decltype(cp)>;
+        launch_overlapped(ctx, reduce_kernel<S, C, KIND>, ctx->red_blocks, kThreads, ctx->scratch,
+                          ctx->red_done, (const S*)ctx->pop[ctx->cur], ctx->lp,
+                          (C)ctx->p.phi_ref, pt, ctx->p.x0, ctx->p.y0, ctx->p.dx, ref, ctx->hres, ctx->dflag, host_flag(ctx));
     });
 }
 
 cudaError_t launch_reduce(trtr_ctx* ctx, int kind, const double* ref) {
-    const PulseTime pt = pulse_at(ctx->pulse, (double)ctx->step * ctx->p.dt);
-    ctx->launches += 2;
-    return dispatch(ctx, [&](auto* sp, auto* cp) {
-        using S = std::remove_pointer_t<decltype(sp)>;
-        using C = std::remove_pointer_t<decltype(cp)>;
-        reduce_kernel<S, C><<<ctx->red_blocks, kThreads, 0, ctx->stream>>>(
-            ctx->scratch, (const S*)ctx->pop[ctx->cur], ctx->lp, (C)ctx->p.phi_ref, kind, pt, ctx->p.x0, ctx->p.y0,
-            ctx->p.dx, ref);
-        finish_kernel<<<1, kThreads, 0, ctx->stream>>>(ctx->dres, ctx->scratch, ctx->red_blocks);
-    });
+    switch (kind) {
+        case kReduceMass: return launch_reduce_kind<kReduceMass>(ctx, ref);
+        case kReducePulse: return launch_reduce_kind<kReducePulse>(ctx, ref);
+        case kReduceField: return launch_reduce_kind<kReduceField>(ctx, ref);
+        case kReduceNonFinite: return launch_reduce_kind<kReduceNonFinite>(ctx, ref);
+        case kReduceBadField: return launch_reduce_kind<kReduceBadField>(ctx, ref);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_get_populations(trtr_ctx* ctx, double* g) {
@@ -443,8 +636,8 @@ cudaError_t launch_get_populations(trtr_ctx* ctx, double* g) {
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        get_pop_kernel<S, C><<<grid_for(ctx, n), kThreads, 0, ctx->stream>>>(g, (const S*)ctx->pop[ctx->cur], ctx->lp,
-                                                                             (C)ctx->p.phi_ref);
+        launch_overlapped(ctx, get_pop_kernel<S, C>, grid_for(ctx, n), kThreads, g, (const S*)ctx->pop[ctx->cur], ctx->lp,
+                          (C)ctx->p.phi_ref, ctx->dflag, host_flag(ctx));
     });
 }
 
@@ -454,8 +647,8 @@ cudaError_t launch_set_populations(trtr_ctx* ctx, const double* g) {
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        set_pop_kernel<S, C><<<grid_for(ctx, n), kThreads, 0, ctx->stream>>>((S*)ctx->pop[ctx->cur], g, ctx->lp,
-                                                                             (C)ctx->p.phi_ref);
+        launch_overlapped(ctx, set_pop_kernel<S, C>, grid_for(ctx, n), kThreads, (S*)ctx->pop[ctx->cur], g, ctx->lp,
+                          (C)ctx->p.phi_ref);
     });
 }
 

@@ -301,9 +301,9 @@ struct trtr_ctx {
     bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
-    double* dres;     // device result of the reductions (4 doubles)
-    double* hres;     // pinned host copy
-    int* dflag;       // device timeout flag; dflag[2], dflag[3]: tile counters of the step kernels
+    double* hres;     // pinned host memory that kernels write: the reductions' two results; [3]: copy of the timeout flag
+    unsigned* red_done;  // blocks of a reduction that have finished (zero between reductions)
+    int* dflag;       // device timeout flag; dflag[2], dflag[3]: tile counters
     double* dtmp;     // device staging for double I/O
     size_t dtmp_len;  // in doubles
     double* phib;     // Dirichlet values of the edge nodes (TRTR_BC_DIRICHLET_NEE)
