@@ -135,6 +135,7 @@ __global__ void pack_f64_kernel(double* pack, const double* uv, const double* Dh
 cudaError_t launch_pack_f64(trtr_ctx* ctx) {
     const size_t n = (size_t)ctx->p.nx * ctx->p.ny, want = (n + 127) / 128, cap = (size_t)ctx->num_sms * 16;
     ctx->launches += 1;
+    ctx->tables_new = true;
     const bool fixed = ctx->p.tau2_mode == TRTR_TAU2_FIXED;
     pack_f64_kernel<<<(unsigned)(want < cap ? want : cap), 128, 0, ctx->stream>>>(
         static_cast<double*>(ctx->pack64), static_cast<const double*>(ctx->uv), static_cast<const double*>(ctx->Dh),
@@ -145,16 +146,14 @@ cudaError_t launch_pack_f64(trtr_ctx* ctx) {
 // One step from buffer `src` into dst as step `step`.  Blocks of one warp while they leave no SM with
 // more than 16 of them, of four warps above.
 cudaError_t launch_step_f64(trtr_ctx* ctx, const void* src, void* dst, long step) {
-    bool overlap = true;
     if (!ctx->pack64_ready) {
         const cudaError_t e = launch_pack_f64(ctx);
         if (e != cudaSuccess) return e;
         ctx->pack64_ready = true;
-        overlap = false;
     }
-    // the tables and packed planes are read before the wait for the kernels before this one: a launch
-    // that follows their writer starts after it has completed
-    overlap = overlap && !ctx->tables_new;
+    // the tables and packed planes are read before the wait for the kernels before this one: the first
+    // launch after their writer starts when that has completed
+    const bool overlap = !ctx->tables_new;
     ctx->tables_new = false;
     F64Args a;
     a.src = static_cast<const double*>(src);

@@ -297,7 +297,7 @@ struct trtr_ctx {
     void* tab_y;
     void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
     long ptab_first;  // time level of its first entry
-    bool tables_new;  // filled since the last FP64 step launch
+    bool tables_new;  // the tables or pack64 were written since the last FP64 step launch
     bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
@@ -369,6 +369,9 @@ cudaError_t launch_bounds_probe(trtr_ctx* ctx);
 void free_adjoint(trtr_ctx* ctx);
 cudaError_t launch_convert_fields(trtr_ctx* ctx, const double* ux, const double* uy, const double* D);
 cudaError_t launch_pulse_fields(trtr_ctx* ctx);
+// The same into another buffer of the packed fields' layout, and the FP64 step's packed planes.
+cudaError_t launch_pack_fields2_into(trtr_ctx* ctx, void* dst);
+cudaError_t launch_pack_f64(trtr_ctx* ctx);
 // Pulse tables: makes sure that they hold the time levels step - 1 .. step + steps - 1 (a launch
 // where they do not), and the pointer that a launch from step `step` reads.
 cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps);

@@ -321,20 +321,33 @@ cudaError_t encode_maps2(trtr_ctx* ctx) {
     });
 }
 
-cudaError_t launch_pack_fields2(trtr_ctx* ctx) {
+static cudaError_t pack_into(trtr_ctx* ctx, void* dst, bool tables) {
     const size_t n = (size_t)(ctx->p.nx + 2 * kGhostT) * (ctx->p.ny + 2 * kGhostT);
     const size_t want = (n + 255) / 256, cap = (size_t)ctx->num_sms * 8;
     ctx->launches += 1;
     PulseLevels levels = {};
-    if (ctx->ptab) levels = pulse_levels_of(ctx, ctx->step - 1);
+    PulseFill fill = pulse_fill_of(ctx);
+    if (tables)
+        levels = pulse_levels_of(ctx, ctx->step - 1);
+    else
+        fill.tab = nullptr;
     pack_fields2_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, ctx->stream>>>(
-        static_cast<float*>(ctx->fld2), static_cast<const float*>(ctx->uv), static_cast<const float*>(ctx->Dh),
-        ctx->lt, ctx->lf, pulse_fill_of(ctx), levels);
-    const cudaError_t e = cudaGetLastError();
-    ctx->ptab_first = ctx->step - 1;
-    ctx->ptab_ready = ctx->ptab != nullptr && e == cudaSuccess;
+        static_cast<float*>(dst), static_cast<const float*>(ctx->uv), static_cast<const float*>(ctx->Dh), ctx->lt, ctx->lf,
+        fill, levels);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_fields2(trtr_ctx* ctx) {
+    const bool tables = ctx->p.src_mode == TRTR_SRC_PULSE;
+    const cudaError_t e = pack_into(ctx, ctx->fld2, tables);
+    if (tables) {
+        ctx->ptab_first = ctx->step - 1;
+        ctx->ptab_ready = e == cudaSuccess;
+    }
     return e;
 }
+
+cudaError_t launch_pack_fields2_into(trtr_ctx* ctx, void* dst) { return pack_into(ctx, dst, false); }
 
 cudaError_t launch_refresh_ghosts2_buffer(trtr_ctx* ctx, void* P) {
     const int n = 2 * (ctx->p.nx + 2 * kGhostP) + 2 * (ctx->p.ny + 2 * kGhostP - 2);

@@ -235,9 +235,18 @@ __device__ __forceinline__ void step2_second(const S* sp, const float* sf, int i
         const int i = i0 + c2, j = j0 + r2;
         if (i >= nx || j >= ny) continue;
         if constexpr (P1) {  // the step-1 value of node (r2, c2) = R1 node (r2 + 1, c2 + 2), plane by plane
+            const bool inner = i >= 1 && i + 2 < nx && j >= 1 && j + 1 < ny;  // no ghost copies
+            S* p1 = dst1 + a.lp.at_g<kGhostP>(i, j);
 #pragma unroll
             for (int q = 0; q < kQ; ++q) {
                 const S* v = sp + q * kT2PopPlane + (r2 + 2 - lattice_ey(q)) * kT2W + c2 + T::HX - lattice_ex(q);
+                if (inner) {
+                    S2 w;
+                    reinterpret_cast<S*>(&w)[0] = v[0];
+                    reinterpret_cast<S*>(&w)[1] = v[1];
+                    *reinterpret_cast<S2*>(p1 + q * pl) = w;
+                    continue;
+                }
                 store_with_ghosts<1, kGhostP>(dst1 + q * pl, a.lp, i, j, v[0]);
                 if (i + 1 < nx) store_with_ghosts<1, kGhostP>(dst1 + q * pl, a.lp, i + 1, j, v[1]);
             }
