@@ -38,10 +38,10 @@ constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 
 cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
     const bool two = most >= 2 && two_step_applies(ctx);
     const long nodes = (long)ctx->p.nx * ctx->p.ny;
-    const bool four = two && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
+    const bool four = most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
                       sweep_applies(ctx);
     cudaError_t e = cudaSuccess;
-    if (two && !ctx->fld2_ready) {
+    if ((two || four) && !ctx->fld2_ready) {
         *what = "field packing launch";
         e = launch_pack_fields2(ctx);
         if (e != cudaSuccess) return e;
@@ -53,7 +53,9 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
     if (e != cudaSuccess) return e;
     if (four) {
         *what = "four-step launch";
-        if (!ctx->ghost4_ready) e = launch_ghost_columns(ctx);
+        if (ctx->p.src_mode == TRTR_SRC_FIELD && !ctx->src_ready) e = launch_pack_source(ctx);
+        ctx->src_ready = e == cudaSuccess;
+        if (e == cudaSuccess && !ctx->ghost4_ready) e = launch_ghost_columns(ctx);
         if (e == cudaSuccess) e = launch_sweep(ctx);
     } else if (two) {
         *what = "two-step launch";
@@ -71,7 +73,7 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
         if (e != cudaSuccess) return e;
     }
     ctx->ghost4_ready = four;
-    ctx->ghost2_ready = two;  // the one-step kernel writes the one-wide frame
+    ctx->ghost2_ready = two || four;  // the one-step kernel writes the one-wide frame
     ctx->cur ^= 1;
     ctx->step += *taken;
     return cudaSuccess;
@@ -284,13 +286,12 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
     ctx->lf = lf;
     ctx->S_cur = ctx->S_prev = -1;
     ctx->steps_per_launch = 2;
-    // the two-step kernel's packed fields (FP32 or 2-byte storage, periodic, no field source; the
-    // 2-byte kernel rounds the one-step kernel's node pairs, so nx is even there)
+    // the two- and four-step kernels' packed fields (FP32 or 2-byte storage, periodic; the
+    // 2-byte kernels round the one-step kernel's node pairs, so nx is even there)
     const bool two_step_storage =
         p->precision == TRTR_F32 ||
         ((p->precision == TRTR_F16_OFS || p->precision == TRTR_BF16_OFS) && p->nx % 2 == 0);
-    const bool two_step = two_step_storage && p->bc_mode == TRTR_BC_PERIODIC && p->src_mode != TRTR_SRC_FIELD &&
-                          p->nx >= 2 && p->ny >= 2;
+    const bool two_step = two_step_storage && p->bc_mode == TRTR_BC_PERIODIC && p->nx >= 2 && p->ny >= 2;
     ctx->lt = trtr::make_layout(p->nx, p->ny, 4, trtr::kGhostT);
 
     cudaError_t e = cudaGetDevice(&ctx->device);
@@ -327,7 +328,7 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         {(void**)&ctx->phib,
          p->bc_mode == TRTR_BC_DIRICHLET_NEE ? (size_t)trtr::edge_count(p->nx, p->ny) * sizeof(double) : 0, true},
         {&ctx->pack64, p->precision == TRTR_F64 ? 4 * fld_bytes : 0, true},
-        {&ctx->fld2, two_step ? 5 * ctx->lt.plane * sizeof(float) : 0, true},
+        {&ctx->fld2, two_step ? (p->src_mode == TRTR_SRC_FIELD ? 6 : 5) * ctx->lt.plane * sizeof(float) : 0, true},
     };
     // fault injection for tests: TRTR_FAULT_ALLOC=k makes the k-th device allocation here fail
     const char* fault = getenv("TRTR_FAULT_ALLOC");
@@ -390,6 +391,7 @@ static trtr_status set_source_impl(trtr_ctx* ctx, const double* S, int on_device
     s = check_launch(ctx, trtr::launch_convert_source(ctx, dev, dst), "source conversion");
     if (s != TRTR_OK) return s;
     ctx->S_cur = dst;
+    ctx->src_ready = false;
     return TRTR_OK;
 }
 
@@ -740,6 +742,7 @@ trtr_status trtr_load(trtr_ctx* ctx, const void* host_buf, size_t bytes) {
         TRTR_CUDA(ctx, cudaMemcpyAsync(ctx->S, b + sizeof(h) + pop_bytes, src_bytes, cudaMemcpyHostToDevice, ctx->stream),
                   "load copy");
         ctx->S_cur = h.S_cur;
+        ctx->src_ready = false;
         ctx->S_prev = h.S_prev;
     }
     TRTR_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "load");

@@ -27,11 +27,7 @@ PlaneLayout make_layout(int nx, int ny, int elem_bytes, int ghost) {
 
 namespace {
 
-__constant__ int c_ex[kQ] = {0, 1, -1, 0, 0, 1, -1, 1, -1};
-__constant__ int c_ey[kQ] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
-__constant__ double c_w[kQ] = {4.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0, 1.0 / 9.0,
-                               1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0};
-
+using core::weight;
 constexpr int kThreads = 256;
 
 // The kernels of a time loop are launched with programmatic dependent launch: set up while the kernel
@@ -121,9 +117,9 @@ __device__ __forceinline__ double pulse_phi(const PulseTime& pt, double x, doubl
 // w_i phi [1 + 3 eu + 4.5 ((eu)^2 - |u|^2/3) + 4.5 ((eu)^3 - eu |u|^2)], eu = e_i . uhat.
 template <typename T>
 __device__ __forceinline__ T equilibrium(int q, T phi, T u, T v) {
-    const T eu = T(c_ex[q]) * u + T(c_ey[q]) * v;
+    const T eu = T(lattice_ex(q)) * u + T(lattice_ey(q)) * v;
     const T uu = u * u + v * v;
-    return T(c_w[q]) * phi *
+    return weight<T>(q) * phi *
            (T(1) + T(3) * eu + T(4.5) * (eu * eu - uu / T(3)) + T(4.5) * (eu * eu * eu - eu * uu));
 }
 
@@ -132,9 +128,9 @@ template <typename S>
 __device__ __forceinline__ void store_pulled(S* P, const PlaneLayout& L, int q, int i, int j, bool inner, S v) {
     S* plane = P + q * L.plane;
     if (inner)  // the slot and its neighbours are away from the ghost frame
-        plane[L.at(i - c_ex[q], j - c_ey[q])] = v;
+        plane[L.at(i - lattice_ex(q), j - lattice_ey(q))] = v;
     else
-        store_with_ghosts(plane, L, wrap(i - c_ex[q], L.nx), wrap(j - c_ey[q], L.ny), v);
+        store_with_ghosts(plane, L, wrap(i - lattice_ex(q), L.nx), wrap(j - lattice_ey(q), L.ny), v);
 }
 __device__ __forceinline__ bool inner_node(const PlaneLayout& L, int i, int j) {
     return i > L.gy && i < L.nx - 1 - L.gy && j > L.gy && j < L.ny - 1 - L.gy;
@@ -171,7 +167,7 @@ __global__ void __launch_bounds__(128)
         const bool inner = inner_node(lp, i, j);
 #pragma unroll
         for (int q = 0; q < kQ; ++q)
-            store_pulled(P, lp, q, i, j, inner, Store<S>::encode(equilibrium<C>(q, phi, u, v), (C)(c_w[q]) * phi_ref));
+            store_pulled(P, lp, q, i, j, inner, Store<S>::encode(equilibrium<C>(q, phi, u, v), weight<C>(q) * phi_ref));
     }
 }
 
@@ -198,15 +194,15 @@ __global__ void dirichlet_nee_kernel(S* P, const C* uv, const double* phib, Plan
         double gq = 0.0, phif = 0.0;
 #pragma unroll
         for (int p = 0; p < kQ; ++p) {
-            const double gf = (double)Store<S>::decode(P[p * lp.plane + lp.at(fi - c_ex[p], fj - c_ey[p])],
-                                                       (C)(c_w[p]) * phi_ref);
+            const double gf = (double)Store<S>::decode(P[p * lp.plane + lp.at(fi - lattice_ex(p), fj - lattice_ey(p))],
+                                                       weight<C>(p) * phi_ref);
             phif += gf;
             if (p == q) gq = gf;
         }
         const double ub = (double)uv[lf.at(i, j)], vb = (double)uv[lf.plane + lf.at(i, j)];
         const double uf = (double)uv[lf.at(fi, fj)], vf = (double)uv[lf.plane + lf.at(fi, fj)];
         const double g = equilibrium(q, phib[k], ub, vb) + gq - equilibrium(q, phif, uf, vf);
-        P[q * lp.plane + lp.at(i - c_ex[q], j - c_ey[q])] = Store<S>::encode((C)g, (C)(c_w[q]) * phi_ref);
+        P[q * lp.plane + lp.at(i - lattice_ex(q), j - lattice_ey(q))] = Store<S>::encode((C)g, weight<C>(q) * phi_ref);
     }
 }
 
@@ -224,7 +220,7 @@ __global__ void gather_edges_kernel(double* phib, const double* phi, int nx, int
 // holds the periodic image, or the Dirichlet pass's value (TRTR_BC_DIRICHLET_NEE).
 template <typename S, typename C>
 __device__ __forceinline__ C pulled(const S* P, int q, int i, int j, const PlaneLayout& L, C phi_ref) {
-    return Store<S>::decode(P[q * L.plane + L.at(i - c_ex[q], j - c_ey[q])], (C)(c_w[q]) * phi_ref);
+    return Store<S>::decode(P[q * L.plane + L.at(i - lattice_ex(q), j - lattice_ey(q))], weight<C>(q) * phi_ref);
 }
 
 template <typename S, typename C>
@@ -488,7 +484,7 @@ __global__ void set_pop_kernel(S* P, const double* g, PlaneLayout L, C phi_ref) 
         const bool inner = inner_node(L, i, j);
 #pragma unroll
         for (int q = 0; q < kQ; ++q)
-            store_pulled(P, L, q, i, j, inner, Store<S>::encode((C)g[(size_t)q * n + k], (C)(c_w[q]) * phi_ref));
+            store_pulled(P, L, q, i, j, inner, Store<S>::encode((C)g[(size_t)q * n + k], weight<C>(q) * phi_ref));
     }
 }
 

@@ -312,8 +312,10 @@ struct trtr_ctx {
     // two-step kernel (FP32 storage, periodic boundaries, no source or the pulse source)
     CUtensorMap maps2[3];   // populations (buffers 0, 1) and packed fields, its tile boxes
     CUtensorMap maps4[5];   // four-step kernel: population rows (buffers 0, 1), interior stores (0, 1), field rows
-    void* fld2;             // [5][rows][pitch] float: uhat_x, uhat_y, a_x, a_y, Dh, two-wide periodic ghosts
+    void* fld2;             // [5 or 6][rows][pitch] float: uhat_x, uhat_y, a_x, a_y, Dh (and the stationary
+                            // source term, TRTR_SRC_FIELD), four-wide periodic ghosts
     trtr::PlaneLayout lt;   // layout of fld2
+    bool src_ready;         // its source plane (TRTR_SRC_FIELD) holds the current S^n
     bool fld2_ready;        // fld2 holds the current fields
     bool ghost4_ready;      // its four-wide ghost columns are up to date (interior rows)
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
@@ -358,6 +360,7 @@ bool sweep_applies(const trtr_ctx* ctx);
 cudaError_t encode_maps4(trtr_ctx* ctx);
 cudaError_t launch_sweep(trtr_ctx* ctx);
 cudaError_t launch_ghost_columns(trtr_ctx* ctx);
+cudaError_t launch_pack_source(trtr_ctx* ctx);  // the source term's plane of the packed fields, from S^n
 // The next launch of a run that may advance `most` (>= 1) steps, of a call that takes `call` in all:
 // four, two or one steps, with what the launch needs; advances the context's state.  *taken: the
 // steps; *what: names the failing launch on an error.

@@ -1,8 +1,8 @@
 // trtr_sweep.cu -- four time steps of the evolution equation (14) per launch: each CTA sweeps a
 // strip of columns from bottom to top and carries four time levels behind one another through
 // shared memory (wavefront temporal blocking), for FP32 storage or FP16 / BF16 offset storage
-// (FP32 arithmetic), periodic boundaries and no source or the manufactured pulse source.  The
-// node update is the one-step kernel's, roundings included, so the results have the same bits.
+// (FP32 arithmetic), periodic boundaries and no source, the manufactured pulse source or a
+// stationary source field.  The node update is the one-step kernel's, roundings included, so the results have the same bits.
 //
 // Strip: X = 120 output columns from i0; every level computes the 128 columns [i0 - 4, i0 + 124)
 // (two warps a row, a node pair a lane), of which level s is valid on all but s - 1 at each side.
@@ -28,39 +28,27 @@ using namespace core;
 constexpr int kT = 4;                 // time levels of a launch
 constexpr int kX = 120, kWC = 128;    // output and computed columns of a strip
 constexpr int kW = kWC + 2 * kT;      // staged population columns
-constexpr int kNF = 5;                // packed fields
+// packed fields: u, a, D and, with a stationary source field, the source term
+__host__ __device__ constexpr int fields_of(int src) { return src == TRTR_SRC_FIELD ? 6 : 5; }
 constexpr int kGhostX = 4;            // ghost columns that the strips read
 
-#ifndef TRTR_SWEEP_R
-#define TRTR_SWEEP_R 3
-#endif
-#ifndef TRTR_SWEEP_AHEAD
-#define TRTR_SWEEP_AHEAD 1
-#endif
-#ifndef TRTR_SWEEP_OUTS
-#define TRTR_SWEEP_OUTS 3
-#endif
-#ifndef TRTR_SWEEP_AHEADH
-#define TRTR_SWEEP_AHEADH 3
-#endif
-#ifndef TRTR_SWEEP_RH
-#define TRTR_SWEEP_RH 4
-#endif
-
-template <typename S, int R_>
+template <typename S, int SRC>
 struct Sweep {
-    static constexpr int R = R_, ES = (int)sizeof(S);
+    static constexpr int ES = (int)sizeof(S), NF = fields_of(SRC);
+    // rows of an iteration, blocks loaded ahead: FP32 has room for 3 rows with five fields a row, 2 with
+    // the source's (4096^2 without a source: 3 rows 163 GLUPS, 2 rows 146); 2-byte storages 4 rows
+    static constexpr int R = ES == 2 ? 4 : (SRC == TRTR_SRC_FIELD ? 2 : 3);
+    static constexpr int Ahead = ES == 2 ? 3 : (SRC == TRTR_SRC_FIELD ? 2 : 1);
     static constexpr int Lag = R + 1;
     static constexpr int C = ((kT - 1) * (Lag + 1) + R - 1) / R * R;  // ramp rows of a segment
-    static constexpr int Ahead = ES == 2 ? TRTR_SWEEP_AHEADH : TRTR_SWEEP_AHEAD;  // blocks loaded ahead
     static constexpr int Ring = ((kT - 1) * Lag + kT + 1 + (Ahead + 1) * R + R - 1) / R * R;
     static constexpr int Blocks = Ring / R;
-    static constexpr int PopRow = kQ * kW * ES, FldRow = kNF * kWC * 4;
+    static constexpr int PopRow = kQ * kW * ES, FldRow = NF * kWC * 4;
     static constexpr int OutBytes = (kQ * R * kX * ES + 127) / 128 * 128;
     static constexpr int FldOff = Ring * ((PopRow + 127) / 128 * 128);
     static constexpr int PopPitch = (PopRow + 127) / 128 * 128;       // TMA destinations on 128 bytes
     static constexpr int OutOff = FldOff + Ring * FldRow;
-    static constexpr int Outs = ES == 2 ? 3 : TRTR_SWEEP_OUTS;                                    // output buffers
+    static constexpr int Outs = 3;                                    // output buffers (with 2 the last level waits for them: -20 %)
     static constexpr int BarOff = OutOff + Outs * OutBytes;
     static constexpr int Depth = 8;                                   // barriers of a level (iterations in flight)
     static constexpr int Smem = BarOff + (Blocks + kT * Depth + Outs) * 8 + 128;
@@ -111,7 +99,7 @@ __device__ __forceinline__ void store_sweep_ghosts(T* plane, const PlaneLayout& 
 // slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
 // the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
 // rows within kGhostP of an edge).
-template <typename S, int LV, bool SR, class G>
+template <typename S, int LV, int SRC, bool SR, class G>
 __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[2], const SweepArgs& a,
                                           const uint32_t rk[2], S* out_row, int lane, int i, int j) {
     constexpr bool kOfs = sizeof(S) == 2;
@@ -122,7 +110,7 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
         return row + q * kW - LV * lattice_ex(q) + 64 * h;
     };
     auto even = [](int q) { return LV % 2 == 0 || lattice_ex(q) == 0; };
-    F2 g[2][kQ], fld[2][kNF];
+    F2 g[2][kQ], fld[2][G::NF];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
 #pragma unroll
@@ -131,11 +119,12 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
             g[h][q] = even(q) ? Pair<S>::raw(*reinterpret_cast<const S2*>(s)) : Pair<S>::raw(s[0], s[1]);
         }
 #pragma unroll
-        for (int m = 0; m < kNF; ++m) fld[h][m] = F2(*reinterpret_cast<const float2*>(f + m * kWC + 64 * h));
+        for (int m = 0; m < G::NF; ++m) fld[h][m] = F2(*reinterpret_cast<const float2*>(f + m * kWC + 64 * h));
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
-        collide_node<F2, kOfs>(g[h], fld[h][0], fld[h][1], fld[h][2], fld[h][3], fld[h][4], src[h], F2(a.magic),
+        collide_node<F2, kOfs>(g[h], fld[h][0], fld[h][1], fld[h][2], fld[h][3], fld[h][4],
+                               SRC == TRTR_SRC_FIELD ? fld[h][G::NF - 1] : src[h], F2(a.magic),
                                F2(a.omega2_fixed), a.tau2_fixed, out[h], F2(a.phi_ref));
     auto enc = [&](int q, int h) -> S2 {
         if constexpr (SR)
@@ -390,7 +379,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 S* pm = base + below * kPitch;
                 S* p0 = base + ring * kPitch;
                 S* pp = base + above * kPitch;
-                const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (kNF * kWC) + 2 * lane;
+                const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (G::NF * kWC) + 2 * lane;
                 uint32_t rk[2] = {0u, 0u};
                 if (SR) {
                     rk[0] = sr_pair_key(wx[0], yw, nx, rkey);
@@ -398,10 +387,10 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 }
                 S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane - kT;
                 switch (level) {
-                    case 1: sweep_row<S, 1, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 2: sweep_row<S, 2, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 3: sweep_row<S, 3, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    default: sweep_row<S, 4, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 1: sweep_row<S, 1, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 2: sweep_row<S, 2, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 3: sweep_row<S, 3, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    default: sweep_row<S, 4, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
                 }
             }
             if (level == kT) fence_proxy_async_smem();  // the rows, for the TMA store
@@ -428,7 +417,7 @@ __global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
 
 template <typename S, int SRC, bool SR>
 cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
-    using G = Sweep<S, sizeof(S) == 2 ? TRTR_SWEEP_RH : TRTR_SWEEP_R>;
+    using G = Sweep<S, SRC>;
     auto kernel = sweep_kernel<S, SRC, SR, G>;
     static int configured_device = -1;
     if (configured_device != ctx->device) {
@@ -479,9 +468,9 @@ cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     return cudaLaunchKernelEx(&cfg, kernel, ctx->maps4[ctx->cur], ctx->maps4[4], ctx->maps4[2 + (ctx->cur ^ 1)], a);
 }
 
-template <typename S>
+template <typename S, int SRC>
 cudaError_t encode4_typed(trtr_ctx* ctx) {
-    using G = Sweep<S, sizeof(S) == 2 ? TRTR_SWEEP_RH : TRTR_SWEEP_R>;
+    using G = Sweep<S, SRC>;
     bool ok = true;
     PlaneLayout in = ctx->lp;  // the interior alone, so that stores are clipped to it
     in.nx = bulk_cols_of<S>(in.nx);
@@ -489,7 +478,7 @@ cudaError_t encode4_typed(trtr_ctx* ctx) {
         ok = ok && encode(&ctx->maps4[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], ctx->lp, kQ, kW, 1, kQ);
         ok = ok && encode_interior(&ctx->maps4[2 + b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], in, kQ, kX, G::R, kQ);
     }
-    ok = ok && encode(&ctx->maps4[4], tma_type<float>(), 4, ctx->fld2, ctx->lt, kNF, kWC, 1, kNF);
+    ok = ok && encode(&ctx->maps4[4], tma_type<float>(), 4, ctx->fld2, ctx->lt, G::NF, kWC, 1, G::NF);
     return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -500,16 +489,42 @@ static bool sweep_size(const trtr_ctx* ctx) { return ctx->p.nx >= 16 && ctx->p.n
 
 cudaError_t encode_maps4(trtr_ctx* ctx) {
     if (!ctx->fld2 || !sweep_size(ctx)) return cudaSuccess;
+    const bool field = ctx->p.src_mode == TRTR_SRC_FIELD;
     switch (ctx->p.precision) {
-        case TRTR_F32: return encode4_typed<float>(ctx);
-        case TRTR_F16_OFS: return encode4_typed<__half>(ctx);
-        case TRTR_BF16_OFS: return encode4_typed<__nv_bfloat16>(ctx);
+        case TRTR_F32: return field ? encode4_typed<float, TRTR_SRC_FIELD>(ctx) : encode4_typed<float, TRTR_SRC_NONE>(ctx);
+        case TRTR_F16_OFS:
+            return field ? encode4_typed<__half, TRTR_SRC_FIELD>(ctx) : encode4_typed<__half, TRTR_SRC_NONE>(ctx);
+        case TRTR_BF16_OFS:
+            return field ? encode4_typed<__nv_bfloat16, TRTR_SRC_FIELD>(ctx) : encode4_typed<__nv_bfloat16, TRTR_SRC_NONE>(ctx);
         default: return cudaErrorInvalidValue;
     }
 }
 
+// Source fields: while S^n is S^{n-1}, so that every step of the launch has the same source term.
 bool sweep_applies(const trtr_ctx* ctx) {
-    return two_step_applies(ctx) && sweep_size(ctx);
+    if (!ctx->fld2 || ctx->steps_per_launch != 2 || ctx->p.bc_mode != TRTR_BC_PERIODIC || !sweep_size(ctx)) return false;
+    return ctx->p.src_mode != TRTR_SRC_FIELD || ctx->S_prev < 0 || ctx->S_prev == ctx->S_cur;
+}
+
+// The source term of a stationary field, with the one-step kernel's roundings of 1.5 S - 0.5 S, at every
+// node of the packed fields' ghost frame.
+__global__ void pack_source_kernel(float* dst, const float* S, PlaneLayout lt, PlaneLayout lf) {
+    const unsigned gw = lt.nx + 2 * kGhostT, n = gw * (unsigned)(lt.ny + 2 * kGhostT);
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int j = (int)(k / gw) - kGhostT, i = (int)(k % gw) - kGhostT;
+        const float s = S[lf.at((i % lt.nx + lt.nx) % lt.nx, (j % lt.ny + lt.ny) % lt.ny)];
+        dst[lt.at(i, j)] = __fmaf_rn(1.5f, s, __fmul_rn(-0.5f, s));
+    }
+}
+
+cudaError_t launch_pack_source(trtr_ctx* ctx) {
+    const unsigned n = (unsigned)(ctx->p.nx + 2 * kGhostT) * (unsigned)(ctx->p.ny + 2 * kGhostT);
+    const unsigned want = (n + 255) / 256, cap = (unsigned)ctx->num_sms * 8;
+    ctx->launches += 1;
+    pack_source_kernel<<<want < cap ? want : cap, 256, 0, ctx->stream>>>(
+        static_cast<float*>(ctx->fld2) + 5 * ctx->lt.plane,
+        static_cast<const float*>(ctx->S) + (size_t)ctx->S_cur * ctx->lf.plane, ctx->lt, ctx->lf);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ghost_columns(trtr_ctx* ctx) {
@@ -526,8 +541,11 @@ cudaError_t launch_ghost_columns(trtr_ctx* ctx) {
 
 template <typename S, bool SR>
 static cudaError_t launch_sweep_src(trtr_ctx* ctx) {
-    return ctx->p.src_mode == TRTR_SRC_PULSE ? launch_sweep_typed<S, TRTR_SRC_PULSE, SR>(ctx)
-                                             : launch_sweep_typed<S, TRTR_SRC_NONE, SR>(ctx);
+    switch (ctx->p.src_mode) {
+        case TRTR_SRC_FIELD: return launch_sweep_typed<S, TRTR_SRC_FIELD, SR>(ctx);
+        case TRTR_SRC_PULSE: return launch_sweep_typed<S, TRTR_SRC_PULSE, SR>(ctx);
+        default: return launch_sweep_typed<S, TRTR_SRC_NONE, SR>(ctx);
+    }
 }
 
 cudaError_t launch_sweep(trtr_ctx* ctx) {

@@ -11,6 +11,7 @@ if not torch.cuda.is_available():
 
 from paper_2312_10316_gb300 import trtr as T  # noqa: E402
 
+from ._gpu_util import random_case  # noqa: E402
 from .test_gpu_step2 import _pulse_solver, _random_solver  # noqa: E402
 
 PREC = {"f32": T.TRTR_F32, "f16": T.TRTR_F16_OFS, "bf16": T.TRTR_BF16_OFS}
@@ -42,6 +43,37 @@ def test_sweeps_equal_one_step_launches_bitwise(nx, ny, prec, kind, rounding):
             assert l1 - l0 == 2 + 4  # field packing, ghost columns, four sweeps
     assert np.array_equal(out[1][0], out[2][0], equal_nan=True)
     assert np.array_equal(out[1][1], out[2][1], equal_nan=True)
+
+
+@pytest.mark.parametrize("nx,ny", [(16, 32), (130, 41), (243, 64)])
+@pytest.mark.parametrize("prec", ["f32", "f16"])
+def test_sweeps_with_a_source_field_equal_one_step_launches_bitwise(nx, ny, prec):
+    """Sweeps run while the field stays the same; after each change one single step comes first."""
+    case = random_case(31 + nx, nx, ny)
+    nx2 = nx - nx % 2 if prec == "f16" else nx
+    case = {k: (np.ascontiguousarray(v[..., :nx2]) if isinstance(v, np.ndarray) else v) for k, v in case.items()}
+    out = {}
+    for k in (1, 2):
+        p = T.Params(nx=nx2, ny=ny, dx=case["dx"], dt=case["dt"], precision=PREC[prec], src_mode=T.TRTR_SRC_FIELD,
+                     grad_mode=T.TRTR_GRAD_PERIODIC)
+        with T.Solver(p) as s:
+            s.set_steps_per_launch(k)
+            s.set_fields(case["ux"], case["uy"], case["D"], case["S1"])
+            s.set_populations(case["g"])
+            l0 = s.launches
+            s.step(16)
+            l1 = s.launches
+            s.set_source(case["S2"])
+            s.step(19)
+            blob = s.save()
+            s.set_source(case["S1"])
+            s.step(14)
+            s.load(blob)
+            s.step(12)
+            out[k] = s.get_populations()
+        if k == 2:
+            assert l1 - l0 == 3 + 4  # fields, source term, ghost columns, four sweeps
+    assert np.array_equal(out[1], out[2])
 
 
 def test_sweeps_stop_at_the_stability_checks():
