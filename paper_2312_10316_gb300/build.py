@@ -20,7 +20,7 @@ LIB = os.path.join(HERE, "libtrtr.so")
 # debug build whose kernels check their memory accesses (TRTR_BOUNDS_CHECK=1)
 LIB_CHECKED = os.path.join(HERE, "libtrtr_checked.so")
 
-SOURCES = ["trtr_api.cu", "trtr_step.cu", "trtr_step2.cu", "trtr_sweep.cu", "trtr_f64.cu",
+SOURCES = ["trtr_api.cu", "trtr_step.cu", "trtr_step2.cu", "trtr_sweep.cu", "trtr_small.cu", "trtr_f64.cu",
            "trtr_aux.cu", "trtr_noalloc.cu", "trtr_batch.cu",
            "trtr_adjoint.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -16,7 +16,8 @@ namespace trtr {
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out) {
     out[0] = out[1] = out[2] = 0ull;
     cudaError_t (*units[])(cudaStream_t, unsigned long long*) = {bounds_take_step, bounds_take_aux, bounds_take_batch,
-                                                                  bounds_take_adjoint, bounds_take_step2, bounds_take_sweep, bounds_take_f64};
+                                                                  bounds_take_adjoint, bounds_take_step2, bounds_take_sweep, bounds_take_f64,
+                                                                  bounds_take_small};
     for (auto take : units) {
         unsigned long long u[3];
         const cudaError_t e = take(s, u);
@@ -40,6 +41,7 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
     const long nodes = (long)ctx->p.nx * ctx->p.ny;
     const bool four = most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
                       sweep_applies(ctx);
+    const bool small = four && small_applies(ctx);
     cudaError_t e = cudaSuccess;
     if ((two || four) && !ctx->fld2_ready) {
         *what = "field packing launch";
@@ -55,8 +57,12 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
         *what = "four-step launch";
         if (ctx->p.src_mode == TRTR_SRC_FIELD && !ctx->src_ready) e = launch_pack_source(ctx);
         ctx->src_ready = e == cudaSuccess;
-        if (e == cudaSuccess && !ctx->ghost4_ready) e = launch_ghost_columns(ctx);
-        if (e == cudaSuccess) e = launch_sweep(ctx);
+        if (small) {
+            if (e == cudaSuccess) e = launch_small(ctx);
+        } else {
+            if (e == cudaSuccess && !ctx->ghost4_ready) e = launch_ghost_columns(ctx);
+            if (e == cudaSuccess) e = launch_sweep(ctx);
+        }
     } else if (two) {
         *what = "two-step launch";
         if (!ctx->ghost2_ready) e = launch_refresh_ghosts2(ctx);  // after one-step launches: complete the two-wide frame
@@ -72,7 +78,7 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
         e = launch_dirichlet(ctx, ctx->pop[ctx->cur ^ 1]);
         if (e != cudaSuccess) return e;
     }
-    ctx->ghost4_ready = four;
+    ctx->ghost4_ready = four && !small;
     ctx->ghost2_ready = two || four;  // the one-step kernel writes the one-wide frame
     ctx->cur ^= 1;
     ctx->step += *taken;
@@ -286,12 +292,8 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
     ctx->lf = lf;
     ctx->S_cur = ctx->S_prev = -1;
     ctx->steps_per_launch = 2;
-    // the two- and four-step kernels' packed fields (FP32 or 2-byte storage, periodic; the
-    // 2-byte kernels round the one-step kernel's node pairs, so nx is even there)
-    const bool two_step_storage =
-        p->precision == TRTR_F32 ||
-        ((p->precision == TRTR_F16_OFS || p->precision == TRTR_BF16_OFS) && p->nx % 2 == 0);
-    const bool two_step = two_step_storage && p->bc_mode == TRTR_BC_PERIODIC && p->nx >= 2 && p->ny >= 2;
+    // the packed fields of the two- and four-step kernels (FP32-computing storage, periodic)
+    const bool two_step = p->precision != TRTR_F64 && p->bc_mode == TRTR_BC_PERIODIC && p->nx >= 2 && p->ny >= 2;
     ctx->lt = trtr::make_layout(p->nx, p->ny, 4, trtr::kGhostT);
 
     cudaError_t e = cudaGetDevice(&ctx->device);

@@ -906,7 +906,7 @@ trtr_status trtr_batch_create(const trtr_instance* inst, int count, void* cuda_s
     // two steps per launch where every instance has the two-step kernel's packed fields
     b->steps_per_launch = 2;
     b->two_step = s == TRTR_OK;  // where every instance has the two-step fields (FP32, or 2-byte with even nx)
-    for (int k = 0; k < count && b->two_step; ++k) b->two_step = b->ctx[k]->fld2 != nullptr;
+    for (int k = 0; k < count && b->two_step; ++k) b->two_step = trtr::two_step_applies(b->ctx[k]);
     if (s == TRTR_OK && b->two_step &&
         cudaMalloc(&b->d_desc2, sizeof(trtr::InstanceDesc2) * count) != cudaSuccess) {
         cudaGetLastError();

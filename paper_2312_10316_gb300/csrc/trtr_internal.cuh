@@ -110,6 +110,7 @@ cudaError_t bounds_take_adjoint(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_step2(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_sweep(cudaStream_t s, unsigned long long* out);
 cudaError_t bounds_take_f64(cudaStream_t s, unsigned long long* out);
+cudaError_t bounds_take_small(cudaStream_t s, unsigned long long* out);
 // All units: the summed count, and the kind and place of the first unit's first access.
 cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out);
 
@@ -297,7 +298,8 @@ struct trtr_ctx {
     void* tab_y;
     void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
     long ptab_first;  // time level of its first entry
-    bool tables_new;  // the tables or pack64 were written since the last FP64 step launch
+    bool tables_new;  // the tables or packed fields were written since the last launch that reads them early
+                      // (before it waits for the launch before it)
     bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
@@ -360,6 +362,9 @@ bool sweep_applies(const trtr_ctx* ctx);
 cudaError_t encode_maps4(trtr_ctx* ctx);
 cudaError_t launch_sweep(trtr_ctx* ctx);
 cudaError_t launch_ghost_columns(trtr_ctx* ctx);
+// the same four steps on a small grid (trtr_small.cu; reads no ghost cells)
+bool small_applies(const trtr_ctx* ctx);
+cudaError_t launch_small(trtr_ctx* ctx);
 cudaError_t launch_pack_source(trtr_ctx* ctx);  // the source term's plane of the packed fields, from S^n
 // The next launch of a run that may advance `most` (>= 1) steps, of a call that takes `call` in all:
 // four, two or one steps, with what the launch needs; advances the context's state.  *taken: the

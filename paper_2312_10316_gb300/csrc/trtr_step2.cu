@@ -273,7 +273,8 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
 }  // namespace
 
 bool two_step_applies(const trtr_ctx* ctx) {
-    return ctx->fld2 != nullptr && ctx->steps_per_launch == 2 && ctx->p.bc_mode == TRTR_BC_PERIODIC &&
+    // 2-byte storages: even widths, whose halo pairs are the one-step kernel's pairs
+    return ctx->fld2 != nullptr && (ctx->esize == 4 || ctx->p.nx % 2 == 0) && ctx->steps_per_launch == 2 && ctx->p.bc_mode == TRTR_BC_PERIODIC &&
            (ctx->p.src_mode == TRTR_SRC_NONE || ctx->p.src_mode == TRTR_SRC_PULSE);
 }
 
@@ -325,6 +326,7 @@ static cudaError_t pack_into(trtr_ctx* ctx, void* dst, bool tables) {
     const size_t n = (size_t)(ctx->p.nx + 2 * kGhostT) * (ctx->p.ny + 2 * kGhostT);
     const size_t want = (n + 255) / 256, cap = (size_t)ctx->num_sms * 8;
     ctx->launches += 1;
+    ctx->tables_new = true;
     PulseLevels levels = {};
     PulseFill fill = pulse_fill_of(ctx);
     if (tables)

@@ -414,6 +414,13 @@ __device__ __forceinline__ uint32_t sr_bits(uint32_t rk, int q) {
     return rk;
 }
 
+// The bits of two nodes that are not one pair: each takes its half (h: 0 the first, 1 the second node of
+// a pair) of its own pair's bits.
+__device__ __forceinline__ uint32_t sr_mixed_bits(uint32_t ka, uint32_t kb, int ha, int hb, int q) {
+    const uint32_t a = sr_bits(ka, q) >> (16 * ha), b = sr_bits(kb, q) >> (16 * hb);
+    return (a & 0xffffu) | (b << 16);
+}
+
 template <typename S>
 struct Pair;
 template <>

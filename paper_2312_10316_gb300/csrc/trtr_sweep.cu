@@ -94,14 +94,22 @@ __device__ __forceinline__ void store_sweep_ghosts(T* plane, const PlaneLayout& 
     }
 }
 
+// How a sweep rounds 2-byte values: to nearest (or FP32, not at all); stochastically; stochastically on
+// an odd width, where halo pairs fall between the one-step kernel's pairs and every pair takes the
+// bits of its two nodes' own pairs (two keys and a byte permutation, 8 % more instructions).
+enum SweepRounding { kRoundNearest = 0, kRoundPairs = 1, kRoundNodes = 2 };
+struct RoundKey {
+    uint32_t a, b, sel;  // the two nodes' keys; the permutation that takes each one's half
+};
+
 // Level LV of row j for one lane: its node pairs at the columns c = 2 lane and c + 64 (h = 0, 1),
 // computed side by side so that each hides the other's latency.  pm / p0 / pp: the ring rows of the
 // slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
 // the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
 // rows within kGhostP of an edge).
-template <typename S, int LV, int SRC, bool SR, class G>
+template <typename S, int LV, int SRC, int RND, class G>
 __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[2], const SweepArgs& a,
-                                          const uint32_t rk[2], S* out_row, int lane, int i, int j) {
+                                          const RoundKey rk[2], S* out_row, int lane, int i, int j) {
     constexpr bool kOfs = sizeof(S) == 2;
     using S2 = typename Pair<S>::type;
     F2 out[2][kQ];
@@ -127,8 +135,10 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
                                SRC == TRTR_SRC_FIELD ? fld[h][G::NF - 1] : src[h], F2(a.magic),
                                F2(a.omega2_fixed), a.tau2_fixed, out[h], F2(a.phi_ref));
     auto enc = [&](int q, int h) -> S2 {
-        if constexpr (SR)
-            return Pair<S>::encode_sr(out[h][q], sr_bits(rk[h], q));
+        if constexpr (RND == kRoundPairs)
+            return Pair<S>::encode_sr(out[h][q], sr_bits(rk[h].a, q));
+        else if constexpr (RND == kRoundNodes)
+            return Pair<S>::encode_sr(out[h][q], __byte_perm(sr_bits(rk[h].a, q), sr_bits(rk[h].b, q), rk[h].sel));
         else
             return Pair<S>::encode_raw(out[h][q]);
     };
@@ -196,7 +206,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-template <typename S, int SRC, bool SR, class G>
+template <typename S, int SRC, int RND, class G>
 __global__ void __launch_bounds__(G::Threads, 1)
     sweep_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mf,
                  const __grid_constant__ CUtensorMap mo, const __grid_constant__ SweepArgs a) {
@@ -323,7 +333,8 @@ __global__ void __launch_bounds__(G::Threads, 1)
         // per strip: the pairs' columns, their images for the rounding keys, their pulse factors
         const int i = t.i0 - kT + 2 * lane;
         F2 p1p[2], p2p[2], p1n[2], p2n[2];
-        int wx[2];
+        int wa[2], wb[2];
+        uint32_t sel[2];
         const float* lev = a.pulse + (level - 1) * a.pt.level;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -333,8 +344,11 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + i + 64 * h)));
                 p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + a.pt.p2 + i + 64 * h)));
             }
-            wx[h] = i + 64 * h < 0 ? i + 64 * h + nx : i + 64 * h;
-            wx[h] = wx[h] >= nx ? wx[h] - nx : wx[h];
+            auto wrap = [&](int v) { return v < 0 ? v + nx : (v >= nx ? v - nx : v); };
+            const int xa = wrap(i + 64 * h), xb = wrap(i + 64 * h + 1);
+            wa[h] = xa & ~1;
+            wb[h] = xb & ~1;
+            sel[h] = (xa & 1 ? 0x32u : 0x10u) | (xb & 1 ? 0x7600u : 0x5400u);
         }
         const float* ty = lev + a.pt.y;
 
@@ -347,7 +361,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
         for (int k = 0; k < t.iters; ++k, j += R, ++it) {
             F2 src[2] = {F2(0.f), F2(0.f)};
             int yw = 0;
-            if (SRC == TRTR_SRC_PULSE || SR) yw = j < 0 ? j + ny : (j >= ny ? j - ny : j);
+            if (SRC == TRTR_SRC_PULSE || RND != kRoundNearest) yw = j < 0 ? j + ny : (j >= ny ? j - ny : j);
             if (SRC == TRTR_SRC_PULSE) {  // as pulse_source_dt
                 const float2 qp = __ldg(reinterpret_cast<const float2*>(ty + 2 * yw));
                 const float2 qn = __ldg(reinterpret_cast<const float2*>(ty + a.pt.level + 2 * yw));
@@ -380,17 +394,21 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 S* p0 = base + ring * kPitch;
                 S* pp = base + above * kPitch;
                 const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (G::NF * kWC) + 2 * lane;
-                uint32_t rk[2] = {0u, 0u};
-                if (SR) {
-                    rk[0] = sr_pair_key(wx[0], yw, nx, rkey);
-                    rk[1] = sr_pair_key(wx[1], yw, nx, rkey);
+                RoundKey rk[2] = {};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (RND != kRoundNearest) rk[h].a = sr_pair_key(wa[h], yw, nx, rkey);
+                    if (RND == kRoundNodes) {
+                        rk[h].b = sr_pair_key(wb[h], yw, nx, rkey);
+                        rk[h].sel = sel[h];
+                    }
                 }
                 S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane - kT;
                 switch (level) {
-                    case 1: sweep_row<S, 1, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 2: sweep_row<S, 2, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 3: sweep_row<S, 3, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    default: sweep_row<S, 4, SRC, SR, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    default: sweep_row<S, 4, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
                 }
             }
             if (level == kT) fence_proxy_async_smem();  // the rows, for the TMA store
@@ -415,10 +433,10 @@ __global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
     }
 }
 
-template <typename S, int SRC, bool SR>
+template <typename S, int SRC, int RND>
 cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     using G = Sweep<S, SRC>;
-    auto kernel = sweep_kernel<S, SRC, SR, G>;
+    auto kernel = sweep_kernel<S, SRC, RND, G>;
     static int configured_device = -1;
     if (configured_device != ctx->device) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
@@ -521,6 +539,7 @@ cudaError_t launch_pack_source(trtr_ctx* ctx) {
     const unsigned n = (unsigned)(ctx->p.nx + 2 * kGhostT) * (unsigned)(ctx->p.ny + 2 * kGhostT);
     const unsigned want = (n + 255) / 256, cap = (unsigned)ctx->num_sms * 8;
     ctx->launches += 1;
+    ctx->tables_new = true;
     pack_source_kernel<<<want < cap ? want : cap, 256, 0, ctx->stream>>>(
         static_cast<float*>(ctx->fld2) + 5 * ctx->lt.plane,
         static_cast<const float*>(ctx->S) + (size_t)ctx->S_cur * ctx->lf.plane, ctx->lt, ctx->lf);
@@ -539,22 +558,26 @@ cudaError_t launch_ghost_columns(trtr_ctx* ctx) {
     return cudaGetLastError();
 }
 
-template <typename S, bool SR>
+template <typename S, int RND>
 static cudaError_t launch_sweep_src(trtr_ctx* ctx) {
     switch (ctx->p.src_mode) {
-        case TRTR_SRC_FIELD: return launch_sweep_typed<S, TRTR_SRC_FIELD, SR>(ctx);
-        case TRTR_SRC_PULSE: return launch_sweep_typed<S, TRTR_SRC_PULSE, SR>(ctx);
-        default: return launch_sweep_typed<S, TRTR_SRC_NONE, SR>(ctx);
+        case TRTR_SRC_FIELD: return launch_sweep_typed<S, TRTR_SRC_FIELD, RND>(ctx);
+        case TRTR_SRC_PULSE: return launch_sweep_typed<S, TRTR_SRC_PULSE, RND>(ctx);
+        default: return launch_sweep_typed<S, TRTR_SRC_NONE, RND>(ctx);
     }
 }
 
+template <typename S>
+static cudaError_t launch_sweep_2byte(trtr_ctx* ctx) {
+    if (ctx->p.rounding != TRTR_ROUND_STOCHASTIC) return launch_sweep_src<S, kRoundNearest>(ctx);
+    return ctx->p.nx % 2 == 0 ? launch_sweep_src<S, kRoundPairs>(ctx) : launch_sweep_src<S, kRoundNodes>(ctx);
+}
+
 cudaError_t launch_sweep(trtr_ctx* ctx) {
-    const bool sr = ctx->p.rounding == TRTR_ROUND_STOCHASTIC;
     switch (ctx->p.precision) {
-        case TRTR_F32: return launch_sweep_src<float, false>(ctx);
-        case TRTR_F16_OFS: return sr ? launch_sweep_src<__half, true>(ctx) : launch_sweep_src<__half, false>(ctx);
-        case TRTR_BF16_OFS:
-            return sr ? launch_sweep_src<__nv_bfloat16, true>(ctx) : launch_sweep_src<__nv_bfloat16, false>(ctx);
+        case TRTR_F32: return launch_sweep_src<float, kRoundNearest>(ctx);
+        case TRTR_F16_OFS: return launch_sweep_2byte<__half>(ctx);
+        case TRTR_BF16_OFS: return launch_sweep_2byte<__nv_bfloat16>(ctx);
         default: return cudaErrorInvalidValue;
     }
 }

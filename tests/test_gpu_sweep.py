@@ -1,5 +1,5 @@
-"""Four steps per launch (strips swept by four time levels behind one another): the bits of one
-launch per step, at the edges of strips (120 columns), of row blocks and of the ghost frames."""
+"""Four steps per launch (strips swept by four time levels behind one another, tiles on small grids): the
+bits of one launch per step, at the edges of strips (120 columns), tiles, row blocks and ghost frames."""
 import numpy as np
 import pytest
 
@@ -15,7 +15,9 @@ from ._gpu_util import random_case  # noqa: E402
 from .test_gpu_step2 import _pulse_solver, _random_solver  # noqa: E402
 
 PREC = {"f32": T.TRTR_F32, "f16": T.TRTR_F16_OFS, "bf16": T.TRTR_BF16_OFS}
-GRIDS = [(16, 32), (38, 40), (120, 64), (122, 35), (124, 33), (240, 34), (250, 300), (37, 50), (1101, 133)]
+# the smallest, the two tile heights of small grids (32 x 4 and 32 x 8 nodes) and sweeps (from 450 x 450
+# on), ragged in both directions; odd widths, where halo pairs fall between the rounding's pairs
+GRIDS = [(16, 32), (17, 33), (37, 50), (122, 35), (250, 300), (263, 301), (481, 470), (600, 330), (1201, 133)]
 
 
 @pytest.mark.parametrize("nx,ny", GRIDS)
@@ -39,22 +41,20 @@ def test_sweeps_equal_one_step_launches_bitwise(nx, ny, prec, kind, rounding):
             s.step(15)  # sweeps from the one-wide frame that it left, a pair and a single step
             s.step(66)  # past the levels of the pulse tables' first fill
             out[k] = (s.get_populations(), s.moments())
-        if k == 2 and (prec == "f32" or nx % 2 == 0):
-            assert l1 - l0 == 2 + 4  # field packing, ghost columns, four sweeps
+        if k == 2:  # field packing, (pulse tables at odd widths of 2-byte storage), ghost columns, four launches
+            assert 1 + 4 <= l1 - l0 <= 2 + 4
     assert np.array_equal(out[1][0], out[2][0], equal_nan=True)
     assert np.array_equal(out[1][1], out[2][1], equal_nan=True)
 
 
-@pytest.mark.parametrize("nx,ny", [(16, 32), (130, 41), (243, 64)])
+@pytest.mark.parametrize("nx,ny", [(16, 32), (243, 64), (1300, 130)])
 @pytest.mark.parametrize("prec", ["f32", "f16"])
 def test_sweeps_with_a_source_field_equal_one_step_launches_bitwise(nx, ny, prec):
     """Sweeps run while the field stays the same; after each change one single step comes first."""
     case = random_case(31 + nx, nx, ny)
-    nx2 = nx - nx % 2 if prec == "f16" else nx
-    case = {k: (np.ascontiguousarray(v[..., :nx2]) if isinstance(v, np.ndarray) else v) for k, v in case.items()}
     out = {}
     for k in (1, 2):
-        p = T.Params(nx=nx2, ny=ny, dx=case["dx"], dt=case["dt"], precision=PREC[prec], src_mode=T.TRTR_SRC_FIELD,
+        p = T.Params(nx=nx, ny=ny, dx=case["dx"], dt=case["dt"], precision=PREC[prec], src_mode=T.TRTR_SRC_FIELD,
                      grad_mode=T.TRTR_GRAD_PERIODIC)
         with T.Solver(p) as s:
             s.set_steps_per_launch(k)
@@ -72,7 +72,7 @@ def test_sweeps_with_a_source_field_equal_one_step_launches_bitwise(nx, ny, prec
             s.step(12)
             out[k] = s.get_populations()
         if k == 2:
-            assert l1 - l0 == 3 + 4  # fields, source term, ghost columns, four sweeps
+            assert 2 + 4 <= l1 - l0 <= 3 + 4  # fields, source term, (ghost columns), four launches
     assert np.array_equal(out[1], out[2])
 
 
