@@ -32,13 +32,6 @@ namespace {
 
 using namespace core;
 
-struct BatchClock {
-    long long n;        // step of the instances
-    unsigned int done;  // CTAs of the running launch that have finished
-    unsigned int next;  // next work-list entry of a dynamically scheduled launch
-    long long first;    // time level of the pulse tables' first entry
-};
-
 template <typename C>
 struct alignas(64) InstanceDesc {
     CUtensorMap mp[2];    // populations, source buffer 0 / 1
@@ -106,19 +99,6 @@ __device__ __forceinline__ void cp_async_16(void* sdst, const void* gsrc, int by
             "cp.async.cg.shared.global [%0], [g], 16;\n\t}" ::"r"(smem_addr(static_cast<char*>(sdst) + o)),
             "l"(static_cast<const char*>(gsrc) + o)
             : "memory");
-}
-
-// A CTA's end of a launch of `steps` steps (one thread): the last CTA to finish advances the step
-// clock and sets the work-list counter back.
-__device__ __forceinline__ void advance_clock(BatchClock* clk, int steps) {
-    __threadfence();
-    if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {
-        __threadfence();
-        clk->n += steps;
-        clk->next = 0;
-        clk->done = 0;
-        __threadfence();
-    }
 }
 
 template <int BY>
@@ -388,6 +368,10 @@ struct trtr_batch {
     int ntiles2;
     int grid2;
     bool two_step;
+    // four steps per launch (trtr_sweep.cu): its descriptors and work-list, and whether it is the faster
+    trtr::SweepBatch sweep;
+    bool four_step;
+    bool odd;  // an instance of odd width
     int steps_per_launch;
     cudaGraphExec_t graph2;
     bool graph2_valid;
@@ -633,6 +617,27 @@ trtr_status setup_two_step(trtr_batch* b) {
     return with_batch2(b, [&](auto l) { return decltype(l)::setup(b); });
 }
 
+// The sweep over the batch where it ends before two two-step launches would: its busiest CTA's rows at
+// 1.15 us for three rows (FP32; 1.87 us for four, 2-byte) against 110 (125) G nodes/s and at least 6 us a
+// two-step launch, as measured on GB300 (48 instances of 64^2 .. 1024^2: see trtr_batch_step).
+trtr_status setup_four_step(trtr_batch* b) {
+    b->four_step = true;
+    for (int k = 0; k < b->count; ++k) {
+        b->four_step = b->four_step && sweep_applies(b->ctx[k]);
+        b->odd = b->odd || b->ctx[k]->p.nx % 2 != 0;
+    }
+    if (!b->four_step) return TRTR_OK;
+    if (sweep_batch_setup(b->ctx, b->count, b->stream, &b->sweep) != cudaSuccess) {
+        cudaGetLastError();
+        return TRTR_ENOMEM;
+    }
+    const bool f32 = b->precision == TRTR_F32;
+    const double sweep = (double)b->sweep.rows / b->sweep.iteration_rows * (f32 ? 1.15 : 1.87);
+    const double two = 2.0 * std::max(6.0, 2.0 * (double)b->nodes / (f32 ? 110e3 : 125e3));
+    b->four_step = sweep < two || !b->two_step;
+    return TRTR_OK;
+}
+
 size_t desc_size(int precision) {
     return precision == TRTR_F64 ? sizeof(InstanceDesc<double>) : sizeof(InstanceDesc<float>);
 }
@@ -784,15 +789,34 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
     int par = b->parity;
     bool last_two = false;
     auto levels = [&](int steps) { return ensure_levels(b, b->step + (n - left), steps) == cudaSuccess; };
-    if (b->two_step && steps_per_launch == 2 && left >= 2) {
+    const bool four = b->four_step && steps_per_launch == 2 && left >= 4;
+    if (four || (b->two_step && steps_per_launch == 2 && left >= 2)) {
         for (int k = 0; k < b->count; ++k) {
             trtr_ctx* c = b->ctx[k];  // instances share the batch's stream
             if (!c->fld2_ready) {
                 if (launch_pack_fields2(c) != cudaSuccess) return TRTR_ECUDA;
                 c->fld2_ready = true;
+                b->ptab_ready = false;  // the packing fills the instance's tables from its step on
             }
-            if (!c->ghost2_ready && launch_refresh_ghosts2(c) != cudaSuccess) return TRTR_ECUDA;
         }
+    }
+    bool last_four = false;
+    if (four) {
+        bool columns = true;
+        for (int k = 0; k < b->count; ++k) columns = columns && b->ctx[k]->ghost4_ready;
+        if (!columns && sweep_batch_ghost_columns(b->sweep, b->count, b->ctx[0]->esize, par, b->stream) != cudaSuccess)
+            return TRTR_ECUDA;
+        for (; left >= 4; left -= 4, par ^= 1)
+            if (!levels(4) || sweep_batch_launch(b->sweep, b->d_clk, b->d_flag, par, b->precision, b->src, b->sr, b->odd,
+                                                 b->stream) != cudaSuccess)
+                return TRTR_ECUDA;
+        last_two = last_four = true;
+    }
+    if (b->two_step && steps_per_launch == 2 && left >= 2) {
+        if (!four)
+            for (int k = 0; k < b->count; ++k)
+                if (!b->ctx[k]->ghost2_ready && launch_refresh_ghosts2(b->ctx[k]) != cudaSuccess) return TRTR_ECUDA;
+        last_four = false;
         if (par == 1) {
             if (!levels(2) || launch_two(b, 1) != cudaSuccess) return TRTR_ECUDA;
             par = 0;
@@ -811,7 +835,7 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
         }
         last_two = true;
     }
-    if (left > 0) last_two = false;  // one-step launches follow: the one-wide ghost frame
+    if (left > 0) last_two = last_four = false;  // one-step launches follow: the one-wide ghost frame
     if (left > 0 && par == 1) {  // bring the ping-pong to parity 0 for the graph
         if (!levels(1) || launch_one(b, 1) != cudaSuccess) return TRTR_ECUDA;
         par = 0;
@@ -833,7 +857,7 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
         b->ctx[k]->step = b->step;
         b->ctx[k]->cur = b->parity;
         if (n > 0) b->ctx[k]->ghost2_ready = last_two;
-        if (n > 0) b->ctx[k]->ghost4_ready = false;
+        if (n > 0) b->ctx[k]->ghost4_ready = last_four;
         b->ctx[k]->launches += n;
     }
     return TRTR_OK;
@@ -913,6 +937,7 @@ trtr_status trtr_batch_create(const trtr_instance* inst, int count, void* cuda_s
         s = TRTR_ENOMEM;
     }
     if (s == TRTR_OK && b->two_step) s = trtr::setup_two_step(b);
+    if (s == TRTR_OK) s = trtr::setup_four_step(b);
     if (s == TRTR_OK) s = trtr::reset_clock(b);
     if (s != TRTR_OK) {
         trtr_batch_destroy(b);
@@ -927,6 +952,7 @@ trtr_status trtr_batch_destroy(trtr_batch* b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->graph_valid) cudaGraphExecDestroy(b->graph);
     if (b->graph2_valid) cudaGraphExecDestroy(b->graph2);
+    trtr::sweep_batch_free(&b->sweep);
     for (int k = 0; k < b->count; ++k)
         if (b->ctx && b->ctx[k]) trtr_destroy(b->ctx[k]);
     void* ptrs[] = {b->d_desc, b->d_tiles, b->d_fill, b->d_clk, b->d_flag, b->d_desc2, b->d_tiles2};

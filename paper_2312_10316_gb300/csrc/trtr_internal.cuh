@@ -265,6 +265,22 @@ constexpr long kDynMinTilesPerCta = 8;
 
 enum MapId { kMapPop0 = 0, kMapPop1 = 1, kMapU = 2, kMapD = 3, kMapS = 4, kNumMaps = 5 };
 
+// Device clock of a batch.
+struct BatchClock {
+    long long n;        // step of the instances
+    unsigned int done;  // CTAs of the running launch that have finished
+    unsigned int next;  // next work-list entry of a dynamically scheduled launch
+    long long first;    // time level of the pulse tables' first entry
+};
+
+// The four-step kernel over a batch: its descriptors and work-list (device), and the work-list's length
+// (rows of its busiest CTA, ramps included, and rows of an iteration).
+struct SweepBatch {
+    void *d_desc = nullptr, *d_units = nullptr, *d_first = nullptr;
+    int ctas = 0, iteration_rows = 1;
+    long rows = 0;
+};
+
 // What the table fill needs of a context or of a batch's instance.
 struct PulseFill {
     void* tab;                       // [kPulseLevels][level]
@@ -370,6 +386,13 @@ cudaError_t launch_pack_source(trtr_ctx* ctx);  // the source term's plane of th
 // four, two or one steps, with what the launch needs; advances the context's state.  *taken: the
 // steps; *what: names the failing launch on an error.
 cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what);
+// the same over a batch's instances (all of sweep_applies): setup, the ghost columns of buffer `parity`,
+// one launch of four steps from buffer `parity` (odd: an instance of odd width)
+cudaError_t sweep_batch_setup(trtr_ctx* const* ctx, int count, cudaStream_t stream, SweepBatch* out);
+void sweep_batch_free(SweepBatch* b);
+cudaError_t sweep_batch_ghost_columns(const SweepBatch& b, int count, int esize, int parity, cudaStream_t stream);
+cudaError_t sweep_batch_launch(const SweepBatch& b, BatchClock* clk, int* flag, int parity, int precision, int src, bool sr,
+                               bool odd, cudaStream_t stream);
 // one block whose bounded wait on a barrier that nothing completes gives up after `cycles`
 cudaError_t launch_wait_timeout(trtr_ctx* ctx, long long cycles);
 // one thread that gives the bounds checks four bad arguments and accesses nothing with them

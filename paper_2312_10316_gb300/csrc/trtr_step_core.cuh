@@ -171,6 +171,19 @@ __device__ __forceinline__ bool bulk_ok(const S* gdst, const void* src, int i0, 
     return true;
 }
 
+// A CTA's end of a batch launch of `steps` steps (one thread): the last CTA to finish advances the step
+// clock and sets the work-list counter back.
+__device__ __forceinline__ void advance_clock(BatchClock* clk, int steps) {
+    __threadfence();
+    if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        clk->n += steps;
+        clk->next = 0;
+        clk->done = 0;
+        __threadfence();
+    }
+}
+
 // Walks the linear tile indices t, t + stride, t + 2 stride, ... of a persistent CTA as
 // (t mod m, t div m) without a division per tile: one division at the start, then an add and a
 // carry per step (m: tiles per row of the order's rows).

@@ -18,6 +18,11 @@
 //
 // Work units are (strip, segment of rows); a segment costs C rows of ramp (its first output row
 // needs C / R iterations), so the host picks the number of segments that ends soonest.
+#include <algorithm>
+#include <queue>
+#include <utility>
+#include <vector>
+
 #include "trtr_step_core.cuh"
 
 namespace trtr {
@@ -71,6 +76,29 @@ struct SweepArgs {
     int tau2_fixed;
     float magic, omega2_fixed, phi_ref;
     uint32_t rkey[kT];
+};
+
+// What a launch works on.  OneGrid: the strips of one context, unit u = (strip, segment), taken by the CTAs
+// in turn.  ManyGrids: the strips of a batch's instances, unit u = units[u] = (instance, i0, j0, j1), CTA b's
+// from first[b] on; the step and its tables' levels come from the batch's clock.
+struct OneGrid {
+    static constexpr bool kBatch = false;
+    CUtensorMap mp, mf, mo;  // population rows of the source, field rows, interior of the result
+    SweepArgs a;
+};
+struct alignas(64) SweepDesc {
+    CUtensorMap mp[2], mo[2], mf;  // by buffer
+    SweepArgs a[2];                // by source buffer; pulse: the tables' first level
+    void* pop[2];
+};
+struct ManyGrids {
+    static constexpr bool kBatch = true;
+    const SweepDesc* desc;
+    const int4* units;
+    const int* first;
+    BatchClock* clk;
+    int* flag;
+    int parity;
 };
 
 // Columns of an nx-wide row in whole 16-byte chunks.
@@ -206,10 +234,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-template <typename S, int SRC, int RND, class G>
-__global__ void __launch_bounds__(G::Threads, 1)
-    sweep_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mf,
-                 const __grid_constant__ CUtensorMap mo, const __grid_constant__ SweepArgs a) {
+template <typename S, int SRC, int RND, class G, class Src>
+__global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_constant__ Src p) {
+    using Args = std::conditional_t<Src::kBatch, SweepArgs, const SweepArgs&>;  // (batch: copied once a unit)
     constexpr int R = G::R;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_abort;
@@ -219,7 +246,6 @@ __global__ void __launch_bounds__(G::Threads, 1)
     uint64_t* done = full + G::Blocks;                               // [kT][Depth]: a level has finished an iteration
     uint64_t* freed = done + kT * G::Depth;                          // [Outs]: an output buffer has been stored
     const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
-    const int nx = a.lp.nx, ny = a.lp.ny;
     if (tid == 0) {
         s_abort = 0;
         for (int b = 0; b < G::Blocks; ++b) mbar_init(&full[b], 1);
@@ -248,26 +274,67 @@ __global__ void __launch_bounds__(G::Threads, 1)
     // Iterations are numbered through all units of the CTA (`it0` before this one): iteration it of a
     // level completes phase it / Depth of done[level][it % Depth].
     struct Unit {
-        int i0, j0, j1, iters, a0;
+        int inst, i0, j0, j1, iters, a0;
+    };
+    auto args = [&](int inst) -> Args {
+        if constexpr (Src::kBatch)
+            return p.desc[inst].a[p.parity];
+        else
+            return p.a;
     };
     auto unit = [&](int u) {
         Unit t;
-        const int strip = u % a.strips, seg = u / a.strips;
-        t.i0 = strip * kX;
-        t.j0 = seg * a.seg_rows;
-        t.j1 = min(t.j0 + a.seg_rows, ny);
+        if constexpr (Src::kBatch) {
+            const int4 v = p.units[u];
+            t.inst = v.x;
+            t.i0 = v.y;
+            t.j0 = v.z;
+            t.j1 = v.w;
+        } else {
+            const int strip = u % p.a.strips, seg = u / p.a.strips;
+            t.inst = 0;
+            t.i0 = strip * kX;
+            t.j0 = seg * p.a.seg_rows;
+            t.j1 = min(t.j0 + p.a.seg_rows, p.a.lp.ny);
+        }
         t.iters = (t.j1 - t.j0 + G::C + R - 1) / R;
         t.a0 = t.j0 + (kT - 1) * G::Lag - G::C;  // level 1's first row
         return t;
     };
+    int u_first = blockIdx.x, u_end = 0, u_step = gridDim.x;
+    long long step = 0;   // batch: the step of this launch, and its level n - 1 in the pulse tables
+    int table_level = 0;
+    if constexpr (Src::kBatch) {
+        u_first = p.first[blockIdx.x];
+        u_end = p.first[blockIdx.x + 1];
+        u_step = 1;
+        const volatile BatchClock* c = p.clk;
+        step = c->n;
+        table_level = (int)(step - 1 - c->first);
+    } else {
+        u_end = p.a.units;
+    }
 
     if (w == G::Warps) {
         // The mover: lane 0 loads the blocks (block m of a unit: the rows a0 + 1 - R + m R ..; iteration
         // k needs the blocks up to k + 1) and stores the rows the last level has finished.
         unsigned phase = 0, it0 = 0, pending = 0;
         bool ok = true;
-        for (int u = blockIdx.x; u < a.units && ok; u += gridDim.x) {
+        for (int u = u_first; u < u_end && ok; u += u_step) {
             const Unit t = unit(u);
+            Args a = args(t.inst);
+            const int nx = a.lp.nx, ny = a.lp.ny;
+            const CUtensorMap *mp, *mf, *mo;
+            if constexpr (Src::kBatch) {
+                const SweepDesc* d = p.desc + t.inst;
+                mp = &d->mp[p.parity];
+                mf = &d->mf;
+                mo = &d->mo[p.parity ^ 1];
+            } else {
+                mp = &p.mp;
+                mf = &p.mf;
+                mo = &p.mo;
+            }
             const int blocks = t.iters + 1;
             auto load = [&](int m) {
                 const unsigned b = (phase + m) % G::Blocks;
@@ -279,8 +346,8 @@ __global__ void __launch_bounds__(G::Threads, 1)
                     unsigned char* pd = smem + (b * R + r) * G::PopPitch;
                     unsigned char* fd = smem + G::FldOff + (b * R + r) * G::FldRow;
                     const int xp = t.i0 - 2 * kT + a.lp.gx, xf = t.i0 - kT + a.gxf;
-                    if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, &mp, &full[b], xp, y + kGhostP, 0);
-                    if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, &mf, &full[b], xf, y + a.gyf, 0);
+                    if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, mp, &full[b], xp, y + kGhostP, 0);
+                    if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, mf, &full[b], xf, y + a.gyf, 0);
                 }
             };
             const bool edges = t.i0 == 0 || t.i0 + kX > min(nx - kGhostX, bulk_cols_of<S>(nx));
@@ -297,7 +364,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
                         fence_proxy_async_smem();
                         load(k + 2 + G::Ahead);
                     }
-                    if (y >= t.j0) tma_store_3d(&mo, buf, t.i0, y, 0);
+                    if (y >= t.j0) tma_store_3d(mo, buf, t.i0, y, 0);
                     bulk_commit();
                 }
                 if (edges && y >= t.j0) copy_edge_columns<S, G>(reinterpret_cast<const S*>(buf), a, t.i0, y, t.j1, lane);
@@ -314,28 +381,39 @@ __global__ void __launch_bounds__(G::Threads, 1)
         }
         if (lane == 0) {
             if (!ok) {  // let the loads issued into this CTA's shared memory land (bounded)
-                atomicExch(a.flag, 1);
+                if constexpr (Src::kBatch)
+                    atomicExch(p.flag, 1);
+                else
+                    atomicExch(p.a.flag, 1);
                 const unsigned n = pending < (unsigned)G::Blocks ? pending : (unsigned)G::Blocks;
                 for (unsigned m = pending - n; m < pending; ++m)
                     mbar_wait_bounded(&full[m % G::Blocks], (m / G::Blocks) & 1);
             }
             bulk_wait_all();
+            // every warp has read the clock: the last level has finished its units (or a wait gave up)
+            if constexpr (Src::kBatch) advance_clock(p.clk, ok ? kT : 0);
         }
         return;
     }
 
     // Level `level`, row r0 of every iteration.
     const int level = w / R + 1, r0 = w % R;
-    const uint32_t rkey = a.rkey[level - 1];
+    uint32_t rkey = 0u;
+    if constexpr (Src::kBatch)
+        rkey = RND != kRoundNearest ? sr_step_key((long)step + level - 1) : 0u;
+    else
+        rkey = p.a.rkey[level - 1];
     unsigned phase = 0, it = 0;
-    for (int u = blockIdx.x; u < a.units; u += gridDim.x) {
+    for (int u = u_first; u < u_end; u += u_step) {
         const Unit t = unit(u);
+        Args a = args(t.inst);
+        const int nx = a.lp.nx, ny = a.lp.ny;
         // per strip: the pairs' columns, their images for the rounding keys, their pulse factors
         const int i = t.i0 - kT + 2 * lane;
         F2 p1p[2], p2p[2], p1n[2], p2n[2];
         int wa[2], wb[2];
         uint32_t sel[2];
-        const float* lev = a.pulse + (level - 1) * a.pt.level;
+        const float* lev = a.pulse + (size_t)(table_level + level - 1) * a.pt.level;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (SRC == TRTR_SRC_PULSE) {
@@ -423,7 +501,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
 
 // The kGhostX ghost columns of every interior row and plane from the interior (periodic).
 template <typename E>
-__global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
+__device__ __forceinline__ void refresh_ghost_columns(E* P, const PlaneLayout& L) {
     const int n = kQ * L.ny * 2 * kGhostX;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int g = k % (2 * kGhostX), row = k / (2 * kGhostX), q = row / L.ny, j = row - q * L.ny;
@@ -432,28 +510,48 @@ __global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
         p[to] = p[g < kGhostX ? L.nx + to : to - L.nx];
     }
 }
+template <typename E>
+__global__ void refresh_ghost_columns_kernel(E* P, PlaneLayout L) {
+    refresh_ghost_columns(P, L);
+}
+
+// The arguments of one context: from buffer `from` into the other.
+template <typename S>
+SweepArgs sweep_args(const trtr_ctx* ctx, int from) {
+    SweepArgs a;
+    memset(static_cast<void*>(&a), 0, sizeof(a));
+    a.pt = PulseTab::make(ctx->p.nx, ctx->p.ny);
+    a.dst = ctx->pop[from ^ 1];
+    a.lp = ctx->lp;
+    a.gxf = ctx->lt.gx;
+    a.gyf = ctx->lt.gy;
+    a.strips = (ctx->p.nx + kX - 1) / kX;
+    a.tau2_fixed = ctx->p.tau2_mode == TRTR_TAU2_FIXED;
+    a.magic = (float)ctx->p.magic;
+    a.omega2_fixed = (float)(ctx->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / ctx->p.tau2 : 0.0);
+    a.phi_ref = (float)ctx->p.phi_ref;
+    return a;
+}
 
 template <typename S, int SRC, int RND>
 cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     using G = Sweep<S, SRC>;
-    auto kernel = sweep_kernel<S, SRC, RND, G>;
+    auto kernel = sweep_kernel<S, SRC, RND, G, OneGrid>;
     static int configured_device = -1;
     if (configured_device != ctx->device) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
         if (e != cudaSuccess) return e;
         configured_device = ctx->device;
     }
-    const int nx = ctx->p.nx, ny = ctx->p.ny;
-    SweepArgs a;
-    memset(static_cast<void*>(&a), 0, sizeof(a));
-    a.pt = PulseTab::make(nx, ny);
+    const int ny = ctx->p.ny;
+    OneGrid p;
+    p.mp = ctx->maps4[ctx->cur];
+    p.mf = ctx->maps4[4];
+    p.mo = ctx->maps4[2 + (ctx->cur ^ 1)];
+    SweepArgs& a = p.a;
+    a = sweep_args<S>(ctx, ctx->cur);
     a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<float>(ctx, a.pt, ctx->step) : nullptr;
-    a.dst = ctx->pop[ctx->cur ^ 1];
     a.flag = ctx->dflag;
-    a.lp = ctx->lp;
-    a.gxf = ctx->lt.gx;
-    a.gyf = ctx->lt.gy;
-    a.strips = (nx + kX - 1) / kX;
     // the number of segments a strip that ends soonest: rounds of the SMs times a unit's rows
     long best = 0;
     int segs = 1;
@@ -468,10 +566,6 @@ cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     }
     a.seg_rows = ((ny + segs - 1) / segs + G::R - 1) / G::R * G::R;
     a.units = a.strips * ((ny + a.seg_rows - 1) / a.seg_rows);
-    a.tau2_fixed = ctx->p.tau2_mode == TRTR_TAU2_FIXED;
-    a.magic = (float)ctx->p.magic;
-    a.omega2_fixed = (float)(ctx->p.tau2_mode == TRTR_TAU2_FIXED ? 1.0 / ctx->p.tau2 : 0.0);
-    a.phi_ref = (float)ctx->p.phi_ref;
     for (int s = 0; s < kT; ++s) a.rkey[s] = sr_step_key(ctx->step + s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.units < ctx->num_sms ? a.units : ctx->num_sms));
@@ -483,21 +577,137 @@ cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, ctx->maps4[ctx->cur], ctx->maps4[4], ctx->maps4[2 + (ctx->cur ^ 1)], a);
+    return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
-template <typename S, int SRC>
-cudaError_t encode4_typed(trtr_ctx* ctx) {
-    using G = Sweep<S, SRC>;
+// The maps of one context: population rows (buffers 0, 1), interior stores (0, 1; whole 16-byte chunks of a
+// row), field rows.
+template <typename S, class G>
+bool encode_maps_of(const trtr_ctx* ctx, CUtensorMap* rows, CUtensorMap* stores, CUtensorMap* fields) {
     bool ok = true;
     PlaneLayout in = ctx->lp;  // the interior alone, so that stores are clipped to it
     in.nx = bulk_cols_of<S>(in.nx);
     for (int b = 0; b < 2; ++b) {
-        ok = ok && encode(&ctx->maps4[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], ctx->lp, kQ, kW, 1, kQ);
-        ok = ok && encode_interior(&ctx->maps4[2 + b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], in, kQ, kX, G::R, kQ);
+        ok = ok && encode(&rows[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], ctx->lp, kQ, kW, 1, kQ);
+        ok = ok && encode_interior(&stores[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], in, kQ, kX, G::R, kQ);
     }
-    ok = ok && encode(&ctx->maps4[4], tma_type<float>(), 4, ctx->fld2, ctx->lt, G::NF, kWC, 1, G::NF);
-    return ok ? cudaSuccess : cudaErrorInvalidValue;
+    return ok && encode(fields, tma_type<float>(), 4, ctx->fld2, ctx->lt, G::NF, kWC, 1, G::NF);
+}
+
+template <typename S, int SRC>
+cudaError_t encode4_typed(trtr_ctx* ctx) {
+    return encode_maps_of<S, Sweep<S, SRC>>(ctx, &ctx->maps4[0], &ctx->maps4[2], &ctx->maps4[4]) ? cudaSuccess
+                                                                                                 : cudaErrorInvalidValue;
+}
+
+// ---- batches -------------------------------------------------------------------------------------
+
+// The four ghost columns of every instance's current buffer.
+template <typename E>
+__global__ void batch_ghost_columns_kernel(const SweepDesc* desc, int parity) {
+    const SweepDesc& d = desc[blockIdx.y];
+    refresh_ghost_columns(static_cast<E*>(d.pop[parity]), d.a[0].lp);
+}
+
+// The work-list: strips cut into segments, the units dealt longest first to the CTA with the least work
+// so far.  Returns the rows (ramps included) of the busiest CTA.
+template <class G>
+long deal_units(trtr_ctx* const* ctx, int count, int ctas, long most_rows, std::vector<int4>& units, std::vector<int>& first) {
+    std::vector<std::pair<long, int4>> all;
+    for (int k = 0; k < count; ++k) {
+        const int nx = ctx[k]->p.nx, ny = ctx[k]->p.ny;
+        const int segs = (int)((ny + most_rows - 1) / most_rows);
+        const int rows = ((ny + segs - 1) / segs + G::R - 1) / G::R * G::R;
+        for (int j0 = 0; j0 < ny; j0 += rows)
+            for (int i0 = 0; i0 < nx; i0 += kX) {
+                const int j1 = std::min(j0 + rows, ny);
+                all.push_back({j1 - j0 + G::C + 4, make_int4(k, i0, j0, j1)});
+            }
+    }
+    std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    using Load = std::pair<long, int>;
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
+    std::vector<std::vector<int4>> mine(ctas);
+    for (int c = 0; c < ctas; ++c) load.push({0, c});
+    long busiest = 0;
+    for (const auto& u : all) {
+        Load l = load.top();
+        load.pop();
+        mine[l.second].push_back(u.second);
+        l.first += u.first;
+        busiest = std::max(busiest, l.first);
+        load.push(l);
+    }
+    units.clear();
+    first.assign(1, 0);
+    for (const auto& m : mine) {
+        units.insert(units.end(), m.begin(), m.end());
+        first.push_back((int)units.size());
+    }
+    return busiest;
+}
+
+template <typename S>
+cudaError_t setup_batch_typed(trtr_ctx* const* ctx, int count, cudaStream_t stream, SweepBatch* out) {
+    using G = Sweep<S, TRTR_SRC_NONE>;  // (the pulse's is the same)
+    static_assert(Sweep<S, TRTR_SRC_PULSE>::R == G::R && Sweep<S, TRTR_SRC_PULSE>::NF == G::NF, "one geometry");
+    const int ctas = ctx[0]->num_sms;
+    long total = 0;
+    for (int k = 0; k < count; ++k) total += (long)((ctx[k]->p.nx + kX - 1) / kX) * ctx[k]->p.ny;
+    std::vector<int4> units, best_units;
+    std::vector<int> first, best_first;
+    long best = -1;
+    for (int parts = 1; parts <= 6; ++parts) {
+        const long rows = std::max((long)G::R * 2, total / ((long)ctas * parts) + 1);
+        const long busiest = deal_units<G>(ctx, count, ctas, rows, units, first);
+        if (best < 0 || busiest < best) {
+            best = busiest;
+            best_units = units;
+            best_first = first;
+        }
+    }
+    out->rows = best;
+    out->iteration_rows = G::R;
+    std::vector<SweepDesc> h(count);
+    for (int k = 0; k < count; ++k) {
+        const trtr_ctx* c = ctx[k];
+        SweepDesc& d = h[k];
+        if (!encode_maps_of<S, G>(c, d.mp, d.mo, &d.mf)) return cudaErrorInvalidValue;
+        for (int b = 0; b < 2; ++b) {
+            d.a[b] = sweep_args<S>(c, b);
+            d.a[b].pulse = c->ptab ? static_cast<const float*>(c->ptab) + kTabGhost : nullptr;
+            d.pop[b] = c->pop[b];
+        }
+    }
+    out->ctas = ctas;
+    cudaError_t e = cudaMalloc(&out->d_desc, sizeof(SweepDesc) * count);
+    if (e == cudaSuccess) e = cudaMalloc(&out->d_units, sizeof(int4) * best_units.size());
+    if (e == cudaSuccess) e = cudaMalloc(&out->d_first, sizeof(int) * best_first.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out->d_desc, h.data(), sizeof(SweepDesc) * count, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out->d_units, best_units.data(), sizeof(int4) * best_units.size(), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(out->d_first, best_first.data(), sizeof(int) * best_first.size(), cudaMemcpyHostToDevice, stream);
+    const cudaError_t s = cudaStreamSynchronize(stream);  // the vectors go out of scope
+    return e != cudaSuccess ? e : s;
+}
+
+template <typename S, int SRC, int RND>
+cudaError_t launch_batch_typed(const SweepBatch& b, BatchClock* clk, int* flag, int parity, cudaStream_t stream) {
+    using G = Sweep<S, SRC>;
+    auto kernel = sweep_kernel<S, SRC, RND, G, ManyGrids>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
+    if (e != cudaSuccess) return e;
+    ManyGrids p;
+    p.desc = static_cast<const SweepDesc*>(b.d_desc);
+    p.units = static_cast<const int4*>(b.d_units);
+    p.first = static_cast<const int*>(b.d_first);
+    p.clk = clk;
+    p.flag = flag;
+    p.parity = parity;
+    kernel<<<b.ctas, G::Threads, G::Smem, stream>>>(p);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -578,6 +788,56 @@ cudaError_t launch_sweep(trtr_ctx* ctx) {
         case TRTR_F32: return launch_sweep_src<float, kRoundNearest>(ctx);
         case TRTR_F16_OFS: return launch_sweep_2byte<__half>(ctx);
         case TRTR_BF16_OFS: return launch_sweep_2byte<__nv_bfloat16>(ctx);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t sweep_batch_setup(trtr_ctx* const* ctx, int count, cudaStream_t stream, SweepBatch* out) {
+    switch (ctx[0]->p.precision) {
+        case TRTR_F32: return setup_batch_typed<float>(ctx, count, stream, out);
+        case TRTR_F16_OFS: return setup_batch_typed<__half>(ctx, count, stream, out);
+        case TRTR_BF16_OFS: return setup_batch_typed<__nv_bfloat16>(ctx, count, stream, out);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+void sweep_batch_free(SweepBatch* b) {
+    for (void* p : {b->d_desc, b->d_units, b->d_first})
+        if (p) cudaFree(p);
+    *b = SweepBatch();
+}
+
+cudaError_t sweep_batch_ghost_columns(const SweepBatch& b, int count, int esize, int parity, cudaStream_t stream) {
+    for (int k = 0; k < count; k += 65535) {
+        const SweepDesc* d = static_cast<const SweepDesc*>(b.d_desc) + k;
+        const dim3 grid(16, count - k < 65535 ? count - k : 65535);
+        if (esize == 4)
+            batch_ghost_columns_kernel<float><<<grid, 256, 0, stream>>>(d, parity);
+        else
+            batch_ghost_columns_kernel<unsigned short><<<grid, 256, 0, stream>>>(d, parity);
+    }
+    return cudaGetLastError();
+}
+
+template <typename S, int RND>
+static cudaError_t launch_batch_src(const SweepBatch& b, BatchClock* clk, int* flag, int parity, int src, cudaStream_t stream) {
+    return src == TRTR_SRC_PULSE ? launch_batch_typed<S, TRTR_SRC_PULSE, RND>(b, clk, flag, parity, stream)
+                                 : launch_batch_typed<S, TRTR_SRC_NONE, RND>(b, clk, flag, parity, stream);
+}
+template <typename S>
+static cudaError_t launch_batch_2byte(const SweepBatch& b, BatchClock* clk, int* flag, int parity, int src, bool sr, bool odd,
+                                      cudaStream_t stream) {
+    if (!sr) return launch_batch_src<S, kRoundNearest>(b, clk, flag, parity, src, stream);
+    return odd ? launch_batch_src<S, kRoundNodes>(b, clk, flag, parity, src, stream)
+               : launch_batch_src<S, kRoundPairs>(b, clk, flag, parity, src, stream);
+}
+
+cudaError_t sweep_batch_launch(const SweepBatch& b, BatchClock* clk, int* flag, int parity, int precision, int src, bool sr,
+                               bool odd, cudaStream_t stream) {
+    switch (precision) {
+        case TRTR_F32: return launch_batch_src<float, kRoundNearest>(b, clk, flag, parity, src, stream);
+        case TRTR_F16_OFS: return launch_batch_2byte<__half>(b, clk, flag, parity, src, sr, odd, stream);
+        case TRTR_BF16_OFS: return launch_batch_2byte<__nv_bfloat16>(b, clk, flag, parity, src, sr, odd, stream);
         default: return cudaErrorInvalidValue;
     }
 }

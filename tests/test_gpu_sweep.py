@@ -1,7 +1,11 @@
 """Four steps per launch (strips swept by four time levels behind one another, tiles on small grids): the
 bits of one launch per step, at the edges of strips (120 columns), tiles, row blocks and ghost frames."""
+import dataclasses
+
 import numpy as np
 import pytest
+
+from paper_2312_10316_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -83,3 +87,23 @@ def test_sweeps_stop_at_the_stability_checks():
             s.step(30)
             res[k] = s.get_populations()
     assert np.array_equal(res[1], res[2])
+
+
+@pytest.mark.parametrize("prec", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("D_amp", [0.0, 0.5])
+def test_batched_sweeps_equal_single_solves_bitwise(prec, D_amp):
+    """Uneven instances (odd widths, more than one strip, several segments) through the batch's four-step
+    launches, with steps left over for the two- and one-step ones."""
+    pulses = [W.Pulse(n=n, D_amp=D_amp, courant=0.3, sigma0=0.1 + 0.01 * k) for k, n in enumerate((700, 33, 250, 123, 641))]
+    if prec != "f32":
+        pulses = [dataclasses.replace(p, n=p.n + k % 2) for k, p in enumerate(pulses)]
+    with T.Batch([T.pulse_instance(p, PREC[prec]) for p in pulses]) as b:
+        b.step(8)
+        b.step(7)
+        b.step(70)
+        got = [b.instance(k).get_populations() for k in range(len(pulses))]
+    for p, g in zip(pulses, got):
+        with T.pulse_solver(p, precision=PREC[prec]) as s:
+            s.set_steps_per_launch(1)
+            s.step(85)
+            assert np.array_equal(s.get_populations(), g), p.n
