@@ -135,9 +135,9 @@ struct RoundKey {
 // slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
 // the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
 // rows within kGhostP of an edge).
-template <typename S, int LV, int SRC, int RND, class G>
+template <typename S, int LV, int SRC, int RND, class G, class Wait>
 __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[2], const SweepArgs& a,
-                                          const RoundKey rk[2], S* out_row, int lane, int i, int j) {
+                                          const RoundKey rk[2], S* out_row, int lane, int i, int j, Wait&& buffer_free) {
     constexpr bool kOfs = sizeof(S) == 2;
     using S2 = typename Pair<S>::type;
     F2 out[2][kQ];
@@ -185,6 +185,7 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
                 }
             }
     } else {
+        if (!buffer_free()) return;  // (a wait gave up: the warp leaves at its next wait)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
@@ -360,10 +361,8 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
                 const int y = t.a0 + k * R - (kT - 1) * G::Lag;  // the last level's rows
                 unsigned char* buf = smem + G::OutOff + o * G::OutBytes;
                 if (lane == 0) {
-                    if (k + 2 + G::Ahead < blocks) {
-                        fence_proxy_async_smem();
-                        load(k + 2 + G::Ahead);
-                    }
+                    fence_proxy_async_smem();  // what the levels wrote in the ring and the buffer, for TMA
+                    if (k + 2 + G::Ahead < blocks) load(k + 2 + G::Ahead);
                     if (y >= t.j0) tma_store_3d(mo, buf, t.i0, y, 0);
                     bulk_commit();
                 }
@@ -449,7 +448,7 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
                                   F2(-0.5f) * vfma(p1p[h], F2(qp.x), p2p[h] * F2(qp.y)));
             }
             // level 1 waits for its rows, the others for the level before to have finished the iteration
-            // before this one; the last level also for its output buffer
+            // before this one; the last level also, before it writes, for its output buffer
             bool ok;
             if (level == 1) {
                 if (++block == G::Blocks) {
@@ -461,7 +460,6 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
                 ok = it == 0 || wait(&done[(level - 2) * G::Depth + (it - 1) % G::Depth], ((it - 1) / G::Depth) & 1);
             }
             const unsigned o = it % G::Outs;
-            if (level == kT && it >= (unsigned)G::Outs) ok = ok && wait(&freed[o], (it / G::Outs - 1) & 1);
             if (!ok) return;
             if (j >= t.j0 - (kT - level) && j < t.j1 + (kT - level)) {
                 const int below = ring >= level ? ring - level : ring - level + G::Ring;
@@ -482,14 +480,14 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
                     }
                 }
                 S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane - kT;
+                auto buffer_free = [&]() { return it < (unsigned)G::Outs || wait(&freed[o], (it / G::Outs - 1) & 1); };
                 switch (level) {
-                    case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
-                    default: sweep_row<S, 4, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j); break;
+                    case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
+                    case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
+                    case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
+                    default: sweep_row<S, 4, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
                 }
             }
-            if (level == kT) fence_proxy_async_smem();  // the rows, for the TMA store
             __syncwarp();
             if (lane == 0) mbar_arrive(&done[(level - 1) * G::Depth + it % G::Depth]);
             ring += R;
