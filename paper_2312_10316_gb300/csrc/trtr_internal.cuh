@@ -335,6 +335,7 @@ struct trtr_ctx {
     trtr::PlaneLayout lt;   // layout of fld2
     bool src_ready;         // its source plane (TRTR_SRC_FIELD) holds the current S^n
     bool fld2_ready;        // fld2 holds the current fields
+    int sweep_rows;         // rows of its segments
     bool ghost4_ready;      // its four-wide ghost columns are up to date (interior rows)
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
     void* pack64;           // FP64: [4][rows][pitch] a_x, a_y, k1, k2 (the layout of uv)

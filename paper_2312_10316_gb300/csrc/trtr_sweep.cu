@@ -78,21 +78,14 @@ struct SweepArgs {
     uint32_t rkey[kT];
 };
 
-// What a launch works on.  OneGrid: the strips of one context, unit u = (strip, segment), taken by the CTAs
-// in turn.  ManyGrids: the strips of a batch's instances, unit u = units[u] = (instance, i0, j0, j1), CTA b's
-// from first[b] on; the step and its tables' levels come from the batch's clock.
-struct OneGrid {
-    static constexpr bool kBatch = false;
-    CUtensorMap mp, mf, mo;  // population rows of the source, field rows, interior of the result
-    SweepArgs a;
-};
+// A batch launch works on the strips of its instances: unit u = units[u] = (instance, i0, j0, j1), CTA b's from
+// first[b] on; the step and its tables' levels come from the batch's clock.
 struct alignas(64) SweepDesc {
     CUtensorMap mp[2], mo[2], mf;  // by buffer
     SweepArgs a[2];                // by source buffer; pulse: the tables' first level
     void* pop[2];
 };
 struct ManyGrids {
-    static constexpr bool kBatch = true;
     const SweepDesc* desc;
     const int4* units;
     const int* first;
@@ -235,9 +228,14 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-template <typename S, int SRC, int RND, class G, class Src>
-__global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_constant__ Src p) {
-    using Args = std::conditional_t<Src::kBatch, SweepArgs, const SweepArgs&>;  // (batch: copied once a unit)
+// One context (BATCH = false): mp_ population rows of the source, mf_ field rows, mo_ interior of the result;
+// unit u = (strip, segment), taken by the CTAs in turn.  BATCH: many alone.
+template <typename S, int SRC, int RND, class G, bool BATCH>
+__global__ void __launch_bounds__(G::Threads, 1)
+    sweep_kernel(const __grid_constant__ CUtensorMap mp_, const __grid_constant__ CUtensorMap mf_,
+                 const __grid_constant__ CUtensorMap mo_, const __grid_constant__ SweepArgs a_,
+                 const __grid_constant__ ManyGrids p) {
+    using Args = std::conditional_t<BATCH, SweepArgs, const SweepArgs&>;  // (batch: copied once a unit)
     constexpr int R = G::R;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_abort;
@@ -278,25 +276,25 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
         int inst, i0, j0, j1, iters, a0;
     };
     auto args = [&](int inst) -> Args {
-        if constexpr (Src::kBatch)
+        if constexpr (BATCH)
             return p.desc[inst].a[p.parity];
         else
-            return p.a;
+            return a_;
     };
     auto unit = [&](int u) {
         Unit t;
-        if constexpr (Src::kBatch) {
+        if constexpr (BATCH) {
             const int4 v = p.units[u];
             t.inst = v.x;
             t.i0 = v.y;
             t.j0 = v.z;
             t.j1 = v.w;
         } else {
-            const int strip = u % p.a.strips, seg = u / p.a.strips;
+            const int strip = u % a_.strips, seg = u / a_.strips;
             t.inst = 0;
             t.i0 = strip * kX;
-            t.j0 = seg * p.a.seg_rows;
-            t.j1 = min(t.j0 + p.a.seg_rows, p.a.lp.ny);
+            t.j0 = seg * a_.seg_rows;
+            t.j1 = min(t.j0 + a_.seg_rows, a_.lp.ny);
         }
         t.iters = (t.j1 - t.j0 + G::C + R - 1) / R;
         t.a0 = t.j0 + (kT - 1) * G::Lag - G::C;  // level 1's first row
@@ -305,7 +303,7 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
     int u_first = blockIdx.x, u_end = 0, u_step = gridDim.x;
     long long step = 0;   // batch: the step of this launch, and its level n - 1 in the pulse tables
     int table_level = 0;
-    if constexpr (Src::kBatch) {
+    if constexpr (BATCH) {
         u_first = p.first[blockIdx.x];
         u_end = p.first[blockIdx.x + 1];
         u_step = 1;
@@ -313,7 +311,7 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
         step = c->n;
         table_level = (int)(step - 1 - c->first);
     } else {
-        u_end = p.a.units;
+        u_end = a_.units;
     }
 
     if (w == G::Warps) {
@@ -326,15 +324,15 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
             Args a = args(t.inst);
             const int nx = a.lp.nx, ny = a.lp.ny;
             const CUtensorMap *mp, *mf, *mo;
-            if constexpr (Src::kBatch) {
+            if constexpr (BATCH) {
                 const SweepDesc* d = p.desc + t.inst;
                 mp = &d->mp[p.parity];
                 mf = &d->mf;
                 mo = &d->mo[p.parity ^ 1];
             } else {
-                mp = &p.mp;
-                mf = &p.mf;
-                mo = &p.mo;
+                mp = &mp_;
+                mf = &mf_;
+                mo = &mo_;
             }
             const int blocks = t.iters + 1;
             auto load = [&](int m) {
@@ -380,17 +378,17 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
         }
         if (lane == 0) {
             if (!ok) {  // let the loads issued into this CTA's shared memory land (bounded)
-                if constexpr (Src::kBatch)
+                if constexpr (BATCH)
                     atomicExch(p.flag, 1);
                 else
-                    atomicExch(p.a.flag, 1);
+                    atomicExch(a_.flag, 1);
                 const unsigned n = pending < (unsigned)G::Blocks ? pending : (unsigned)G::Blocks;
                 for (unsigned m = pending - n; m < pending; ++m)
                     mbar_wait_bounded(&full[m % G::Blocks], (m / G::Blocks) & 1);
             }
             bulk_wait_all();
             // every warp has read the clock: the last level has finished its units (or a wait gave up)
-            if constexpr (Src::kBatch) advance_clock(p.clk, ok ? kT : 0);
+            if constexpr (BATCH) advance_clock(p.clk, ok ? kT : 0);
         }
         return;
     }
@@ -398,10 +396,10 @@ __global__ void __launch_bounds__(G::Threads, 1) sweep_kernel(const __grid_const
     // Level `level`, row r0 of every iteration.
     const int level = w / R + 1, r0 = w % R;
     uint32_t rkey = 0u;
-    if constexpr (Src::kBatch)
+    if constexpr (BATCH)
         rkey = RND != kRoundNearest ? sr_step_key((long)step + level - 1) : 0u;
     else
-        rkey = p.a.rkey[level - 1];
+        rkey = a_.rkey[level - 1];
     unsigned phase = 0, it = 0;
     for (int u = u_first; u < u_end; u += u_step) {
         const Unit t = unit(u);
@@ -534,36 +532,18 @@ SweepArgs sweep_args(const trtr_ctx* ctx, int from) {
 template <typename S, int SRC, int RND>
 cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     using G = Sweep<S, SRC>;
-    auto kernel = sweep_kernel<S, SRC, RND, G, OneGrid>;
+    auto kernel = sweep_kernel<S, SRC, RND, G, false>;
     static int configured_device = -1;
     if (configured_device != ctx->device) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
         if (e != cudaSuccess) return e;
         configured_device = ctx->device;
     }
-    const int ny = ctx->p.ny;
-    OneGrid p;
-    p.mp = ctx->maps4[ctx->cur];
-    p.mf = ctx->maps4[4];
-    p.mo = ctx->maps4[2 + (ctx->cur ^ 1)];
-    SweepArgs& a = p.a;
-    a = sweep_args<S>(ctx, ctx->cur);
+    SweepArgs a = sweep_args<S>(ctx, ctx->cur);
     a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<float>(ctx, a.pt, ctx->step) : nullptr;
     a.flag = ctx->dflag;
-    // the number of segments a strip that ends soonest: rounds of the SMs times a unit's rows
-    long best = 0;
-    int segs = 1;
-    for (int s = 1; s <= (ny + G::R - 1) / G::R && s <= 4 * ctx->num_sms; ++s) {
-        const int rows = ((ny + s - 1) / s + G::R - 1) / G::R * G::R;
-        const long units = (long)a.strips * ((ny + rows - 1) / rows);
-        const long cost = ((units + ctx->num_sms - 1) / ctx->num_sms) * (rows + G::C + 4);
-        if (s == 1 || cost < best) {
-            best = cost;
-            segs = s;
-        }
-    }
-    a.seg_rows = ((ny + segs - 1) / segs + G::R - 1) / G::R * G::R;
-    a.units = a.strips * ((ny + a.seg_rows - 1) / a.seg_rows);
+    a.seg_rows = ctx->sweep_rows;
+    a.units = a.strips * ((ctx->p.ny + a.seg_rows - 1) / a.seg_rows);
     for (int s = 0; s < kT; ++s) a.rkey[s] = sr_step_key(ctx->step + s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.units < ctx->num_sms ? a.units : ctx->num_sms));
@@ -575,7 +555,8 @@ cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    return cudaLaunchKernelEx(&cfg, kernel, ctx->maps4[ctx->cur], ctx->maps4[4], ctx->maps4[2 + (ctx->cur ^ 1)], a,
+                              ManyGrids());
 }
 
 // The maps of one context: population rows (buffers 0, 1), interior stores (0, 1; whole 16-byte chunks of a
@@ -592,8 +573,28 @@ bool encode_maps_of(const trtr_ctx* ctx, CUtensorMap* rows, CUtensorMap* stores,
     return ok && encode(fields, tma_type<float>(), 4, ctx->fld2, ctx->lt, G::NF, kWC, 1, G::NF);
 }
 
+// Rows of a segment: the number of segments a strip that ends soonest, by rounds of the SMs times a unit's
+// rows (once per context: the search took longer than a launch of a 512^2 grid).
+template <class G>
+int segment_rows(const trtr_ctx* ctx) {
+    const int ny = ctx->p.ny, strips = (ctx->p.nx + kX - 1) / kX;
+    long best = 0;
+    int best_rows = ny;
+    for (int s = 1; s <= (ny + G::R - 1) / G::R && s <= 4 * ctx->num_sms; ++s) {
+        const int rows = ((ny + s - 1) / s + G::R - 1) / G::R * G::R;
+        const long units = (long)strips * ((ny + rows - 1) / rows);
+        const long cost = ((units + ctx->num_sms - 1) / ctx->num_sms) * (rows + G::C + 4);
+        if (s == 1 || cost < best) {
+            best = cost;
+            best_rows = rows;
+        }
+    }
+    return best_rows;
+}
+
 template <typename S, int SRC>
 cudaError_t encode4_typed(trtr_ctx* ctx) {
+    ctx->sweep_rows = segment_rows<Sweep<S, SRC>>(ctx);
     return encode_maps_of<S, Sweep<S, SRC>>(ctx, &ctx->maps4[0], &ctx->maps4[2], &ctx->maps4[4]) ? cudaSuccess
                                                                                                  : cudaErrorInvalidValue;
 }
@@ -694,7 +695,7 @@ cudaError_t setup_batch_typed(trtr_ctx* const* ctx, int count, cudaStream_t stre
 template <typename S, int SRC, int RND>
 cudaError_t launch_batch_typed(const SweepBatch& b, BatchClock* clk, int* flag, int parity, cudaStream_t stream) {
     using G = Sweep<S, SRC>;
-    auto kernel = sweep_kernel<S, SRC, RND, G, ManyGrids>;
+    auto kernel = sweep_kernel<S, SRC, RND, G, true>;
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, G::Smem);
     if (e != cudaSuccess) return e;
     ManyGrids p;
@@ -704,7 +705,7 @@ cudaError_t launch_batch_typed(const SweepBatch& b, BatchClock* clk, int* flag, 
     p.clk = clk;
     p.flag = flag;
     p.parity = parity;
-    kernel<<<b.ctas, G::Threads, G::Smem, stream>>>(p);
+    kernel<<<b.ctas, G::Threads, G::Smem, stream>>>(CUtensorMap(), CUtensorMap(), CUtensorMap(), SweepArgs(), p);
     return cudaGetLastError();
 }
 
