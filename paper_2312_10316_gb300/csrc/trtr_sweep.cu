@@ -101,18 +101,14 @@ __host__ __device__ __forceinline__ int bulk_cols_of(int nx) {
     return nx / kChunk * kChunk;
 }
 
-// The ghost copies of one value of interior node (i, j): kGhostX columns, kGhostP rows.
+// The copies of one value of interior node (i, j) in the kGhostP ghost rows, corners included.
 template <typename T>
-__device__ __forceinline__ void store_sweep_ghosts(T* plane, const PlaneLayout& L, int i, int j, T v) {
-    T* row = plane + (size_t)(j + kGhostP) * L.pitch + L.gx;
+__device__ __forceinline__ void store_row_ghosts(T* plane, const PlaneLayout& L, int i, int j, T v) {
     const int xs = i < kGhostX ? L.nx : (i >= L.nx - kGhostX ? -L.nx : 0);
-    const int ys = j < kGhostP ? L.ny : (j >= L.ny - kGhostP ? -L.ny : 0);
+    const int ys = j < kGhostP ? L.ny : -L.ny;
+    T* row = plane + (ptrdiff_t)(j + kGhostP + ys) * L.pitch + L.gx;
+    row[i] = v;
     if (xs) row[i + xs] = v;
-    if (ys) {
-        row += (ptrdiff_t)ys * L.pitch;
-        row[i] = v;
-        if (xs) row[i + xs] = v;
-    }
 }
 
 // How a sweep rounds 2-byte values: to nearest (or FP32, not at all); stochastically; stochastically on
@@ -179,42 +175,44 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
             }
     } else {
         if (!buffer_free()) return;  // (a wait gave up: the warp leaves at its next wait)
+        const int nx = a.lp.nx, nc = bulk_cols_of<S>(nx);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
+            const int ih = i + 64 * h;
+            S2 v[kQ];
 #pragma unroll
-            for (int q = 0; q < kQ; ++q) *reinterpret_cast<S2*>(out_row + q * (G::R * kX) + 64 * h) = enc(q, h);
+            for (int q = 0; q < kQ; ++q) {
+                v[q] = enc(q, h);
+                *reinterpret_cast<S2*>(out_row + q * (G::R * kX) + 64 * h) = v[q];
+            }
+            // the edge columns from the registers
+            if (ih < kGhostX || ih + 1 >= min(nx - kGhostX, nc)) {
+                S* row = static_cast<S*>(a.dst) + (size_t)(j + kGhostP) * a.lp.pitch + a.lp.gx + ih;
+                const int to = ih < kGhostX ? nx : -nx;
+                const bool g0 = ih < kGhostX || (ih >= nx - kGhostX && ih < nx);
+                const bool g1 = ih < kGhostX || (ih + 1 >= nx - kGhostX && ih + 1 < nx);
+                const bool t0 = ih >= nc && ih < nx, t1 = ih + 1 >= nc && ih + 1 < nx;
+#pragma unroll
+                for (int q = 0; q < kQ; ++q) {
+                    S* r = row + q * a.lp.plane;
+                    const S v0 = reinterpret_cast<const S*>(&v[q])[0], v1 = reinterpret_cast<const S*>(&v[q])[1];
+                    if (g0) r[to] = v0;
+                    if (g1) r[to + 1] = v1;
+                    if (t0) r[0] = v0;
+                    if (t1) r[1] = v1;
+                }
+            }
             if (j < kGhostP || j >= a.lp.ny - kGhostP) {
 #pragma unroll 1
                 for (int q = 0; q < kQ; ++q) {
                     const S* v = out_row + q * (G::R * kX) + 64 * h;
                     S* plane = static_cast<S*>(a.dst) + q * a.lp.plane;
-                    if (i + 64 * h < a.lp.nx) store_sweep_ghosts(plane, a.lp, i + 64 * h, j, v[0]);
-                    if (i + 64 * h + 1 < a.lp.nx) store_sweep_ghosts(plane, a.lp, i + 64 * h + 1, j, v[1]);
+                    if (ih < nx) store_row_ghosts(plane, a.lp, ih, j, v[0]);
+                    if (ih + 1 < nx) store_row_ghosts(plane, a.lp, ih + 1, j, v[1]);
                 }
             }
         }
-    }
-}
-
-// The edge columns of the rows y .. y + R - 1 (below j1) of a strip from the output buffer, by one
-// warp: the ghost copies, and the last columns where a row is no whole number of 16-byte chunks (the
-// TMA store's map ends with the last whole one).
-template <typename S, class G>
-__device__ __forceinline__ void copy_edge_columns(const S* buf, const SweepArgs& a, int i0, int y, int j1, int lane) {
-    const int nx = a.lp.nx, nc = bulk_cols_of<S>(nx);
-    const int right = max(i0, min(nc, nx - kGhostX)), left = i0 == 0 ? kGhostX : 0;
-    const int n = left + max(0, min(i0 + kX, nx) - right), t = lane & 15;
-    const int i = t < left ? t : right + t - left;
-    if (t >= n) return;
-    for (int qr = lane >> 4; qr < kQ * G::R; qr += 2) {
-        const int q = qr / G::R, j = y + qr - q * G::R;
-        if (j >= j1) continue;
-        S* row = static_cast<S*>(a.dst) + q * a.lp.plane + (size_t)(j + kGhostP) * a.lp.pitch + a.lp.gx;
-        const S v = buf[qr * kX + i - i0];
-        if (i < kGhostX) row[i + nx] = v;
-        if (i >= nx - kGhostX) row[i - nx] = v;
-        if (i >= nc) row[i] = v;
     }
 }
 
@@ -322,7 +320,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
         for (int u = u_first; u < u_end && ok; u += u_step) {
             const Unit t = unit(u);
             Args a = args(t.inst);
-            const int nx = a.lp.nx, ny = a.lp.ny;
+            const int ny = a.lp.ny;
             const CUtensorMap *mp, *mf, *mo;
             if constexpr (BATCH) {
                 const SweepDesc* d = p.desc + t.inst;
@@ -349,7 +347,6 @@ __global__ void __launch_bounds__(G::Threads, 1)
                     if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, mf, &full[b], xf, y + a.gyf, 0);
                 }
             };
-            const bool edges = t.i0 == 0 || t.i0 + kX > min(nx - kGhostX, bulk_cols_of<S>(nx));
             int loaded = min(blocks, 2 + G::Ahead);
             if (lane == 0)
                 for (int m = 0; m < loaded; ++m) load(m);
@@ -364,8 +361,6 @@ __global__ void __launch_bounds__(G::Threads, 1)
                     if (y >= t.j0) tma_store_3d(mo, buf, t.i0, y, 0);
                     bulk_commit();
                 }
-                if (edges && y >= t.j0) copy_edge_columns<S, G>(reinterpret_cast<const S*>(buf), a, t.i0, y, t.j1, lane);
-                __syncwarp();
                 if (lane == 0) {  // the store before this one has left its buffer
                     asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     if (it > 0) mbar_arrive(&freed[(it - 1) % G::Outs]);
