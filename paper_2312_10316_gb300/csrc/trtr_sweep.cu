@@ -5,7 +5,7 @@
 // stationary source field.  The node update is the one-step kernel's, roundings included, so the results have the same bits.
 //
 // Strip: X = 120 output columns from i0; every level computes the 128 columns [i0 - 4, i0 + 124)
-// (two warps a row, a node pair a lane), of which level s is valid on all but s - 1 at each side.
+// (two node pairs a lane, or two warps a row), of which level s is valid on all but s - 1 at each side.
 // Rows arrive through TMA, one box of the nine populations (136 columns from i0 - 8) and one of
 // the five packed fields (128 columns from i0 - 4) a row, into a ring of kRing rows; y wraps by the
 // row index, x through a four-wide ghost frame of columns.  Populations live in place: node x at
@@ -57,7 +57,13 @@ struct Sweep {
     static constexpr int BarOff = OutOff + Outs * OutBytes;
     static constexpr int Depth = 8;                                   // barriers of a level (iterations in flight)
     static constexpr int Smem = BarOff + (Blocks + kT * Depth + Outs) * 8 + 128;
-    static constexpr int Warps = kT * R;                              // a warp per level and row
+    // Node pairs of a lane.  One (two warps a row) hides more latency, two (one warp) spend fewer instructions
+    // on addresses and waits.  4096^2 FP32, us a step, one / two: no source 89.4 / 95.5, source field 13 % apart
+    // (1101 x 1101), pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three rows:
+    // four would be 33 warps) / 96.
+    static constexpr int P = ES == 4 && SRC != TRTR_SRC_PULSE ? 1 : 2;
+    static constexpr int Row = 2 / P;                                 // warps of a row
+    static constexpr int Warps = kT * R * Row;                        // warps of a level: R rows
     static constexpr int Threads = (Warps + 1) * 32;                  // and one warp that moves the data
     static_assert(FldRow % 128 == 0, "TMA destinations on 128 bytes");
     // level 4 may finish iteration k when level 2 has finished k - 2, and level 1 may then be in k + 1 + Ahead
@@ -119,25 +125,26 @@ struct RoundKey {
     uint32_t a, b, sel;  // the two nodes' keys; the permutation that takes each one's half
 };
 
-// Level LV of row j for one lane: its node pairs at the columns c = 2 lane and c + 64 (h = 0, 1),
-// computed side by side so that each hides the other's latency.  pm / p0 / pp: the ring rows of the
+// Level LV of row j for one lane: its G::P node pairs, at the columns c = 64 part + 2 lane and c + 64 (h = 0, 1),
+// computed side by side.  pm / p0 / pp: the ring rows of the
 // slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
 // the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
 // rows within kGhostP of an edge).
 template <typename S, int LV, int SRC, int RND, class G, class Wait>
-__device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[2], const SweepArgs& a,
-                                          const RoundKey rk[2], S* out_row, int lane, int i, int j, Wait&& buffer_free) {
+__device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, const F2 src[G::P], const SweepArgs& a,
+                                          const RoundKey rk[G::P], S* out_row, int lane, int part, int i, int j,
+                                          Wait&& buffer_free) {
     constexpr bool kOfs = sizeof(S) == 2;
     using S2 = typename Pair<S>::type;
-    F2 out[2][kQ];
+    F2 out[G::P][kQ];
     auto slot = [&](int q, int h) -> S* {
         S* row = lattice_ey(q) == 1 ? pm : (lattice_ey(q) == -1 ? pp : p0);
         return row + q * kW - LV * lattice_ex(q) + 64 * h;
     };
     auto even = [](int q) { return LV % 2 == 0 || lattice_ex(q) == 0; };
-    F2 g[2][kQ], fld[2][G::NF];
+    F2 g[G::P][kQ], fld[G::P][G::NF];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < G::P; ++h) {
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
             const S* s = slot(q, h);
@@ -147,7 +154,7 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
         for (int m = 0; m < G::NF; ++m) fld[h][m] = F2(*reinterpret_cast<const float2*>(f + m * kWC + 64 * h));
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < G::P; ++h)
         collide_node<F2, kOfs>(g[h], fld[h][0], fld[h][1], fld[h][2], fld[h][3], fld[h][4],
                                SRC == TRTR_SRC_FIELD ? fld[h][G::NF - 1] : src[h], F2(a.magic),
                                F2(a.omega2_fixed), a.tau2_fixed, out[h], F2(a.phi_ref));
@@ -161,7 +168,7 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
     };
     if constexpr (LV < kT) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < G::P; ++h)
 #pragma unroll
             for (int q = 0; q < kQ; ++q) {
                 const S2 v = enc(q, h);
@@ -177,8 +184,8 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
         if (!buffer_free()) return;  // (a wait gave up: the warp leaves at its next wait)
         const int nx = a.lp.nx, nc = bulk_cols_of<S>(nx);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
+        for (int h = 0; h < G::P; ++h) {
+            if (part + h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
             const int ih = i + 64 * h;
             S2 v[kQ];
 #pragma unroll
@@ -246,7 +253,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
     if (tid == 0) {
         s_abort = 0;
         for (int b = 0; b < G::Blocks; ++b) mbar_init(&full[b], 1);
-        for (int b = 0; b < kT * G::Depth; ++b) mbar_init(&done[b], R);
+        for (int b = 0; b < kT * G::Depth; ++b) mbar_init(&done[b], R * G::Row);
         for (int b = 0; b < G::Outs; ++b) mbar_init(&freed[b], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -388,8 +395,8 @@ __global__ void __launch_bounds__(G::Threads, 1)
         return;
     }
 
-    // Level `level`, row r0 of every iteration.
-    const int level = w / R + 1, r0 = w % R;
+    // Level `level`, row r0 of every iteration, its columns from 64 part on.
+    const int level = w / (R * G::Row) + 1, r0 = w / G::Row % R, part = w % G::Row;
     uint32_t rkey = 0u;
     if constexpr (BATCH)
         rkey = RND != kRoundNearest ? sr_step_key((long)step + level - 1) : 0u;
@@ -401,13 +408,13 @@ __global__ void __launch_bounds__(G::Threads, 1)
         Args a = args(t.inst);
         const int nx = a.lp.nx, ny = a.lp.ny;
         // per strip: the pairs' columns, their images for the rounding keys, their pulse factors
-        const int i = t.i0 - kT + 2 * lane;
-        F2 p1p[2], p2p[2], p1n[2], p2n[2];
-        int wa[2], wb[2];
-        uint32_t sel[2];
+        const int i = t.i0 - kT + 2 * lane + 64 * part;
+        F2 p1p[G::P], p2p[G::P], p1n[G::P], p2n[G::P];
+        int wa[G::P], wb[G::P];
+        uint32_t sel[G::P];
         const float* lev = a.pulse + (size_t)(table_level + level - 1) * a.pt.level;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < G::P; ++h) {
             if (SRC == TRTR_SRC_PULSE) {
                 p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + i + 64 * h)));
                 p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.p2 + i + 64 * h)));
@@ -428,17 +435,29 @@ __global__ void __launch_bounds__(G::Threads, 1)
         ring = ring < 0 ? ring + G::Ring : (ring >= G::Ring ? ring - G::Ring : ring);
         unsigned block = phase % G::Blocks, parity = (phase / G::Blocks) & 1;
         if (level == 1 && !wait(&full[block], parity)) return;
+        // The row's pulse factors.  FP32 loads them an iteration ahead (4096^2: 102.5 -> 98.9 us a step; the 2-byte
+        // storages, with more arithmetic in flight, lose 2 %).
+        constexpr bool kAheadFactors = G::ES == 4;
+        float2 qp = make_float2(0.f, 0.f), qn = qp;
+        auto load_factors = [&](int y) {
+            y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+            qp = __ldg(reinterpret_cast<const float2*>(ty + 2 * y));
+            qn = __ldg(reinterpret_cast<const float2*>(ty + a.pt.level + 2 * y));
+        };
+        if (SRC == TRTR_SRC_PULSE && kAheadFactors) load_factors(j);
         for (int k = 0; k < t.iters; ++k, j += R, ++it) {
-            F2 src[2] = {F2(0.f), F2(0.f)};
-            int yw = 0;
-            if (SRC == TRTR_SRC_PULSE || RND != kRoundNearest) yw = j < 0 ? j + ny : (j >= ny ? j - ny : j);
-            if (SRC == TRTR_SRC_PULSE) {  // as pulse_source_dt
-                const float2 qp = __ldg(reinterpret_cast<const float2*>(ty + 2 * yw));
-                const float2 qn = __ldg(reinterpret_cast<const float2*>(ty + a.pt.level + 2 * yw));
+            F2 src[G::P];
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
+            for (int h = 0; h < G::P; ++h) src[h] = F2(0.f);
+            int yw = 0;
+            if (RND != kRoundNearest) yw = j < 0 ? j + ny : (j >= ny ? j - ny : j);
+            if (SRC == TRTR_SRC_PULSE) {  // as pulse_source_dt
+                if (!kAheadFactors) load_factors(j);
+#pragma unroll
+                for (int h = 0; h < G::P; ++h)
                     src[h] = vfma(F2(1.5f), vfma(p1n[h], F2(qn.x), p2n[h] * F2(qn.y)),
                                   F2(-0.5f) * vfma(p1p[h], F2(qp.x), p2p[h] * F2(qp.y)));
+                if (kAheadFactors) load_factors(j + R);
             }
             // level 1 waits for its rows, the others for the level before to have finished the iteration
             // before this one; the last level also, before it writes, for its output buffer
@@ -458,27 +477,27 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 const int below = ring >= level ? ring - level : ring - level + G::Ring;
                 const int above = ring + level < G::Ring ? ring + level : ring + level - G::Ring;
                 constexpr int kPitch = G::PopPitch / G::ES;
-                S* base = reinterpret_cast<S*>(smem) + 2 * lane + kT;
+                S* base = reinterpret_cast<S*>(smem) + 2 * lane + 64 * part + kT;
                 S* pm = base + below * kPitch;
                 S* p0 = base + ring * kPitch;
                 S* pp = base + above * kPitch;
-                const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (G::NF * kWC) + 2 * lane;
-                RoundKey rk[2] = {};
+                const float* f = reinterpret_cast<const float*>(smem + G::FldOff) + ring * (G::NF * kWC) + 2 * lane + 64 * part;
+                RoundKey rk[G::P] = {};
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int h = 0; h < G::P; ++h) {
                     if (RND != kRoundNearest) rk[h].a = sr_pair_key(wa[h], yw, nx, rkey);
                     if (RND == kRoundNodes) {
                         rk[h].b = sr_pair_key(wb[h], yw, nx, rkey);
                         rk[h].sel = sel[h];
                     }
                 }
-                S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane - kT;
+                S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane + 64 * part - kT;
                 auto buffer_free = [&]() { return it < (unsigned)G::Outs || wait(&freed[o], (it / G::Outs - 1) & 1); };
                 switch (level) {
-                    case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
-                    case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
-                    case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
-                    default: sweep_row<S, 4, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, i, j, buffer_free); break;
+                    case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
+                    case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
+                    case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
+                    default: sweep_row<S, 4, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
                 }
             }
             __syncwarp();
