@@ -2,8 +2,8 @@
 """Throughput of the fused TRT-R step (GLUPS) on the rotating-pulse workloads.
 
 One bench step is one TRT-R time step (pull-stream, phi, TRT-R relaxation, auxiliary term,
-source, store) over every node of the workload's grid; where the two-step kernel applies, one
-launch advances two of them.  Prints ONE JSON line on rank 0: the workload's throughput with
+source, store) over every node of the workload's grid; where the sweep or the two-step kernel
+applies, one launch advances four or two of them.  Prints ONE JSON line on rank 0: the workload's throughput with
 its roofline, the relative L2 error of a full-length solve against the GPU FP64 path, an
 end-to-end run from host buffers and, for the FP32 pulse workloads, the same grid with FP16
 storage (`fp16_storage`).
@@ -67,7 +67,8 @@ TABLE2_PRINTED = os.path.join(ROOT, "tests", "golden", "table2_convergence.txt")
 _CORE = ["paper_2312_10316_gb300/csrc/trtr_step_core.cuh", "paper_2312_10316_gb300/csrc/trtr_internal.cuh"]
 KERNEL_SOURCES = {"step_kernel": ["paper_2312_10316_gb300/csrc/trtr_step.cu"] + _CORE,
                   "step2_kernel": ["paper_2312_10316_gb300/csrc/trtr_step2.cu",
-                                   "paper_2312_10316_gb300/csrc/trtr_step2_core.cuh"] + _CORE}
+                                   "paper_2312_10316_gb300/csrc/trtr_step2_core.cuh"] + _CORE,
+                  "sweep_kernel": ["paper_2312_10316_gb300/csrc/trtr_sweep.cu"] + _CORE}
 
 
 def parse_args():
@@ -88,7 +89,8 @@ def parse_args():
                     help="steps of the FP64 GPU comparison run that states the L2 error, independent of "
                          "--steps (-1: the workload's configured length, 10000 steps; 0: skip)")
     ap.add_argument("--steps-per-launch", default="auto", choices=["auto", "1", "2"],
-                    help="auto: two steps per launch where the two-step kernel applies; 1: one step per launch "
+                    help="auto: four or two steps per launch where the sweep or the two-step kernel applies; "
+                         "1: one step per launch "
                          "(the one-step kernel); 2: as auto")
     ap.add_argument("--rounding", default="auto", choices=["auto", "nearest", "stochastic"],
                     help="rounding of the 2-byte storages (auto: the library's default, stochastic; FP32 ignores it)")
@@ -104,7 +106,7 @@ def algorithmic_bytes_per_node(pop_bytes: int, field_bytes: int = 4) -> int:
 
 
 def two_step_bytes_per_node(pop_bytes: int = 4, field_bytes: int = 4) -> int:
-    """One launch of the two-step kernel (two time steps): 9 populations read + 9 written, plus
+    """One launch of the two-step kernel or of the sweep (two or four time steps): 9 populations read + 9 written, plus
     the packed u_x, u_y, a_x, a_y, D read once per node."""
     return 2 * 9 * pop_bytes + 5 * field_bytes
 
@@ -288,6 +290,15 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
     if src_override == T.TRTR_SRC_FIELD:
         solver.set_source(W.source(pulse, 0.0))  # the manufactured source as a stationary field
     solver.step(args.warmup)
+    # one event interval per launch: four steps where trtr_step takes four at once (the sweep), two
+    # where the two-step kernel applies
+    if args.steps_per_launch == "1":
+        solver.set_steps_per_launch(1)
+    spl = solver.steps_per_launch
+    before = solver.launches
+    solver.step(4)
+    if solver.launches - before == 1:
+        spl = 4
     solver.sync()
     barrier(world)
     torch.cuda.synchronize()
@@ -296,10 +307,6 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
     clocks = ClockSampler(("GPU-" + uuid) if uuid and not uuid.startswith("GPU-") else uuid)
     clocks.start()
     time.sleep(0.4)  # let the sampler take a reading at the start of the region
-    # one event interval per launch: two steps per launch where the two-step kernel applies
-    if args.steps_per_launch == "1":
-        solver.set_steps_per_launch(1)
-    spl = solver.steps_per_launch
     n_launch, tail = divmod(args.steps, spl)
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(n_launch + 1 + (1 if tail else 0))]
     launches0 = solver.launches
@@ -323,13 +330,15 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
     value = n_nodes * args.steps * world / (total_ms * 1e-3) / 1e9
     avg_launch_ms = sum(per_launch) / len(per_launch)
 
-    if spl == 2:
+    if spl == 4:
+        bpn, kernel = two_step_bytes_per_node(pop_bytes), "sweep_kernel"  # the same planes, once per four steps
+    elif spl == 2:
         bpn, kernel = two_step_bytes_per_node(pop_bytes), "step2_kernel"
     else:
         bpn, kernel = algorithmic_bytes_per_node(pop_bytes), "step_kernel"
     # S^n and S^{n-1} planes in the compute type
     extra = 2 * (8 if prec == T.TRTR_F64 else 4) if src_override == T.TRTR_SRC_FIELD else 0
-    bpn += extra
+    bpn += extra // 2 if spl == 4 else extra  # (the sweep reads the source term, packed from both)
     peak, peak_kind = measured_hbm_peak()
     achieved = bpn * n_nodes / (avg_launch_ms * 1e-3) / 1e9
     traffic = ncu_traffic(workload, kernel) if src_override is None else None
@@ -627,10 +636,10 @@ def run_batch(args):
 
             dist.destroy_process_group()
         return None
-    # pairs of steps through the two-step kernel where it applies (92 B per node and launch in
-    # FP32, 56 B for the 2-byte storages)
+    # two steps per launch, or four where the batch's sweep is the faster (the batch decides; counted as
+    # four, so bytes and launches are lower bounds): 92 B per node and launch in FP32, 56 B for 2-byte storages
     if spl == 2:
-        bpn, kernel = two_step_bytes_per_node(pop_bytes), "batch2_kernel"
+        bpn, kernel, spl = two_step_bytes_per_node(pop_bytes), "batch sweep_kernel or batch2_kernel", 4
     else:
         bpn, kernel = algorithmic_bytes_per_node(pop_bytes), "batch_kernel"
     peak, peak_kind = measured_hbm_peak()

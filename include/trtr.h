@@ -175,16 +175,18 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
  * storage on a grid of even nx, periodic boundaries and src_mode NONE or PULSE, pairs of steps
  * run as one launch of the two-step kernel (the same arithmetic and roundings, the same results
  * bit for bit; populations read and written once per two steps; see
- * trtr_set_steps_per_launch); an odd last step, or a pair whose middle step is a check_every
+ * trtr_set_steps_per_launch).  A call of 12 steps or more (4 on 2^18 nodes or more) takes four
+ * steps a launch, with odd nx and a source field that stays the same from step to step too, again
+ * with the same bits.  An odd last step, or a pair whose middle step is a check_every
  * point, runs one step per launch.  Short launches use programmatic dependent launch: each
  * waits for the work before it on the stream before reading its results. */
 trtr_status trtr_step(trtr_ctx* ctx, long n);
 
-/* k = 2 (the default): trtr_step uses the two-step kernel where it applies; k = 1: one step per
- * launch always.  TRTR_EINVAL for other k. */
+/* k = 2 (the default): trtr_step takes two steps a launch, or four, where it can; k = 1: one step
+ * per launch always.  TRTR_EINVAL for other k. */
 trtr_status trtr_set_steps_per_launch(trtr_ctx* ctx, int k);
 
-/* The steps one launch of trtr_step advances where it can on this context: 2 when the two-step
+/* The steps one launch of a short trtr_step call advances where it can on this context: 2 when the two-step
  * kernel applies (FP32, or FP16 / BF16 with even nx; periodic; src_mode NONE or PULSE; not
  * disabled), else 1. */
 trtr_status trtr_get_steps_per_launch(const trtr_ctx* ctx, int* k);
@@ -252,8 +254,8 @@ trtr_status trtr_launch_count(const trtr_ctx* ctx, long* launches);
 
 /* Advances n >= 1 steps from the current state, keeping a copy of the state every
  * `interval` steps (0: ceil(sqrt(n))), and remembers the run for trtr_adjoint.  Allocates
- * about (n/interval + interval) population arrays of device memory (freed by the next
- * record or by trtr_destroy). */
+ * about (n/interval + interval) population arrays of device memory, kept for the next record of
+ * the same steps and interval (freed by another record or by trtr_destroy). */
 trtr_status trtr_forward_record(trtr_ctx* ctx, long steps, int interval);
 
 /* Backward sweep of the recorded run: dJ_dphi = dJ/dphi(x, t_end) [ny][nx] (host or device);
@@ -266,8 +268,8 @@ trtr_status trtr_adjoint(trtr_ctx* ctx, const double* dJ_dphi, int on_device, do
  * Many independent problems of uneven sizes advanced together, each by the same step of
  * Eq. (14).  The paper solves one problem at a time; this is a throughput mode of its step.
  * Persistent kernel launches walk a work-list of (instance, tile) pairs spanning every
- * instance: one time step per launch, or two (the two-step kernel) where every instance has
- * FP32 storage, or 2-byte storage with even nx;
+ * instance: one time step per launch, two (the two-step kernel) where every instance has
+ * FP32 storage, or 2-byte storage with even nx, or four where that ends sooner;
  * trtr_batch_step replays two-launch CUDA graphs of them.
  * Each instance is an ordinary context (trtr_batch_instance gives it out for queries). */
 typedef struct {
@@ -307,14 +309,14 @@ trtr_status trtr_batch_set_config(trtr_batch* b, int config);
 
 /* Advances every instance by n >= 0 steps (asynchronous on the batch's stream).  Where the
  * two-step kernel applies (every instance FP32, or 2-byte with even nx), pairs of steps run as
- * launches of it over a work-list of its tiles (the same results bit for bit; see
- * trtr_batch_set_steps_per_launch), the other steps
- * with the configured one-step kernel.  Instances must not be stepped through their own
+ * launches of it over a work-list of its tiles, or four steps as one launch over the instances'
+ * strips where that ends sooner (the same results bit for bit; see
+ * trtr_batch_set_steps_per_launch), the other steps with the configured one-step kernel.  Instances must not be stepped through their own
  * contexts in between (TRTR_ESTATE). */
 trtr_status trtr_batch_step(trtr_batch* b, long n);
 
-/* k = 2 (the default): trtr_batch_step runs pairs of steps with the two-step kernel where it
- * applies (FP32 instances, or 2-byte instances of even nx); k = 1: every step with the
+/* k = 2 (the default): trtr_batch_step takes two steps a launch, or four, where it can (two: FP32
+ * instances, or 2-byte instances of even nx); k = 1: every step with the
  * configured one-step kernel.
  * TRTR_EINVAL for other k. */
 trtr_status trtr_batch_set_steps_per_launch(trtr_batch* b, int k);

@@ -3,9 +3,9 @@
 //
 // Forward (trtr_forward_record): n steps of the ordinary step kernel, keeping a copy of
 // the state every k steps (k = ceil(sqrt(n)) by default).  Backward (trtr_adjoint): for
-// each segment, last to first, the state at the segment start is copied into a pool and
-// the segment's states are recomputed by the step kernel; then one backward kernel per
-// step runs from the segment's end to its start.  Total work: two forward sweeps and one
+// each segment, last to first, the segment's states are recomputed from its checkpoint into
+// a pool by the step kernels; then one backward kernel per step runs from the segment's end
+// to its start.  Total work: two forward sweeps and one
 // backward sweep; memory: about 2 sqrt(n) states.
 //
 // Notation (lattice units, S = 0).  The stored array holds P_i(x) = post_i(g(x)) with

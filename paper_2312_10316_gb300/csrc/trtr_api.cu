@@ -1,6 +1,6 @@
 // trtr_api.cu -- the C ABI declared in include/trtr.h: validation, device memory of a
 // context, ping-pong bookkeeping and the host side of every call.  All compute runs in the
-// kernels of trtr_step.cu and trtr_aux.cu.
+// kernels of the other files (launch_steps chooses between them).
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>

@@ -2,8 +2,8 @@
 //
 // Every instance is an ordinary context (its own ghosted planes, fields and reductions).
 // A persistent kernel launch walks a work-list of (instance, tile) pairs spanning all
-// instances, one time step per launch (batch_kernel) or, for FP32 instances, two
-// (batch2_kernel, the two-step kernel's tile code).  Per tile the producer thread issues the
+// instances, one time step per launch (batch_kernel), two (batch2_kernel, the two-step
+// kernel's tile code) or four (the sweep of trtr_sweep.cu over every instance's strips).  Per tile the producer thread issues the
 // instance's TMA loads, then copies the instance's step arguments from a device descriptor
 // into a shared-memory slot of the stage and gives the stage's mbarrier its second arrival,
 // so the consumers read the arguments after their acquire-wait.  The arithmetic per node is

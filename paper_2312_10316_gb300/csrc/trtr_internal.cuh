@@ -5,7 +5,8 @@
 // node (i, j) sits at row j + gy and column gx + i of a [rows][pitch] plane, where gx is one
 // 128-byte line of columns, so interior rows start on a 128-byte boundary, and the gy columns
 // before / after the interior and the gy rows above / below it hold ghost copies (gy = 2 for
-// the populations, 1 for the fields of the one-step kernel):
+// the populations, 1 for the fields of the one-step kernel, 4 for the packed fields; the sweep keeps
+// four ghost columns of the populations):
 //
 //   populations  2 x [9][rows][pitch] in the storage type: the post-collision values P_i(x)
 //                of the previous step; the pre-collision population is the pull
@@ -17,7 +18,11 @@
 //                extrapolation 2u(edge) - u(edge -+ 1) (TRTR_GRAD_ONESIDED_EDGE), for which the
 //                central difference at the edge node equals the one-sided difference.
 //   source       [2][rows][pitch] dt*S in the compute type (TRTR_SRC_FIELD only)
-//   pulse tab    [2][nx] sin(pi x_i), cos(pi x_i) and [2][ny] sin(pi y_j), cos(pi y_j)
+//   packed       [5 or 6][rows][pitch] FP32: u, a = (u . grad) u, Dh and, with a source field, the
+//                source term, for the kernels that take several steps; FP64: [4][rows][pitch]
+//                a, k1, k2 (pack64)
+//   pulse tab    [2][nx] sin(pi x_i), cos(pi x_i) and [2][ny] sin(pi y_j), cos(pi y_j); and the
+//                separable factors of the pulse source at kPulseLevels time levels (PulseTab)
 //   edge values  [2 nx + 2 (ny - 2)] FP64 Dirichlet values of the edge nodes
 //                (TRTR_BC_DIRICHLET_NEE), in the order of edge_node()
 //   scratch      FP64 partial sums of the reductions, one pair per reduction block

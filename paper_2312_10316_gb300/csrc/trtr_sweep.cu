@@ -2,22 +2,32 @@
 // strip of columns from bottom to top and carries four time levels behind one another through
 // shared memory (wavefront temporal blocking), for FP32 storage or FP16 / BF16 offset storage
 // (FP32 arithmetic), periodic boundaries and no source, the manufactured pulse source or a
-// stationary source field.  The node update is the one-step kernel's, roundings included, so the results have the same bits.
+// stationary source field.  The node update is the one-step kernel's, roundings included, so the
+// results have the same bits.
 //
 // Strip: X = 120 output columns from i0; every level computes the 128 columns [i0 - 4, i0 + 124)
 // (two node pairs a lane, or two warps a row), of which level s is valid on all but s - 1 at each side.
 // Rows arrive through TMA, one box of the nine populations (136 columns from i0 - 8) and one of
-// the five packed fields (128 columns from i0 - 4) a row, into a ring of kRing rows; y wraps by the
-// row index, x through a four-wide ghost frame of columns.  Populations live in place: node x at
+// the five or six packed fields (128 columns from i0 - 4) a row, into a ring of Ring rows; y wraps by
+// the row index, x through a four-wide ghost frame of columns.  Populations live in place: node x at
 // level s reads and writes the slots x - s e_q of the ring, which no other node touches at that
 // level, so one ring serves every level (level s = 1 .. 4 of row j uses the slot rows j - s, j,
-// j + s).  In iteration k level s works on R rows, kLag rows behind level s - 1, which has then
-// finished the row above them; one CTA barrier an iteration orders everything.  The last level
-// writes its rows to a shared-memory buffer that one TMA store an iteration moves out, clipped to
-// the grid; nodes near an edge also store their ghost copies.
+// j + s).  In iteration k level s works on R rows, Lag rows behind level s - 1, which has then
+// finished the row above them; an mbarrier per level and iteration is all that orders the warps (one
+// CTA barrier an iteration: 144 GLUPS against 155).  The last level writes its rows to a shared-memory
+// buffer that one TMA store an iteration moves out, clipped to the grid's whole 16-byte chunks; its
+// lanes store the edge columns' ghost copies and the last columns themselves.
 //
 // Work units are (strip, segment of rows); a segment costs C rows of ramp (its first output row
 // needs C / R iterations), so the host picks the number of segments that ends soonest.
+//
+// What bounds it: latency and issue, not memory.  At 2048^2 FP32 without a source 0.58 instructions are
+// issued a cycle and scheduler, the shared-memory data path is 59 % busy, and DRAM carries 0.38 GB of the
+// 0.39 GB a launch has to move; the warps wait for the level before theirs (a third of their time) and on
+// fixed latencies.  Four steps move the populations once (92 B a node instead of 4 x 84), and 128 columns
+// keep the work done twice at 128 / 120 plus the ramp.  Measured (GB300), us a step, the two-step kernel
+// before -> now: FP32 pulse 4096^2 147 -> 99, no source 128 -> 89, FP16 pulse 139 -> 108; 200 steps of the
+// FP32 pulse at 1024^2 with their set-up 3.43 -> 1.94 ms.
 #include <algorithm>
 #include <queue>
 #include <utility>
@@ -53,14 +63,14 @@ struct Sweep {
     static constexpr int FldOff = Ring * ((PopRow + 127) / 128 * 128);
     static constexpr int PopPitch = (PopRow + 127) / 128 * 128;       // TMA destinations on 128 bytes
     static constexpr int OutOff = FldOff + Ring * FldRow;
-    static constexpr int Outs = 3;                                    // output buffers (with 2 the last level waits for them: -20 %)
+    static constexpr int Outs = 3;                                    // output buffers (two measured the same)
     static constexpr int BarOff = OutOff + Outs * OutBytes;
     static constexpr int Depth = 8;                                   // barriers of a level (iterations in flight)
     static constexpr int Smem = BarOff + (Blocks + kT * Depth + Outs) * 8 + 128;
     // Node pairs of a lane.  One (two warps a row) hides more latency, two (one warp) spend fewer instructions
     // on addresses and waits.  4096^2 FP32, us a step, one / two: no source 89.4 / 95.5, source field 13 % apart
-    // (1101 x 1101), pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three rows:
-    // four would be 33 warps) / 96.
+    // (1101 x 1101), pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three
+    // rows: four would be 33 warps) / 96.
     static constexpr int P = ES == 4 && SRC != TRTR_SRC_PULSE ? 1 : 2;
     static constexpr int Row = 2 / P;                                 // warps of a row
     static constexpr int Warps = kT * R * Row;                        // warps of a level: R rows
@@ -125,8 +135,8 @@ struct RoundKey {
     uint32_t a, b, sel;  // the two nodes' keys; the permutation that takes each one's half
 };
 
-// Level LV of row j for one lane: its G::P node pairs, at the columns c = 64 part + 2 lane and c + 64 (h = 0, 1),
-// computed side by side.  pm / p0 / pp: the ring rows of the
+// Level LV of row j for one lane: its G::P node pairs, at the columns c = 64 part + 2 lane and, with two,
+// c + 64 (h = 0, 1), computed side by side.  pm / p0 / pp: the ring rows of the
 // slots j - LV, j, j + LV, f: the row's fields, src: the source terms, rk: the rounding keys, at
 // the first pair.  LV < kT writes the slots back, LV = kT the output buffer (and the ghost copies of
 // rows within kGhostP of an edge).
@@ -193,7 +203,8 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
                 v[q] = enc(q, h);
                 *reinterpret_cast<S2*>(out_row + q * (G::R * kX) + 64 * h) = v[q];
             }
-            // the edge columns from the registers
+            // the edge columns from the registers (copied from the buffer by the data mover, the edge strips took
+            // 2950 cycles an iteration, the others 2200: a 1024^2 step 10.1 us, now 8.6)
             if (ih < kGhostX || ih + 1 >= min(nx - kGhostX, nc)) {
                 S* row = static_cast<S*>(a.dst) + (size_t)(j + kGhostP) * a.lp.pitch + a.lp.gx + ih;
                 const int to = ih < kGhostX ? nx : -nx;
