@@ -72,6 +72,9 @@ struct Sweep {
     // (1101 x 1101), pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three
     // rows: four would be 33 warps) / 96.
     static constexpr int P = ES == 4 && SRC != TRTR_SRC_PULSE ? 1 : 2;
+    // The fields and the pulse tables are older than the launch before and are read while it still runs: FP32, us a
+    // step, 512^2 3.09 -> 2.99, 1024^2 7.83 -> 7.63; FP16 pulse 4096^2 108.2 -> 109.1, so 2-byte storages wait first.
+    static constexpr bool Early = ES == 4;
     static constexpr int Row = 2 / P;                                 // warps of a row
     static constexpr int Warps = kT * R * Row;                        // warps of a level: R rows
     static constexpr int Threads = (Warps + 1) * 32;                  // and one warp that moves the data
@@ -240,6 +243,10 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void*
                  : "memory");
 }
 
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -270,7 +277,10 @@ __global__ void __launch_bounds__(G::Threads, 1)
     }
     __syncthreads();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The launch before may still run from here on (a batch waits at once: that launch moves its clock).
+    constexpr bool kEarly = !BATCH && G::Early;
+    auto wait_for_grid = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
+    if (!kEarly) wait_for_grid();
 
     // A wait that gives up sets s_abort; every warp then leaves at its next wait.
     volatile int* abort_flag = &s_abort;
@@ -334,11 +344,46 @@ __global__ void __launch_bounds__(G::Threads, 1)
         // The mover: lane 0 loads the blocks (block m of a unit: the rows a0 + 1 - R + m R ..; iteration
         // k needs the blocks up to k + 1) and stores the rows the last level has finished.
         unsigned phase = 0, it0 = 0, pending = 0;
-        bool ok = true;
+        bool ok = true, fields_loaded = false;
+        // block m of unit t: its populations, its fields
+        auto load_populations = [&](const Unit& t, const SweepArgs& a, const CUtensorMap* mp, int m) {
+            const unsigned b = (phase + m) % G::Blocks;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                int y = t.a0 + 1 - R + m * R + r;
+                y = y < 0 ? y + a.lp.ny : (y >= a.lp.ny ? y - a.lp.ny : y);
+                unsigned char* pd = smem + (b * R + r) * G::PopPitch;
+                const int xp = t.i0 - 2 * kT + a.lp.gx;
+                if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, mp, &full[b], xp, y + kGhostP, 0);
+            }
+        };
+        auto load_fields = [&](const Unit& t, const SweepArgs& a, const CUtensorMap* mf, int m) {
+            const unsigned b = (phase + m) % G::Blocks;
+            mbar_expect_tx(&full[b], R * (G::PopRow + G::FldRow));
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                int y = t.a0 + 1 - R + m * R + r;
+                y = y < 0 ? y + a.lp.ny : (y >= a.lp.ny ? y - a.lp.ny : y);
+                unsigned char* fd = smem + G::FldOff + (b * R + r) * G::FldRow;
+                const int xf = t.i0 - kT + a.gxf;
+                if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, mf, &full[b], xf, y + a.gyf, 0);
+            }
+        };
+        if constexpr (kEarly) {
+            if (lane == 0) {
+                prefetch_tensormap(&mp_);
+                prefetch_tensormap(&mo_);
+                if (u_first < u_end) {
+                    const Unit t = unit(u_first);
+                    for (int m = 0; m < min(t.iters + 1, 2 + G::Ahead); ++m) load_fields(t, a_, &mf_, m);
+                }
+            }
+            fields_loaded = true;
+            wait_for_grid();
+        }
         for (int u = u_first; u < u_end && ok; u += u_step) {
             const Unit t = unit(u);
             Args a = args(t.inst);
-            const int ny = a.lp.ny;
             const CUtensorMap *mp, *mf, *mo;
             if constexpr (BATCH) {
                 const SweepDesc* d = p.desc + t.inst;
@@ -352,22 +397,16 @@ __global__ void __launch_bounds__(G::Threads, 1)
             }
             const int blocks = t.iters + 1;
             auto load = [&](int m) {
-                const unsigned b = (phase + m) % G::Blocks;
-                mbar_expect_tx(&full[b], R * (G::PopRow + G::FldRow));
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    int y = t.a0 + 1 - R + m * R + r;
-                    y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
-                    unsigned char* pd = smem + (b * R + r) * G::PopPitch;
-                    unsigned char* fd = smem + G::FldOff + (b * R + r) * G::FldRow;
-                    const int xp = t.i0 - 2 * kT + a.lp.gx, xf = t.i0 - kT + a.gxf;
-                    if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, mp, &full[b], xp, y + kGhostP, 0);
-                    if (tma_ok(fd, xf, y, 4)) tma_load_3d(fd, mf, &full[b], xf, y + a.gyf, 0);
-                }
+                load_fields(t, a, mf, m);
+                load_populations(t, a, mp, m);
             };
             int loaded = min(blocks, 2 + G::Ahead);
             if (lane == 0)
-                for (int m = 0; m < loaded; ++m) load(m);
+                for (int m = 0; m < loaded; ++m) {
+                    if (!fields_loaded) load_fields(t, a, mf, m);
+                    load_populations(t, a, mp, m);
+                }
+            fields_loaded = false;
             for (int k = 0; k < t.iters; ++k) {
                 const unsigned it = it0 + k, o = it % G::Outs;
                 if (!(ok = wait(&done[(kT - 1) * G::Depth + it % G::Depth], (it / G::Depth) & 1))) break;
@@ -439,6 +478,8 @@ __global__ void __launch_bounds__(G::Threads, 1)
             sel[h] = (xa & 1 ? 0x32u : 0x10u) | (xb & 1 ? 0x7600u : 0x5400u);
         }
         const float* ty = lev + a.pt.y;
+
+        if (kEarly && u == u_first) wait_for_grid();
 
         // the warp's row of the iteration and its ring row (block m = 0 starts at row a0 + 1 - R)
         int j = t.a0 - (level - 1) * G::Lag + r0;
@@ -578,6 +619,10 @@ cudaError_t launch_sweep_typed(trtr_ctx* ctx) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    if (G::Early) {  // not over the kernel that wrote what is read early
+        attr[0].val.programmaticStreamSerializationAllowed = !ctx->tables_new;
+        ctx->tables_new = false;
+    }
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, ctx->maps4[ctx->cur], ctx->maps4[4], ctx->maps4[2 + (ctx->cur ^ 1)], a,
