@@ -1,7 +1,7 @@
 // trtr_small.cu -- four time steps of the evolution equation (14) per launch for small grids (FP32
 // storage or FP16 / BF16 offset storage, periodic; no source, the pulse source or a stationary source
-// field).  On a grid of a few hundred nodes a side a launch is latency: the sweep's ramp
-// (trtr_sweep.cu) makes it 9 us for four steps whatever the size, the two-step kernel takes 5 - 6 us
+// field).  On a grid of up to 300 nodes a side a launch is latency: the sweep's ramp
+// (trtr_sweep.cu) makes it 6 - 10 us for four steps whatever the size, the two-step kernel takes 5 - 6 us
 // for two.  Here a CTA takes one small tile with its four-node halo (32 x 8: 40 x 16 nodes), one node pair a
 // thread, and every thread keeps its pair through the four steps: the fields, the source terms and the
 // rounding keys stay in registers and are loaded while the launch before still runs, and only the
@@ -166,13 +166,15 @@ template <class G>
 long small_tiles(const trtr_ctx* ctx) {
     return (long)((ctx->p.nx + G::BX - 1) / G::BX) * ((ctx->p.ny + G::BY - 1) / G::BY);
 }
-// 32 x 4 tiles up to two CTAs an SM, then 32 x 8 up to four, then the sweep.  Measured (GB300, FP32
-// without a source, us a step; 32 x 4 / 32 x 8 / sweep): 64^2 1.14 / 1.28 / 2.25, 192^2 1.47 / 1.73 / 2.30,
-// 256^2 2.17 / 1.78 / 2.64, 384^2 - / 2.89 / 3.32, 448^2 - / 3.57 / 3.29 (16 x 8 and 16 x 4 tiles: 1.31 and
-// 1.39 at 64^2, 1.63 and 1.65 at 192^2).  FP16 and the pulse source have the same crossings.
+// 32 x 4 tiles up to two CTAs an SM, then 32 x 8 up to two (FP32 without the pulse) or three, then the sweep.
+// Measured (GB300, us a step; 32 x 4 / 32 x 8 / sweep).  FP32 without a source: 64^2 1.14 / 1.28 / -, 192^2 1.47 /
+// 1.73 / 1.56, 256^2 2.17 / 1.78 / 1.84, 272^2 - / 2.15 / 1.83, 384^2 - / 2.90 / 2.47; a source field: 288^2 - / 2.24 /
+// 1.94; the pulse, whose sweep has one warp a row: 256^2 - / 1.97 / 2.42, 320^2 - / 2.60 / 2.73, 336^2 - / 2.95 / 2.72;
+// FP16: 256^2 - / 1.77 / 2.52, 320^2 - / 2.39 / 2.55, 352^2 - / 2.75 / 2.56.  (16 x 8 and 16 x 4 tiles: 1.31 and 1.39
+// at 64^2, 1.63 and 1.65 at 192^2.)
 using SmallA = SmallTile<32, 4>;
 using SmallB = SmallTile<32, 8>;
-constexpr long kSmallACtas = 2, kSmallBCtas = 4;
+constexpr long kSmallACtas = 2, kSmallBCtas = 3, kSmallBCtasF32 = 2;
 
 template <typename S, int SRC, bool SR, class G>
 cudaError_t launch_small_typed(trtr_ctx* ctx) {
@@ -224,7 +226,8 @@ cudaError_t launch_small_src(trtr_ctx* ctx) {
 
 // Instead of the sweep (sizes: SmallA).
 bool small_applies(const trtr_ctx* ctx) {
-    return sweep_applies(ctx) && small_tiles<SmallB>(ctx) <= kSmallBCtas * ctx->num_sms;
+    const long ctas = ctx->p.precision == TRTR_F32 && ctx->p.src_mode != TRTR_SRC_PULSE ? kSmallBCtasF32 : kSmallBCtas;
+    return sweep_applies(ctx) && small_tiles<SmallB>(ctx) <= ctas * ctx->num_sms;
 }
 
 cudaError_t launch_small(trtr_ctx* ctx) {

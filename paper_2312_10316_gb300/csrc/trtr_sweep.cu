@@ -68,8 +68,8 @@ struct Sweep {
     static constexpr int Depth = 8;                                   // barriers of a level (iterations in flight)
     static constexpr int Smem = BarOff + (Blocks + kT * Depth + Outs) * 8 + 128;
     // Node pairs of a lane.  One (two warps a row) hides more latency, two (one warp) spend fewer instructions
-    // on addresses and waits.  4096^2 FP32, us a step, one / two: no source 89.4 / 95.5, source field 13 % apart
-    // (1101 x 1101), pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three
+    // on addresses and waits.  4096^2 FP32, us a step, one / two: no source 89.4 / 95.5, source field
+    // (2048^2) 29.9 / 36.3, pulse (whose row factors every warp loads) 105.8 / 98.9; 2-byte storages 103 (three
     // rows: four would be 33 warps) / 96.
     static constexpr int P = ES == 4 && SRC != TRTR_SRC_PULSE ? 1 : 2;
     // The fields and the pulse tables are older than the launch before and are read while it still runs: FP32, us a
