@@ -329,6 +329,12 @@ trtr_status trtr_batch_get_steps_per_launch(const trtr_batch* b, int* k);
  * (TRTR_EBOUNDS in the bounds-checked build if a kernel access out of bounds was caught). */
 trtr_status trtr_batch_sync(trtr_batch* b);
 
+/* Checks the timeout path of the batch's kernels: one block waits on a barrier that nothing completes for
+ * `cycles` clock cycles (1 .. 2^31), gives up and leaves as a block of a one-step launch does.  The step
+ * counts (trtr_batch_info) although its results are void, as after any timeout: set the instances'
+ * populations anew.  Returns what trtr_batch_sync does: TRTR_ETIMEOUT. */
+trtr_status trtr_batch_check_timeout_path(trtr_batch* b, long long cycles);
+
 /* The context of instance k (owned by the batch): moments, mass, error, populations. */
 trtr_status trtr_batch_instance(trtr_batch* b, int k, trtr_ctx** ctx);
 

@@ -84,13 +84,6 @@ __global__ void __launch_bounds__(256) batch_pulse_tables_kernel(const InstanceF
     fill_pulse_tables<float>(f.fill, levels, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
-// Level n - 1 of the pulse tables within them (the clock is advanced only after every CTA of the
-// launch has finished its tiles).
-__device__ __forceinline__ int pulse_level_at(const BatchClock* clk) {
-    const volatile BatchClock* c = clk;
-    return (int)(c->n - 1 - c->first);
-}
-
 // Asynchronous copy of `bytes` (a multiple of 16) from global to shared memory.
 __device__ __forceinline__ void cp_async_16(void* sdst, const void* gsrc, int bytes) {
     for (int o = 0; o < bytes; o += 16)
@@ -183,7 +176,7 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
     // stochastic rounding of the 2-byte storages: the key of this step (the clock is advanced
     // only after every CTA of the launch has finished its tiles)
     const uint32_t rkey = sr ? sr_step_key((long)*reinterpret_cast<volatile long long*>(&clk->n)) : 0u;
-    const int level = SRC == TRTR_SRC_PULSE ? pulse_level_at(clk) : 0;
+    const int level = SRC == TRTR_SRC_PULSE ? table_entry_at(clk, 1, desc[0].base[0].flag) : 0;
     __syncthreads();  // s_t of the first stages
 
     for (int k = 0;; ++k) {
@@ -225,12 +218,7 @@ __global__ void __launch_bounds__(32 * BY, min_blocks<BY>())
                 atomicExch(desc[t.x].base[0].flag, 1);
                 for (int kk = k + 1; kk < k + STAGES; ++kk)
                     if (s_t[kk % STAGES].x >= 0) mbar_wait_bounded(&full[kk % STAGES], (kk / STAGES) & 1);
-                // the counters go back to zero when the last CTA is out (the step's results are void)
-                __threadfence();
-                if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {
-                    atomicExch(&clk->next, 0u);
-                    atomicExch(&clk->done, 0u);
-                }
+                advance_clock(clk, 1);  // the step's results are void, but the host counts it
             }
             return;
         }
@@ -258,7 +246,7 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(16) StepArgs<float> sargs[STAGES];
     __shared__ int s_abort;
-    const int level = SRC == TRTR_SRC_PULSE ? pulse_level_at(clk) : 0;
+    const int level = SRC == TRTR_SRC_PULSE ? table_entry_at(clk, 2, desc[0].base[0].flag) : 0;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                            ~static_cast<uintptr_t>(127));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * T::Stage);
@@ -328,11 +316,7 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
                 atomicExch(desc[t.x].base[0].flag, 1);
                 for (int kk = k + 1; kk < k + STAGES; ++kk)
                     if (s_t[kk % STAGES].x >= 0) mbar_wait_bounded(&full[kk % STAGES], (kk / STAGES) & 1);
-                __threadfence();
-                if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {
-                    atomicExch(&clk->next, 0u);
-                    atomicExch(&clk->done, 0u);
-                }
+                advance_clock(clk, 2);
             }
             return;
         }
@@ -742,7 +726,7 @@ trtr_status build_graph2(trtr_batch* b) {
 // The pulse tables of the levels step - 1 .. step + steps - 1 in every instance.
 cudaError_t ensure_levels(trtr_batch* b, long step, int steps) {
     if (b->src != TRTR_SRC_PULSE) return cudaSuccess;
-    if (b->ptab_ready && step - 1 >= b->ptab_first && step + steps <= b->ptab_first + kPulseLevels) return cudaSuccess;
+    if (b->ptab_ready && levels_within(b->ptab_first, step, steps)) return cudaSuccess;
     for (int k = 0; k < b->count; k += 65535) {
         const int n = b->count - k < 65535 ? b->count - k : 65535;
         batch_pulse_tables_kernel<<<dim3(32, n), 256, 0, b->stream>>>(static_cast<const InstanceFill*>(b->d_fill) + k,
@@ -779,16 +763,21 @@ trtr_status setup_fills(trtr_batch* b) {
     return TRTR_OK;
 }
 
-// n steps: pairs through the two-step kernel where it applies (steps_per_launch 2), the rest
-// (an odd step, or all with steps_per_launch 1) through the one-step kernel of the configured
-// geometry.  Both kernels advance the device clock, so they interleave.
-trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
-    for (int k = 0; k < b->count; ++k)
-        if (b->ctx[k]->step != b->step || b->ctx[k]->cur != b->parity) return TRTR_ESTATE;
-    long left = n;
-    int par = b->parity;
-    bool last_two = false;
-    auto levels = [&](int steps) { return ensure_levels(b, b->step + (n - left), steps) == cudaSuccess; };
+// What the launches of one call have done: steps left, the parity and ghost frames that they leave.
+struct Advance {
+    long left;
+    int par;
+    bool last_two = false, last_four = false;
+};
+
+// The steps `at.left`: four at a time or pairs through the two-step kernel where these apply (steps_per_launch
+// 2), the rest (an odd step, or all with steps_per_launch 1) through the one-step kernel of the configured
+// geometry.  All kernels advance the device clock, so they interleave.  `at` follows every launch.
+trtr_status advance_launches(trtr_batch* b, int steps_per_launch, Advance& at) {
+    const long end = b->step + at.left;
+    long& left = at.left;
+    int& par = at.par;
+    auto levels = [&](int steps) { return ensure_levels(b, end - left, steps) == cudaSuccess; };
     const bool four = b->four_step && steps_per_launch == 2 && left >= 4;
     if (four || (b->two_step && steps_per_launch == 2 && left >= 2)) {
         for (int k = 0; k < b->count; ++k) {
@@ -800,7 +789,6 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
             }
         }
     }
-    bool last_four = false;
     if (four) {
         bool columns = true;
         for (int k = 0; k < b->count; ++k) columns = columns && b->ctx[k]->ghost4_ready;
@@ -810,13 +798,13 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
             if (!levels(4) || sweep_batch_launch(b->sweep, b->d_clk, b->d_flag, par, b->precision, b->src, b->sr, b->odd,
                                                  b->stream) != cudaSuccess)
                 return TRTR_ECUDA;
-        last_two = last_four = true;
+        at.last_two = at.last_four = true;
     }
     if (b->two_step && steps_per_launch == 2 && left >= 2) {
         if (!four)
             for (int k = 0; k < b->count; ++k)
                 if (!b->ctx[k]->ghost2_ready && launch_refresh_ghosts2(b->ctx[k]) != cudaSuccess) return TRTR_ECUDA;
-        last_four = false;
+        at.last_four = false;
         if (par == 1) {
             if (!levels(2) || launch_two(b, 1) != cudaSuccess) return TRTR_ECUDA;
             par = 0;
@@ -833,9 +821,9 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
             par = 1;
             left -= 2;
         }
-        last_two = true;
+        at.last_two = true;
     }
-    if (left > 0) last_two = last_four = false;  // one-step launches follow: the one-wide ghost frame
+    if (left > 0) at.last_two = at.last_four = false;  // one-step launches follow: the one-wide ghost frame
     if (left > 0 && par == 1) {  // bring the ping-pong to parity 0 for the graph
         if (!levels(1) || launch_one(b, 1) != cudaSuccess) return TRTR_ECUDA;
         par = 0;
@@ -850,17 +838,42 @@ trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
     if (left == 1) {
         if (!levels(1) || launch_one(b, 0) != cudaSuccess) return TRTR_ECUDA;
         par = 1;
+        left = 0;
     }
-    b->step += n;
-    b->parity = par;
+    return TRTR_OK;
+}
+
+// n steps, and what the launches have done in the batch and its instances: also where one of them fails after
+// others went out, so that the host's step stays the device clock's.
+trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
+    for (int k = 0; k < b->count; ++k)
+        if (b->ctx[k]->step != b->step || b->ctx[k]->cur != b->parity) return TRTR_ESTATE;
+    Advance at;
+    at.left = n;
+    at.par = b->parity;
+    const trtr_status s = advance_launches(b, steps_per_launch, at);
+    if (s != TRTR_OK) at.last_two = at.last_four = false;
+    const long done = n - at.left;
+    b->step += done;
+    b->parity = at.par;
     for (int k = 0; k < b->count; ++k) {
         b->ctx[k]->step = b->step;
         b->ctx[k]->cur = b->parity;
-        if (n > 0) b->ctx[k]->ghost2_ready = last_two;
-        if (n > 0) b->ctx[k]->ghost4_ready = last_four;
-        b->ctx[k]->launches += n;
+        if (done > 0) b->ctx[k]->ghost2_ready = at.last_two;
+        if (done > 0) b->ctx[k]->ghost4_ready = at.last_four;
+        b->ctx[k]->launches += done;
     }
-    return TRTR_OK;
+    return s;
+}
+
+// One block whose bounded wait gives up and which then leaves as a block of a one-step launch does.
+__global__ void batch_wait_timeout_kernel(BatchClock* clk, int* flag, long long cycles) {
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x != 0) return;
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (!mbar_wait_bounded(&bar, 0, cycles)) atomicExch(flag, 1);
+    advance_clock(clk, 1);
 }
 
 }  // namespace
@@ -999,6 +1012,22 @@ trtr_status trtr_batch_step(trtr_batch* b, long n) {
     trtr::TraceRange trace("trtr_batch_step");
     if (!b || n < 0) return TRTR_EINVAL;
     return trtr::advance(b, n, b->steps_per_launch);
+}
+
+trtr_status trtr_batch_check_timeout_path(trtr_batch* b, long long cycles) {
+    if (!b || cycles < 1 || cycles > (1LL << 31)) return TRTR_EINVAL;
+    for (int k = 0; k < b->count; ++k)
+        if (b->ctx[k]->step != b->step || b->ctx[k]->cur != b->parity) return TRTR_ESTATE;
+    trtr::batch_wait_timeout_kernel<<<1, 32, 0, b->stream>>>(b->d_clk, b->d_flag, cycles);
+    if (cudaGetLastError() != cudaSuccess) return TRTR_ECUDA;
+    b->step += 1;
+    b->parity ^= 1;
+    for (int k = 0; k < b->count; ++k) {
+        b->ctx[k]->step = b->step;
+        b->ctx[k]->cur = b->parity;
+        b->ctx[k]->ghost2_ready = b->ctx[k]->ghost4_ready = false;
+    }
+    return trtr_batch_sync(b);
 }
 
 trtr_status trtr_batch_sync(trtr_batch* b) {

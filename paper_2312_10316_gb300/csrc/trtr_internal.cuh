@@ -270,12 +270,27 @@ constexpr long kDynMinTilesPerCta = 8;
 
 enum MapId { kMapPop0 = 0, kMapPop1 = 1, kMapU = 2, kMapD = 3, kMapS = 4, kNumMaps = 5 };
 
-// Device clock of a batch.
+// Whether tables that hold kPulseLevels time levels from `first` on hold those of a launch of `steps` steps
+// from step `step`: step - 1 .. step + steps - 1.
+__host__ __device__ inline bool levels_within(long first, long step, int steps) {
+    return step - 1 >= first && step + steps <= first + kPulseLevels;
+}
+
+// Device clock of a batch.  Every launch that the host has counted advances it, one whose wait gave up
+// too: the host's step and the clock's never part, and the tables' levels that the host has filled are those
+// that the launches look up.
 struct BatchClock {
     long long n;        // step of the instances
     unsigned int done;  // CTAs of the running launch that have finished
     unsigned int next;  // next work-list entry of a dynamically scheduled launch
     long long first;    // time level of the pulse tables' first entry
+    // Entry of level n - 1 for a launch of `steps` steps, which reads the entries up to steps behind it.  A
+    // clock outside the tables (*outside) is answered by their nearest entry: no launch reads past them.
+    __host__ __device__ int table_entry(int steps, bool* outside) const {
+        const long long e = n - 1 - first, last = kPulseLevels - 1 - steps;
+        *outside = e < 0 || e > last;
+        return (int)(e < 0 ? 0 : (e > last ? last : e));
+    }
 };
 
 // The four-step kernel over a batch: its descriptors and work-list (device), and the work-list's length

@@ -468,7 +468,7 @@ __global__ void pulse_tables_kernel(const PulseFill fill, const __grid_constant_
 
 cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
     if (ctx->p.src_mode != TRTR_SRC_PULSE) return cudaSuccess;
-    if (ctx->ptab_ready && step - 1 >= ctx->ptab_first && step + steps <= ctx->ptab_first + kPulseLevels) return cudaSuccess;
+    if (ctx->ptab_ready && levels_within(ctx->ptab_first, step, steps)) return cudaSuccess;
     const long entries = (long)kPulseLevels * (ctx->p.nx + ctx->p.ny + 4 * kTabGhost);
     const long want = (entries + 255) / 256, cap = (long)ctx->num_sms * 8;
     const unsigned grid = (unsigned)(want < cap ? want : cap);

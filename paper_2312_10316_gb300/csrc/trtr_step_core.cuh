@@ -171,8 +171,21 @@ __device__ __forceinline__ bool bulk_ok(const S* gdst, const void* src, int i0, 
     return true;
 }
 
-// A CTA's end of a batch launch of `steps` steps (one thread): the last CTA to finish advances the step
-// clock and sets the work-list counter back.
+// Entry of level n - 1 in the pulse tables for a batch launch of `steps` steps (the clock is advanced only
+// after every CTA of the launch has finished its tiles); a clock outside the tables sets the flag.
+__device__ __forceinline__ int table_entry_at(const BatchClock* clk, int steps, int* flag) {
+    const volatile BatchClock* v = clk;
+    BatchClock c = {};
+    c.n = v->n;
+    c.first = v->first;
+    bool outside;
+    const int e = c.table_entry(steps, &outside);
+    if (outside && threadIdx.x == 0) atomicExch(flag, 1);
+    return e;
+}
+
+// A CTA's end of a batch launch of `steps` steps (one thread), also of one whose wait gave up: the last CTA
+// to finish advances the step clock and sets the work-list counter back.
 __device__ __forceinline__ void advance_clock(BatchClock* clk, int steps) {
     __threadfence();
     if (atomicAdd(&clk->done, 1u) == gridDim.x - 1) {

@@ -333,9 +333,8 @@ __global__ void __launch_bounds__(G::Threads, 1)
         u_first = p.first[blockIdx.x];
         u_end = p.first[blockIdx.x + 1];
         u_step = 1;
-        const volatile BatchClock* c = p.clk;
-        step = c->n;
-        table_level = (int)(step - 1 - c->first);
+        step = const_cast<const volatile BatchClock*>(p.clk)->n;
+        if (SRC == TRTR_SRC_PULSE) table_level = table_entry_at(p.clk, kT, p.flag);
     } else {
         u_end = a_.units;
     }
@@ -428,6 +427,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
             phase += blocks;
             it0 += t.iters;
         }
+        if (*abort_flag) ok = false;  // (the last level's last buffer)
         if (lane == 0) {
             if (!ok) {  // let the loads issued into this CTA's shared memory land (bounded)
                 if constexpr (BATCH)
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
             }
             bulk_wait_all();
             // every warp has read the clock: the last level has finished its units (or a wait gave up)
-            if constexpr (BATCH) advance_clock(p.clk, ok ? kT : 0);
+            if constexpr (BATCH) advance_clock(p.clk, kT);
         }
         return;
     }

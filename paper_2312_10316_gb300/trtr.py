@@ -93,6 +93,7 @@ _SIGNATURES = {
     "trtr_batch_set_config": (_st, [_vp, ctypes.c_int]),
     "trtr_batch_step": (_st, [_vp, ctypes.c_long]),
     "trtr_batch_sync": (_st, [_vp]),
+    "trtr_batch_check_timeout_path": (_st, [_vp, ctypes.c_longlong]),
     "trtr_batch_instance": (_st, [_vp, ctypes.c_int, ctypes.POINTER(_vp)]),
     "trtr_batch_info": (_st, [_vp, ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_longlong),
                               ctypes.POINTER(ctypes.c_long), ctypes.POINTER(ctypes.c_int)]),
@@ -592,6 +593,11 @@ def trtr_batch_get_steps_per_launch(b) -> int:
 
 def trtr_batch_sync(b):
     _bcheck(lib.trtr_batch_sync(b), "trtr_batch_sync")
+
+
+def trtr_batch_check_timeout_path(b, cycles: int) -> int:
+    """The status (TRTR_ETIMEOUT where the path works)."""
+    return int(lib.trtr_batch_check_timeout_path(b, int(cycles)))
 
 
 def trtr_batch_instance(b, k: int):
