@@ -343,8 +343,9 @@ struct trtr_batch {
     int4* d_tiles;
     int ntiles;
     void* d_fill;     // InstanceFill of every instance (src PULSE)
-    long ptab_first;  // time level of the pulse tables' first entry
-    bool ptab_ready;
+    std::vector<trtr::Pulse> pulses;  // of the instances, as the batch was given them
+    long ptab_first;  // the level that the device clock has for the pulse tables' first entry ...
+    bool ptab_ready;  // ... and whether every instance's tables hold its levels from there on
     // two steps per launch (FP32 instances): descriptors and work-list of the two-step kernel,
     // its graph, and whether pairs of steps use it
     void* d_desc2;
@@ -732,9 +733,21 @@ cudaError_t ensure_levels(trtr_batch* b, long step, int steps) {
         batch_pulse_tables_kernel<<<dim3(32, n), 256, 0, b->stream>>>(static_cast<const InstanceFill*>(b->d_fill) + k,
                                                                       b->d_clk, step - 1);
     }
+    const cudaError_t e = cudaGetLastError();
+    for (int k = 0; k < b->count; ++k) tables_filled(b->ctx[k], b->pulses[k], step - 1, e);
     b->ptab_first = step - 1;
-    b->ptab_ready = cudaPeekAtLastError() == cudaSuccess;
-    return cudaGetLastError();
+    b->ptab_ready = e == cudaSuccess;
+    return e;
+}
+
+// Whether the instances' tables are still the batch's last fill: an instance's own calls refill them too.
+bool tables_held(const trtr_batch* b) {
+    bool held = b->ptab_ready;
+    for (int k = 0; k < b->count && held; ++k) {
+        const trtr_ctx* c = b->ctx[k];
+        held = c->ptab_ready && c->ptab_first == b->ptab_first && c->ptab_pulse == b->pulses[k];
+    }
+    return held;
 }
 
 // Instances without tables of their own (src NONE beside PULSE instances) get them; the fills go to
@@ -751,6 +764,7 @@ trtr_status setup_fills(trtr_batch* b) {
             }
         }
         h[k] = InstanceFill{pulse_fill_of(c), c->pulse, c->p.dt};
+        b->pulses.push_back(c->pulse);
     }
     if (cudaMalloc(&b->d_fill, sizeof(InstanceFill) * b->count) != cudaSuccess) {
         cudaGetLastError();
@@ -848,6 +862,7 @@ trtr_status advance_launches(trtr_batch* b, int steps_per_launch, Advance& at) {
 trtr_status advance(trtr_batch* b, long n, int steps_per_launch) {
     for (int k = 0; k < b->count; ++k)
         if (b->ctx[k]->step != b->step || b->ctx[k]->cur != b->parity) return TRTR_ESTATE;
+    if (b->src == TRTR_SRC_PULSE) b->ptab_ready = tables_held(b);
     Advance at;
     at.left = n;
     at.par = b->parity;

@@ -46,6 +46,9 @@ constexpr int kQ = 9;
 struct Pulse {
     double omega, xc, yc, sigma0, D0, D_amp;
 };
+inline bool operator==(const Pulse& a, const Pulse& b) {
+    return a.omega == b.omega && a.xc == b.xc && a.yc == b.yc && a.sigma0 == b.sigma0 && a.D0 == b.D0 && a.D_amp == b.D_amp;
+}
 
 // Per-time uniforms of the pulse source / closed form, computed on the host in double.
 struct PulseTime {
@@ -333,10 +336,12 @@ struct trtr_ctx {
     void* tab_x;
     void* tab_y;
     void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
-    long ptab_first;  // time level of its first entry
+    // what they hold, whoever filled them last (the context or its batch), if ptab_ready
+    trtr::Pulse ptab_pulse;
+    long ptab_first;  // time level of the first entry
+    bool ptab_ready;
     bool tables_new;  // the tables or packed fields were written since the last launch that reads them early
                       // (before it waits for the launch before it)
-    bool ptab_ready;  // it holds the levels from ptab_first on, of the current pulse
     double* scratch;  // reduction partials
     int red_blocks;
     double* hres;     // pinned host memory that kernels write: the reductions' two results; [3]: copy of the timeout flag

@@ -468,7 +468,7 @@ __global__ void pulse_tables_kernel(const PulseFill fill, const __grid_constant_
 
 cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
     if (ctx->p.src_mode != TRTR_SRC_PULSE) return cudaSuccess;
-    if (ctx->ptab_ready && levels_within(ctx->ptab_first, step, steps)) return cudaSuccess;
+    if (ctx->ptab_ready && ctx->ptab_pulse == ctx->pulse && levels_within(ctx->ptab_first, step, steps)) return cudaSuccess;
     const long entries = (long)kPulseLevels * (ctx->p.nx + ctx->p.ny + 4 * kTabGhost);
     const long want = (entries + 255) / 256, cap = (long)ctx->num_sms * 8;
     const unsigned grid = (unsigned)(want < cap ? want : cap);
@@ -479,8 +479,7 @@ cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
     else
         pulse_tables_kernel<float><<<grid, 256, 0, ctx->stream>>>(pulse_fill_of(ctx), pulse_levels_of(ctx, step - 1));
     const cudaError_t e = cudaGetLastError();
-    ctx->ptab_first = step - 1;
-    ctx->ptab_ready = e == cudaSuccess;
+    tables_filled(ctx, ctx->pulse, step - 1, e);
     ctx->tables_new = true;
     return e;
 }

@@ -342,10 +342,7 @@ static cudaError_t pack_into(trtr_ctx* ctx, void* dst, bool tables) {
 cudaError_t launch_pack_fields2(trtr_ctx* ctx) {
     const bool tables = ctx->p.src_mode == TRTR_SRC_PULSE;
     const cudaError_t e = pack_into(ctx, ctx->fld2, tables);
-    if (tables) {
-        ctx->ptab_first = ctx->step - 1;
-        ctx->ptab_ready = e == cudaSuccess;
-    }
+    if (tables) tables_filled(ctx, ctx->pulse, ctx->step - 1, e);
     return e;
 }
 

@@ -321,6 +321,13 @@ inline PulseFill pulse_fill_of(const trtr_ctx* ctx) {
     return f;
 }
 
+// A fill of the context's tables with `pulse` from level `first` on has been launched (e: how that went).
+inline void tables_filled(trtr_ctx* ctx, const Pulse& pulse, long first, cudaError_t e) {
+    ctx->ptab_pulse = pulse;
+    ctx->ptab_first = first;
+    ctx->ptab_ready = e == cudaSuccess;
+}
+
 // The tables of a launch from step `step`: coordinate 0 of level step - 1.
 template <typename C>
 inline const C* pulse_level(const trtr_ctx* ctx, const PulseTab& t, long step) {
