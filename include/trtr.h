@@ -179,7 +179,9 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
  * steps a launch, with odd nx and a source field that stays the same from step to step too, again
  * with the same bits.  An odd last step, or a pair whose middle step is a check_every
  * point, runs one step per launch.  Short launches use programmatic dependent launch: each
- * waits for the work before it on the stream before reading its results. */
+ * waits for the work before it on the stream before reading its results.  A call captured into a CUDA
+ * graph takes one and two steps a launch and prepares what they read in the graph: a replay goes on from
+ * the state in the buffer that was current at the capture, at the captured times. */
 trtr_status trtr_step(trtr_ctx* ctx, long n);
 
 /* k = 2 (the default): trtr_step takes two steps a launch, or four, where it can; k = 1: one step

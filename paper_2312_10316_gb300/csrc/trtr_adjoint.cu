@@ -401,19 +401,23 @@ trtr_status trtr_forward_record(trtr_ctx* ctx, long steps, int interval) {
     }
     // the recorded run keeps only the checkpoint states, so several steps between two checkpoints may
     // run as one launch (the same states bit for bit)
+    trtr::begin_steps(ctx);
+    const char* what = "";
     for (long k = 0; k < steps;) {
+        what = "checkpoint copy";
         if (k % a->interval == 0 &&
             cudaMemcpyAsync(a->ckpt[k / a->interval], ctx->pop[ctx->cur], a->state_bytes, cudaMemcpyDeviceToDevice,
                             ctx->stream) != cudaSuccess)
-            return adj_fail(ctx, TRTR_ECUDA, "checkpoint copy failed");
+            break;
         const long to_checkpoint = a->interval - k % a->interval;
-        const char* what = "";
         int taken = 0;
         if (trtr::launch_steps(ctx, to_checkpoint < steps - k ? to_checkpoint : steps - k, steps, &taken, &what) != cudaSuccess)
-            return adj_fail(ctx, TRTR_ECUDA, what);
+            break;
         k += taken;
+        what = nullptr;
     }
-    return TRTR_OK;
+    trtr::end_steps(ctx);
+    return what ? adj_fail(ctx, TRTR_ECUDA, what) : TRTR_OK;
 }
 
 trtr_status trtr_adjoint(trtr_ctx* ctx, const double* dJ_dphi, int on_device, double* grad_D, int grad_on_device) {

@@ -31,6 +31,30 @@ cudaError_t bounds_take_all(cudaStream_t s, unsigned long long* out) {
     return cudaSuccess;
 }
 
+// A call that is captured into a graph is replayed later, with other calls in between: it prepares what its
+// launches read (packed fields, tables, ghost frames) itself and hands nothing prepared on, for none of it
+// has run; and it keeps to one and two steps a launch, so that a call of an even number of them leaves the
+// state in the buffer where its replays look for it.  Calls on a context that has been captured find
+// tables and ghost frames as a replay left them.
+static void forget_prepared(trtr_ctx* ctx, bool fields) {
+    ctx->ptab_ready = ctx->ghost2_ready = ctx->ghost4_ready = false;
+    if (fields) ctx->fld2_ready = ctx->pack64_ready = ctx->src_ready = false;
+}
+void begin_steps(trtr_ctx* ctx) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &status) != cudaSuccess) {
+        cudaGetLastError();
+        status = cudaStreamCaptureStatusNone;
+    }
+    ctx->capturing = status == cudaStreamCaptureStatusActive;
+    ctx->captured = ctx->captured || ctx->capturing;
+    if (ctx->captured) forget_prepared(ctx, ctx->capturing);
+}
+void end_steps(trtr_ctx* ctx) {
+    if (ctx->capturing) forget_prepared(ctx, true);
+    ctx->capturing = false;
+}
+
 // Four steps a launch (trtr_sweep.cu) where the call takes enough of them: the launch that brings the
 // ghost columns up to date costs what two sweeps of a small grid save over two-step launches (200^2
 // FP32, 8 steps: 22 us either way), on a large one it is lost in the first.
@@ -39,7 +63,7 @@ constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 
 cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
     const bool two = most >= 2 && two_step_applies(ctx);
     const long nodes = (long)ctx->p.nx * ctx->p.ny;
-    const bool four = most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
+    const bool four = !ctx->capturing && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
                       sweep_applies(ctx);
     const bool small = four && small_applies(ctx);
     cudaError_t e = cudaSuccess;
@@ -520,19 +544,8 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
     return TRTR_OK;
 }
 
-trtr_status trtr_step(trtr_ctx* ctx, long n) {
-    trtr::TraceRange trace("trtr_step");
-    if (!ctx) return TRTR_EINVAL;
-    if (n < 0) return fail(ctx, TRTR_EINVAL, "negative step count");
+static trtr_status take_steps(trtr_ctx* ctx, long n) {
     trtr_status s;
-    if (!ready(ctx, &s)) return s;
-    if (ctx->p.src_mode == TRTR_SRC_FIELD && ctx->S_cur < 0)
-        return fail(ctx, TRTR_ESTATE, "src_mode FIELD needs a source (trtr_set_source)");
-    if (ctx->p.src_mode == TRTR_SRC_PULSE && !ctx->pulse_set)
-        return fail(ctx, TRTR_ESTATE, "src_mode PULSE needs trtr_set_pulse");
-    const bool nee = ctx->p.bc_mode == TRTR_BC_DIRICHLET_NEE;
-    if (nee && !ctx->dirichlet_set)
-        return fail(ctx, TRTR_ESTATE, "bc_mode DIRICHLET_NEE needs boundary values (trtr_set_dirichlet)");
     const long every = ctx->p.check_every;
     for (long k = 0; k < n;) {
         // no launch passes over a step that the stability check looks at
@@ -552,6 +565,25 @@ trtr_status trtr_step(trtr_ctx* ctx, long n) {
         }
     }
     return TRTR_OK;
+}
+
+trtr_status trtr_step(trtr_ctx* ctx, long n) {
+    trtr::TraceRange trace("trtr_step");
+    if (!ctx) return TRTR_EINVAL;
+    if (n < 0) return fail(ctx, TRTR_EINVAL, "negative step count");
+    trtr_status s;
+    if (!ready(ctx, &s)) return s;
+    if (ctx->p.src_mode == TRTR_SRC_FIELD && ctx->S_cur < 0)
+        return fail(ctx, TRTR_ESTATE, "src_mode FIELD needs a source (trtr_set_source)");
+    if (ctx->p.src_mode == TRTR_SRC_PULSE && !ctx->pulse_set)
+        return fail(ctx, TRTR_ESTATE, "src_mode PULSE needs trtr_set_pulse");
+    const bool nee = ctx->p.bc_mode == TRTR_BC_DIRICHLET_NEE;
+    if (nee && !ctx->dirichlet_set)
+        return fail(ctx, TRTR_ESTATE, "bc_mode DIRICHLET_NEE needs boundary values (trtr_set_dirichlet)");
+    trtr::begin_steps(ctx);
+    s = take_steps(ctx, n);
+    trtr::end_steps(ctx);
+    return s;
 }
 
 trtr_status trtr_moments(trtr_ctx* ctx, double* phi_out, int on_device) {

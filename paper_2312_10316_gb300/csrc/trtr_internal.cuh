@@ -365,6 +365,8 @@ struct trtr_ctx {
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
     void* pack64;           // FP64: [4][rows][pitch] a_x, a_y, k1, k2 (the layout of uv)
     bool pack64_ready;      // it holds the current fields
+    bool capturing;         // trtr_step is being captured into a graph: no four-step launches
+    bool captured;          // a call of it has been: replays may change the tables and ghost frames between calls
     int steps_per_launch;   // 2: trtr_step uses the two-step kernel where it applies; 1: never
     trtr::Pulse pulse;
     long step;
@@ -412,6 +414,9 @@ cudaError_t launch_pack_source(trtr_ctx* ctx);  // the source term's plane of th
 // four, two or one steps, with what the launch needs; advances the context's state.  *taken: the
 // steps; *what: names the failing launch on an error.
 cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what);
+// before the first and after the last launch_steps of a call (captured or not)
+void begin_steps(trtr_ctx* ctx);
+void end_steps(trtr_ctx* ctx);
 // the same over a batch's instances (all of sweep_applies): setup, the ghost columns of buffer `parity`,
 // one launch of four steps from buffer `parity` (odd: an instance of odd width)
 cudaError_t sweep_batch_setup(trtr_ctx* const* ctx, int count, cudaStream_t stream, SweepBatch* out);
