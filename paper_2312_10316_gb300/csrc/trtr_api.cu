@@ -63,9 +63,10 @@ constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 
 cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
     const bool two = most >= 2 && two_step_applies(ctx);
     const long nodes = (long)ctx->p.nx * ctx->p.ny;
-    const bool four = !ctx->capturing && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
-                      sweep_applies(ctx);
-    const bool small = four && small_applies(ctx);
+    const bool can = !ctx->capturing && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
+                     sweep_applies(ctx);
+    const bool small = can && small_applies(ctx);
+    const bool four = small || (can && (ctx->sweep_sooner || !two));
     cudaError_t e = cudaSuccess;
     if ((two || four) && !ctx->fld2_ready) {
         *what = "field packing launch";

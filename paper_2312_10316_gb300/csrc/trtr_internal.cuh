@@ -361,6 +361,7 @@ struct trtr_ctx {
     bool src_ready;         // its source plane (TRTR_SRC_FIELD) holds the current S^n
     bool fld2_ready;        // fld2 holds the current fields
     int sweep_rows;         // rows of its segments
+    bool sweep_sooner;      // its four steps end before those of two two-step launches
     bool ghost4_ready;      // its four-wide ghost columns are up to date (interior rows)
     bool ghost2_ready;      // the current population buffer's whole two-wide ghost frame is up to date
     void* pack64;           // FP64: [4][rows][pitch] a_x, a_y, k1, k2 (the layout of uv)
@@ -403,6 +404,8 @@ cudaError_t launch_step2_from(trtr_ctx* ctx, const CUtensorMap* src_map, void* d
 // The four-step kernel (trtr_sweep.cu): whether it applies to the context, its maps (at creation),
 // one launch advancing the state by four steps, and the ghost columns that it reads.
 bool sweep_applies(const trtr_ctx* ctx);
+double sweep_us(int precision, int src, double iterations);     // estimate of a launch of so many iterations a CTA
+double two_step_us(int precision, int src, int num_sms, int nx, int ny);  // of a two-step launch (trtr_step2.cu)
 cudaError_t encode_maps4(trtr_ctx* ctx);
 cudaError_t launch_sweep(trtr_ctx* ctx);
 cudaError_t launch_ghost_columns(trtr_ctx* ctx);

@@ -272,6 +272,22 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
 
 }  // namespace
 
+// A two-step launch on GB300 in us, for the choice between it and the sweep: a start, a term for each round of
+// its tiles (`ctas` of them at once) and one for the tiles at the left and right edges, which store ghost copies
+// column by column (a 16-column grid's 32-column tiles half of them); at least `least`.
+double two_step_us(int precision, int src, int num_sms, int nx, int ny) {
+    const bool f32 = precision == TRTR_F32, pulse = src == TRTR_SRC_PULSE;
+    const int bx = f32 ? Geom2Of<TRTR_SRC_NONE, 4>::T::X : Geom2Of<TRTR_SRC_NONE, 2>::T::X;
+    const int by = f32 ? Geom2Of<TRTR_SRC_NONE, 4>::T::Y : Geom2Of<TRTR_SRC_NONE, 2>::T::Y;
+    const int ctas = num_sms * (f32 ? Geom2Of<TRTR_SRC_NONE, 4>::kCtas : Geom2Of<TRTR_SRC_NONE, 2>::kCtas);
+    const double start = f32 ? (pulse ? 1.55 : 1.4) : (pulse ? 4.2 : 4.0), round = f32 ? (pulse ? 2.75 : 2.5) : (pulse ? 5.7 : 5.0),
+                 edge = f32 ? (pulse ? 0.0058 : 0.0055) : (pulse ? 0.016 : 0.015), least = f32 ? (pulse ? 7.0 : 6.5) : (pulse ? 9.0 : 8.0);
+    const long cols = (nx + bx - 1) / bx, rows = (ny + by - 1) / by, rounds = (cols * rows + ctas - 1) / ctas;
+    const double edges = cols > 1 ? 2.0 : (f32 && nx < bx ? (double)nx / bx : 1.0);
+    const double us = start + round * (double)rounds + edge * edges * (double)rows;
+    return us > least ? us : least;
+}
+
 bool two_step_applies(const trtr_ctx* ctx) {
     // 2-byte storages: even widths, whose halo pairs are the one-step kernel's pairs
     return ctx->fld2 != nullptr && (ctx->esize == 4 || ctx->p.nx % 2 == 0) && ctx->steps_per_launch == 2 && ctx->p.bc_mode == TRTR_BC_PERIODIC &&

@@ -644,9 +644,9 @@ bool encode_maps_of(const trtr_ctx* ctx, CUtensorMap* rows, CUtensorMap* stores,
 }
 
 // Rows of a segment: the number of segments a strip that ends soonest, by rounds of the SMs times a unit's
-// rows (once per context: the search took longer than a launch of a 512^2 grid).
+// rows (once per context: the search took longer than a launch of a 512^2 grid).  *iterations: of a CTA.
 template <class G>
-int segment_rows(const trtr_ctx* ctx) {
+int segment_rows(const trtr_ctx* ctx, double* iterations) {
     const int ny = ctx->p.ny, strips = (ctx->p.nx + kX - 1) / kX;
     long best = 0;
     int best_rows = ny;
@@ -659,12 +659,22 @@ int segment_rows(const trtr_ctx* ctx) {
             best_rows = rows;
         }
     }
+    *iterations = (double)best / G::R;
     return best_rows;
 }
 
 template <typename S, int SRC>
 cudaError_t encode4_typed(trtr_ctx* ctx) {
-    ctx->sweep_rows = segment_rows<Sweep<S, SRC>>(ctx);
+    // A strip costs its 128 columns however few of them the grid has, and a segment its ramp: grids of up to 32
+    // columns (FP32) or of about 40 rows take longer than two two-step launches.  Measured (GB300, FP32 pulse, us for
+    // four steps, sweep / two-step launches): 16 x 8000 33.7 / 26.8, 32 x 20000 73.2 / 69.2, 20000 x 32 42.8 / 34.5,
+    // 48 x 8000 34.0 / 44.5, 121 x 1000 14.2 / 15.8, 4000 x 64 15.4 / 20.7, 500^2 14.9 / 22.7; without a source
+    // 16 x 8000 26.6 / 24.8, 20000 x 32 34.0 / 31.8; FP16 20000 x 32 38.4 / 37.6, 16 x 8000 31.7 / 44.9.  Both sides are
+    // estimated to 15 %, most within 8: the sweep has to win by that.
+    double iterations = 0.0;
+    ctx->sweep_rows = segment_rows<Sweep<S, SRC>>(ctx, &iterations);
+    ctx->sweep_sooner = 1.08 * sweep_us(ctx->p.precision, ctx->p.src_mode, iterations) <
+                        2.0 * two_step_us(ctx->p.precision, ctx->p.src_mode, ctx->num_sms, ctx->p.nx, ctx->p.ny);
     return encode_maps_of<S, Sweep<S, SRC>>(ctx, &ctx->maps4[0], &ctx->maps4[2], &ctx->maps4[4]) ? cudaSuccess
                                                                                                  : cudaErrorInvalidValue;
 }
@@ -783,6 +793,14 @@ cudaError_t launch_batch_typed(const SweepBatch& b, BatchClock* clk, int* flag, 
 
 // Rows wrap once around the grid, and a row holds at least one whole 16-byte chunk.
 static bool sweep_size(const trtr_ctx* ctx) { return ctx->p.nx >= 16 && ctx->p.ny >= 32; }
+
+// Fitted to launches of 5 to 140 iterations on GB300 (FP32 to 6 %, FP16 to 13 %; the first iterations, which only
+// load, are shorter): us an iteration of three rows (two with a source field; four of the 2-byte storages).
+double sweep_us(int precision, int src, double iterations) {
+    if (precision != TRTR_F32) return src == TRTR_SRC_PULSE ? 2.1 * iterations - 5.0 : 1.8 * iterations - 3.6;
+    const double us = src == TRTR_SRC_PULSE ? 1.40 : (src == TRTR_SRC_FIELD ? 0.89 : 1.13);
+    return us * iterations - 1.8;
+}
 
 cudaError_t encode_maps4(trtr_ctx* ctx) {
     if (!ctx->fld2 || !sweep_size(ctx)) return cudaSuccess;
