@@ -305,11 +305,12 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         if (!ok) s_abort = 1;
         S* sp = reinterpret_cast<S*>(smem + s * T::Stage);
         const float* sf = reinterpret_cast<const float*>(smem + s * T::Stage + T::FldOff);
-        auto tables = [&](int l) { return SRC == TRTR_SRC_PULSE ? sargs[s].pulse + (size_t)(level + l) * sargs[s].pt.level : nullptr; };
-        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, t.y, t.z, sargs[s], tables(0), tid, rkey1);
+        TableSource source{nullptr, &sargs[s].pt};
+        if (SRC == TRTR_SRC_PULSE) source.lev = sargs[s].pulse + (size_t)level * sargs[s].pt.level;
+        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, t.y, t.z, sargs[s], source, tid, rkey1);
         __syncthreads();  // step 1 complete (and s_abort visible)
         if (ok && !s_abort)
-            step2_second<S, SRC, T, NT, false, SR>(sp, sf, t.y, t.z, sargs[s], tables(1), tid, nullptr, rkey2);
+            step2_second<S, SRC, T, NT, false, SR>(sp, sf, t.y, t.z, sargs[s], source, tid, nullptr, rkey2);
         __syncthreads();  // stage s and its argument slot fully read
         if (s_abort) {
             if (tid == 0) {

@@ -228,7 +228,7 @@ constexpr int kSchedDynamic = 1, kSchedReverse = 2;
 template <typename C>
 struct alignas(16) StepArgs {
     void* dst;              // P written by this step (plain stores, with ghosts)
-    const C* pulse;         // pulse tables (TRTR_SRC_PULSE): coordinate 0 of level n - 1 (level n follows)
+    const C* pulse;         // pulse tables of a batch's instance: coordinate 0 of their first level
     int* flag;              // set when a bounded wait gives up
     unsigned* tile_ctr;     // [next tile, CTAs done] of kernels that hand out tiles dynamically (zero between launches)
     PlaneLayout lp;         // populations
@@ -238,7 +238,8 @@ struct alignas(16) StepArgs {
     C magic;                // Lambda
     C omega2_fixed;         // 1 / tau2 (TRTR_TAU2_FIXED)
     C phi_ref;
-    PulseTab pt;            // layout of the pulse tables
+    PulseTab pt;            // their layout
+    int entry;              // of level n - 1 in the pulse tables (TRTR_SRC_PULSE; a context's)
     uint32_t rkey;          // stochastic rounding of the 2-byte storages: the step's key (sr_step_key)
     int sched;              // kSchedDynamic | kSchedReverse (below)
 };
@@ -271,7 +272,8 @@ constexpr long kPdlMaxTilesPerCta = 8;
 // (the 512^2 adjoint's forward steps: 11 -> 18 us per two-step launch).
 constexpr long kDynMinTilesPerCta = 8;
 
-enum MapId { kMapPop0 = 0, kMapPop1 = 1, kMapU = 2, kMapD = 3, kMapS = 4, kNumMaps = 5 };
+// (kMapS: the source planes, or the x factors of the pulse tables, whose y factors are kMapY)
+enum MapId { kMapPop0 = 0, kMapPop1 = 1, kMapU = 2, kMapD = 3, kMapS = 4, kMapY = 5, kNumMaps = 6 };
 
 // Whether tables that hold kPulseLevels time levels from `first` on hold those of a launch of `steps` steps
 // from step `step`: step - 1 .. step + steps - 1.
@@ -353,7 +355,7 @@ struct trtr_ctx {
     bool fields_set, pulse_set, initialized, maps_ready, dirichlet_set;
     bool small_tiles;  // step kernel geometry for small grids (chosen by encode_maps)
     // two-step kernel (FP32 storage, periodic boundaries, no source or the pulse source)
-    CUtensorMap maps2[3];   // populations (buffers 0, 1) and packed fields, its tile boxes
+    CUtensorMap maps2[5];   // populations (buffers 0, 1), packed fields and pulse tables (x, y), its tile boxes
     CUtensorMap maps4[5];   // four-step kernel: population rows (buffers 0, 1), interior stores (0, 1), field rows
     void* fld2;             // [5 or 6][rows][pitch] float: uhat_x, uhat_y, a_x, a_y, Dh (and the stationary
                             // source term, TRTR_SRC_FIELD), four-wide periodic ghosts

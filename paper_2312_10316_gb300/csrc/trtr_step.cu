@@ -147,20 +147,28 @@ struct SmallPipe {
 #define TRTR_STEP_PDL 1  // 0: never launch the step with programmatic dependent launch (sweeps)
 #endif
 
+// A stage: the tile's boxes and, with the pulse source, its tables.
+template <class T, class Tab, int SRC>
+constexpr int stage_bytes() {
+    return (int)T::STAGE + (SRC == TRTR_SRC_PULSE ? Tab::Bytes : 0);
+}
+
 template <typename S, int SRC, int STAGES, class G, bool SR>
 __global__ void __launch_bounds__(G::THREADS, G::CTAS)
     step_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mu,
-                const __grid_constant__ CUtensorMap md, const __grid_constant__ CUtensorMap ms,
+                const __grid_constant__ CUtensorMap md, const __grid_constant__ CUtensorMap ms, const __grid_constant__ CUtensorMap my,
                 const StepArgs<typename Store<S>::C> a) {
     constexpr int kBX = G::BX, kBY = G::BY, kWPR = G::WPR, kPairsPerLane = G::PAIRS;
     constexpr bool kTST = G::TST;
     using T = Tile<S, SRC, kBX, kBY>;
+    using Tab = TileTables<kBX, kBY, 2>;
+    constexpr int kStage = stage_bytes<T, Tab, SRC>();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_abort;
     // stages on a 128-byte boundary (TMA destination alignment), barriers after them
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                            ~static_cast<uintptr_t>(127));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * T::STAGE);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * kStage);
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r = w / kWPR;                // tile row of this warp
@@ -225,13 +233,17 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
             }
         }
     };
+    auto issue = [&](int t, int s) {
+        const int x0 = tile_x0(t), y0 = tile_y0(t);
+        issue_tile<S, SRC, kBX, kBY>(smem + s * kStage, &full[s], &mp, &mu, &md, &ms, x0, y0, a, SRC == TRTR_SRC_PULSE ? Tab::TX : 0);
+        if (SRC == TRTR_SRC_PULSE) Tab::issue(smem + s * kStage + T::STAGE, &full[s], &ms, &my, a.entry, x0, y0);
+    };
     if (tid == 0) {
         s_more = 1;
         for (int k = 0; k < STAGES; ++k) {
             const int t = take(k);
             s_tile[k] = t;
-            if (t >= 0) issue_tile<S, SRC, kBX, kBY>(smem + k * T::STAGE, &full[k], &mp, &mu, &md, &ms, tile_x0(t),
-                                                     tile_y0(t), a);
+            if (t >= 0) issue(t, k);
         }
     }
     __syncthreads();
@@ -243,18 +255,15 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
         const int i0 = tile_x0(t), j0 = tile_y0(t);
         const int j = j0 + r;
 
-        // the pulse source of this lane's pairs, from its tables before the wait (hides their latency)
-        F2 psrc[kPairsPerLane];
-        if (SRC == TRTR_SRC_PULSE && j < ny) {
-#pragma unroll
-            for (int m = 0; m < kPairsPerLane; ++m)
-                psrc[m] = pulse_source_dt(reinterpret_cast<const float*>(a.pulse), a.pt, i0 + c0 + 64 * m + 2 * lane, j);
-        }
-
         const bool ok = mbar_wait_bounded(&full[s], (k / STAGES) & 1);
         if (!ok) s_abort = 1;
         if (ok && j < ny) {
-            const unsigned char* st = smem + s * T::STAGE;
+            const unsigned char* st = smem + s * kStage;
+            F2 psrc[kPairsPerLane];  // the pulse source of this lane's pairs
+            if (SRC == TRTR_SRC_PULSE) {
+#pragma unroll
+                for (int m = 0; m < kPairsPerLane; ++m) psrc[m] = Tab::source(st + T::STAGE, 0, c0 + 64 * m + 2 * lane, r);
+            }
             tile_row_pairs<S, SRC, kBX, kBY, kPairsPerLane, kTST, G::UNR, SR>(st, r, lane, i0, j, a, psrc, c0);
         }
         __syncthreads();  // stage s fully read (and s_abort visible)
@@ -272,9 +281,7 @@ __global__ void __launch_bounds__(G::THREADS, G::CTAS)
         if (tid == 0) {
             const int tn = take(k + STAGES);
             s_tile[s] = tn;
-            if (tn >= 0)
-                issue_tile<S, SRC, kBX, kBY>(smem + s * T::STAGE, &full[s], &mp, &mu, &md, &ms, tile_x0(tn),
-                                             tile_y0(tn), a);
+            if (tn >= 0) issue(tn, s);
         }
         if constexpr (STAGES == 1) __syncthreads();  // s_tile[0] is read again at once
     }
@@ -312,7 +319,7 @@ __global__ void bounds_probe_kernel(PlaneLayout L) {
 // Stages per CTA: G::STAGES, or fewer while they do not fit in the 227 KB a CTA may use.
 template <typename S, int SRC, class G>
 constexpr int stages_for() {
-    constexpr int kStage = Tile<S, SRC, G::BX, G::BY>::STAGE;
+    constexpr int kStage = stage_bytes<Tile<S, SRC, G::BX, G::BY>, TileTables<G::BX, G::BY, 2>, SRC>();
     static_assert(kStage + 256 <= 227 * 1024, "one tile stage must fit in shared memory");
     int s = G::STAGES;
     while (s > 1 && s * kStage + 256 > 227 * 1024) --s;
@@ -334,6 +341,9 @@ cudaError_t encode_typed(trtr_ctx* ctx) {
     ok = ok && encode(&ctx->maps[kMapD], tma_type<C>(), sizeof(C), ctx->Dh, ctx->lf, 1, kBX, kBY, 1);
     if (ctx->S) ok = ok && encode(&ctx->maps[kMapS], tma_type<C>(), sizeof(C), ctx->S, ctx->lf, 2, kBX, kBY, 1);
     else ctx->maps[kMapS] = ctx->maps[kMapD];
+    ctx->maps[kMapY] = ctx->maps[kMapS];
+    if (SRC == TRTR_SRC_PULSE)
+        ok = ok && encode_tables(&ctx->maps[kMapS], &ctx->maps[kMapY], ctx->ptab, PulseTab::make(ctx->p.nx, ctx->p.ny), kBX, kBY, 2);
     return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -346,7 +356,7 @@ cudaError_t launch_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, l
     using T = Tile<S, SRC, kBX, kBY>;
     constexpr int kStages = stages_for<S, SRC, G>();
     auto kernel = step_kernel<S, SRC, kStages, G, SR>;
-    const size_t smem = (size_t)kStages * T::STAGE + 128 + kStages * sizeof(uint64_t);
+    const size_t smem = (size_t)kStages * stage_bytes<T, TileTables<kBX, kBY, 2>, SRC>() + 128 + kStages * sizeof(uint64_t);
     static int configured_device = -1;
     static int ctas_per_sm = 1;
     if (configured_device != ctx->device) {
@@ -359,8 +369,8 @@ cudaError_t launch_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, l
     }
     StepArgs<C> a;
     a.dst = dst;
-    a.pt = PulseTab::make(ctx->p.nx, ctx->p.ny);
-    a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<C>(ctx, a.pt, step) : nullptr;
+    a.pulse = nullptr;
+    a.entry = SRC == TRTR_SRC_PULSE ? (int)(step - 1 - ctx->ptab_first) : 0;
     a.flag = ctx->dflag;
     a.tile_ctr = reinterpret_cast<unsigned*>(ctx->dflag + 2);
     a.lp = ctx->lp;
@@ -388,7 +398,7 @@ cudaError_t launch_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, l
     attr[0].val.programmaticStreamSerializationAllowed = TRTR_STEP_PDL && ntiles <= kPdlMaxTilesPerCta * grid;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, src_map, ctx->maps[kMapU], ctx->maps[kMapD], ctx->maps[kMapS], a);
+    return cudaLaunchKernelEx(&cfg, kernel, src_map, ctx->maps[kMapU], ctx->maps[kMapD], ctx->maps[kMapS], ctx->maps[kMapY], a);
 }
 
 template <typename S, int SRC>

@@ -36,17 +36,24 @@ namespace {
 
 using namespace core;
 
+template <int SRC, class T>
+constexpr int stage_bytes() {
+    return SRC == TRTR_SRC_PULSE ? T::StageTab : T::Stage;
+}
+
 template <typename S, int SRC, class G, bool P1, bool SR>
 __global__ void __launch_bounds__(G::kThreads, G::kCtas)
-    step2_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mf, const Step2Args args) {
+    step2_kernel(const __grid_constant__ CUtensorMap mp, const __grid_constant__ CUtensorMap mf,
+                 const __grid_constant__ CUtensorMap mtx, const __grid_constant__ CUtensorMap mty, const Step2Args args) {
     constexpr int STAGES = G::kStages, NT = G::kThreads;
     using T = typename G::T;
+    constexpr int kStage = stage_bytes<SRC, T>();
     const StepArgs<float>& a = args.a;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_abort;
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) &
                                                            ~static_cast<uintptr_t>(127));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * T::Stage);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * kStage);
 
     const int tid = threadIdx.x;
     const int nx = a.lp.nx, ny = a.lp.ny;
@@ -114,8 +121,10 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         const int2 o = take();
         s_org[s] = o;
         if (o.x >= 0) {
-            mbar_expect_tx(&full[s], T::TX);
-            step2_issue<T>(smem + s * T::Stage, &full[s], &mp, &mf, o.x, o.y, a.lp.gx, a.lf.gx);
+            mbar_expect_tx(&full[s], SRC == TRTR_SRC_PULSE ? T::TX + T::Tab::TX : T::TX);
+            step2_issue<T>(smem + s * kStage, &full[s], &mp, &mf, o.x, o.y, a.lp.gx, a.lf.gx);
+            if (SRC == TRTR_SRC_PULSE)
+                T::Tab::issue(smem + s * kStage + T::Stage, &full[s], &mtx, &mty, a.entry, o.x - 4, o.y - 2);
         }
     };
 
@@ -140,12 +149,13 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
         const int i0 = o.x, j0 = o.y;
         const bool ok = mbar_wait_bounded(&full[s], (k / STAGES) & 1);
         if (!ok) s_abort = 1;
-        S* sp = reinterpret_cast<S*>(smem + s * T::Stage);
-        const float* sf = reinterpret_cast<const float*>(smem + s * T::Stage + T::FldOff);
-        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, i0, j0, a, a.pulse, tid, a.rkey);
+        S* sp = reinterpret_cast<S*>(smem + s * kStage);
+        const float* sf = reinterpret_cast<const float*>(smem + s * kStage + T::FldOff);
+        const StagedSource<T> source{smem + s * kStage + T::Stage};
+        if (ok) step2_first<S, SRC, T, NT, SR>(sp, sf, i0, j0, a, source, tid, a.rkey);
         __syncthreads();  // P1 complete (and s_abort visible)
         if (ok && !s_abort)
-            step2_second<S, SRC, T, NT, P1, SR>(sp, sf, i0, j0, a, a.pulse + a.pt.level, tid,
+            step2_second<S, SRC, T, NT, P1, SR>(sp, sf, i0, j0, a, source, tid,
                                                  static_cast<S*>(args.dst1), args.rkey2);
         __syncthreads();  // stage s fully read
         if (s_abort) {
@@ -225,7 +235,7 @@ __global__ void refresh_ghosts2_kernel(E* P, PlaneLayout L) {
 template <typename S, int SRC, class G, bool P1, bool SR>
 cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, void* dst1, long step) {
     auto kernel = step2_kernel<S, SRC, G, P1, SR>;
-    const size_t smem = (size_t)G::kStages * G::T::Stage + 128 + G::kStages * sizeof(uint64_t);
+    const size_t smem = (size_t)G::kStages * stage_bytes<SRC, typename G::T>() + 128 + G::kStages * sizeof(uint64_t);
     static int configured_device = -1;
     static int ctas_per_sm = 1;
     if (configured_device != ctx->device) {
@@ -241,8 +251,7 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
     memset(static_cast<void*>(&args), 0, sizeof(args));
     a.dst = dst;
     args.dst1 = dst1;
-    a.pt = PulseTab::make(ctx->p.nx, ctx->p.ny);
-    a.pulse = SRC == TRTR_SRC_PULSE ? pulse_level<float>(ctx, a.pt, step) : nullptr;
+    a.entry = SRC == TRTR_SRC_PULSE ? (int)(step - 1 - ctx->ptab_first) : 0;
     a.flag = ctx->dflag;
     a.tile_ctr = reinterpret_cast<unsigned*>(ctx->dflag + 2);
     a.lp = ctx->lp;
@@ -267,7 +276,7 @@ cudaError_t launch2_typed(trtr_ctx* ctx, const CUtensorMap& src_map, void* dst, 
     attr[0].val.programmaticStreamSerializationAllowed = TRTR_STEP2_PDL && ntiles <= kPdlMaxTilesPerCta * grid;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, src_map, ctx->maps2[2], args);
+    return cudaLaunchKernelEx(&cfg, kernel, src_map, ctx->maps2[2], ctx->maps2[3], ctx->maps2[4], args);
 }
 
 }  // namespace
@@ -308,6 +317,9 @@ cudaError_t encode2_typed(trtr_ctx* ctx) {
     for (int b = 0; b < 2; ++b)
         ok = ok && encode(&ctx->maps2[b], tma_type<S>(), (int)sizeof(S), ctx->pop[b], ctx->lp, kQ, T::W, T::PR, kQ);
     ok = ok && encode(&ctx->maps2[2], tma_type<float>(), 4, ctx->fld2, ctx->lt, kT2NF, T::WF, T::FR, kT2NF);
+    if (ctx->p.src_mode == TRTR_SRC_PULSE)
+        ok = ok && encode_tables(&ctx->maps2[3], &ctx->maps2[4], ctx->ptab, PulseTab::make(ctx->p.nx, ctx->p.ny),
+                                 T::X + 8, T::Y + 4, 3);
     return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 

@@ -31,6 +31,9 @@ struct Tile2 {
     static constexpr int FldBytes = kT2NF * FldPlane * 4;
     static constexpr int TX = PopBytes + FldBytes;       // bytes per tile (boxes include any fill)
     static constexpr int Stage = (FldOff + FldBytes + 127) / 128 * 128;
+    // with the pulse source a stage ends with the tables of three levels, columns from i0 - 4 and rows from j0 - 2 on
+    using Tab = TileTables<BX + 8, BY + 4, 3>;
+    static constexpr int StageTab = Stage + Tab::Bytes;
     static_assert(ES == 4 || ES == 2, "FP32 or 2-byte populations");
     static_assert((BX * ES) % 16 == 0 && BX % 4 == 0, "tile origins on 16-byte boundaries");
     static_assert(W <= 256 && WF <= 256 && PR <= 256, "TMA box dimensions are at most 256");
@@ -40,7 +43,7 @@ template <int STAGES, int CTAS, int THREADS, int BX, int BY, int ES = 4>
 struct Geom2 {
     static constexpr int kStages = STAGES, kCtas = CTAS, kThreads = THREADS;
     using T = Tile2<BX, BY, ES>;
-    static_assert(STAGES * T::Stage + 256 <= 227 * 1024, "the stages must fit in shared memory");
+    static_assert(STAGES * T::StageTab + 256 <= 227 * 1024, "the stages must fit in shared memory");
 };
 // Geometry per source mode and population size (stages, CTAs per SM, threads, tile width, tile
 // height), from the sweeps of rebuilds with -DTRTR_STEP2_STAGES=S -DTRTR_STEP2_CTAS=C
@@ -94,7 +97,7 @@ using Geom2Of = typename Geom2For<SRC, ES>::type;
 #endif
 
 struct alignas(16) Step2Args {
-    StepArgs<float> a;  // pulse, rkey: the pulse tables and rounding key of the first step
+    StepArgs<float> a;  // rkey: the rounding key of the first step
     void* dst1;             // if not null: also store the first step's state here (one-wide ghosts)
     uint32_t rkey2;         // the second step's rounding key (stochastic rounding of 2-byte storages)
 };
@@ -161,13 +164,30 @@ __device__ __forceinline__ typename Pair<S>::type encode2(F2 v, uint32_t rk, int
         return Pair<S>::encode_raw(v);
 }
 
+// Source terms from a stage's tables: the pair at column i0 + c, row j0 + r in the tile's step 0 or 1.
+template <class T>
+struct StagedSource {
+    const unsigned char* tables;
+    __device__ __forceinline__ F2 operator()(int step, int c, int r, int, int) const {
+        return T::Tab::source(tables, step, c + 4, r + 2);
+    }
+};
+// The same from the tables in global memory (a batch, whose instances' tables are its tiles' to look up).
+struct TableSource {
+    const float* lev;
+    const PulseTab* t;
+    __device__ __forceinline__ F2 operator()(int step, int, int, int i, int j) const {
+        return pulse_source_dt(lev + step * t->level, *t, i, j);
+    }
+};
+
 // Step 1 over the tile's halo region R1, in place in the stage (thread tid of NT).  2-byte
 // storages: the step-1 values are rounded to the storage format with the first step's key rkey1, as
 // a one-step launch stores them (halo nodes with the key of the wrapped node; nx is even, so
 // the wrapped pairs are the one-step kernel's pairs).
-template <typename S, int SRC, class T, int NT, bool SR = false>
+template <typename S, int SRC, class T, int NT, bool SR = false, class Source>
 __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int j0, const StepArgs<float>& a,
-                                            const float* pulse, int tid, uint32_t rkey1 = 0u) {
+                                            const Source& source, int tid, uint32_t rkey1 = 0u) {
     constexpr int kT2W = T::W, kT2WF = T::WF, kT2PopPlane = T::PopPlane, kT2FldPlane = T::FldPlane;
     constexpr bool kOfs = sizeof(S) == 2;  // offsets folded into the moments, as in the one-step kernel
     constexpr int kC = T::HX - 2;          // stage column of R1 column 0
@@ -203,7 +223,7 @@ __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int 
         const F2 Dh = ld2(f + 4 * kT2FldPlane, fa);
         const int x = i0 - 2 + c, y = j0 - 1 + r;
         F2 src(0.f);  // halo nodes: the tables' periodic images
-        if (SRC == TRTR_SRC_PULSE) src = pulse_source_dt(pulse, a.pt, x, y);
+        if (SRC == TRTR_SRC_PULSE) src = source(0, c - 2, r - 1, x, y);
         F2 out[kQ];
         collide_node<F2, kOfs>(g, ux, uy, ax, ay, Dh, src, magic, w2f, a.tau2_fixed, out, F2(a.phi_ref));
         const uint32_t rk = SR ? sr_pair_key(wrap_clamp(x, nx), wrap_clamp(y, ny), nx, rkey1) : 0u;
@@ -218,9 +238,9 @@ __device__ __forceinline__ void step2_first(S* sp, const float* sf, int i0, int 
 // Step 2 on the tile's output nodes from the step-1 values in the stage, stored to a.dst with
 // the ghost copies of nodes within two of an edge.  P1: the step-1 state of the output nodes is
 // stored to dst1 too, with the one-wide ghost frame that one-step kernels read.
-template <typename S, int SRC, class T, int NT, bool P1 = false, bool SR = false>
+template <typename S, int SRC, class T, int NT, bool P1 = false, bool SR = false, class Source>
 __device__ __forceinline__ void step2_second(const S* sp, const float* sf, int i0, int j0,
-                                             const StepArgs<float>& a, const float* pulse, int tid,
+                                             const StepArgs<float>& a, const Source& source, int tid,
                                              S* dst1 = nullptr, uint32_t rkey2 = 0u) {
     constexpr int kT2X = T::X, kT2W = T::W, kT2WF = T::WF, kT2R2 = T::R2, kT2PopPlane = T::PopPlane,
                   kT2FldPlane = T::FldPlane;
@@ -263,7 +283,7 @@ __device__ __forceinline__ void step2_second(const S* sp, const float* sf, int i
         const F2 ay(*reinterpret_cast<const float2*>(f + 3 * kT2FldPlane));
         const F2 Dh(*reinterpret_cast<const float2*>(f + 4 * kT2FldPlane));
         F2 src(0.f);
-        if (SRC == TRTR_SRC_PULSE) src = pulse_source_dt(pulse, a.pt, i, j);
+        if (SRC == TRTR_SRC_PULSE) src = source(1, c2, r2, i, j);
         F2 out[kQ];
         collide_node<F2, kOfs>(g, ux, uy, ax, ay, Dh, src, magic, w2f, a.tau2_fixed, out, F2(a.phi_ref));
         const uint32_t rk = SR ? sr_pair_key(i, j, nx, rkey2) : 0u;

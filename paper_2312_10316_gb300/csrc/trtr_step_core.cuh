@@ -238,11 +238,12 @@ __device__ __forceinline__ F2 vdiv(F2 a, F2 b) { return F2(__fdividef(a.v.x, b.v
 // s = dt S^n + dt/2 (S^n - S^{n-1}) = 1.5 dt S^n - 0.5 dt S^{n-1} (a7, Eqs. (3) and (14)) of the
 // manufactured source at the node pair (i, i + 1) (i even, images included) or the node i of row
 // j, from the tables of the levels n - 1 and n (`lev`: level n - 1).
+__device__ __forceinline__ F2 pulse_level_dt(F2 p1, F2 p2, float2 q) { return vfma(p1, F2(q.x), p2 * F2(q.y)); }
 __device__ __forceinline__ F2 pulse_source_dt(const float* lev, const PulseTab& t, int i, int j) {
     auto level = [&](const float* p) {
         const float2 q = __ldg(reinterpret_cast<const float2*>(p + t.y + 2 * j));
         const F2 p1(__ldg(reinterpret_cast<const float2*>(p + i))), p2(__ldg(reinterpret_cast<const float2*>(p + t.p2 + i)));
-        return vfma(p1, F2(q.x), p2 * F2(q.y));
+        return pulse_level_dt(p1, p2, q);
     };
     return vfma(F2(1.5f), level(lev + t.level), F2(-0.5f) * level(lev));
 }
@@ -253,6 +254,36 @@ __device__ __forceinline__ double pulse_source_dt(const double* lev, const Pulse
     };
     return fma(1.5, level(lev + t.level), -0.5 * level(lev));
 }
+
+// The pulse tables of a tile of BX columns and BY rows in its stage: a box of LEVELS levels of P1 and P2 and, on
+// the next 128-byte boundary, one of (Q1, Q2), loaded with the tile's populations.  Read from global
+// memory by the lanes, the six loads a pair came behind the TMA loads of the tile and waited for L2, a level's
+// entries being new to every launch (GB300, us a step, by the lanes / with the boxes; one step a launch: FP32 400^2
+// 6.79 / 6.50, 16 x 8000 27.8 / 24.4, FP16 16 x 8000 20.6 / 18.1; two: FP32 400^2 4.75 / 4.57, 20000 x 32 9.50 / 8.88,
+// FP16 2048^2 43.8 / 41.5).
+template <int BX, int BY, int LEVELS>
+struct TileTables {
+    static constexpr int YOff = (LEVELS * 2 * BX * 4 + 127) / 128 * 128;
+    static constexpr int TX = LEVELS * 2 * (BX + BY) * 4, Bytes = (YOff + LEVELS * 2 * BY * 4 + 127) / 128 * 128;
+    static_assert(BX % 4 == 0 && BY % 2 == 0, "boxes on 16-byte boundaries");
+    // columns from i0, rows from j0; entry: of the first level in the tables
+    static __device__ __forceinline__ void issue(unsigned char* at, uint64_t* bar, const CUtensorMap* mx,
+                                                 const CUtensorMap* my, int entry, int i0, int j0) {
+        const int x = kTabGhost + i0, y = 2 * (kTabGhost + j0);
+        if (tma_ok(at, x, entry, 4)) tma_load_3d(at, mx, bar, x, 0, entry);
+        if (tma_ok(at + YOff, y, entry, 4)) tma_load_2d(at + YOff, my, bar, y, entry);
+    }
+    // the source term of the pair at column i0 + c, row j0 + r from the levels l and l + 1, as pulse_source_dt
+    static __device__ __forceinline__ F2 source(const unsigned char* at, int l, int c, int r) {
+        auto level = [&](int k) {
+            const float* x = reinterpret_cast<const float*>(at) + 2 * BX * k + c;
+            const float* y = reinterpret_cast<const float*>(at + YOff) + 2 * BY * k + 2 * r;
+            return pulse_level_dt(F2(*reinterpret_cast<const float2*>(x)), F2(*reinterpret_cast<const float2*>(x + BX)),
+                                  *reinterpret_cast<const float2*>(y));
+        };
+        return vfma(F2(1.5f), level(l + 1), F2(-0.5f) * level(l));
+    }
+};
 
 // The E(r) factor of the pulse tables from its exponent -r^2 / (2 s^2): FP64 as it is; FP32 with the
 // exponent split into an integer and a fraction in FP64, so that a large exponent costs no digits.
@@ -523,9 +554,9 @@ struct Pair<__nv_bfloat16> {
 template <typename S, int SRC, int BX, int BY>
 __device__ __forceinline__ void issue_tile(unsigned char* stage, uint64_t* bar, const CUtensorMap* mp,
                                            const CUtensorMap* mu, const CUtensorMap* md, const CUtensorMap* ms,
-                                           int i0, int j0, const StepArgs<typename Store<S>::C>& a) {
+                                           int i0, int j0, const StepArgs<typename Store<S>::C>& a, uint32_t more = 0) {
     using T = Tile<S, SRC, BX, BY>;
-    mbar_expect_tx(bar, T::TX);
+    mbar_expect_tx(bar, T::TX + more);
     constexpr int kPe = (int)sizeof(S), kFe = (int)sizeof(typename Store<S>::C);
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
@@ -735,7 +766,24 @@ inline bool encode(CUtensorMap* m, CUtensorMapDataType t, int elem, void* base, 
               kPromotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The same with bounds at the interior (coordinate 0 is node 0): loads outside it read zero, stores
+// The pulse tables as boxes of `levels` levels: `bx` columns of P1 and P2 (x), `by` rows of (Q1, Q2) (y).
+inline bool encode_tables(CUtensorMap* x, CUtensorMap* y, void* tab, const PulseTab& t, int bx, int by, int levels) {
+    auto fn = get_encoder();
+    if (!fn) return false;
+    const cuuint64_t xd[3] = {(cuuint64_t)t.p2, 2, (cuuint64_t)kPulseLevels};
+    const cuuint64_t xs[2] = {(cuuint64_t)t.p2 * 4, (cuuint64_t)t.level * 4};
+    const cuuint64_t yd[2] = {(cuuint64_t)(t.level - 2 * t.p2), (cuuint64_t)kPulseLevels};
+    const cuuint64_t ys[1] = {(cuuint64_t)t.level * 4};
+    const cuuint32_t xb[3] = {(cuuint32_t)bx, 2, (cuuint32_t)levels}, yb[2] = {(cuuint32_t)(2 * by), (cuuint32_t)levels};
+    const cuuint32_t es[3] = {1, 1, 1};
+    const auto f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    return fn(x, f32, 3, tab, xd, xs, xb, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, kPromotion,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
+           fn(y, f32, 2, static_cast<float*>(tab) + 2 * t.p2, yd, ys, yb, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, kPromotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// As encode, with bounds at the interior (coordinate 0 is node 0): loads outside it read zero, stores
 // write nothing there.
 inline bool encode_interior(CUtensorMap* m, CUtensorMapDataType t, int elem, void* base, const PlaneLayout& L, int depth,
                             int bw, int bh, int bd) {
