@@ -342,8 +342,8 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
         {&ctx->uv, 2 * fld_bytes, true},
         {&ctx->Dh, fld_bytes, true},
         {&ctx->S, p->src_mode == TRTR_SRC_FIELD ? 2 * fld_bytes : 0, true},
-        {&ctx->tab_x, 2 * (size_t)p->nx * ctx->csize, true},
-        {&ctx->tab_y, 2 * (size_t)p->ny * ctx->csize, true},
+        {&ctx->tab_x, 4 * (size_t)p->nx * ctx->csize, true},
+        {&ctx->tab_y, 4 * (size_t)p->ny * ctx->csize, true},
         {&ctx->ptab,
          p->src_mode == TRTR_SRC_PULSE
              ? trtr::PulseTab::make(p->nx, p->ny).values(trtr::kPulseLevels) * ctx->csize

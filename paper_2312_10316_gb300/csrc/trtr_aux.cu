@@ -87,14 +87,14 @@ __global__ void pulse_fields_kernel(C* uv, C* Dh, C* tab_x, C* tab_y, PlaneLayou
         if (i < 0 || i >= L.nx || j < 0 || j >= L.ny) continue;
         const double x = x0 + i * dx, y = y0 + j * dx;
         Dh[L.at(i, j)] = C(use_const ? dh_const : pp.D0 * (1.0 + pp.D_amp * sin(M_PI * x) * sin(M_PI * y)) * ds);
-        if (j == 0) {
-            tab_x[i] = C(sin(M_PI * x));
-            tab_x[L.nx + i] = C(cos(M_PI * x));
-        }
-        if (i == 0) {
-            tab_y[j] = C(sin(M_PI * y));
-            tab_y[L.ny + j] = C(cos(M_PI * y));
-        }
+        auto axis = [](C* tab, int n, int at, double v) {
+            tab[at] = C(sin(M_PI * v));
+            tab[n + at] = C(cos(M_PI * v));
+            tab[2 * n + at] = C(v);
+            tab[3 * n + at] = C(v - (double)C(v));
+        };
+        if (j == 0) axis(tab_x, L.nx, i, x);
+        if (i == 0) axis(tab_y, L.ny, j, y);
     }
 }
 

@@ -76,9 +76,9 @@ constexpr int schedule_mode(int schedule) { return schedule == 0 ? 1 : (schedule
 
 // Pulse tables of every instance (blockIdx.y) from time level `first` on.
 __global__ void __launch_bounds__(256) batch_pulse_tables_kernel(const InstanceFill* fills, BatchClock* clk, long long first) {
-    __shared__ PulseTime levels[kPulseLevels];
+    __shared__ PulseLevel<float> levels[kPulseLevels];
     const InstanceFill& f = fills[blockIdx.y];
-    if (threadIdx.x < kPulseLevels) levels[threadIdx.x] = pulse_at(f.pulse, (double)(first + threadIdx.x) * f.dt);
+    if (threadIdx.x < kPulseLevels) levels[threadIdx.x].set(pulse_at(f.pulse, (double)(first + threadIdx.x) * f.dt), f.fill.amp);
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) clk->first = first;
     __syncthreads();
     fill_pulse_tables<float>(f.fill, levels, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);

@@ -21,7 +21,7 @@
 //   packed       [5 or 6][rows][pitch] FP32: u, a = (u . grad) u, Dh and, with a source field, the
 //                source term, for the kernels that take several steps; FP64: [4][rows][pitch]
 //                a, k1, k2 (pack64)
-//   pulse tab    [2][nx] sin(pi x_i), cos(pi x_i) and [2][ny] sin(pi y_j), cos(pi y_j); and the
+//   pulse tab    [4][nx] sin(pi x_i), cos(pi x_i), x_i (two floats) and [4][ny] of y_j; and the
 //                separable factors of the pulse source at kPulseLevels time levels (PulseTab)
 //   edge values  [2 nx + 2 (ny - 2)] FP64 Dirichlet values of the edge nodes
 //                (TRTR_BC_DIRICHLET_NEE), in the order of edge_node()
@@ -309,7 +309,7 @@ struct SweepBatch {
 // What the table fill needs of a context or of a batch's instance.
 struct PulseFill {
     void* tab;                       // [kPulseLevels][level]
-    const void *tab_x, *tab_y;       // sin and cos of pi x, pi y in the compute type
+    const void *tab_x, *tab_y;       // of the axes (trtr_ctx::tab_x)
     double x0, y0, dx, amp;          // amp: dt D0 D_amp
     int nx, ny;
 };
@@ -335,7 +335,7 @@ struct trtr_ctx {
     void* S;          // [2][rows][pitch] (TRTR_SRC_FIELD)
     int S_cur;        // buffer holding S^n (-1: none set)
     int S_prev;       // buffer holding S^{n-1} (-1: use S^n)
-    void* tab_x;
+    void* tab_x;      // [4][nx] sin and cos of pi x in the compute type; FP32: x as the sum of two floats
     void* tab_y;
     void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
     // what they hold, whoever filled them last (the context or its batch), if ptab_ready

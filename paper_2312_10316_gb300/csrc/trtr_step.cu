@@ -471,24 +471,38 @@ cudaError_t encode_maps(trtr_ctx* ctx) {
     }
 }
 
+// One entry a thread, computed while the launches before still run: their tables are written over when they have
+// completed.
 template <typename C>
-__global__ void pulse_tables_kernel(const PulseFill fill, const __grid_constant__ PulseLevels levels) {
-    fill_pulse_tables<C>(fill, levels.t, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+__global__ void pulse_tables_kernel(const PulseFill fill, const __grid_constant__ PulseLevels<C> levels) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    auto wait = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
+    const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < table_entries(fill.nx, fill.ny))
+        fill_pulse_entry<C>(fill, levels.t, k, wait);
+    else
+        wait();
+}
+template <typename C>
+cudaError_t launch_pulse_tables(trtr_ctx* ctx, long first) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((table_entries(ctx->p.nx, ctx->p.ny) + 127) / 128);
+    cfg.blockDim = dim3(128);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, pulse_tables_kernel<C>, pulse_fill_of(ctx), pulse_levels_of<C>(ctx, first));
 }
 
 cudaError_t ensure_pulse_levels(trtr_ctx* ctx, long step, int steps) {
     if (ctx->p.src_mode != TRTR_SRC_PULSE) return cudaSuccess;
     if (ctx->ptab_ready && ctx->ptab_pulse == ctx->pulse && levels_within(ctx->ptab_first, step, steps)) return cudaSuccess;
-    const long entries = (long)kPulseLevels * (ctx->p.nx + ctx->p.ny + 4 * kTabGhost);
-    const long want = (entries + 255) / 256, cap = (long)ctx->num_sms * 8;
-    const unsigned grid = (unsigned)(want < cap ? want : cap);
     ctx->ptab_ready = false;
     ctx->launches += 1;
-    if (ctx->csize == 8)
-        pulse_tables_kernel<double><<<grid, 256, 0, ctx->stream>>>(pulse_fill_of(ctx), pulse_levels_of(ctx, step - 1));
-    else
-        pulse_tables_kernel<float><<<grid, 256, 0, ctx->stream>>>(pulse_fill_of(ctx), pulse_levels_of(ctx, step - 1));
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = ctx->csize == 8 ? launch_pulse_tables<double>(ctx, step - 1) : launch_pulse_tables<float>(ctx, step - 1);
     tables_filled(ctx, ctx->pulse, step - 1, e);
     ctx->tables_new = true;
     return e;

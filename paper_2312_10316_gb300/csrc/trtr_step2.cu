@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(G::kThreads, G::kCtas)
 // differences 0.5 (u(+1) - u(-1)).
 // Fills the pulse tables too (fill.tab not null).
 __global__ void pack_fields2_kernel(float* f2, const float* uv, const float* Dh, PlaneLayout lt, PlaneLayout lf,
-                                    const PulseFill fill, const __grid_constant__ PulseLevels levels) {
+                                    const PulseFill fill, const __grid_constant__ PulseLevels<float> levels) {
     if (fill.tab) fill_pulse_tables<float>(fill, levels.t, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
     const int gw = lt.nx + 2 * kGhostT, gh = lt.ny + 2 * kGhostT;
     const size_t n = (size_t)gw * gh;
@@ -355,10 +355,10 @@ static cudaError_t pack_into(trtr_ctx* ctx, void* dst, bool tables) {
     const size_t want = (n + 255) / 256, cap = (size_t)ctx->num_sms * 8;
     ctx->launches += 1;
     ctx->tables_new = true;
-    PulseLevels levels = {};
+    PulseLevels<float> levels = {};
     PulseFill fill = pulse_fill_of(ctx);
     if (tables)
-        levels = pulse_levels_of(ctx, ctx->step - 1);
+        levels = pulse_levels_of<float>(ctx, ctx->step - 1);
     else
         fill.tab = nullptr;
     pack_fields2_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, ctx->stream>>>(

@@ -285,55 +285,103 @@ struct TileTables {
     }
 };
 
-// The E(r) factor of the pulse tables from its exponent -r^2 / (2 s^2): FP64 as it is; FP32 with the
-// exponent split into an integer and a fraction in FP64, so that a large exponent costs no digits.
-__device__ __forceinline__ double pulse_exp(double z, double) { return exp(z); }
-__device__ __forceinline__ float pulse_exp(double z, float) {
-    const double a = z * 1.4426950408889634074;  // log2(e)
-    const double n = rint(a);
-    return n < -160.0 ? 0.f : scalbnf(exp2f((float)(a - n)), (int)n);
+// The table fill.  FP64 takes r = x - c, z = r^2 / s^2 and exp(-z / 2) as they stand.  FP32 carries r, r^2, z and
+// the exponent as unevaluated sums of two floats (exact products and sums: 45 bits and more), so that neither
+// r near the pulse nor a large exponent costs digits, with no instruction of the FP64 pipe: in FP64, 14 of them an
+// entry (16 cycles a warp each) made a fill of 20000 + 32 coordinates 39 us (GB300), now 12.5.
+template <typename C>
+struct PulseLevel;  // the pulse at one time level
+template <>
+struct PulseLevel<double> {
+    double cx, cy, inv_s2, A;  // A: dt D0 D_amp s0^2 / s^4
+    __host__ __device__ void set(const PulseTime& t, double amp) {
+        cx = t.cx;
+        cy = t.cy;
+        inv_s2 = t.inv_s2;
+        A = amp * t.amp * t.inv_s2;
+    }
+};
+template <>
+struct PulseLevel<float> {
+    float2 cx, cy, inv_s2, e;  // (value, remainder); e: -log2(e) / (2 s^2)
+    float A;
+    static __host__ __device__ float2 split(double v) {
+        float2 r;
+        r.x = (float)v;
+        r.y = (float)(v - (double)r.x);
+        return r;
+    }
+    __host__ __device__ void set(const PulseTime& t, double amp) {
+        cx = split(t.cx);
+        cy = split(t.cy);
+        inv_s2 = split(t.inv_s2);
+        e = split(-0.5 * 1.4426950408889634074 * t.inv_s2);
+        A = (float)(amp * t.amp * t.inv_s2);
+    }
+};
+
+// (E sin, E [pi cos r + sin (1 - z)]) of coordinate w of the n along an axis at a level of centre c.
+__device__ __forceinline__ double2 pulse_factors(const double* tab, int n, int w, double x0, double dx, double c,
+                                                 const PulseLevel<double>& l) {
+    const double sn = tab[w], cs = tab[n + w], r = x0 + w * dx - c, z = r * r * l.inv_s2, E = exp(-0.5 * z);
+    return make_double2(E * sn, E * (3.14159265358979323846 * cs * r + sn * (1.0 - z)));
+}
+__device__ __forceinline__ float2 pulse_factors(const float* tab, int n, int w, double, double, float2 c,
+                                                const PulseLevel<float>& l) {
+    const float sn = tab[w], cs = tab[n + w], xh = tab[2 * n + w], xl = tab[3 * n + w];
+    const float s = xh - c.x, b = s - xh;
+    const float t = ((xh - (s - b)) - (c.x + b)) + (xl - c.y);
+    const float rh = s + t, rl = t - (rh - s);  // r
+    const float p = rh * rh, pe = fmaf(2.f * rh, rl, fmaf(rh, rh, -p));  // r^2
+    const float a = p * l.e.x, ae = fmaf(p, l.e.x, -a) + fmaf(p, l.e.y, pe * l.e.x);
+    const float k = rintf(a);
+    const float E = k < -160.f ? 0.f : scalbnf(exp2f((a - k) + ae), (int)k);
+    const float z = p * l.inv_s2.x, ze = fmaf(p, l.inv_s2.x, -z) + fmaf(p, l.inv_s2.y, pe * l.inv_s2.x);
+    if (E == 0.f) return make_float2(0.f, 0.f);
+    return make_float2(E * sn, E * (3.14159265358979323846f * cs * rh + sn * ((1.f - z) - ze)));
 }
 
-// Entries k, k + stride, ... of the tables: one coordinate of one level each (levels[l]: the pulse
-// at level l of the table), coordinates outside the grid as their periodic images.
-template <typename C>
-__device__ __forceinline__ void fill_pulse_tables(const PulseFill& f, const PulseTime* levels, unsigned k,
-                                                  unsigned stride) {
+// Entry k of the tables, one coordinate of one level (levels[l]: of level l), coordinates outside the grid as
+// their periodic images; `ready`: called before the stores.
+constexpr unsigned table_entries(int nx, int ny) { return (unsigned)(nx + ny + 4 * kTabGhost) * kPulseLevels; }
+template <typename C, class Ready>
+__device__ __forceinline__ void fill_pulse_entry(const PulseFill& f, const PulseLevel<C>* levels, unsigned k, Ready&& ready) {
     const PulseTab t = PulseTab::make(f.nx, f.ny);
     const unsigned gx = f.nx + 2 * kTabGhost, per = gx + f.ny + 2 * kTabGhost;
-    const C pi = C(3.14159265358979323846);
-    for (const unsigned total = per * kPulseLevels; k < total; k += stride) {
-        const unsigned lev = k / per, e = k - lev * per;
-        const bool along_x = e < gx;
-        const int n = along_x ? f.nx : f.ny, at = (int)(along_x ? e : e - gx) - kTabGhost;
-        int w = at % n;
-        w = w < 0 ? w + n : w;
-        const PulseTime pt = levels[lev];
-        const C* tab = static_cast<const C*>(along_x ? f.tab_x : f.tab_y);
-        const C sn = tab[w], cs = tab[n + w];
-        const double r = along_x ? f.x0 + w * f.dx - pt.cx : f.y0 + w * f.dx - pt.cy;
-        const double z = r * r * pt.inv_s2;
-        const C E = pulse_exp(-0.5 * z, C(0));
-        const C slope = E * (pi * cs * C(r) + sn * C(1.0 - z)), value = E * sn;
-        C* out = static_cast<C*>(f.tab) + kTabGhost + (size_t)lev * t.level;
-        if (along_x) {
-            out[at] = slope;
-            out[t.p2 + at] = value;
-        } else {
-            const C A = C(f.amp * pt.amp * pt.inv_s2);
-            out[t.y + 2 * at] = A * value;
-            out[t.y + 2 * at + 1] = A * slope;
-        }
+    const unsigned lev = k / per, e = k - lev * per;
+    const bool along_x = e < gx;
+    const int n = along_x ? f.nx : f.ny, at = (int)(along_x ? e : e - gx) - kTabGhost;
+    int w = at % n;
+    w = w < 0 ? w + n : w;
+    const PulseLevel<C>& l = levels[lev];
+    const auto v = pulse_factors(static_cast<const C*>(along_x ? f.tab_x : f.tab_y), n, w, along_x ? f.x0 : f.y0, f.dx,
+                                 along_x ? l.cx : l.cy, l);
+    C* out = static_cast<C*>(f.tab) + kTabGhost + (size_t)lev * t.level;
+    ready();
+    if (along_x) {
+        out[at] = v.y;
+        out[t.p2 + at] = v.x;
+    } else {
+        out[t.y + 2 * at] = l.A * v.x;
+        out[t.y + 2 * at + 1] = l.A * v.y;
     }
+}
+// Entries k, k + stride, ...
+template <typename C>
+__device__ __forceinline__ void fill_pulse_tables(const PulseFill& f, const PulseLevel<C>* levels, unsigned k, unsigned stride) {
+    for (const unsigned total = table_entries(f.nx, f.ny); k < total; k += stride) fill_pulse_entry(f, levels, k, [] {});
 }
 
 // The pulse at the time levels of one fill of the tables, computed on the host.
+template <typename C>
 struct PulseLevels {
-    PulseTime t[kPulseLevels];
+    PulseLevel<C> t[kPulseLevels];
 };
-inline PulseLevels pulse_levels_of(const trtr_ctx* ctx, long first) {
-    PulseLevels l;
-    for (int k = 0; k < kPulseLevels; ++k) l.t[k] = pulse_at(ctx->pulse, (double)(first + k) * ctx->p.dt);
+template <typename C>
+inline PulseLevels<C> pulse_levels_of(const trtr_ctx* ctx, long first) {
+    PulseLevels<C> l;
+    const double amp = ctx->p.dt * ctx->pulse.D0 * ctx->pulse.D_amp;
+    for (int k = 0; k < kPulseLevels; ++k) l.t[k].set(pulse_at(ctx->pulse, (double)(first + k) * ctx->p.dt), amp);
     return l;
 }
 
