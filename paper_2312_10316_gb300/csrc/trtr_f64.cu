@@ -77,8 +77,10 @@ __global__ void __launch_bounds__(128) f64_step_kernel(const __grid_constant__ F
     const unsigned nx = a.lp.nx, ny = a.lp.ny;
     const bool in = k < nx * ny;
     const unsigned j = k / nx, i = k - j * nx;
-    // what earlier steps do not write is loaded while they may still run (programmatic dependent launch)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // What earlier steps do not write is loaded while they may still run (programmatic dependent launch).  The next
+    // launch may come from the wait on: let in at the start, several launches' blocks waited side by side and a
+    // launch's own blocks went to the SMs that had room, a few of the 152 (us a step: 16 x 2000 20.9, now 6.7;
+    // 1000 x 33 21.2, now 6.5; 130^2 8.2, now 4.6; 64^2 4.4, now 4.2).
     double ux = 0, uy = 0, ax = 0, ay = 0, k1 = 0, k2 = 0, s = 0;
     if (in) {
         const size_t o = a.lf.at_g<kGhostF>(i, j), pl = a.lf.plane;
@@ -91,6 +93,7 @@ __global__ void __launch_bounds__(128) f64_step_kernel(const __grid_constant__ F
         if (SRC == TRTR_SRC_PULSE) s = pulse_source_dt(a.pulse, a.pt, i, j);
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!in) return;
     double g[kQ], out[kQ];
     const size_t at = a.lp.at_g<kGhostP>(i, j);
