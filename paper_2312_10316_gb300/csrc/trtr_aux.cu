@@ -136,39 +136,49 @@ __device__ __forceinline__ bool inner_node(const PlaneLayout& L, int i, int j) {
     return i > L.gy && i < L.nx - 1 - L.gy && j > L.gy && j < L.ny - 1 - L.gy;
 }
 
-// Initial condition g_i(x) = g_i^eq(phi0(x), u(x)) in the pull layout: node x evaluates phi0
-// once (FP64) and its nine equilibria in the compute type, and stores g_i(x) where x pulls it,
-// P_i(x - e_i), periodic images included (each slot has exactly one writer).  A thread takes `rows`
-// rows of one column; the pulse's phi0 is the product of a factor of x, taken once a thread, and one
-// of y, taken once a block and row: an FP64 exponential a node is 45 FP64 instructions and made this
-// kernel 0.9 ms at 4096^2.
-constexpr int kInitRows = 32;
+// Initial condition g_i(x) = g_i^eq(phi0(x), u(x)) in the pull layout: node x takes its nine equilibria in
+// the compute type and stores g_i(x) where x pulls it, P_i(x - e_i), periodic images included (each slot
+// has exactly one writer).
 template <typename S, typename C>
-__global__ void __launch_bounds__(128)
-    init_eq_kernel(S* P, const C* uv, const double* phi0, PlaneLayout lp, PlaneLayout lf, double x0, double y0, double dx,
-                   PulseTime pt, C phi_ref, int rows) {
-    __shared__ double fy[kInitRows];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j0 = blockIdx.y * rows;
-    double fx = 0.0;
-    if (!phi0) {
-        const double rx = x0 + i * dx - pt.cx;
-        fx = pt.amp * exp(-0.5 * rx * rx * pt.inv_s2);
-        if (threadIdx.x < (unsigned)rows) {
-            const double ry = y0 + (j0 + (int)threadIdx.x) * dx - pt.cy;
-            fy[threadIdx.x] = exp(-0.5 * ry * ry * pt.inv_s2);
-        }
-        __syncthreads();
-    }
-    if (i >= lp.nx) return;
-    for (int r = 0; r < rows && j0 + r < lp.ny; ++r) {
-        const int j = j0 + r;
-        const C phi = (C)(phi0 ? phi0[(size_t)j * lp.nx + i] : fx * fy[r]);
-        const C u = uv[lf.at(i, j)], v = uv[lf.plane + lf.at(i, j)];
-        const bool inner = inner_node(lp, i, j);
+__device__ __forceinline__ void init_node(S* P, const C* uv, const PlaneLayout& lp, const PlaneLayout& lf, int i, int j, C phi,
+                                          C phi_ref) {
+    const C u = uv[lf.at(i, j)], v = uv[lf.plane + lf.at(i, j)];
+    const bool inner = inner_node(lp, i, j);
 #pragma unroll
-        for (int q = 0; q < kQ; ++q)
-            store_pulled(P, lp, q, i, j, inner, Store<S>::encode(equilibrium<C>(q, phi, u, v), weight<C>(q) * phi_ref));
+    for (int q = 0; q < kQ; ++q)
+        store_pulled(P, lp, q, i, j, inner, Store<S>::encode(equilibrium<C>(q, phi, u, v), weight<C>(q) * phi_ref));
+}
+
+// From the caller's phi0: a node a thread (GB300, us, with 26 rows of a column a thread / now: FP32 2048^2
+// 104 / 77, 40 x 4000 16.6 / 10.4).
+template <typename S, typename C>
+__global__ void __launch_bounds__(kThreads)
+    init_eq_kernel(S* P, const C* uv, const double* phi0, PlaneLayout lp, PlaneLayout lf, C phi_ref) {
+    const unsigned n = (unsigned)lp.nx * lp.ny;
+    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        const int j = (int)(k / lp.nx), i = (int)(k - (unsigned)j * lp.nx);
+        init_node<S, C>(P, uv, lp, lf, i, j, (C)phi0[k], phi_ref);
     }
+}
+
+// The pulse at t = 0, the product of a factor of x and one of y, each taken once a block (w columns, `rows` rows):
+// an FP64 exponential a node is 45 FP64 instructions and made this kernel 0.9 ms at 4096^2.
+constexpr int kInitRows = 32, kInitThreads = 128;
+template <typename S, typename C>
+__global__ void __launch_bounds__(kInitThreads)
+    init_pulse_kernel(S* P, const C* uv, PlaneLayout lp, PlaneLayout lf, double x0, double y0, double dx, PulseTime pt,
+                      C phi_ref, int log_w, int rows) {
+    __shared__ double f[kInitThreads + kInitRows];
+    const int w = 1 << log_w, tid = threadIdx.x, i0 = blockIdx.x << log_w, j0 = blockIdx.y * rows;
+    for (int t = tid; t < w + rows; t += kInitThreads) {
+        const double r = t < w ? x0 + (i0 + t) * dx - pt.cx : y0 + (j0 + t - w) * dx - pt.cy;
+        f[t] = (t < w ? pt.amp : 1.0) * exp(-0.5 * r * r * pt.inv_s2);
+    }
+    __syncthreads();
+    const int c = tid & (w - 1), i = i0 + c;
+    if (i >= lp.nx) return;
+    for (int r = tid >> log_w; r < rows && j0 + r < lp.ny; r += kInitThreads >> log_w)
+        init_node<S, C>(P, uv, lp, lf, i, j0 + r, (C)(f[c] * f[w + r]), phi_ref);
 }
 
 // Dirichlet boundary by non-equilibrium extrapolation (Sec. 3) over the buffer P that a step
@@ -576,18 +586,29 @@ cudaError_t launch_convert_source(trtr_ctx* ctx, const double* S, int buffer) {
 }
 
 cudaError_t launch_init_equilibrium(trtr_ctx* ctx, const double* phi0) {
-    // rows a thread: as many as leave eight blocks an SM
-    const int columns = (ctx->p.nx + 127) / 128;
-    const long share = (long)ctx->p.ny * columns / (8L * ctx->num_sms);
-    const int rows = share < 1 ? 1 : (share > kInitRows ? kInitRows : (int)share);
-    const PulseTime pt = pulse_at(ctx->pulse, 0.0);
     ctx->launches += 1;
+    const int nx = ctx->p.nx, ny = ctx->p.ny;
+    // the pulse: columns of a block, fewer where the last block of a row would leave more than a tenth of them
+    // empty (GB300, us, 128 columns always / now: FP32 16 x 4000 26.9 / 8.0, 40 x 4000 24.9 / 10.5), and as many rows as
+    // leave eight blocks an SM
+    int log_w = 7;
+    auto blocks = [&](int l) { return (nx + (1 << l) - 1) >> l; };
+    while (log_w > 4 && 10L * (blocks(log_w) << log_w) > 11L * nx) --log_w;
+    const int step = kInitThreads >> log_w, columns = blocks(log_w);
+    const long share = (long)ny * columns / (8L * ctx->num_sms);
+    const int rows = ((int)(share < 1 ? 1 : (share > kInitRows ? kInitRows : share)) + step - 1) / step * step;
+    const PulseTime pt = pulse_at(ctx->pulse, 0.0);
     return dispatch(ctx, [&](auto* sp, auto* cp) {
         using S = std::remove_pointer_t<decltype(sp)>;
         using C = std::remove_pointer_t<decltype(cp)>;
-        init_eq_kernel<S, C><<<dim3(columns, (ctx->p.ny + rows - 1) / rows), 128, 0, ctx->stream>>>(
-            (S*)ctx->pop[ctx->cur], (const C*)ctx->uv, phi0, ctx->lp, ctx->lf, ctx->p.x0, ctx->p.y0, ctx->p.dx, pt,
-            (C)ctx->p.phi_ref, rows);
+        S* P = (S*)ctx->pop[ctx->cur];
+        const C* uv = (const C*)ctx->uv;
+        const C phi_ref = (C)ctx->p.phi_ref;
+        if (phi0)
+            init_eq_kernel<S, C><<<grid_for(ctx, (size_t)nx * ny), kThreads, 0, ctx->stream>>>(P, uv, phi0, ctx->lp, ctx->lf, phi_ref);
+        else
+            init_pulse_kernel<S, C><<<dim3(columns, (ny + rows - 1) / rows), kInitThreads, 0, ctx->stream>>>(
+                P, uv, ctx->lp, ctx->lf, ctx->p.x0, ctx->p.y0, ctx->p.dx, pt, phi_ref, log_w, rows);
     });
 }
 
