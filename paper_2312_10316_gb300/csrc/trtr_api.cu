@@ -332,6 +332,10 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
 
     const size_t pop_bytes = trtr::kQ * lp.plane * es;
     const size_t fld_bytes = lf.plane * ctx->csize;
+    // the pulse tables stand behind tab_y (an allocation and its release are some 100 us for a few MB)
+    const size_t axis_bytes = (4 * (size_t)p->ny * ctx->csize + 255) / 256 * 256;
+    const size_t ptab_bytes =
+        p->src_mode == TRTR_SRC_PULSE ? trtr::PulseTab::make(p->nx, p->ny).values(trtr::kPulseLevels) * ctx->csize : 0;
     struct {
         void** ptr;
         size_t bytes;
@@ -339,22 +343,16 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
     } allocs[] = {
         {&ctx->pop[0], pop_bytes, true},
         {&ctx->pop[1], pop_bytes, true},
-        {&ctx->uv, 2 * fld_bytes, true},
+        {&ctx->uv, (p->precision == TRTR_F64 ? 6 : 2) * fld_bytes, true},  // (FP64: the packed planes behind u)
         {&ctx->Dh, fld_bytes, true},
         {&ctx->S, p->src_mode == TRTR_SRC_FIELD ? 2 * fld_bytes : 0, true},
         {&ctx->tab_x, 4 * (size_t)p->nx * ctx->csize, true},
-        {&ctx->tab_y, 4 * (size_t)p->ny * ctx->csize, true},
-        {&ctx->ptab,
-         p->src_mode == TRTR_SRC_PULSE
-             ? trtr::PulseTab::make(p->nx, p->ny).values(trtr::kPulseLevels) * ctx->csize
-             : 0,
-         true},
+        {&ctx->tab_y, axis_bytes + ptab_bytes, true},
         {(void**)&ctx->scratch, 2 * (size_t)ctx->red_blocks * sizeof(double), false},
         {(void**)&ctx->red_done, sizeof(unsigned), true},
         {(void**)&ctx->dflag, 4 * sizeof(int), true},  // the timeout flag, then the tile counters
         {(void**)&ctx->phib,
          p->bc_mode == TRTR_BC_DIRICHLET_NEE ? (size_t)trtr::edge_count(p->nx, p->ny) * sizeof(double) : 0, true},
-        {&ctx->pack64, p->precision == TRTR_F64 ? 4 * fld_bytes : 0, true},
         {&ctx->fld2, two_step ? (p->src_mode == TRTR_SRC_FIELD ? 6 : 5) * ctx->lt.plane * sizeof(float) : 0, true},
     };
     // fault injection for tests: TRTR_FAULT_ALLOC=k makes the k-th device allocation here fail
@@ -375,6 +373,8 @@ trtr_status trtr_create(const trtr_params* p, void* cuda_stream, trtr_ctx** out)
             return TRTR_ECUDA;
         }
     }
+    if (p->precision == TRTR_F64) ctx->pack64 = static_cast<char*>(ctx->uv) + 2 * fld_bytes;
+    if (ptab_bytes) ctx->ptab = static_cast<char*>(ctx->tab_y) + axis_bytes;
     if (cudaMallocHost((void**)&ctx->hres, 4 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         trtr_destroy(ctx);
@@ -395,7 +395,7 @@ trtr_status trtr_destroy(trtr_ctx* ctx) {
     cudaGetLastError();
     trtr::free_adjoint(ctx);
     void* ptrs[] = {ctx->pop[0], ctx->pop[1],  ctx->uv,   ctx->Dh,    ctx->S,    ctx->tab_x,
-                    ctx->tab_y,  ctx->scratch, ctx->red_done, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab, ctx->pack64};
+                    ctx->tab_y,  ctx->scratch, ctx->red_done, ctx->dflag, ctx->dtmp, ctx->phib, ctx->fld2, ctx->ptab_own};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (ctx->hres) cudaFreeHost(ctx->hres);

@@ -759,10 +759,11 @@ trtr_status setup_fills(trtr_batch* b) {
         trtr_ctx* c = b->ctx[k];
         if (!c->ptab) {
             const size_t bytes = PulseTab::make(c->p.nx, c->p.ny).values(kPulseLevels) * sizeof(float);
-            if (cudaMalloc(&c->ptab, bytes) != cudaSuccess || cudaMemsetAsync(c->ptab, 0, bytes, b->stream) != cudaSuccess) {
+            if (cudaMalloc(&c->ptab_own, bytes) != cudaSuccess || cudaMemsetAsync(c->ptab_own, 0, bytes, b->stream) != cudaSuccess) {
                 cudaGetLastError();
                 return TRTR_ENOMEM;
             }
+            c->ptab = c->ptab_own;
         }
         h[k] = InstanceFill{pulse_fill_of(c), c->pulse, c->p.dt};
         b->pulses.push_back(c->pulse);

@@ -301,7 +301,7 @@ struct BatchClock {
 // The four-step kernel over a batch: its descriptors and work-list (device), and the work-list's length
 // (rows of its busiest CTA, ramps included, and rows of an iteration).
 struct SweepBatch {
-    void *d_desc = nullptr, *d_units = nullptr, *d_first = nullptr;
+    void *d_desc = nullptr, *d_units = nullptr, *d_first = nullptr;  // (one allocation)
     int ctas = 0, iteration_rows = 1;
     long rows = 0;
 };
@@ -337,7 +337,8 @@ struct trtr_ctx {
     int S_prev;       // buffer holding S^{n-1} (-1: use S^n)
     void* tab_x;      // [4][nx] sin and cos of pi x in the compute type; FP32: x as the sum of two floats
     void* tab_y;
-    void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE)
+    void* ptab;       // [kPulseLevels] pulse tables (TRTR_SRC_PULSE), behind tab_y ...
+    void* ptab_own;   // ... or in an allocation of their own (an instance without a source beside ones with it)
     // what they hold, whoever filled them last (the context or its batch), if ptab_ready
     trtr::Pulse ptab_pulse;
     long ptab_first;  // time level of the first entry

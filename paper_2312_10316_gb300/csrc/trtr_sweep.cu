@@ -688,11 +688,17 @@ __global__ void batch_ghost_columns_kernel(const SweepDesc* desc, int parity) {
     refresh_ghost_columns(static_cast<E*>(d.pop[parity]), d.a[0].lp);
 }
 
-// The work-list: strips cut into segments, the units dealt longest first to the CTA with the least work
-// so far.  Returns the rows (ramps included) of the busiest CTA.
+// The work-list: strips cut into segments of at most most_rows rows, the units dealt longest first to the CTA with
+// the least work so far.  Returns the rows (ramps included) of the busiest CTA; with lists, also the units
+// in the CTAs' order.
+struct Unit {
+    int rows, cta;
+    int4 at;
+};
 template <class G>
-long deal_units(trtr_ctx* const* ctx, int count, int ctas, long most_rows, std::vector<int4>& units, std::vector<int>& first) {
-    std::vector<std::pair<long, int4>> all;
+long deal_units(trtr_ctx* const* ctx, int count, int ctas, long most_rows, std::vector<Unit>& all, std::vector<int4>* units,
+                std::vector<int>* first) {
+    all.clear();
     for (int k = 0; k < count; ++k) {
         const int nx = ctx[k]->p.nx, ny = ctx[k]->p.ny;
         const int segs = (int)((ny + most_rows - 1) / most_rows);
@@ -700,28 +706,30 @@ long deal_units(trtr_ctx* const* ctx, int count, int ctas, long most_rows, std::
         for (int j0 = 0; j0 < ny; j0 += rows)
             for (int i0 = 0; i0 < nx; i0 += kX) {
                 const int j1 = std::min(j0 + rows, ny);
-                all.push_back({j1 - j0 + G::C + 4, make_int4(k, i0, j0, j1)});
+                all.push_back(Unit{j1 - j0 + G::C + 4, 0, make_int4(k, i0, j0, j1)});
             }
     }
-    std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    std::stable_sort(all.begin(), all.end(), [](const Unit& a, const Unit& b) { return a.rows > b.rows; });
     using Load = std::pair<long, int>;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
-    std::vector<std::vector<int4>> mine(ctas);
-    for (int c = 0; c < ctas; ++c) load.push({0, c});
+    std::vector<Load> heap(ctas);
+    for (int c = 0; c < ctas; ++c) heap[c] = {0, c};
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load(std::greater<Load>(), std::move(heap));
     long busiest = 0;
-    for (const auto& u : all) {
+    for (Unit& u : all) {
         Load l = load.top();
         load.pop();
-        mine[l.second].push_back(u.second);
-        l.first += u.first;
+        u.cta = l.second;
+        l.first += u.rows;
         busiest = std::max(busiest, l.first);
         load.push(l);
     }
-    units.clear();
-    first.assign(1, 0);
-    for (const auto& m : mine) {
-        units.insert(units.end(), m.begin(), m.end());
-        first.push_back((int)units.size());
+    if (units) {
+        first->assign(ctas + 1, 0);
+        for (const Unit& u : all) ++(*first)[u.cta + 1];
+        for (int c = 0; c < ctas; ++c) (*first)[c + 1] += (*first)[c];
+        std::vector<int> next(first->begin(), first->end() - 1);
+        units->resize(all.size());
+        for (const Unit& u : all) (*units)[next[u.cta]++] = u.at;
     }
     return busiest;
 }
@@ -733,18 +741,21 @@ cudaError_t setup_batch_typed(trtr_ctx* const* ctx, int count, cudaStream_t stre
     const int ctas = ctx[0]->num_sms;
     long total = 0;
     for (int k = 0; k < count; ++k) total += (long)((ctx[k]->p.nx + kX - 1) / kX) * ctx[k]->p.ny;
-    std::vector<int4> units, best_units;
-    std::vector<int> first, best_first;
-    long best = -1;
+    std::vector<Unit> scratch;
+    std::vector<int4> best_units;
+    std::vector<int> best_first;
+    long best = -1, best_rows = 0, last_rows = 0;
     for (int parts = 1; parts <= 6; ++parts) {
         const long rows = std::max((long)G::R * 2, total / ((long)ctas * parts) + 1);
-        const long busiest = deal_units<G>(ctx, count, ctas, rows, units, first);
+        if (rows == last_rows) continue;
+        last_rows = rows;
+        const long busiest = deal_units<G>(ctx, count, ctas, rows, scratch, nullptr, nullptr);
         if (best < 0 || busiest < best) {
             best = busiest;
-            best_units = units;
-            best_first = first;
+            best_rows = rows;
         }
     }
+    deal_units<G>(ctx, count, ctas, best_rows, scratch, &best_units, &best_first);
     out->rows = best;
     out->iteration_rows = G::R;
     std::vector<SweepDesc> h(count);
@@ -759,16 +770,18 @@ cudaError_t setup_batch_typed(trtr_ctx* const* ctx, int count, cudaStream_t stre
         }
     }
     out->ctas = ctas;
-    cudaError_t e = cudaMalloc(&out->d_desc, sizeof(SweepDesc) * count);
-    if (e == cudaSuccess) e = cudaMalloc(&out->d_units, sizeof(int4) * best_units.size());
-    if (e == cudaSuccess) e = cudaMalloc(&out->d_first, sizeof(int) * best_first.size());
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out->d_desc, h.data(), sizeof(SweepDesc) * count, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out->d_units, best_units.data(), sizeof(int4) * best_units.size(), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out->d_first, best_first.data(), sizeof(int) * best_first.size(), cudaMemcpyHostToDevice, stream);
-    const cudaError_t s = cudaStreamSynchronize(stream);  // the vectors go out of scope
+    const size_t desc_bytes = sizeof(SweepDesc) * count, unit_bytes = sizeof(int4) * best_units.size();
+    const size_t first_bytes = sizeof(int) * best_first.size();
+    std::vector<char> all(desc_bytes + unit_bytes + first_bytes);
+    memcpy(all.data(), h.data(), desc_bytes);
+    memcpy(all.data() + desc_bytes, best_units.data(), unit_bytes);
+    memcpy(all.data() + desc_bytes + unit_bytes, best_first.data(), first_bytes);
+    cudaError_t e = cudaMalloc(&out->d_desc, all.size());
+    if (e != cudaSuccess) return e;
+    out->d_units = static_cast<char*>(out->d_desc) + desc_bytes;
+    out->d_first = static_cast<char*>(out->d_units) + unit_bytes;
+    e = cudaMemcpyAsync(out->d_desc, all.data(), all.size(), cudaMemcpyHostToDevice, stream);
+    const cudaError_t s = cudaStreamSynchronize(stream);  // the vector goes out of scope
     return e != cudaSuccess ? e : s;
 }
 
@@ -889,8 +902,7 @@ cudaError_t sweep_batch_setup(trtr_ctx* const* ctx, int count, cudaStream_t stre
 }
 
 void sweep_batch_free(SweepBatch* b) {
-    for (void* p : {b->d_desc, b->d_units, b->d_first})
-        if (p) cudaFree(p);
+    if (b->d_desc) cudaFree(b->d_desc);
     *b = SweepBatch();
 }
 
