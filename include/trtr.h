@@ -193,6 +193,10 @@ trtr_status trtr_set_steps_per_launch(trtr_ctx* ctx, int k);
  * disabled), else 1. */
 trtr_status trtr_get_steps_per_launch(const trtr_ctx* ctx, int* k);
 
+/* The steps that the first launch of trtr_step(ctx, n), n >= 1, would advance from the context's state: 4, 2
+ * or 1.  TRTR_EINVAL for NULL arguments or n < 1. */
+trtr_status trtr_get_launch_steps(const trtr_ctx* ctx, long n, int* k);
+
 /* phi(x, t_n) = sum_i g_i(x, t_n) of the pre-collision populations (B_0^neq = 0, Sec. 2.2),
  * written as doubles [ny][nx].  Synchronises. */
 trtr_status trtr_moments(trtr_ctx* ctx, double* phi_out, int on_device);
@@ -326,6 +330,10 @@ trtr_status trtr_batch_set_steps_per_launch(trtr_batch* b, int k);
 /* The steps one launch of trtr_batch_step advances where it can: 2 when the two-step kernel
  * applies to the batch and is not disabled, else 1.  TRTR_EINVAL for NULL arguments. */
 trtr_status trtr_batch_get_steps_per_launch(const trtr_batch* b, int* k);
+
+/* The steps that the first launch of trtr_batch_step(b, n), n >= 1, would advance: 4, 2 or 1.  TRTR_EINVAL
+ * for NULL arguments or n < 1. */
+trtr_status trtr_batch_get_launch_steps(const trtr_batch* b, long n, int* k);
 
 /* Waits for the batch's stream; TRTR_ETIMEOUT if a step kernel gave up a bounded wait
  * (TRTR_EBOUNDS in the bounds-checked build if a kernel access out of bounds was caught). */

@@ -60,13 +60,19 @@ void end_steps(trtr_ctx* ctx) {
 // FP32, 8 steps: 22 us either way), on a large one it is lost in the first.
 constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 1L << 18;
 
-cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
+int steps_of_launch(const trtr_ctx* ctx, long most, long call, bool* small) {
     const bool two = most >= 2 && two_step_applies(ctx);
     const long nodes = (long)ctx->p.nx * ctx->p.ny;
     const bool can = !ctx->capturing && most >= 4 && call >= (nodes >= kSweepLargeNodes ? kSweepMinStepsLarge : kSweepMinSteps) &&
                      sweep_applies(ctx);
-    const bool small = can && small_applies(ctx);
-    const bool four = small || (can && (ctx->sweep_sooner || !two));
+    *small = can && small_applies(ctx);
+    return *small || (can && (ctx->sweep_sooner || !two)) ? 4 : (two ? 2 : 1);
+}
+
+cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const char** what) {
+    bool small;
+    *taken = steps_of_launch(ctx, most, call, &small);
+    const bool four = *taken == 4, two = *taken == 2;
     cudaError_t e = cudaSuccess;
     if ((two || four) && !ctx->fld2_ready) {
         *what = "field packing launch";
@@ -75,7 +81,6 @@ cudaError_t launch_steps(trtr_ctx* ctx, long most, long call, int* taken, const 
         ctx->fld2_ready = true;
     }
     *what = "pulse tables launch";
-    *taken = four ? 4 : (two ? 2 : 1);
     e = ensure_pulse_levels(ctx, ctx->step, *taken);
     if (e != cudaSuccess) return e;
     if (four) {
@@ -545,15 +550,19 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
     return TRTR_OK;
 }
 
+// The steps that the next launch of a call may take, `left` of them to go: no launch passes over a step that the
+// stability check looks at.
+static long most_steps(const trtr_ctx* ctx, long left) {
+    const long every = ctx->p.check_every, to_check = every > 0 ? every - ctx->step % every : left;
+    return to_check < left ? to_check : left;
+}
+
 static trtr_status take_steps(trtr_ctx* ctx, long n) {
     trtr_status s;
-    const long every = ctx->p.check_every;
     for (long k = 0; k < n;) {
-        // no launch passes over a step that the stability check looks at
-        const long most = every > 0 ? (every - ctx->step % every < n - k ? every - ctx->step % every : n - k) : n - k;
         const char* what = "";
         int taken = 0;
-        cudaError_t e = trtr::launch_steps(ctx, most, n, &taken, &what);
+        cudaError_t e = trtr::launch_steps(ctx, most_steps(ctx, n - k), n, &taken, &what);
         if (e != cudaSuccess) return cuda_fail(ctx, e, what);
         k += taken;
         if (ctx->p.src_mode == TRTR_SRC_FIELD) ctx->S_prev = ctx->S_cur;
@@ -821,6 +830,13 @@ trtr_status trtr_set_steps_per_launch(trtr_ctx* ctx, int k) {
 trtr_status trtr_get_steps_per_launch(const trtr_ctx* ctx, int* k) {
     if (!ctx || !k) return TRTR_EINVAL;
     *k = trtr::two_step_applies(ctx) ? 2 : 1;
+    return TRTR_OK;
+}
+
+trtr_status trtr_get_launch_steps(const trtr_ctx* ctx, long n, int* k) {
+    if (!ctx || !k || n < 1) return TRTR_EINVAL;
+    bool small;
+    *k = trtr::steps_of_launch(ctx, most_steps(ctx, n), n, &small);
     return TRTR_OK;
 }
 

@@ -603,9 +603,25 @@ trtr_status setup_two_step(trtr_batch* b) {
     return with_batch2(b, [&](auto l) { return decltype(l)::setup(b); });
 }
 
-// The sweep over the batch where it ends before two two-step launches would: its busiest CTA's rows at
-// 1.15 us for three rows (FP32; 1.87 us for four, 2-byte) against 110 (125) G nodes/s and at least 6 us a
-// two-step launch, as measured on GB300 (48 instances of 64^2 .. 1024^2: see trtr_batch_step).
+// us of a batch launch on GB300: of the sweep whose busiest CTA takes so many iterations, and of the two-step
+// kernel over so many nodes (in million).  Fitted to batches of 1 to 100 instances of 34^2 to 1025^2, most within
+// 8 % (the smallest two-step launches to 15 %).
+double batch_sweep_us(int precision, int src, double iterations) {
+    const bool pulse = src == TRTR_SRC_PULSE;
+    return precision == TRTR_F32 ? (pulse ? 6.5 + 1.12 * iterations : 4.0 + 1.07 * iterations)
+                                 : (pulse ? 6.5 + 1.62 * iterations : 6.0 + 1.50 * iterations);
+}
+double batch_two_step_us(int precision, int src, double mnodes) {
+    const bool pulse = src == TRTR_SRC_PULSE;
+    return precision == TRTR_F32 ? (pulse ? 28.0 + 20.5 * mnodes : 26.0 + 17.3 * mnodes)
+                                 : (pulse ? 30.0 + 18.5 * mnodes : 28.0 + 15.5 * mnodes);
+}
+
+// The sweep over the batch where every instance can and it ends before two two-step launches would, or where
+// these do not apply.  Measured (us for four steps, sweep / two-step launches): 30 FP32 instances of 64^2 17 / 69,
+// with the pulse source 20 / 75; 60 of 96^2 41 / 72 and 50 / 81; 30 of 256^2 93 / 142 and 102 / 166; 5 of 1024^2
+// 150 / 233 and 158 / 270; FP16 108 / 135 and 121 / 156 for 30 of 256^2.  What the estimate finds slower is a
+// batch of narrow instances, whose strips are mostly empty columns.
 trtr_status setup_four_step(trtr_batch* b) {
     b->four_step = true;
     for (int k = 0; k < b->count; ++k) {
@@ -617,10 +633,8 @@ trtr_status setup_four_step(trtr_batch* b) {
         cudaGetLastError();
         return TRTR_ENOMEM;
     }
-    const bool f32 = b->precision == TRTR_F32;
-    const double sweep = (double)b->sweep.rows / b->sweep.iteration_rows * (f32 ? 1.15 : 1.87);
-    const double two = 2.0 * std::max(6.0, 2.0 * (double)b->nodes / (f32 ? 110e3 : 125e3));
-    b->four_step = sweep < two || !b->two_step;
+    const double sweep = batch_sweep_us(b->precision, b->src, (double)b->sweep.rows / b->sweep.iteration_rows);
+    b->four_step = !b->two_step || sweep < 2.0 * batch_two_step_us(b->precision, b->src, 1e-6 * (double)b->nodes);
     return TRTR_OK;
 }
 
@@ -786,6 +800,12 @@ struct Advance {
     bool last_two = false, last_four = false;
 };
 
+// The steps of the first launch of a call of n steps.
+int steps_of_launch(const trtr_batch* b, int steps_per_launch, long n) {
+    if (steps_per_launch != 2 || n < 2) return 1;
+    return b->four_step && n >= 4 ? 4 : (b->two_step ? 2 : 1);
+}
+
 // The steps `at.left`: four at a time or pairs through the two-step kernel where these apply (steps_per_launch
 // 2), the rest (an odd step, or all with steps_per_launch 1) through the one-step kernel of the configured
 // geometry.  All kernels advance the device clock, so they interleave.  `at` follows every launch.
@@ -794,7 +814,7 @@ trtr_status advance_launches(trtr_batch* b, int steps_per_launch, Advance& at) {
     long& left = at.left;
     int& par = at.par;
     auto levels = [&](int steps) { return ensure_levels(b, end - left, steps) == cudaSuccess; };
-    const bool four = b->four_step && steps_per_launch == 2 && left >= 4;
+    const bool four = steps_of_launch(b, steps_per_launch, left) == 4;
     if (four || (b->two_step && steps_per_launch == 2 && left >= 2)) {
         for (int k = 0; k < b->count; ++k) {
             trtr_ctx* c = b->ctx[k];  // instances share the batch's stream
@@ -1022,6 +1042,12 @@ trtr_status trtr_batch_set_steps_per_launch(trtr_batch* b, int k) {
 trtr_status trtr_batch_get_steps_per_launch(const trtr_batch* b, int* k) {
     if (!b || !k) return TRTR_EINVAL;
     *k = b->two_step && b->steps_per_launch == 2 ? 2 : 1;
+    return TRTR_OK;
+}
+
+trtr_status trtr_batch_get_launch_steps(const trtr_batch* b, long n, int* k) {
+    if (!b || !k || n < 1) return TRTR_EINVAL;
+    *k = trtr::steps_of_launch(b, b->steps_per_launch, n);
     return TRTR_OK;
 }
 

@@ -109,6 +109,8 @@ _SIGNATURES = {
     "trtr_batch_set_steps_per_launch": (_st, [_vp, ctypes.c_int]),
     "trtr_batch_get_steps_per_launch": (_st, [_vp, ctypes.POINTER(ctypes.c_int)]),
     "trtr_get_steps_per_launch": (_st, [_vp, ctypes.POINTER(ctypes.c_int)]),
+    "trtr_get_launch_steps": (_st, [_vp, ctypes.c_long, ctypes.POINTER(ctypes.c_int)]),
+    "trtr_batch_get_launch_steps": (_st, [_vp, ctypes.c_long, ctypes.POINTER(ctypes.c_int)]),
 }
 
 
@@ -370,6 +372,12 @@ def trtr_get_steps_per_launch(ctx) -> int:
     return int(k.value)
 
 
+def trtr_get_launch_steps(ctx, n: int) -> int:
+    k = ctypes.c_int()
+    _check(ctx, lib.trtr_get_launch_steps(ctx, int(n), ctypes.byref(k)))
+    return k.value
+
+
 def trtr_check_bounds_path(ctx) -> int:
     """Status of the bounds-check probe (TRTR_EBOUNDS in the checked build, TRTR_OK otherwise)."""
     return int(lib.trtr_check_bounds_path(ctx))
@@ -470,6 +478,10 @@ class Solver:
     @property
     def steps_per_launch(self) -> int:
         return trtr_get_steps_per_launch(self.ctx)
+
+    def launch_steps(self, n: int) -> int:
+        """The steps that the first launch of step(n) advances."""
+        return trtr_get_launch_steps(self.ctx, n)
 
     def moments(self, out=None):
         if out is None:
@@ -591,6 +603,12 @@ def trtr_batch_get_steps_per_launch(b) -> int:
     return k.value
 
 
+def trtr_batch_get_launch_steps(b, n: int) -> int:
+    k = ctypes.c_int()
+    _bcheck(lib.trtr_batch_get_launch_steps(b, int(n), ctypes.byref(k)), "trtr_batch_get_launch_steps")
+    return k.value
+
+
 def trtr_batch_sync(b):
     _bcheck(lib.trtr_batch_sync(b), "trtr_batch_sync")
 
@@ -676,6 +694,10 @@ class Batch:
     @property
     def steps_per_launch(self) -> int:
         return trtr_batch_get_steps_per_launch(self.b)
+
+    def launch_steps(self, n: int) -> int:
+        """The steps that the first launch of step(n) advances."""
+        return trtr_batch_get_launch_steps(self.b, n)
 
     def step(self, n: int = 1):
         trtr_batch_step(self.b, n)
