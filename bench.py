@@ -278,6 +278,18 @@ def cpu_baseline(pulse, seconds: float):
 # ------------------------------------------------------------------------------ ours
 
 
+def warm_up(solver, steps):
+    """Exactly `steps` untimed steps, the last of them in calls like the timed ones; the steps of a timed
+    call, which is one launch: four where the sweep takes calls of four, two where the two-step kernel
+    applies."""
+    spl = solver.launch_steps(4)
+    if steps % spl:
+        solver.step(steps % spl)
+    for _ in range(steps // spl):
+        solver.step(spl)
+    return spl
+
+
 def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world, stream, sh, local):
     """W warm-up steps, then K steps of `workload` timed with one CUDA event per launch on the
     library's stream, clocks sampled meanwhile: (GLUPS, ms per step, roofline, launches, clocks)."""
@@ -289,17 +301,9 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
     solver = T.pulse_solver(pulse, precision=prec, stream=sh, src_mode=src_override, rounding=rnd)
     if src_override == T.TRTR_SRC_FIELD:
         solver.set_source(W.source(pulse, 0.0))  # the manufactured source as a stationary field
-    solver.step(args.warmup)
-    # one event interval per launch: four steps where trtr_step takes four at once (the sweep), two
-    # where the two-step kernel applies
     if args.steps_per_launch == "1":
         solver.set_steps_per_launch(1)
-    spl = solver.steps_per_launch
-    before = solver.launches
-    for _ in range(8):
-        solver.step(4)
-    if solver.launches - before < 12:  # (8, and now and then one that fills tables or ghost columns)
-        spl = 4
+    spl = warm_up(solver, args.warmup)
     solver.sync()
     barrier(world)
     torch.cuda.synchronize()
@@ -347,7 +351,8 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
     # fields, whatever the kernel moves), and the DRAM bytes the committed counters measured
     per_update_bpn = algorithmic_bytes_per_node(pop_bytes) + extra
     per_update = per_update_bpn * n_nodes * spl / (avg_launch_ms * 1e-3) / 1e9
-    roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
+    # (the sweep's launches are bound by latency and instruction issue, the others by HBM)
+    roofline = {"bound": "latency" if spl == 4 else "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic,
                 "frac_per_node_update": round(per_update / peak, 4),
                 "bytes_per_node_update": per_update_bpn,
@@ -589,7 +594,7 @@ def run_batch(args):
     value = nodes * args.steps * world / (ms * 1e-3) / 1e9
     step_ms = ms / args.steps
     solves_per_s = len(pulses) * world * args.steps / pulses[0].steps / (ms * 1e-3)
-    spl = batch.steps_per_launch
+    spl = batch.launch_steps(args.steps)
     batch.close()
 
     # one launch per instance per step, same instances, same stream
@@ -637,10 +642,9 @@ def run_batch(args):
 
             dist.destroy_process_group()
         return None
-    # two steps per launch, or four where the batch's sweep is the faster (the batch decides; counted as
-    # four, so bytes and launches are lower bounds): 92 B per node and launch in FP32, 56 B for 2-byte storages
-    if spl == 2:
-        bpn, kernel, spl = two_step_bytes_per_node(pop_bytes), "batch sweep_kernel or batch2_kernel", 4
+    # two or four steps per launch: 92 B per node and launch in FP32, 56 B for 2-byte storages
+    if spl > 1:
+        bpn, kernel = two_step_bytes_per_node(pop_bytes), "batch sweep_kernel" if spl == 4 else "batch2_kernel"
     else:
         bpn, kernel = algorithmic_bytes_per_node(pop_bytes), "batch_kernel"
     peak, peak_kind = measured_hbm_peak()
@@ -660,7 +664,7 @@ def run_batch(args):
                      "frac_per_node_update": round(per_update / peak, 4), "bytes_per_node_update": per_update_bpn,
                      "peak_kind": f"{peak_kind} copy bandwidth",
                      "bytes_per_node": bpn, "kernel": kernel, "steps_per_launch": spl},
-        "gpu_launches": args.steps // spl + args.steps % spl,
+        "gpu_launches": args.steps // spl + (args.steps % spl + 1) // 2 if spl > 1 else args.steps,
         "clocks": clk,
         "e2e": e2e,
         "cpu_baseline": None if args.no_cpu_baseline else cpu_baseline(
