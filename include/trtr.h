@@ -402,9 +402,13 @@ int trtr_abi_version(void);
 
 /* ---- Bounds-checked debug build ---------------------------------------------------------
  * The library built with TRTR_BOUNDS_CHECK=1 (libtrtr_checked.so) checks its kernels' memory
- * accesses against the ghosted plane layout: every plane index, the two-node stores, the bulk
+ * accesses against the ghosted plane layout: every plane index, or where a kernel goes on from one
+ * index with offsets the outermost of them; the pulse tables' entries; the rows and columns of staged
+ * tiles and of the sweep's ring of rows; the two-node stores, the bulk
  * row copies (inside the interior row, 16-byte aligned addresses and size) and the TMA load
  * coordinates (x times the element size a multiple of 16 bytes, 128-byte aligned destination).
+ * Not checked are the caller's arrays, the library's one-dimensional ones (reduction partials, edge
+ * values, work-lists) and TMA stores, which the hardware clips to the interior.
  * A bad access is recorded and skipped (or kept inside the ghost frame); nothing traps.  The
  * next call that synchronises a context's stream (or trtr_batch_sync) then returns
  * TRTR_EBOUNDS with the first access in trtr_last_error.  The default build compiles none of
@@ -415,8 +419,8 @@ int trtr_bounds_checked(void);
 
 /* Synchronises the current device, then returns the record of every kernel since the last
  * report and clears it: out[0] = accesses caught, out[1] = kind of the first (1 plane index,
- * 2 two-node store, 3 bulk row copy, 4 TMA load), out[2] = its column i | row j << 32 (for a
- * TMA load, x | y << 32).  The default build writes zeros.  TRTR_EINVAL: out is NULL;
+ * 2 two-node store, 3 bulk row copy, 4 TMA load, 5 row or column of a staged tile, 6 pulse table),
+ * out[2] = its column i | row j << 32 (for a TMA load, x | y << 32; for 5, the value | the count).  The default build writes zeros.  TRTR_EINVAL: out is NULL;
  * TRTR_ECUDA: a CUDA call failed. */
 trtr_status trtr_bounds_report(unsigned long long out[3]);
 

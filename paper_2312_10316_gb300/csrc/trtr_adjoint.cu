@@ -151,8 +151,10 @@ __global__ void __launch_bounds__(kThreads)
     const unsigned k = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = k < n;
     const int j = in ? (int)(k / per) : 0, i = in ? kN * (int)(k - (unsigned)j * per) : 0;
+    const bool ok = in_frame(a.lp, i - 1, j - 1, 1, 1) && in_frame(a.lp, i + kN, j + 1, kN, 1) &&
+                    in_frame(a.lf, i + kN - 1, j, 1, 0) && in_frame(a.lq, i + kN - 1, j, 1, 0);
     V g[kQ], ux, uy, ax, ay, w1, w2, dt2;
-    if (in) {
+    if (in && ok) {
         const size_t at = a.lp.at(i, j), o = a.lf.at(i, j), pl = a.lf.plane;
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {  // pull (the ghost cells hold the periodic images)
@@ -189,7 +191,7 @@ __global__ void __launch_bounds__(kThreads)
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!in) return;
+    if (!in || !ok) return;
     V Q[kQ], lam[kQ], d1, d2;
     const size_t aq = a.lq.at(i, j);
 #pragma unroll
@@ -210,6 +212,7 @@ __global__ void __launch_bounds__(kThreads)
         if constexpr (kF64) {
             put(i, lam[q]);
         } else if (inner) {
+            if (!in_frame(a.lq, i - lattice_ex(q), j - lattice_ey(q), 0, 0) || !in_frame(a.lq, i + 1 - lattice_ex(q), j, 0, 0)) continue;
             C* p = plane + aq - (ptrdiff_t)lattice_ey(q) * a.lq.pitch - lattice_ex(q);
             if (lattice_ex(q) == 0) {
                 *reinterpret_cast<float2*>(p) = lam[q].v;

@@ -258,8 +258,13 @@ template <typename S>
 __device__ __forceinline__ void pulled_pair(const S* P, int i, int j, const PlaneLayout& L, float phi_ref, F2 g[kQ]) {
     using S2 = typename core::Pair<S>::type;
     const S* at = P + L.at(i, j);
+    const bool ok = in_frame(L, i - 1, j - 1, kGhostP, kGhostP) && in_frame(L, i + 2, j + 1, kGhostP, kGhostP);
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {
+        if (!ok) {
+            g[q] = F2(0.f);
+            continue;
+        }
         const S* p = at + q * L.plane - (ptrdiff_t)lattice_ey(q) * L.pitch - lattice_ex(q);
         const float off = core::weight<float>(q) * phi_ref;
         g[q] = lattice_ex(q) == 0 ? core::Pair<S>::decode(*reinterpret_cast<const S2*>(p), off)

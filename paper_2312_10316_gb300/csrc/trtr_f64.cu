@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(128) f64_step_kernel(const __grid_constant__ F
     if (!in) return;
     double g[kQ], out[kQ];
     const size_t at = a.lp.at_g<kGhostP>(i, j);
+    if (!in_frame(a.lp, (int)i - 1, (int)j - 1, 1, 1) || !in_frame(a.lp, (int)i + 1, (int)j + 1, 1, 1)) return;
 #pragma unroll
     for (int q = 0; q < kQ; ++q)
         g[q] = a.src[q * a.lp.plane + at - (ptrdiff_t)lattice_ey(q) * a.lp.pitch - lattice_ex(q)];

@@ -59,10 +59,13 @@ struct PulseTime {
 
 // ---- bounds-checked builds (TRTR_BOUNDS_CHECK=1) ----------------------------------------
 // The debug build checks the kernels' memory accesses against the layout: every plane index
-// (PlaneLayout::at), the pair stores, the bulk row copies and the TMA load coordinates.  An
-// access out of bounds is recorded in this translation unit's log and then skipped, or kept
-// inside the ghost frame; it never traps, so the context stays usable and the host reports
-// TRTR_EBOUNDS at the next synchronisation.  The default build compiles none of it.
+// (PlaneLayout::at), where a kernel goes on from one index with offsets the outermost of them (in_frame), the
+// pulse tables' entries (in_tables), the rows and columns of staged tiles and of the sweep's ring (in_tile), the
+// pair stores, the bulk row copies and the TMA load coordinates.  An access out of bounds is recorded in this
+// translation unit's log and then skipped, or kept inside the ghost frame; it never traps, so the context
+// stays usable and the host reports TRTR_EBOUNDS at the next synchronisation.  The default build compiles
+// none of it.  Not checked: the caller's [ny][nx] arrays and the library's own one-dimensional ones
+// (reduction partials, edge values, work-lists), and TMA stores, which the hardware clips to the interior.
 #ifndef TRTR_BOUNDS_CHECK
 #define TRTR_BOUNDS_CHECK 0
 #endif
@@ -72,7 +75,8 @@ enum BoundsKind {
     kBoundsPair = 2,   // a two-node store past the row or not aligned to the pair
     kBoundsBulk = 3,   // a bulk row copy outside the interior row, or not 16-byte aligned
     kBoundsTma = 4,    // a TMA load whose x coordinate or destination breaks the alignment rules
-    kBoundsTile = 5,   // a tile column or row outside the tile
+    kBoundsTile = 5,   // a column or row outside a staged tile or the sweep's ring (value, count)
+    kBoundsTable = 6,  // an entry outside the pulse tables
 };
 
 #if TRTR_BOUNDS_CHECK
@@ -152,7 +156,30 @@ struct PlaneLayout {
 #endif
         return (size_t)(j + g) * (size_t)pitch + (size_t)(i + gx);
     }
+    // node (i, j) is in the interior or within wx columns and wy rows of it, and in the allocation
+    __host__ __device__ bool covers(int i, int j, int wx, int wy) const {
+        return i >= -wx && i < nx + wx && j >= -wy && j < ny + wy && i + gx >= 0 && i + gx < pitch && j + gy >= 0 && j + gy < rows;
+    }
 };
+// Checked builds: false, and recorded, where an access is out of bounds, which the caller then skips.
+__device__ __forceinline__ bool in_frame(const PlaneLayout& L, int i, int j, int wx, int wy) {
+#if TRTR_BOUNDS_CHECK
+    if (!L.covers(i, j, wx, wy)) {
+        TRTR_BOUNDS_FAULT(kBoundsPlane, i, j);
+        return false;
+    }
+#endif
+    return true;
+}
+__device__ __forceinline__ bool in_tile(int v, int count) {
+#if TRTR_BOUNDS_CHECK
+    if (v < 0 || v >= count) {
+        TRTR_BOUNDS_FAULT(kBoundsTile, v, count);
+        return false;
+    }
+#endif
+    return true;
+}
 
 PlaneLayout make_layout(int nx, int ny, int elem_bytes, int ghost);
 
@@ -214,7 +241,20 @@ struct PulseTab {
         return t;
     }
     size_t values(int levels) const { return (size_t)level * levels; }
+    // the entries of the columns [i, i + w) and of row j are in a level
+    __host__ __device__ bool covers(int i, int w, int j) const {
+        return i >= -kTabGhost && i + w <= p2 - kTabGhost && j >= -kTabGhost && j < (level - 2 * p2) / 2 - kTabGhost;
+    }
 };
+__device__ __forceinline__ bool in_tables(const PulseTab& t, int i, int w, int j) {
+#if TRTR_BOUNDS_CHECK
+    if (!t.covers(i, w, j)) {
+        TRTR_BOUNDS_FAULT(kBoundsTable, i, j);
+        return false;
+    }
+#endif
+    return true;
+}
 
 // Tile schedule bits of a step launch.  kSchedDynamic: the CTAs take their tiles from tile_ctr
 // (long launches; kDynMinTilesPerCta).  kSchedReverse: the launch walks the tile order from the

@@ -46,6 +46,9 @@ __device__ __forceinline__ void small_step(S* tile, int r, int c, const F2 f[5],
     if (r < LV || r >= kH - LV || c + 1 < LV || c >= kW - LV) return;
     auto slot = [&](int q) { return tile + (q * kH + r - LV * lattice_ey(q)) * kW + c - LV * lattice_ex(q); };
     auto even = [](int q) { return LV % 2 == 0 || lattice_ex(q) == 0; };
+    if (!in_tile(r - LV, kH) || !in_tile(r + LV, kH)) return;
+    // (a pair at the rim of a step's nodes reaches a column into the row beside it; one node of it is not used)
+    if (!in_tile(r * kW + c - LV + 1, kH * kW) || !in_tile(r * kW + c + LV, kH * kW)) return;
     F2 g[kQ], out[kQ];
 #pragma unroll
     for (int q = 0; q < kQ; ++q) {

@@ -240,6 +240,7 @@ __device__ __forceinline__ F2 vdiv(F2 a, F2 b) { return F2(__fdividef(a.v.x, b.v
 // j, from the tables of the levels n - 1 and n (`lev`: level n - 1).
 __device__ __forceinline__ F2 pulse_level_dt(F2 p1, F2 p2, float2 q) { return vfma(p1, F2(q.x), p2 * F2(q.y)); }
 __device__ __forceinline__ F2 pulse_source_dt(const float* lev, const PulseTab& t, int i, int j) {
+    if (!in_tables(t, i, 2, j)) return F2(0.f);
     auto level = [&](const float* p) {
         const float2 q = __ldg(reinterpret_cast<const float2*>(p + t.y + 2 * j));
         const F2 p1(__ldg(reinterpret_cast<const float2*>(p + i))), p2(__ldg(reinterpret_cast<const float2*>(p + t.p2 + i)));
@@ -248,6 +249,7 @@ __device__ __forceinline__ F2 pulse_source_dt(const float* lev, const PulseTab& 
     return vfma(F2(1.5f), level(lev + t.level), F2(-0.5f) * level(lev));
 }
 __device__ __forceinline__ double pulse_source_dt(const double* lev, const PulseTab& t, int i, int j) {
+    if (!in_tables(t, i, 1, j)) return 0.0;
     auto level = [&](const double* p) {
         const double2 q = __ldg(reinterpret_cast<const double2*>(p + t.y + 2 * j));
         return fma(__ldg(p + i), q.x, __ldg(p + t.p2 + i) * q.y);
@@ -275,6 +277,7 @@ struct TileTables {
     }
     // the source term of the pair at column i0 + c, row j0 + r from the levels l and l + 1, as pulse_source_dt
     static __device__ __forceinline__ F2 source(const unsigned char* at, int l, int c, int r) {
+        if (!in_tile(l, LEVELS - 1) || !in_tile(c, BX - 1) || !in_tile(r, BY)) return F2(0.f);
         auto level = [&](int k) {
             const float* x = reinterpret_cast<const float*>(at) + 2 * BX * k + c;
             const float* y = reinterpret_cast<const float*>(at + YOff) + 2 * BY * k + 2 * r;
@@ -358,6 +361,7 @@ __device__ __forceinline__ void fill_pulse_entry(const PulseFill& f, const Pulse
                                  along_x ? l.cx : l.cy, l);
     C* out = static_cast<C*>(f.tab) + kTabGhost + (size_t)lev * t.level;
     ready();
+    if (!in_tables(t, along_x ? at : 0, 1, along_x ? 0 : at)) return;
     if (along_x) {
         out[at] = v.y;
         out[t.p2 + at] = v.x;

@@ -125,6 +125,7 @@ template <typename T>
 __device__ __forceinline__ void store_row_ghosts(T* plane, const PlaneLayout& L, int i, int j, T v) {
     const int xs = i < kGhostX ? L.nx : (i >= L.nx - kGhostX ? -L.nx : 0);
     const int ys = j < kGhostP ? L.ny : -L.ny;
+    if (!in_frame(L, i, j + ys, 0, kGhostP) || !in_frame(L, i + xs, j + ys, kGhostX, kGhostP)) return;
     T* row = plane + (ptrdiff_t)(j + kGhostP + ys) * L.pitch + L.gx;
     row[i] = v;
     if (xs) row[i + xs] = v;
@@ -199,6 +200,7 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
 #pragma unroll
         for (int h = 0; h < G::P; ++h) {
             if (part + h == 0 ? lane < kT / 2 : lane >= 32 - kT / 2) continue;  // outside the output columns
+            if (!in_tile(2 * lane + 64 * (part + h) - kT, kX - 1)) continue;
             const int ih = i + 64 * h;
             S2 v[kQ];
 #pragma unroll
@@ -218,10 +220,10 @@ __device__ __forceinline__ void sweep_row(S* pm, S* p0, S* pp, const float* f, c
                 for (int q = 0; q < kQ; ++q) {
                     S* r = row + q * a.lp.plane;
                     const S v0 = reinterpret_cast<const S*>(&v[q])[0], v1 = reinterpret_cast<const S*>(&v[q])[1];
-                    if (g0) r[to] = v0;
-                    if (g1) r[to + 1] = v1;
-                    if (t0) r[0] = v0;
-                    if (t1) r[1] = v1;
+                    if (g0 && in_frame(a.lp, ih + to, j, kGhostX, 0)) r[to] = v0;
+                    if (g1 && in_frame(a.lp, ih + to + 1, j, kGhostX, 0)) r[to + 1] = v1;
+                    if (t0 && in_frame(a.lp, ih, j, 0, 0)) r[0] = v0;
+                    if (t1 && in_frame(a.lp, ih + 1, j, 0, 0)) r[1] = v1;
                 }
             }
             if (j < kGhostP || j >= a.lp.ny - kGhostP) {
@@ -353,7 +355,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 y = y < 0 ? y + a.lp.ny : (y >= a.lp.ny ? y - a.lp.ny : y);
                 unsigned char* pd = smem + (b * R + r) * G::PopPitch;
                 const int xp = t.i0 - 2 * kT + a.lp.gx;
-                if (tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, mp, &full[b], xp, y + kGhostP, 0);
+                if (in_tile((int)(b * R) + r, G::Ring) && in_tile(y, a.lp.ny) && tma_ok(pd, xp, y, G::ES)) tma_load_3d(pd, mp, &full[b], xp, y + kGhostP, 0);
             }
         };
         auto load_fields = [&](const Unit& t, const SweepArgs& a, const CUtensorMap* mf, int m) {
@@ -466,10 +468,11 @@ __global__ void __launch_bounds__(G::Threads, 1)
 #pragma unroll
         for (int h = 0; h < G::P; ++h) {
             if (SRC == TRTR_SRC_PULSE) {
-                p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + i + 64 * h)));
-                p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.p2 + i + 64 * h)));
-                p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + i + 64 * h)));
-                p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + a.pt.p2 + i + 64 * h)));
+                const float* p = lev + (in_tables(a.pt, i + 64 * h, 2, 0) ? i + 64 * h : 0);
+                p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(p)));
+                p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.p2)));
+                p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.level)));
+                p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.level + a.pt.p2)));
             }
             auto wrap = [&](int v) { return v < 0 ? v + nx : (v >= nx ? v - nx : v); };
             const int xa = wrap(i + 64 * h), xb = wrap(i + 64 * h + 1);
@@ -493,6 +496,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
         float2 qp = make_float2(0.f, 0.f), qn = qp;
         auto load_factors = [&](int y) {
             y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+            if (!in_tables(a.pt, 0, 1, y)) return;
             qp = __ldg(reinterpret_cast<const float2*>(ty + 2 * y));
             qn = __ldg(reinterpret_cast<const float2*>(ty + a.pt.level + 2 * y));
         };
@@ -528,6 +532,10 @@ __global__ void __launch_bounds__(G::Threads, 1)
             if (j >= t.j0 - (kT - level) && j < t.j1 + (kT - level)) {
                 const int below = ring >= level ? ring - level : ring - level + G::Ring;
                 const int above = ring + level < G::Ring ? ring + level : ring + level - G::Ring;
+                const int col = 2 * lane + 64 * part;  // its pairs, and the columns that they reach in the ring
+                const bool inside = in_tile(below, G::Ring) && in_tile(ring, G::Ring) && in_tile(above, G::Ring) &&
+                                    in_tile(col + kT - level, kW) && in_tile(col + kT + 64 * (G::P - 1) + 1 + level, kW) &&
+                                    in_tile(col + 64 * (G::P - 1) + 1, kWC);
                 constexpr int kPitch = G::PopPitch / G::ES;
                 S* base = reinterpret_cast<S*>(smem) + 2 * lane + 64 * part + kT;
                 S* pm = base + below * kPitch;
@@ -545,7 +553,7 @@ __global__ void __launch_bounds__(G::Threads, 1)
                 }
                 S* buf = reinterpret_cast<S*>(smem + G::OutOff + o * G::OutBytes) + r0 * kX + 2 * lane + 64 * part - kT;
                 auto buffer_free = [&]() { return it < (unsigned)G::Outs || wait(&freed[o], (it / G::Outs - 1) & 1); };
-                switch (level) {
+                if (inside) switch (level) {
                     case 1: sweep_row<S, 1, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
                     case 2: sweep_row<S, 2, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
                     case 3: sweep_row<S, 3, SRC, RND, G>(pm, p0, pp, f, src, a, rk, buf, lane, part, i, j, buffer_free); break;
@@ -569,7 +577,8 @@ __device__ __forceinline__ void refresh_ghost_columns(E* P, const PlaneLayout& L
         const int g = k % (2 * kGhostX), row = k / (2 * kGhostX), q = row / L.ny, j = row - q * L.ny;
         E* p = P + (size_t)q * L.plane + (size_t)(j + kGhostP) * L.pitch + L.gx;
         const int to = g < kGhostX ? g - kGhostX : L.nx + g - kGhostX;
-        p[to] = p[g < kGhostX ? L.nx + to : to - L.nx];
+        const int from = g < kGhostX ? L.nx + to : to - L.nx;
+        if (in_frame(L, to, j, kGhostX, 0) && in_frame(L, from, j, 0, 0)) p[to] = p[from];
     }
 }
 template <typename E>
