@@ -429,9 +429,10 @@ __global__ void __launch_bounds__(G::Threads, 1)
             phase += blocks;
             it0 += t.iters;
         }
-        if (*abort_flag) ok = false;  // (the last level's last buffer)
         if (lane == 0) {
-            if (!ok) {  // let the loads issued into this CTA's shared memory land (bounded)
+            // a wait gave up (the flag alone: the last level's for its last buffer): let the loads issued into
+            // this CTA's shared memory land (bounded)
+            if (!ok || *abort_flag) {
                 if constexpr (BATCH)
                     atomicExch(p.flag, 1);
                 else
@@ -467,12 +468,11 @@ __global__ void __launch_bounds__(G::Threads, 1)
         const float* lev = a.pulse + (size_t)(table_level + level - 1) * a.pt.level;
 #pragma unroll
         for (int h = 0; h < G::P; ++h) {
-            if (SRC == TRTR_SRC_PULSE) {
-                const float* p = lev + (in_tables(a.pt, i + 64 * h, 2, 0) ? i + 64 * h : 0);
-                p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(p)));
-                p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.p2)));
-                p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.level)));
-                p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(p + a.pt.level + a.pt.p2)));
+            if (SRC == TRTR_SRC_PULSE && in_tables(a.pt, i + 64 * h, 2, 0)) {
+                p1p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + i + 64 * h)));
+                p2p[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.p2 + i + 64 * h)));
+                p1n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + i + 64 * h)));
+                p2n[h] = F2(__ldg(reinterpret_cast<const float2*>(lev + a.pt.level + a.pt.p2 + i + 64 * h)));
             }
             auto wrap = [&](int v) { return v < 0 ? v + nx : (v >= nx ? v - nx : v); };
             const int xa = wrap(i + 64 * h), xb = wrap(i + 64 * h + 1);
