@@ -57,7 +57,8 @@ void end_steps(trtr_ctx* ctx) {
 
 // Four steps a launch (trtr_sweep.cu) where the call takes enough of them: the launch that brings the
 // ghost columns up to date costs what two sweeps of a small grid save over two-step launches (200^2
-// FP32, 8 steps: 22 us either way), on a large one it is lost in the first.
+// FP32, 8 steps: 22 us either way), on a large one it is lost in the first.  The small-grid kernel
+// (trtr_small.cu) reads no ghost columns and keeps to the same line.
 constexpr long kSweepMinSteps = 12, kSweepMinStepsLarge = 4, kSweepLargeNodes = 1L << 18;
 
 int steps_of_launch(const trtr_ctx* ctx, long most, long call, bool* small) {

@@ -301,11 +301,14 @@ __host__ __device__ __forceinline__ uint32_t sr_step_key(long step) {
     return sr_hash((uint32_t)step * 0x9E3779B9U + (uint32_t)((unsigned long long)step >> 32) + 0x632BE5ABU);
 }
 
-// Programmatic dependent launch of the step kernels: only for launches of a few tiles per CTA,
+// Programmatic dependent launch of the one- and two-step kernels: only for launches of a few tiles per CTA,
 // where the launch latency it hides is a large part of the step.  On long launches it costs time
 // (measured on GB300 without events between the launches: the two-step kernel at 4096^2 0.360
 // against 0.346 ms, at 8192^2 1.97 against 1.41 ms; the one-step FP16 kernel at 8192^2 0.634
-// against 0.612 ms), and a launch that records an event after it does not overlap anyway.
+// against 0.612 ms), and a launch that records an event after it does not overlap anyway.  The sweep, whose
+// CTAs have a share of rows each, takes it on every launch (us a step without / with: FP32 512^2 3.75 / 3.00,
+// 1024^2 8.28 / 7.67, 4096^2 90.6 / 89.8, 8192^2 338.5 / 337.6; FP16 pulse 8192^2 408.3 / 409.0), and so do the
+// small-grid and FP64 kernels.
 constexpr long kPdlMaxTilesPerCta = 8;
 // Tiles handed out from a counter: only for launches of more than this many tiles per CTA.  On
 // short launches the CTAs' few sequential atomic round trips cost more than the balancing gains
