@@ -42,7 +42,8 @@ static void forget_prepared(trtr_ctx* ctx, bool fields) {
 }
 void begin_steps(trtr_ctx* ctx) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &status) != cudaSuccess) {
+    const bool legacy = ctx->stream == nullptr || ctx->stream == cudaStreamLegacy;  // (cannot be captured)
+    if (!legacy && cudaStreamIsCapturing(ctx->stream, &status) != cudaSuccess) {
         cudaGetLastError();
         status = cudaStreamCaptureStatusNone;
     }
