@@ -176,8 +176,8 @@ trtr_status trtr_init_equilibrium(trtr_ctx* ctx, const double* phi0, int on_devi
  * run as one launch of the two-step kernel (the same arithmetic and roundings, the same results
  * bit for bit; populations read and written once per two steps; see
  * trtr_set_steps_per_launch).  A call of 12 steps or more (4 on 2^18 nodes or more) takes four
- * steps a launch, with odd nx and a source field that stays the same from step to step too, again
- * with the same bits.  An odd last step, or a pair whose middle step is a check_every
+ * steps a launch where that ends sooner (not on grids of a few columns or rows), with odd nx and a
+ * source field that stays the same from step to step too, again with the same bits.  An odd last step, or a pair whose middle step is a check_every
  * point, runs one step per launch.  Short launches use programmatic dependent launch: each
  * waits for the work before it on the stream before reading its results.  A call captured into a CUDA
  * graph takes one and two steps a launch and prepares what they read in the graph: a replay goes on from
