@@ -303,15 +303,16 @@ def timed_steps(args, pulse, prec, pop_bytes, workload, rnd, src_override, world
         solver.set_source(W.source(pulse, 0.0))  # the manufactured source as a stationary field
     if args.steps_per_launch == "1":
         solver.set_steps_per_launch(1)
-    spl = warm_up(solver, args.warmup)
-    solver.sync()
-    barrier(world)
     torch.cuda.synchronize()
     props = torch.cuda.get_device_properties(local)
     uuid = str(getattr(props, "uuid", "")) or None
     clocks = ClockSampler(("GPU-" + uuid) if uuid and not uuid.startswith("GPU-") else uuid)
     clocks.start()
     time.sleep(0.4)  # let the sampler take a reading at the start of the region
+    spl = warm_up(solver, args.warmup)  # directly before the timed steps: the GPU is not idle in between
+    solver.sync()
+    barrier(world)
+    torch.cuda.synchronize()
     n_launch, tail = divmod(args.steps, spl)
     ev = [torch.cuda.Event(enable_timing=True) for _ in range(n_launch + 1 + (1 if tail else 0))]
     launches0 = solver.launches
