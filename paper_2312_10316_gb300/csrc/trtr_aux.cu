@@ -385,6 +385,8 @@ __device__ __forceinline__ void reduce_nodes(const S* P, const PlaneLayout& L, C
     } else if constexpr (sizeof(S) == 8) {
         const unsigned n = (unsigned)L.nx * L.ny;
         unsigned bad = 0;
+        // four nodes' loads in flight (GB300, FP64 4096^2, us: the mass 370, now 352; against a field 418, now 410)
+#pragma unroll 4
         for (unsigned k = first; k < n; k += stride) {
             const int j = (int)(k / L.nx), i = (int)(k - (unsigned)j * L.nx);
             if constexpr (KIND == kReduceNonFinite) {
